@@ -225,6 +225,91 @@ def run(state):
     return state[1].out
 
 
+# --- the same outputs in 64 bits, in plain torch ------------------------------------------------------------------------
+def _rms(x, gain, eps):
+    return x * torch.rsqrt(x.square().mean(-1, keepdim=True) + eps) * gain
+
+
+def _rope(v, pos, base):                                   # [tokens, heads, Dh], rotate-half pairs (i, i + Dh / 2)
+    half = v.shape[-1] // 2
+    theta = torch.pow(base, -torch.arange(half, dtype=torch.float64, device=v.device) / half)
+    ang = pos.double()[:, None, None] * theta
+    a, b, cos, sin = v[..., :half], v[..., half:], ang.cos(), ang.sin()
+    return torch.cat((a * cos - b * sin, b * cos + a * sin), -1)
+
+
+def _pages(batch):
+    """Every sequence's pages: handed out in order, the contexts' first, then the ones the new tokens grow into."""
+    nxt, tables = 0, [[] for _ in batch.q_len]
+    for lens in (batch.ctx_len, batch.total_len()):
+        for s, t in enumerate(lens):
+            while len(tables[s]) * PAGE < t:
+                tables[s].append(nxt)
+                nxt += 1
+    return tables
+
+
+def _exact_step(case, flags, conditioned, seed):
+    dev = torch.device("cuda", torch.cuda.current_device())
+    dims, batch = _dims(case), _batch(case)
+    Hq, Hk, Dh = dims.n_q_heads, dims.n_kv_heads, dims.head_dim
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(seed + 1)
+    shape = wl.kv_pool_shape(dims, wl.pages_needed(batch) + 8)[1:]
+    pool = [torch.empty(shape, dtype=torch.bfloat16, device=dev).normal_(generator=gen) for _ in range(dims.n_layers)]
+    bias = [[(0.1 * torch.randn(n, generator=gen, device=dev)).to(torch.bfloat16).double()
+             for n in (dims.q_dim, dims.kv_dim, dims.kv_dim)] if case["bias"] else None for _ in range(dims.n_layers)]
+    mod = wl.make_modulation(dims, batch.n_seqs, seed, dev).double() if conditioned else None
+    seq = torch.repeat_interleave(torch.arange(batch.n_seqs), torch.tensor(batch.q_len)).to(dev)
+    pos = torch.cat([torch.arange(c, c + q) for q, c in zip(batch.q_len, batch.ctx_len)]).to(dev)
+    pages = [torch.tensor(t, device=dev) for t in _pages(batch)]
+    slot = torch.cat([pages[s][torch.arange(c, c + q, device=dev) // PAGE] * PAGE
+                      for s, (q, c) in enumerate(zip(batch.q_len, batch.ctx_len))]) + pos % PAGE
+    x = wl.make_x(batch.n_tokens, dims.d_model, seed, dev).double()
+    out = []
+    for l in range(dims.n_layers):
+        w = {k: v.double() for k, v in wl.make_layer_weights(dims, seed, l, dev, "depth_scaled").items()}
+
+        def norm(v, gain, first):
+            h = _rms(v, gain, dims.rms_eps)
+            return h if mod is None else h * (1.0 + mod[l, seq, first + 1]) + mod[l, seq, first]
+
+        def gated(v, which):
+            return v if mod is None else v * mod[l, seq, which]
+
+        h = norm(x, w["g_attn"], 0)
+        q, k, v = (h @ w[n].T + (bias[l][i] if bias[l] else 0.0) for i, n in enumerate(("w_q", "w_k", "w_v")))
+        q = _rope(q.view(-1, Hq, Dh), pos, dims.rope_base)
+        k, v = _rope(k.view(-1, Hk, Dh), pos, dims.rope_base), v.view(-1, Hk, Dh)
+        whole = pool[l].double()                           # a new key or value is read back in the cache's bf16
+        for i, t in enumerate((k, v)):
+            whole[i, slot // PAGE, :, slot % PAGE] = t
+        pool[l] = None
+        o, row = torch.empty_like(q), 0
+        for s, (n, c) in enumerate(zip(batch.q_len, batch.ctx_len)):
+            keys, vals = (whole[i, pages[s]].to(torch.bfloat16).double().permute(1, 0, 2, 3).reshape(Hk, -1, Dh)[:, :n + c]
+                          for i in (0, 1))
+            qs = q[row:row + n].view(n, Hk, Hq // Hk, Dh).permute(1, 2, 0, 3)                  # [Hk, G, n, Dh]
+            sc = qs @ keys[:, None].transpose(-1, -2) / math.sqrt(Dh)
+            if not flags & B.HS_FLAG_BIDIRECTIONAL:
+                sc.masked_fill_(torch.arange(n + c, device=dev) > pos[row:row + n, None], -math.inf)
+            o[row:row + n] = (sc.softmax(-1) @ vals[:, None]).permute(2, 0, 1, 3).reshape(n, Hq, Dh)
+            row += n
+        x = x + gated(o.view(-1, dims.q_dim) @ w["w_o"].T, 2)
+        h = norm(x, w["g_mlp"], 3)
+        x = x + gated((torch.nn.functional.silu(h @ w["w_gate"].T) * (h @ w["w_up"].T)) @ w["w_down"].T, 5)
+        out.append(whole)
+    return [x, *out]
+
+
+def exact(case, seed):
+    if case["kind"] == "head":
+        s = _HeadState(case, seed)
+        h = _rms(s.y[s.rows.long()].double(), s.gain.double(), 1e-6)
+        return [torch.cat([h @ w.double().T for w in s.w.split(16384)], -1), None, None]
+    return [t for i, (c, flags, cond, _) in enumerate(_parts(case)) for t in _exact_step(c, flags, cond, seed + 7919 * i)]
+
+
 # --- what a pass cannot do without ---------------------------------------------------------------------------------
 def work(case):
     if case["kind"] == "head":
