@@ -539,9 +539,9 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
   // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next
-  // kernel would wait on SMs outside the budget, so the launches stay strictly serial.  (Not while the
-  // per-kernel timers run: an event between two kernels serialises them anyway.)
-  const int overlap = (sm_budget == s->sm_count && !s->profile) ? 1 : 0;
+  // kernel would wait on SMs outside the budget, so they are placed only when the last block in front has left (see
+  // OverlapMode).  (Not while the per-kernel timers run: an event between two kernels serialises them anyway.)
+  const int overlap = s->profile ? kOverlapNone : sm_budget == s->sm_count ? kOverlapEarly : kOverlapLate;
   // A operands of a small step are fetched with boxes of 64 or 32 rows instead of 128
   const int a_rows = use_pair ? 128 : (T <= 32 ? 32 : T <= 64 ? 64 : 128);
   const int a_sel = a_rows == 64 ? 0 : 1;
@@ -760,7 +760,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
       // side by side: the decode kernel on the stage's own stream with decode_sms of the budget, the prefill kernel on
       // the caller's stream with the rest; both are joined before the out-projection
       AttnParams ad = a;
-      ad.overlap = 0;
+      ad.overlap = kOverlapNone;
       if (cudaEventRecord(s->ev_fork, stream) != cudaSuccess || cudaStreamWaitEvent(s->aux_stream, s->ev_fork, 0) != cudaSuccess) {
         e = cudaGetLastError(); where = "attention fork"; break;
       }
@@ -784,7 +784,9 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     go.M = T; go.N = d; go.K = q_dim;
     go.mode = kGemmResid;
     go.ab_f16 = f16;
-    go.overlap = overlap;
+    // (behind the two attention kernels side by side the out-projection waits for both: with a partial budget it must
+    // not be placed on the prefill kernel's leaving alone)
+    go.overlap = decode_sms > 0 && overlap == kOverlapLate ? int(kOverlapNone) : overlap;
     go.tm_out = tm_y; go.accumulate = 1;
     go.gate_mod = mod_l; go.tok_seq = meta + s->ml.tok_seq; go.gate_which = 2;
     go.pair = pair_d;
@@ -799,6 +801,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
       SkinnyParams k = skinny_base(o, q_dim, d, kGemmResid);
       k.w[0] = wo.w_o; k.y = x; k.accumulate = 1;
       k.gate_mod = go.gate_mod; k.tok_seq = go.tok_seq; k.gate_which = 2;
+      k.overlap = go.overlap;
       k.smid_log = slots(5);
       if (sk_fold_mlp) sk_fold_out(k, w.g_mlp, skinny(d, F, kGemmGateUp));
       LaunchTimer t(s, 5, stream); where = "out-proj gemm"; e = launch_gemm_skinny(k, sm_budget, stream);

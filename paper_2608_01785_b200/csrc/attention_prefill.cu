@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) attn_prefill_kernel(const __gri
   tc_fence_after_sync();
   const uint32_t tmem = bar->tmem_base;
   griddep_wait();
-  griddep_launch_dependents();
+  griddep_launch_dependents(p.overlap);
 
   int rs = 0;
   uint32_t rph = 0;       // item ring slot / phase

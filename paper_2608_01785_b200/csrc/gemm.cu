@@ -380,7 +380,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     }
   }
   griddep_wait();                 // everything above is set-up; the operands belong to the previous kernel until here
-  griddep_launch_dependents();
+  griddep_launch_dependents(p.overlap);
 
   if (warp == 0) {
     // ------------------------------------------------------- TMA producer --

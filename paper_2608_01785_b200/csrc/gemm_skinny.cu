@@ -401,9 +401,9 @@ template <int MT, int DB, bool F16, bool FOLD>
 __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const SkinnyParams p) {
   extern __shared__ __align__(16) uint8_t sk_smem[];
   log_smid(p.smid_log);
-  gemm_skinny_body<MT, DB, F16, FOLD>(p, sk_smem, int(blockIdx.x), int(gridDim.x), [] {
+  gemm_skinny_body<MT, DB, F16, FOLD>(p, sk_smem, int(blockIdx.x), int(gridDim.x), [&] {
     griddep_wait();
-    griddep_launch_dependents();
+    griddep_launch_dependents(p.overlap);
   });
 }
 

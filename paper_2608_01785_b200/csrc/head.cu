@@ -16,7 +16,6 @@ __global__ void __launch_bounds__(HEAD_THREADS, 1) embed_kernel(const EmbedParam
   extern __shared__ uint8_t unused_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   griddep_wait();
-  griddep_launch_dependents();
   const int d8 = p.d >> 3;
   for (int t = blockIdx.x * warps + warp; t < p.n; t += gridDim.x * warps) {
     const int id = p.tokens[t];
@@ -44,7 +43,6 @@ __global__ void __launch_bounds__(HEAD_THREADS, 1) argmax_kernel(const ArgmaxPar
   float* sv = reinterpret_cast<float*>(argmax_smem);
   int* si = reinterpret_cast<int*>(argmax_smem + HEAD_THREADS * 4);
   griddep_wait();
-  griddep_launch_dependents();
   const int v4 = p.vocab >> 2;
   for (int r = blockIdx.x; r < p.n; r += gridDim.x) {
     const float4* row = reinterpret_cast<const float4*>(p.logits + size_t(r) * p.vocab);

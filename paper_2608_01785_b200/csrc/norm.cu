@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(NORM_THREADS, 1) rmsnorm_kernel(const NormPara
   log_smid(p.smid_log);
   float4* cache = reinterpret_cast<float4*>(norm_smem + warp * NORM_STAGE_FLOATS);
   griddep_wait();
-  griddep_launch_dependents();
+  griddep_launch_dependents(p.overlap);
   const int d8 = p.d >> 3;                         // groups of 8 elements
   const int cached8 = min(d8, NORM_STAGE_FLOATS / 8);
   const uint4* gsrc = reinterpret_cast<const uint4*>(p.gain);
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
   }
   __syncthreads();
   griddep_wait();                 // the gains above are weights; the rows belong to the previous kernel until here
-  griddep_launch_dependents();
+  griddep_launch_dependents(p.overlap);
   uint64_t* full = bars + 2 * warp;
   const int stride = gridDim.x * n_warps, first = blockIdx.x * n_warps + warp;
   const char* src = in_bf16 ? reinterpret_cast<const char*>(p.x_bf16) : reinterpret_cast<const char*>(p.x_f32);
