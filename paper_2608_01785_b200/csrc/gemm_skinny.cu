@@ -95,7 +95,13 @@ __device__ __forceinline__ float row_norm_factor(const float* row_ss, int stride
   const int q = threadIdx.x & 3;
   float sum = 0.f;
   if (row < T)
-    for (int i = q; i < n; i += 4) sum += __ldcg(row_ss + size_t(row) * stride + i);
+    for (int i0 = q; i0 < n; i0 += 4 * 8) {        // eight loads in flight at a time, added in order
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = i0 + 4 * u < n ? __ldcg(row_ss + size_t(row) * stride + i0 + 4 * u) : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) sum += v[u];
+    }
   sum += __shfl_xor_sync(0xffffffffu, sum, 1);
   sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   return rsqrtf(sum / float(width) + eps);
@@ -133,16 +139,14 @@ __device__ __forceinline__ void gemm_skinny_body(const SkinnyParams& p, uint8_t*
 #pragma unroll
     for (int j = 0; j < NT; ++j) wrow[j] = unit_row(p, unit, j, g) + k_off;
   };
-  // activation rows of this lane: rows 16 i + g and 16 i + g + 8 (clamped into the step)
+  // Activation rows of this lane: rows 16 i + g and 16 i + g + 8.  Rows past the step are not copied: whatever their
+  // ring bytes hold reaches only accumulator rows that no epilogue stores.  (Copying the last row in their place made
+  // every lane of every block ask the L2 for the same lines: talker step of one row 334 -> 236 us.)
   const uint8_t* arow[MT][2];
 #pragma unroll
   for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      int r = 16 * i + 8 * h + g;
-      r = r < p.T ? r : p.T - 1;
-      arow[i][h] = static_cast<const uint8_t*>(p.a) + size_t(r) * p.K * 2 + k_off;
-    }
+    for (int h = 0; h < 2; ++h) arow[i][h] = static_cast<const uint8_t*>(p.a) + size_t(16 * i + 8 * h + g) * p.K * 2 + k_off;
   auto issue_b = [&](int s, int slot) {                     // weights of step s of this warp's slice
 #pragma unroll
     for (int j = 0; j < NT; ++j) cp_async16(ring + slot * STAGE_BYTES + j * 512, wrow[j] + size_t(s) * STEP_BYTES);
@@ -152,7 +156,7 @@ __device__ __forceinline__ void gemm_skinny_body(const SkinnyParams& p, uint8_t*
     for (int i = 0; i < MT; ++i)
 #pragma unroll
       for (int h = 0; h < 2; ++h)
-        cp_async16(ring + slot * STAGE_BYTES + (NT + 2 * i + h) * 512, arow[i][h] + size_t(s) * STEP_BYTES);
+        if (16 * i + 8 * h + g < p.T) cp_async16(ring + slot * STAGE_BYTES + (NT + 2 * i + h) * 512, arow[i][h] + size_t(s) * STEP_BYTES);
   };
   auto prologue = [&]() {
 #pragma unroll
