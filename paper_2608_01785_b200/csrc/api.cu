@@ -186,7 +186,7 @@ struct hs_stage {
   const float* modulation = nullptr;          // optional [n_layers][max_seqs][6][d_model] (hs_stage_set_modulation)
   std::vector<hs_layer_weights_t> operands;   // what the projections read: the fp16 copies, or `layers` itself
   std::vector<LayerMaps> maps;
-  CUtensorMap tm_h, tm_o, tm_act, tm_kv;   // operand loads
+  CUtensorMap tm_h, tm_o, tm_act, tm_kv, tm_kv_page;   // operand loads
   CUtensorMap tm_h_s[2], tm_o_s[2], tm_act_s[2];   // the same A operands with 64- and 32-row boxes (small steps)
   CUtensorMap tm_q_st, tm_act_st, tm_h_st; // epilogue stores (box 64 x 32)
   CUtensorMap tm_q_attn;                   // Q tiles of the prefill attention (box 64 x tokens per item)
@@ -336,7 +336,8 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
   ok = ok && encode_2d(&s->tm_q_attn, s->ws_dev + s->ws.q, T, q_dim,
                        prefill_tokens_per_item(cfg->n_q_heads / cfg->n_kv_heads));
   const uint64_t pool_rows = uint64_t(cfg->n_layers) * 2 * cfg->num_pages * cfg->n_kv_heads * kPage;
-  ok = ok && encode_2d(&s->tm_kv, s->kv_pool, pool_rows, cfg->head_dim, 16);
+  ok = ok && encode_2d(&s->tm_kv, s->kv_pool, pool_rows, cfg->head_dim, 16) &&
+       encode_kv_pages(get_encode_fn(), &s->tm_kv_page, s->kv_pool, cfg->n_layers, cfg->num_pages, cfg->n_kv_heads, cfg->head_dim);
   s->maps.resize(cfg->n_layers);
   s->operands = s->layers;
   s->qkv_bias.assign(cfg->n_layers, hs_stage::QkvBias());
@@ -634,6 +635,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   auto make_attn = [&](int l) {
     AttnParams a{};
     a.tm_kv = s->tm_kv;
+    a.tm_kv_page = s->tm_kv_page;
     a.tm_q = s->tm_q_attn;
     a.prefill_tokens = prefill_tokens_per_item(c.n_q_heads / c.n_kv_heads);
     a.o_f16 = f16;

@@ -38,15 +38,10 @@ struct Geom {
 __device__ __forceinline__ int kv_off(int kk, int cc) {
   return (cc >> 3) * 2048 + kk * 128 + (((cc & 7) ^ (kk & 7)) << 4);
 }
-// First pool row (unit: one key's Dh elements of one KV head) of (layer, K|V, page, head).
-__device__ __forceinline__ int pool_row(const AttnParams& p, int layer, int kv, int page, int hk) {
-  return (((layer * 2 + kv) * p.num_pages + page) * p.n_kv_heads + hk) * 16;
-}
+// Requests the K and the V block of (layer, page, KV head) with one copy: [K | V][half][16 keys][128 B].
 template <int DH>
-__device__ __forceinline__ void load_page(const AttnParams& p, int layer, uint8_t* dst, uint64_t* bar, int kv, int page, int hk) {
-  const int row = pool_row(p, layer, kv, page, hk);
-#pragma unroll
-  for (int h = 0; h < Geom<DH>::HALVES; ++h) tma_load_2d(dst + h * 2048, &p.tm_kv, bar, h * 64, row);
+__device__ __forceinline__ void load_page(const AttnParams& p, int layer, uint8_t* dst, uint64_t* bar, int page, int hk) {
+  tma_load_4d(dst, &p.tm_kv_page, bar, 0, (page * p.n_kv_heads + hk) * 16, 0, layer * 2);
 }
 __device__ __forceinline__ float quad_max(float v) {
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -195,7 +190,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
     for (int i = 0; i < DC_WARPS * DC_STAGES; ++i) mbar_init(&full_all[i], 1);
     *abort_flag = 0;
     fence_barrier_init();
-    tma_prefetch_desc(&p.tm_kv);
+    tma_prefetch_desc(&p.tm_kv_page);
   }
   __syncthreads();
 
@@ -205,8 +200,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
   auto issue = [&](int page, int hk) {      // lane 0: request one page of an item
     const uint32_t st = issued % DC_STAGES;
     mbar_expect_tx(&full[st], SLOT_BYTES);
-    load_page<DH>(p, layer, slots + st * SLOT_BYTES, &full[st], 0, page, hk);
-    load_page<DH>(p, layer, slots + st * SLOT_BYTES + G_::PAGE_BYTES, &full[st], 1, page, hk);
+    load_page<DH>(p, layer, slots + st * SLOT_BYTES, &full[st], page, hk);
     ++issued;
   };
 

@@ -93,17 +93,6 @@ hs_status_t setup_device(int dev, const DeviceSetup** out) {
   return HS_OK;
 }
 
-bool encode_pool_map(CUtensorMap* m, const void* pool, uint64_t rows, uint64_t head_dim) {
-  EncodeTiledFn fn = g_encode;
-  cuuint64_t dims[2] = {head_dim, rows};
-  cuuint64_t strides[1] = {head_dim * 2};
-  cuuint32_t box[2] = {64, 16};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(pool), dims,
-            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
 }  // namespace hs
 
@@ -172,7 +161,7 @@ extern "C" hs_status_t hs_op_decode_attention_noalloc(const void* q_dev, const v
 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   AttnParams a{};
-  if (!encode_pool_map(&a.tm_kv, kv_pool_dev, uint64_t(pool_rows), uint64_t(head_dim))) return HS_ERR_CUDA;
+  if (!encode_kv_pages(g_encode, &a.tm_kv_page, kv_pool_dev, n_layers, num_pages, n_kv_heads, head_dim)) return HS_ERR_CUDA;
   // The metadata copy also resets the queue heads and the status word left by the previous call.  The source is
   // ordinary (pageable) host memory: the runtime has taken its contents when the call returns, possibly after
   // waiting for earlier work of the stream.
