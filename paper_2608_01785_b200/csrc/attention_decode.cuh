@@ -26,6 +26,7 @@ namespace hs {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kLazyMax = 8.f;         // the softmax reference moves when a score exceeds it by this much (log2 units)
 
 template <int DH>
 struct Geom {
@@ -196,12 +197,13 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
 
   uint8_t* slots = smem + (worker ? warp : 0) * DC_STAGES * SLOT_BYTES;
   uint64_t* full = full_all + (worker ? warp : 0) * DC_STAGES;
-  uint32_t issued = 0, consumed = 0;      // pages this warp has requested / finished, over all its items
+  int fill = 0;                           // ring slot of the next page to request, over all items of this warp
+  int cur = 0;                            // ring slot of the next page to read, and its phase
+  uint32_t cur_phase = 0;
   auto issue = [&](int page, int hk) {      // lane 0: request one page of an item
-    const uint32_t st = issued % DC_STAGES;
-    mbar_expect_tx(&full[st], SLOT_BYTES);
-    load_page<DH>(p, layer, slots + st * SLOT_BYTES, &full[st], page, hk);
-    ++issued;
+    mbar_expect_tx(&full[fill], SLOT_BYTES);
+    load_page<DH>(p, layer, slots + fill * SLOT_BYTES, &full[fill], page, hk);
+    if (++fill == DC_STAGES) fill = 0;
   };
 
   // A warp's first item is its own index in the grid (no round trip to the queue head before the first page request);
@@ -288,65 +290,83 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
     float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
     bool ok = true;
 
+    // A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
+    // bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs per key
+    // half, the V fragments are fetched while the scores are on their way, and the exponentials are taken against a reference that follows the running maximum only when a score exceeds it by more than 8 in
+    // log2 units (the sum uses the same reference, so O / l is the same quotient): no shuffles and no rescale for most
+    // pages.  Against a loop with one chain of MMAs, a running maximum moved on every page (four shuffles, exp2f) and V
+    // fetched behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker
+    // step of 16 rows 300.5 -> 287.6 us, of 11 rows on 52 SMs 471 -> 448; at config-3 dimensions 9 rows, 4 layers 493 ->
+    // 482 us, 29 rows on 96 SMs 796 -> 779, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.15 ms.
     for (int pi = 0; pi < n_pages; ++pi) {
       // the slot read in the previous iteration is free: keep DC_STAGES - 1 pages in flight
       const int page_ahead = __shfl_sync(0xffffffffu, my_page, (pi + DC_STAGES - 1) & 31);
       if (lane == 0 && pi + DC_STAGES - 1 < n_pages) issue(page_ahead, hk);
-      const uint32_t st = consumed % DC_STAGES;
-      ok = mbar_wait(&full[st], (consumed / DC_STAGES) & 1, abort_flag, p.status);
+      ok = mbar_wait(&full[cur], cur_phase, abort_flag, p.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      ++consumed;
-      const uint32_t k_base = smem_u32(slots + st * SLOT_BYTES);
+      const uint32_t k_base = smem_u32(slots + cur * SLOT_BYTES);
       const uint32_t v_base = k_base + G_::PAGE_BYTES;
+      if (++cur == DC_STAGES) { cur = 0; cur_phase ^= 1; }
       const int n_valid = k1 - (k0 + pi * 16);            // keys of this page that belong to the item
       float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+      float sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-      for (int ks = 0; ks < DH / 16; ++ks) {
-        uint32_t kf[4];
+      for (int ks = 0; ks < DH / 16; ks += 2) {
+        uint32_t kf[4], kg[4];
         const int kk = (lane & 7) + (lane >> 4) * 8, cc = 2 * ks + ((lane >> 3) & 1);
         ldmatrix_x4(kf, k_base + kv_off(kk, cc));
+        ldmatrix_x4(kg, k_base + kv_off(kk, cc + 2));
         mma_bf16_16816(sc[0], qf[ks], kf[0], kf[1]);
         mma_bf16_16816(sc[1], qf[ks], kf[2], kf[3]);
+        mma_bf16_16816(sd[0], qf[ks + 1], kg[0], kg[1]);
+        mma_bf16_16816(sd[1], qf[ks + 1], kg[2], kg[3]);
       }
-      float mx_a = -INFINITY, mx_b = -INFINITY;
+      uint32_t vf[DH / 16][4];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float v = sc[j][e] * scale_log2;
-          if (8 * j + 2 * (lane & 3) + (e & 1) >= n_valid) v = -INFINITY;
-          sc[j][e] = v;
-        }
-        mx_a = fmaxf(mx_a, fmaxf(sc[j][0], sc[j][1]));
-        mx_b = fmaxf(mx_b, fmaxf(sc[j][2], sc[j][3]));
+      for (int dp = 0; dp < DH / 16; ++dp) {
+        const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
+        ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, cc));
       }
-      mx_a = quad_max(mx_a);
-      mx_b = quad_max(mx_b);
-      const float mn_a = fmaxf(m_a, mx_a), mn_b = fmaxf(m_b, mx_b);
-      const float al_a = exp2f(m_a - mn_a), al_b = exp2f(m_b - mn_b);
-      // the running maxima settle after a few pages: skip the rescale of O when no row's maximum moved
-      const bool rescale = __any_sync(0xffffffffu, mn_a != m_a || mn_b != m_b);
-      m_a = mn_a;
-      m_b = mn_b;
-      float sum_a = 0.f, sum_b = 0.f;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        sc[j][0] = exp2f(sc[j][0] - mn_a);
-        sc[j][1] = exp2f(sc[j][1] - mn_a);
-        sc[j][2] = exp2f(sc[j][2] - mn_b);
-        sc[j][3] = exp2f(sc[j][3] - mn_b);
-        sum_a += sc[j][0] + sc[j][1];
-        sum_b += sc[j][2] + sc[j][3];
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sc[j][e] += sd[j][e];
+      if (n_valid < 16) {
+        const int k = 2 * (lane & 3);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (8 * j + k + (e & 1) >= n_valid) sc[j][e] = -INFINITY;
+#pragma unroll
+        for (int dp = 0; dp < DH / 16; ++dp)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], k + 8 * (e & 1), n_valid);
       }
-      l_a = l_a * al_a + sum_a;
-      l_b = l_b * al_b + sum_b;
-      if (rescale) {
+      const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
+      const float mx_b = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2;
+      if (__any_sync(0xffffffffu, mx_a > m_a + kLazyMax || mx_b > m_b + kLazyMax)) {
+        const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = fmaxf(m_b, quad_max(mx_b));
+        const float al_a = fast_exp2(m_a - mn_a), al_b = fast_exp2(m_b - mn_b);
+        m_a = mn_a;
+        m_b = mn_b;
+        l_a *= al_a;
+        l_b *= al_b;
 #pragma unroll
         for (int j = 0; j < DH / 8; ++j) {
           o_acc[j][0] *= al_a; o_acc[j][1] *= al_a;
           o_acc[j][2] *= al_b; o_acc[j][3] *= al_b;
         }
       }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        sc[j][0] = fast_exp2(fmaf(sc[j][0], scale_log2, -m_a));
+        sc[j][1] = fast_exp2(fmaf(sc[j][1], scale_log2, -m_a));
+        sc[j][2] = fast_exp2(fmaf(sc[j][2], scale_log2, -m_b));
+        sc[j][3] = fast_exp2(fmaf(sc[j][3], scale_log2, -m_b));
+      }
+      l_a += (sc[0][0] + sc[0][1]) + (sc[1][0] + sc[1][1]);
+      l_b += (sc[0][2] + sc[0][3]) + (sc[1][2] + sc[1][3]);
       uint32_t pf[4];
       pf[0] = pack_bf16(sc[0][0], sc[0][1]);
       pf[1] = pack_bf16(sc[0][2], sc[0][3]);
@@ -354,18 +374,8 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
       pf[3] = pack_bf16(sc[1][2], sc[1][3]);
 #pragma unroll
       for (int dp = 0; dp < DH / 16; ++dp) {
-        uint32_t vf[4];
-        const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
-        ldmatrix_x4_trans(vf, v_base + kv_off(kk, cc));
-        if (n_valid < 16) {
-          const int k = 2 * (lane & 3);
-          vf[0] = mask_v(vf[0], k, n_valid);
-          vf[1] = mask_v(vf[1], k + 8, n_valid);
-          vf[2] = mask_v(vf[2], k, n_valid);
-          vf[3] = mask_v(vf[3], k + 8, n_valid);
-        }
-        mma_bf16_16816(o_acc[2 * dp], pf, vf[0], vf[1]);
-        mma_bf16_16816(o_acc[2 * dp + 1], pf, vf[2], vf[3]);
+        mma_bf16_16816(o_acc[2 * dp], pf, vf[dp][0], vf[dp][1]);
+        mma_bf16_16816(o_acc[2 * dp + 1], pf, vf[dp][2], vf[dp][3]);
       }
       __syncwarp();                         // every lane is done with this slot before lane 0 refills it
     }

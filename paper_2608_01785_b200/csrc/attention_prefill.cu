@@ -78,12 +78,6 @@ static_assert(sizeof(Barriers) <= 1024, "barrier block");
 __device__ __forceinline__ int pool_row(const AttnParams& p, int kv, int page, int hk) {
   return (((p.layer * 2 + kv) * p.num_pages + page) * p.n_kv_heads + hk) * 16;
 }
-// 2^x on the special-function unit (ex2.approx: exact 0 for -inf, relative error about 2^-22).
-__device__ __forceinline__ float fast_exp2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 // MN-major bf16 operand with the 128-byte swizzle: atoms of 64 (MN, contiguous) x 8 (K) elements;
 // lbo = bytes between atoms along MN, sbo = bytes between atoms along K.
 __device__ __forceinline__ uint64_t umma_desc_mnmajor_sw128(uint32_t smem_addr, uint32_t lbo, uint32_t sbo) {
