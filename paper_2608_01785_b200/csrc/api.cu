@@ -22,7 +22,8 @@ constexpr int kRing = 4;   // pinned staging slots for step metadata
 constexpr int kRowSsStride = 64;   // partial sums of x^2 kept per token: one per 128-column tile of d_model at most
 
 struct WsLayout {
-  size_t rope, h, q, o, act, meta, part_o, part_ml, status, turn, smid, row_ss, row_rs, row_done, w16, w16_layer, total;
+  size_t rope, h, q, o, act, meta, part_o, part_ml, status, turn, smid, row_ss, row_rs, row_done, gemm_part, w16, w16_layer, total;
+  int part_rows;             // rows of d_model floats in gemm_part
 };
 
 // elements of the i-th weight matrix of a layer, in the order w_q, w_k, w_v, w_o, w_gate, w_up, w_down
@@ -57,6 +58,9 @@ WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   w.row_ss = take(std::max(T * kRowSsStride, size_t(64) * size_t(c.d_model / 32 + 1)) * 4);
   w.row_rs = take(T * 4);                            // r of every token
   w.row_done = take((T / 32 + 2) * 4);               // tile columns delivered per group of 32 token rows
+  // partial sums of the K-split residual GEMMs of small and middling steps (gemm_plan_parts): at most ten splits and 40 MB
+  w.part_rows = int(std::min(size_t(10) * align_up(T, 32), (size_t(40) << 20) / (size_t(c.d_model) * 4)));
+  w.gemm_part = take(size_t(w.part_rows) * c.d_model * 4);
   // fp16 copies of the seven weight matrices of every layer (absent with HS_FLAG_BF16_ACTIVATIONS);
   // within a layer: w_q, w_k, w_v, w_o, w_gate, w_up, w_down, each 1024-byte aligned
   w.w16 = off;
@@ -189,6 +193,7 @@ struct hs_stage {
   CUtensorMap tm_h, tm_o, tm_act, tm_kv, tm_kv_page;   // operand loads
   CUtensorMap tm_h_s[2], tm_o_s[2], tm_act_s[2];   // the same A operands with 64- and 32-row boxes (small steps)
   CUtensorMap tm_q_st, tm_act_st, tm_h_st; // epilogue stores (box 64 x 32)
+  CUtensorMap tm_part;                     // partial sums of the K-split residual GEMMs (box 32 x 32 fp32)
   CUtensorMap tm_q_attn;                   // Q tiles of the prefill attention (box 64 x tokens per item)
   int32_t* pinned[kRing] = {};
   cudaEvent_t ev[kRing] = {};
@@ -335,6 +340,7 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
        encode_2d(&s->tm_act_st, s->ws_dev + s->ws.act, T, F, 32) && encode_2d(&s->tm_h_st, s->ws_dev + s->ws.h, T, d, 32);
   ok = ok && encode_2d(&s->tm_q_attn, s->ws_dev + s->ws.q, T, q_dim,
                        prefill_tokens_per_item(cfg->n_q_heads / cfg->n_kv_heads));
+  if (s->ws.part_rows > 0) ok = ok && encode_2d(&s->tm_part, s->ws_dev + s->ws.gemm_part, s->ws.part_rows, d, 32, true);
   const uint64_t pool_rows = uint64_t(cfg->n_layers) * 2 * cfg->num_pages * cfg->n_kv_heads * kPage;
   ok = ok && encode_2d(&s->tm_kv, s->kv_pool, pool_rows, cfg->head_dim, 16) &&
        encode_kv_pages(get_encode_fn(), &s->tm_kv_page, s->kv_pool, cfg->n_layers, cfg->num_pages, cfg->n_kv_heads, cfg->head_dim);
@@ -567,6 +573,38 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const bool fold_norm = !s->modulation && n_ss_tiles <= kRowSsStride && !skinny(d, q_dim + 2 * kv_dim, kGemmQkv) &&
                          !skinny(q_dim, d, kGemmResid) && !skinny(d, F, kGemmGateUp) && !skinny(F, d, kGemmResid) &&
                          pair_d && pair_qkv && pair_gu;
+  // A step with separate norm kernels: the K splits of a residual GEMM leave their partial sums in scratch and the norm
+  // kernel behind it adds them (the last layer's: a launch of the same kernel without a norm).  Nothing waits for its
+  // turn and all splits are equally long, so every SM streams weights until the end.  A choice by shape and stage, never
+  // by budget; a width or a scratch that does not fit keeps the ordered chain.  Measured on B200 against that chain
+  // and the norm kernel of one warp per row: 64 decode rows at config-3 dimensions 5.14 -> 4.96 ms, 29 rows on 96 SMs (4
+  // layers) 780 -> 714 us, a chunk of 394 tokens with 7 decode rows (4 layers) 1239 -> 1127 us, denoising 1125 -> 1034 us.
+  const bool parts_ok = !fold_norm && d <= kNormRowMaxD;
+  auto plan_parts = [&](int K) {
+    ResidPlan r{0, 0, 0, 0.0};
+    if (parts_ok && !(T <= 16 && skinny(K, d, kGemmResid))) r = gemm_plan_parts(T, d, K, s->sm_count, s->ws.part_rows);
+    if (r.ks > 0 && skinny(K, d, kGemmResid) && gemm_skinny_cost_us(T, K, d, kGemmResid, s->sm_count) < r.us) r.ks = 0;
+    return r;
+  };
+  const ResidPlan parts_out = plan_parts(q_dim), parts_down = plan_parts(F);
+  const int part_rows = ceil_div(T, 32) * 32;
+  auto use_parts = [&](GemmParams& gp, const ResidPlan& r) {
+    gp.pair = r.pair;
+    gp.bn = r.bn;
+    gp.ksplit = r.ks;
+    gp.stream_k_slots = 0;
+    gp.gate_mod = nullptr;               // the norm kernel applies the gate to the sum
+    gp.tm_out = s->tm_part;
+    gp.part_rows = part_rows;
+  };
+  auto add_parts = [&](NormParams& n, const ResidPlan& r, const float* mod_of_branch, int gate_which) {
+    if (r.ks == 0) return;
+    n.part = reinterpret_cast<const float*>(s->ws_dev + s->ws.gemm_part);
+    n.n_parts = r.ks;
+    n.part_stride = size_t(part_rows) * d;
+    n.mod_gate = mod_of_branch;
+    n.gate_which = mod_of_branch ? gate_which : 0;
+  };
   // Steps of at most 16 rows: a residual projection on the weight-streaming kernel folds the norm behind it the same
   // way (its epilogue emits h and the row sums, the block that delivers the last unit finalises r); the projection
   // behind the norm -- on either kernel -- scales its rows.  A choice by shape, never by budget.  Measured on B200, the
@@ -688,11 +726,13 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     np.h_f16 = f16;
     np.status = status;
     np.overlap = overlap;
+    np.sm_count = s->sm_count;
     np.smid_log = slots(0);
     const float* mod_l = s->modulation ? s->modulation + size_t(l) * c.max_seqs * 6 * d : nullptr;
     np.mod = mod_l;
     np.tok_seq = meta + s->ml.tok_seq;
     np.mod_which = 0;
+    if (l > 0) add_parts(np, parts_down, mod_l ? mod_l - size_t(c.max_seqs) * 6 * d : nullptr, 5);
     const bool folded_attn_norm = (fold_norm || sk_fold_attn) && l > 0;   // the previous layer's down-projection produced h and the sums
     if (!folded_attn_norm) { LaunchTimer t(s, 0, stream); where = "rmsnorm"; e = launch_rmsnorm(np, sm_budget, stream); }
     if (e != cudaSuccess) break;
@@ -799,7 +839,8 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     go.status = status;
     go.smid_log = slots(5);
     if (fold_norm) fold_out(go, w.g_mlp);
-    if (skinny(q_dim, d, kGemmResid)) {
+    if (parts_out.ks > 0) use_parts(go, parts_out);
+    if (parts_out.ks == 0 && skinny(q_dim, d, kGemmResid)) {
       SkinnyParams k = skinny_base(o, q_dim, d, kGemmResid);
       k.w[0] = wo.w_o; k.y = x; k.accumulate = 1;
       k.gate_mod = go.gate_mod; k.tok_seq = go.tok_seq; k.gate_which = 2;
@@ -813,6 +854,9 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     np.x_bf16 = nullptr;
     np.gain = static_cast<const __nv_bfloat16*>(w.g_mlp);
     np.mod_which = 3;
+    np.n_parts = 0;
+    np.gate_which = 0;
+    add_parts(np, parts_out, mod_l, 2);
     if (!fold_norm && !sk_fold_mlp) { LaunchTimer t(s, 0, stream); where = "rmsnorm"; e = launch_rmsnorm(np, sm_budget, stream); }
     if (e != cudaSuccess) break;
 
@@ -859,14 +903,24 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     gd.status = status;
     gd.smid_log = slots(7);
     if (fold_norm && l + 1 < c.n_layers) fold_out(gd, s->layers[l + 1].g_attn);
-    if (skinny(F, d, kGemmResid)) {
+    if (parts_down.ks > 0) use_parts(gd, parts_down);
+    if (parts_down.ks == 0 && skinny(F, d, kGemmResid)) {
       SkinnyParams k = skinny_base(s->ws_dev + s->ws.act, F, d, kGemmResid);
       k.w[0] = wo.w_down; k.y = x; k.accumulate = 1;
       k.gate_mod = gd.gate_mod; k.tok_seq = gd.tok_seq; k.gate_which = 5;
       k.smid_log = slots(7);
       if (sk_fold_attn && l + 1 < c.n_layers) sk_fold_out(k, s->layers[l + 1].g_attn, skinny(d, q_dim + 2 * kv_dim, kGemmQkv));
       LaunchTimer t(s, 7, stream); where = "down gemm"; e = launch_gemm_skinny(k, sm_budget, stream);
-    } else { LaunchTimer t(s, 7, stream); where = "down gemm"; e = launch_gemm(gd, sm_budget, stream); }
+    } else {
+      LaunchTimer t(s, 7, stream); where = "down gemm"; e = launch_gemm(gd, sm_budget, stream);
+      if (e == cudaSuccess && parts_down.ks > 0 && l + 1 == c.n_layers) {     // no norm follows: the sum alone
+        np.h = nullptr;
+        np.n_parts = 0;
+        np.gate_which = 0;
+        add_parts(np, parts_down, mod_l, 5);
+        where = "partial sums"; e = launch_rmsnorm(np, sm_budget, stream);
+      }
+    }
     if (e != cudaSuccess) break;
   }
   return e == cudaSuccess ? HS_OK : cuda_fail(where, e);
@@ -1109,6 +1163,7 @@ hs_status_t hs_head_step(hs_head_t* h, const float* y, const int32_t* rows, int3
   np.d = d;
   np.eps = h->cfg.rms_eps;
   np.row_index = rows;
+  np.sm_count = h->sm_count;
   np.status = status;
   cudaError_t e = launch_rmsnorm(np, sm_budget, stream);
   if (e != cudaSuccess) return cuda_fail("head rmsnorm", e);

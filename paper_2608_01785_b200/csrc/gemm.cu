@@ -23,6 +23,8 @@
 // stream is never read by the SM), QKV (rotate-half RoPE; bf16 q by TMA store; k, v scattered into the
 // paged cache), gate/up (silu(gate) * up -> bf16 by TMA store).  Output blocks are staged in shared memory
 // in the 128-byte-swizzled layout the tensor maps expect (conflict-free for one-row-per-thread writes).
+#include <algorithm>
+
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -203,7 +205,7 @@ struct Unit { int tile, kb_begin, kb_end, seg, last, half; };
 //                     256-row tiles, each unit twice -- once per 128-row half (`half`) -- so that every output
 //                     element still receives the same partial sums in the same order.
 struct UnitWalk {
-  int stream_k, n_tiles, k_blocks, ksplit, n_workers, n_slots;
+  int stream_k, parts, n_tiles, k_blocks, ksplit, n_workers, n_slots;
   int halves, n_m_tiles, M;  // halves = 2: a single block standing in for a pair
   int cur;                 // unit (plain) or slot (stream-K) being handed out
   int idx, n_seg, first_tile;
@@ -211,11 +213,12 @@ struct UnitWalk {
   __device__ __forceinline__ void init(const GemmParams& p, bool pair, bool emulate_pair, int n_m_tiles_, int n_tiles_,
                                        int k_blocks_, int worker, int n_workers_) {
     stream_k = (pair || emulate_pair) && p.mode == kGemmResid && p.stream_k_slots > 0;
+    parts = p.mode == kGemmResid && p.part_rows > 0;
     halves = emulate_pair ? 2 : 1;
     n_m_tiles = n_m_tiles_;
     M = p.M;
     n_tiles = n_tiles_; k_blocks = k_blocks_; n_workers = n_workers_;
-    ksplit = !pair && p.mode == kGemmResid && p.ksplit > 1 ? p.ksplit : 1;
+    ksplit = (!pair || parts) && p.mode == kGemmResid && p.ksplit > 1 ? p.ksplit : 1;
     n_slots = stream_k ? p.stream_k_slots : n_tiles * ksplit;
     cur = worker - n_workers;
     idx = n_seg = 0; first_tile = 0; lo = hi = 0;
@@ -233,8 +236,8 @@ struct UnitWalk {
       if (cur >= n_slots) return false;
       const int ks = cur / n_tiles;
       u.tile = cur - ks * n_tiles;
-      u.kb_begin = gemm_split_begin(k_blocks, ksplit, ks);
-      u.kb_end = gemm_split_begin(k_blocks, ksplit, ks + 1);
+      u.kb_begin = parts ? k_blocks * ks / ksplit : gemm_split_begin(k_blocks, ksplit, ks);
+      u.kb_end = parts ? k_blocks * (ks + 1) / ksplit : gemm_split_begin(k_blocks, ksplit, ks + 1);
       u.seg = ks;
       u.last = ks == ksplit - 1;
       return true;
@@ -311,7 +314,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // Resid mode, whose epilogue adds partial sums into the output in a fixed order.
   UnitWalk walk;
   walk.init(p, PAIR, emulate_pair, n_m_tiles, n_tiles, k_blocks, worker, n_workers);
-  const bool ordered = walk.stream_k || walk.ksplit > 1;
+  const bool ordered = !walk.parts && (walk.stream_k || walk.ksplit > 1);
   Unit un;
 
   if (threadIdx.x == 0) {
@@ -514,7 +517,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           if (lane == 0) go = spin_until_equal(turn, ks, abort_flag, p.status);
           if (!__shfl_sync(0xffffffffu, go, 0)) break;
         }
-        const bool add = p.accumulate || ks > 0;
+        const bool add = !walk.parts && (p.accumulate || ks > 0);
+        const int out_row = walk.parts ? ks * p.part_rows + row_base : row_base;
+        const bool store_ok = !walk.parts || row_base < p.M;      // (a box past the rows would reach into the next split)
         // conditioned block: the product is scaled by the gate vector of the row's sequence before it is added
         const float* gate = p.gate_mod && row_ok ? p.gate_mod + (size_t(p.tok_seq[row]) * 6 + p.gate_which) * p.N : nullptr;
         if (gate) {   // pull this tile's part of the gate vector into the L1 before the chunk loop needs it
@@ -673,7 +678,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           __syncwarp();
           if (lane == 0) {
             if (add) tma_reduce_add_2d(&p.tm_out, buf, col0, row_base);
-            else tma_store_2d(&p.tm_out, buf, col0, row_base);
+            else if (store_ok) tma_store_2d(&p.tm_out, buf, col0, out_row);
             bulk_commit();
           }
           epi_sel ^= 1;
@@ -877,6 +882,51 @@ int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count) {
   return best;
 }
 
+ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows) {
+  // A block (pair) works K blocks of a tile at the slowest of five rates, measured on B200: issue and tensor core (0.20 us per
+  // K block 128 columns wide, 0.27 for 256 and for pairs), what one SM takes in (120 KB/us) and what of it can be weights
+  // from the HBM (68 KB/us: latency against the ring's bytes in flight), what the L2 hands out to all SMs (14.5 MB/us) and
+  // what the HBM delivers (6.2 MB/us of weights, which the row tiles of a column share).  Rounds of one unit per worker,
+  // 2.5 us of start and end, 1.2 us per further round, and the partial sums are read once more (12 MB/us).
+  // What the choice minimises is the time on the whole device plus 0.15 of those on 13/16, 3/4, 13/20 and 1/2 of it, so that
+  // a stage with a neighbour is not left with a short last round.  Measured on B200, K = 18944, N = 3584, by splits x width
+  // (us per launch, events around it): 64 rows on 148 SMs 3 x 128 36.6, 5 x 128 33.7, 10 x 128 34.2, 10 x 256 34.9; 29
+  // rows on 96 SMs 36.5 / 42.3 / 36.9 / 39.1.
+  const int k_blocks = (K + BK - 1) / BK, part_rows = (M + 31) / 32 * 32;
+  ResidPlan best{0, 0, 0, 1e30};
+  for (int form = 0; form < 3; ++form) {                     // single blocks 128 and 256 columns wide, pairs
+    const bool pair = form == 2;
+    if (pair && M <= BM) continue;
+    const int bn = form == 0 ? 128 : 256;
+    const int m_tiles = pair ? (M + 2 * BM - 1) / (2 * BM) : (M + BM - 1) / BM, tiles = m_tiles * ((N + bn - 1) / bn);
+    const double a_bytes = (!pair && M <= 32 ? 32 : !pair && M <= 64 ? 64 : 128) * BK * 2, b_bytes = (pair ? 128 : bn) * BK * 2;
+    for (int ks = 1; ks <= 10 && ks <= k_blocks && ks * part_rows <= part_cap_rows; ++ks) {
+      const int units = tiles * ks, kb = (k_blocks + ks - 1) / ks;
+      double cost = 0.0;
+      for (const int eightieths : {80, 65, 60, 52, 40}) {
+        const int sms = sm_count * eightieths / 80, W = pair ? sms / 2 : sms;
+        if (W < 1) continue;
+        auto round_us = [&](int n) {
+          const double sm = pair ? 2.0 * n : n;
+          double t = pair || bn == 256 ? 0.27 : 0.20;
+          t = std::max(t, (a_bytes + b_bytes) / 120e3);
+          t = std::max(t, b_bytes / m_tiles / 68e3);
+          t = std::max(t, sm * (a_bytes + b_bytes) / 14.5e6);
+          t = std::max(t, sm * b_bytes / m_tiles / 6.2e6);
+          return kb * t;
+        };
+        const int full = units / W, rest = units - full * W;
+        const double us = full * round_us(W) + (rest ? round_us(rest) : 0.0) + 2.5 + 1.2 * (full + (rest ? 1 : 0) - 1) +
+                          double(ks) * part_rows * N * 4.0 / 12e6;
+        cost += eightieths == 80 ? us : 0.15 * us;
+      }
+      if (cost < best.us - 1e-9) best = ResidPlan{pair ? 1 : 0, bn, ks, cost};
+    }
+  }
+  best.us /= 1.6;
+  return best;
+}
+
 int gemm_pick_stream_k(int M, int N, int K, int sm_count) {
   // Whole 256 x 256 tiles on W pairs take ceil(tiles / W) rounds; cutting the K blocks of all tiles into W equal
   // runs takes tiles / W rounds' worth, at the price of a second (ordered) add for the tiles that a cut falls into.
@@ -903,7 +953,8 @@ cudaError_t launch_gemm(const GemmParams& p, int sm_budget, cudaStream_t stream)
   if (p.pair && sm_budget >= 2) {
     // pairs of blocks (clusters of two SMs) on 256 x 256 tiles; an odd budget leaves one SM unused
     const int pair_tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * n_n_tiles;
-    const int pairs = p.mode == kGemmResid && p.stream_k_slots > 0 ? p.stream_k_slots : pair_tiles;
+    const int pairs = p.mode == kGemmResid && p.stream_k_slots > 0 ? p.stream_k_slots
+                      : p.mode == kGemmResid && p.part_rows > 0 && p.ksplit > 1 ? pair_tiles * p.ksplit : pair_tiles;
     const int grid = 2 * (pairs < sm_budget / 2 ? pairs : sm_budget / 2);
     return launch_step_kernel(gemm_pair_kernel, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
   }

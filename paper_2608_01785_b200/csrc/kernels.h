@@ -40,6 +40,9 @@ struct GemmParams {
   int bn;                    // tile width of this launch (gemm_pick_bn); 256 when unused
   int ksplit;                // K splits per output tile, added in split order (gemm_pick_ksplit); 0/1 = none
   int stream_k_slots;        // pairs only: > 0 = cut the tiles' K blocks into this many equal runs (gemm_pick_stream_k)
+  int part_rows;             // > 0: partial sums -- K split ks of the tile goes, unadded, to rows ks * part_rows ... of
+                             // tm_out (a scratch [ksplit * part_rows, N] fp32 matrix; part_rows a multiple of 32, at
+                             // least M), in equal splits; the RMSNorm behind the GEMM adds them (NormParams::part)
   int* tile_turn;            // [tiles * 4] ([tiles * 8] on pairs) whose-turn words for the ordered adds; zero at entry and at exit
   // Qkv
   int q_dim, kv_dim, head_dim, n_kv_heads;
@@ -109,6 +112,11 @@ inline double gemm_ksplit_cost_us(int k_blocks, int ks, int waves) {
 // Runs for the stream-K form of a Resid-mode GEMM on pairs (one per pair of the device), or 0 when whole tiles
 // already fill their waves well enough (budget independent).
 int gemm_pick_stream_k(int M, int N, int K, int sm_count);
+// Form of a residual GEMM whose K splits leave partial sums for the RMSNorm behind it (GemmParams::part_rows): tile width,
+// pairs or single blocks, and the number of splits, or ks = 0 when no form fits `part_cap_rows` rows of scratch.  `us` is
+// the modelled time with the extra reading of the partials.  A function of the shape and the device's SM count only.
+struct ResidPlan { int pair, bn, ks; double us; };
+ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows);
 // The same three GEMMs for steps of at most 64 rows (gemm_skinny.cu): weight streaming on plain loads and
 // warp-level MMAs, one block per 32 output columns and the whole K range, no K split across blocks.
 struct SkinnyParams {
@@ -155,6 +163,7 @@ struct SkinnyParams {
 };
 // True when the skinny kernel covers this shape (few rows, K a multiple of 32, widths it can tile).
 bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim);
+double gemm_skinny_cost_us(int T, int K, int N, int mode, int sm_count);
 // True when it is also expected to be faster than the tiled kernel for this shape (budget independent).
 bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count);
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream);
@@ -179,12 +188,22 @@ struct NormParams {
   const float* mod;
   const int32_t* tok_seq;
   int mod_which;
+  // optional partial sums of the residual GEMM in front (GemmParams::part_rows): x += gate * (part[0] + part[1] + ...),
+  // added in split order, written to x_f32_out; gate_which > 0 takes the gate vector from `mod_gate` (the layer's vectors
+  // the branch belongs to), else the gate is 1.  h null: only this sum is formed.
+  const float* part;         // [n_parts][part_stride] floats, rows of d
+  int n_parts;
+  size_t part_stride;
+  const float* mod_gate;
+  int gate_which;
+  int sm_count;              // > 0: SMs of the device, for the choice of the kernel (never the budget)
   int h_f16;                 // 1 = write h as fp16, 0 = bf16
   int overlap;               // OverlapMode: how the launch overlaps the previous kernel's drain
   int* status;               // device status word (bounded waits report HS_ERR_TIMEOUT here)
   int* smid_log;             // nullable: SM census slots of this launch
 };
 cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stream);
+constexpr int kNormRowMaxD = 512 * 8 * 4;    // widest row of the kernel that adds partial sums
 
 // Embedding lookup and greedy sampling (head.cu).
 struct EmbedParams {

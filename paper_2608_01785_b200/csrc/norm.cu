@@ -259,6 +259,117 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
   if (!ok) drain_after_abort();
 }
 
+// The same operation for steps of few rows, and the one that adds the partial sums of a K-split residual GEMM first: TPR
+// threads work on a row (as many as leave one round of rows on the device, at most 512), each holds its V groups of
+// four columns in registers, so a launch is one round trip to memory, one reduction and one write.  What bounds it is
+// that latency: one warp per row (the kernel above) took 8.2 us per launch at 64 x 3584 and 9.3 us at 1024 x 1024
+// (conditioned), this one 5.4 us with three partial sums to add and 9.5-10 with two (ncu).  Sums: a thread's groups in order, a butterfly per warp, the warps in
+// order -- a function of the shape and the device's SM count, never of the budget.
+constexpr int ROW_THREADS = 512;
+
+template <int V>
+__global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormParams p, int tpr) {
+  constexpr int PB = V >= 8 ? 2 : V >= 4 ? 4 : 8;      // partial sums requested at a time (V * PB groups in flight)
+  extern __shared__ uint8_t row_unused_smem[];
+  __shared__ float red[2][ROW_THREADS / 32];
+  log_smid(p.smid_log);
+  const int rows_per_block = ROW_THREADS / tpr, group = threadIdx.x / tpr, tid = threadIdx.x - group * tpr;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps_per_row = tpr >> 5, first_warp = group * warps_per_row;
+  const int d4 = p.d >> 2;
+  uint2 gw[V];                                         // gains are weights: fetched before the wait
+#pragma unroll
+  for (int v = 0; v < V; ++v)
+    gw[v] = p.h && tid + v * tpr < d4 ? __ldg(reinterpret_cast<const uint2*>(p.gain) + tid + v * tpr) : make_uint2(0u, 0u);
+  griddep_wait();
+  griddep_launch_dependents(p.overlap);
+  const bool f16 = p.h_f16 != 0;
+  int phase = 0;
+  for (int row = blockIdx.x * rows_per_block + group; row < p.T; row += gridDim.x * rows_per_block, phase ^= 1) {
+    const int src_row = p.row_index ? p.row_index[row] : row;
+    float4 a[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int i = tid + v * tpr;
+      a[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < d4) {
+        if (p.x_bf16) {
+          const uint2 w = reinterpret_cast<const uint2*>(p.x_bf16 + size_t(src_row) * p.d)[i];
+          a[v] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                             __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+        } else {
+          a[v] = __ldcg(reinterpret_cast<const float4*>(p.x_f32 + size_t(src_row) * p.d) + i);
+        }
+      }
+    }
+    const int seq = p.mod || p.gate_which > 0 ? p.tok_seq[row] : 0;
+    if (p.n_parts > 0) {
+      float4 s[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) s[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k0 = 0; k0 < p.n_parts; k0 += PB) {
+        float4 q[PB][V];
+#pragma unroll
+        for (int k = 0; k < PB; ++k)
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            q[k][v] = k0 + k < p.n_parts && tid + v * tpr < d4
+                          ? __ldcg(reinterpret_cast<const float4*>(p.part + (k0 + k) * p.part_stride + size_t(row) * p.d) + tid + v * tpr)
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < PB; ++k)
+#pragma unroll
+          for (int v = 0; v < V; ++v) { s[v].x += q[k][v].x; s[v].y += q[k][v].y; s[v].z += q[k][v].z; s[v].w += q[k][v].w; }
+      }
+      if (p.gate_which > 0) {                          // conditioned block: the branch is scaled by its gate vector
+        const float4* gate = reinterpret_cast<const float4*>(p.mod_gate + (size_t(seq) * 6 + p.gate_which) * p.d);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (tid + v * tpr < d4) {
+            const float4 g = __ldg(gate + tid + v * tpr);
+            s[v].x *= g.x; s[v].y *= g.y; s[v].z *= g.z; s[v].w *= g.w;
+          }
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) { a[v].x += s[v].x; a[v].y += s[v].y; a[v].z += s[v].z; a[v].w += s[v].w; }
+    }
+    if (p.n_parts > 0 || p.x_bf16) {
+      float4* xo = reinterpret_cast<float4*>(p.x_f32_out + size_t(row) * p.d);
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (tid + v * tpr < d4) xo[tid + v * tpr] = a[v];
+    }
+    if (!p.h) continue;
+    float ss = 0.f;
+#pragma unroll
+    for (int v = 0; v < V; ++v) ss += (a[v].x * a[v].x + a[v].y * a[v].y) + (a[v].z * a[v].z + a[v].w * a[v].w);
+    ss = warp_sum(ss);
+    if (warps_per_row > 1) {                           // (the row's warps meet in shared memory; two buffers, one barrier)
+      if (lane == 0) red[phase][warp] = ss;
+      named_barrier_sync(1 + group, tpr);
+      ss = 0.f;
+      for (int w = 0; w < warps_per_row; ++w) ss += red[phase][first_warp + w];
+    }
+    const float r = rsqrtf(ss / float(p.d) + p.eps);
+    uint2* hdst = reinterpret_cast<uint2*>(p.h + size_t(row) * p.d);
+    const float4* shift = p.mod ? reinterpret_cast<const float4*>(p.mod + (size_t(seq) * 6 + p.mod_which) * p.d) : nullptr;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int i = tid + v * tpr;
+      if (i < d4) {
+        float v4[4] = {a[v].x * r * __uint_as_float(gw[v].x << 16), a[v].y * r * __uint_as_float(gw[v].x & 0xffff0000u),
+                       a[v].z * r * __uint_as_float(gw[v].y << 16), a[v].w * r * __uint_as_float(gw[v].y & 0xffff0000u)};
+        if (shift) {                                   // conditioned block: (1 + scale) and shift of the row's sequence
+          const float4 sh = __ldg(shift + i), sc = __ldg(shift + d4 + i);
+          v4[0] = fmaf(v4[0], 1.f + sc.x, sh.x); v4[1] = fmaf(v4[1], 1.f + sc.y, sh.y);
+          v4[2] = fmaf(v4[2], 1.f + sc.z, sh.z); v4[3] = fmaf(v4[3], 1.f + sc.w, sh.w);
+        }
+        if (f16 && p.status) note_f16_saturation(v4, p.status);
+        hdst[i] = make_uint2(pack_act(v4[0], v4[1], f16), pack_act(v4[2], v4[3], f16));
+      }
+    }
+  }
+}
+
 // One-time widening of the significand: bf16 weights -> fp16 copies (n8 groups of 8 values).  A bf16 value
 // is an fp16 value exactly when 2^-17 <= |w| <= 65504; smaller ones round to the fp16 subnormal grid
 // (absolute error <= 2^-25), larger ones saturate.
@@ -285,12 +396,28 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_
 cudaError_t norm_set_attributes() {
   cudaError_t e = set_kernel_smem(rmsnorm_kernel, NORM_SMEM);
   if (e != cudaSuccess) return e;
+  if ((e = set_kernel_smem(rmsnorm_row_kernel<1>, kMinSmemBytes)) != cudaSuccess) return e;
+  if ((e = set_kernel_smem(rmsnorm_row_kernel<2>, kMinSmemBytes)) != cudaSuccess) return e;
+  if ((e = set_kernel_smem(rmsnorm_row_kernel<4>, kMinSmemBytes)) != cudaSuccess) return e;
+  if ((e = set_kernel_smem(rmsnorm_row_kernel<8>, kMinSmemBytes)) != cudaSuccess) return e;
   if ((e = set_kernel_smem(rmsnorm_bulk_kernel<false>, 512 + BULK_SMEM_BUDGET)) != cudaSuccess) return e;
   return set_kernel_smem(rmsnorm_bulk_kernel<true>, 512 + BULK_SMEM_BUDGET);
 }
 
 cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stream) {
   if (p.T <= 0) return cudaSuccess;
+  // few rows (one round of them on the whole device), or partial sums to add: many threads per row
+  if (p.d <= kNormRowMaxD) {
+    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2;
+    int tpr = ROW_THREADS;
+    while (tpr > 32 && (p.T + ROW_THREADS / tpr - 1) / (ROW_THREADS / tpr) > sms && (d4 + tpr / 2 - 1) / (tpr / 2) <= 8) tpr >>= 1;
+    const int rows_per_block = ROW_THREADS / tpr, blocks = (p.T + rows_per_block - 1) / rows_per_block;
+    if (p.n_parts > 0 || (p.sm_count > 0 && blocks <= sms)) {
+      const int grid = blocks < sm_budget ? blocks : sm_budget, V = (d4 + tpr - 1) / tpr;
+      auto kernel = V <= 1 ? rmsnorm_row_kernel<1> : V <= 2 ? rmsnorm_row_kernel<2> : V <= 4 ? rmsnorm_row_kernel<4> : rmsnorm_row_kernel<8>;
+      return launch_step_kernel(kernel, grid, ROW_THREADS, kMinSmemBytes, stream, p.overlap != 0, p, tpr);
+    }
+  }
   // bulk-staged variant: as many warps as have room for two fp32 rows each (a function of d alone, never of
   // the budget); rows too wide for four warps fall back to the register-staged kernel
   const size_t pair_bytes = size_t(p.d) * 4 * 2, gain_bytes = size_t(p.d) * 2;

@@ -373,9 +373,9 @@ __device__ __forceinline__ void griddep_launch_dependents(int overlap) {
 // Host side: launches `kernel`; with `overlap` set, the launch carries the programmatic-stream-serialisation
 // attribute, i.e. its blocks may become resident (and run up to griddep_wait()) as soon as every block of the
 // previous kernel of the stream has triggered or left.
-template <typename P>
-inline cudaError_t launch_step_kernel(void (*kernel)(P), int grid, int block, size_t smem, cudaStream_t stream,
-                                      bool overlap, const P& params) {
+template <typename... P>
+inline cudaError_t launch_step_kernel(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream,
+                                      bool overlap, const P&... params) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid), 1, 1);
   cfg.blockDim = dim3(unsigned(block), 1, 1);
@@ -386,7 +386,7 @@ inline cudaError_t launch_step_kernel(void (*kernel)(P), int grid, int block, si
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, params);
+  return cudaLaunchKernelEx(&cfg, kernel, params...);
 }
 
 // Host side: lets `kernel` use `bytes` of dynamic shared memory and asks for the largest shared-memory
