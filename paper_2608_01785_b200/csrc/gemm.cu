@@ -297,11 +297,11 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint64_t* xbar = reinterpret_cast<uint64_t*>(epi_smem + 4 * EPI_WARP_BYTES + 256);   // [4 warps][4] landing-block barriers (three used)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   log_smid(p.smid_log);
   // In pair mode the two blocks of a cluster share every work unit: a unit's tile is 256 rows tall and
   // block `rank` owns rows 128 * rank .. 128 * rank + 127 of it.
-  const uint32_t rank = PAIR ? cluster_ctarank() : 0;
+  const uint32_t rank = PAIR ? blockIdx.x & 1 : 0;              // (clusters of two along x)
   const int worker = PAIR ? int(blockIdx.x >> 1) : int(blockIdx.x);
   const int n_workers = PAIR ? int(gridDim.x >> 1) : int(gridDim.x);
   // a single block that stands in for a pair (stream-K form at sm_budget 1) walks the pair's 256-row tiles
@@ -346,7 +346,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   __syncthreads();
   if (PAIR) cluster_sync_all();               // the other block's barriers exist before anything targets them
   tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   // A small step's A box holds only the rows that exist (32 or 64 instead of 128): the MMA still reads 128
   // rows starting at the stage's base -- beyond the A box that is the B data of the stage, finite values
   // that only reach accumulator rows no epilogue stores
@@ -373,42 +373,49 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // for the previous kernel, and for the A boxes of those stages after it.
   bool have_unit = false;
   int b_ahead = 0;
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     have_unit = walk.next(un);
     if (have_unit) {
       const int n = un.tile / n_m_tiles;
       const BSource b0 = b_source(p, n, PAIR ? int(rank) : 0), b1 = b_source(p, n, 1);
       b_ahead = un.kb_end - un.kb_begin < STAGES ? un.kb_end - un.kb_begin : STAGES;
-      for (int i = 0; i < b_ahead; ++i) load_b(i, un.kb_begin + i, b0, b1);
+      if (elect_one())
+        for (int i = 0; i < b_ahead; ++i) load_b(i, un.kb_begin + i, b0, b1);
     }
   }
   griddep_wait();                 // everything above is set-up; the operands belong to the previous kernel until here
   griddep_launch_dependents(p.overlap);
 
+  // The producer and the MMA issuer are whole warps in uniform control flow, one elected lane issuing: the descriptors,
+  // coordinates and barrier addresses then live in uniform registers.  With a loop inside `if (lane == 0)` every
+  // instruction fetched its operands through a move of its own, about 60 cycles per MMA, and the issuing thread was
+  // what bounded the main loop (it never waited for data): 565 cycles per 64-wide K block for 128 columns and for pairs
+  // alike; now 405 and 520 (a pair's tensor time is 512).
   if (warp == 0) {
     // ------------------------------------------------------- TMA producer --
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      while (ok && have_unit) {
-        const int tile = un.tile;
-        const int m = tile % n_m_tiles, n = tile / n_m_tiles;
-        const BSource b0 = b_source(p, n, PAIR ? int(rank) : 0), b1 = b_source(p, n, 1);
-        const int kb_end = un.kb_end;
-        for (int kb = un.kb_begin; kb < kb_end; ++kb) {
-          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-          if (b_ahead > 0) --b_ahead;
-          else load_b(s, kb, b0, b1);
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    while (ok && have_unit) {
+      const int tile = un.tile;
+      const int m = tile % n_m_tiles, n = tile / n_m_tiles;
+      const BSource b0 = b_source(p, n, PAIR ? int(rank) : 0), b1 = b_source(p, n, 1);
+      const int kb_end = un.kb_end;
+      for (int kb = un.kb_begin; kb < kb_end; ++kb) {
+        ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        if (elect_one()) {
+          if (b_ahead == 0) load_b(s, kb, b0, b1);
           load_a(s, kb, m, un.half);
-          if (++s == STAGES) { s = 0; ph ^= 1; }
         }
-        have_unit = walk.next(un);
+        if (b_ahead > 0) --b_ahead;
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
+      have_unit = walk.next(un);
     }
   } else if (warp == 1) {
     // --------------------------------------------------------- MMA issuer --
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
@@ -419,38 +426,35 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       bool ok = true;
       const uint64_t a_desc0 = umma_desc_kmajor_sw128(smem_u32(smem));
       while (ok && walk.next(un)) {
-        if (!mbar_wait(&tempty[acc], acc_ph ^ 1, abort_flag, p.status)) break;
+        ok = mbar_wait(&tempty[acc], acc_ph ^ 1, abort_flag, p.status);
+        if (!__all_sync(0xffffffffu, ok)) break;
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * BN;
         const int kb_begin = un.kb_begin, kb_end = un.kb_end;
         for (int kb = kb_begin; kb < kb_end; ++kb) {
-          if (!mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
+          ok = mbar_wait(&full[s], ph, abort_flag, p.status);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           tc_fence_after_sync();
           // descriptors of stage s: those of stage 0 plus the stage's offset in the address field (units of 16 bytes;
-          // shared memory is below 256 KB, so nothing carries out of the field): the issuing thread has as little as
-          // possible between two MMAs
+          // shared memory is below 256 KB, so nothing carries out of the field)
           const uint64_t a_desc = a_desc0 + uint64_t(s * (STAGE_BYTES >> 4));
           const uint64_t b_desc = a_desc + uint64_t(b_off >> 4);
           const uint32_t acc0 = kb != kb_begin ? 1u : 0u;
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {  // 16 bf16 = 32 B along K: +2 in the (address / 16) field
-            if (PAIR) umma_bf16_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : acc0);
-            else umma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : acc0);
-          }
-          // frees the stage (in both blocks) once these MMAs have read it
-          if (PAIR) {
-            umma_commit_pair_both(&empty[s]);
-          } else {
-            umma_commit(&empty[s]);
+            for (int k = 0; k < BK / 16; ++k) {  // 16 bf16 = 32 B along K: +2 in the (address / 16) field
+              if (PAIR) umma_bf16_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : acc0);
+              else umma_bf16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : acc0);
+            }
+            // frees the stage (in both blocks) once these MMAs have read it
+            if (PAIR) umma_commit_pair_both(&empty[s]);
+            else umma_commit(&empty[s]);
           }
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
-        if (ok) {
-          if (PAIR) {
-            umma_commit_pair_both(&tfull[acc]);
-          } else {
-            umma_commit(&tfull[acc]);
-          }
+        if (ok && elect_one()) {
+          if (PAIR) umma_commit_pair_both(&tfull[acc]);
+          else umma_commit(&tfull[acc]);
         }
         acc ^= 1;
         if (acc == 0) acc_ph ^= 1;
