@@ -24,6 +24,7 @@
 // paged cache), gate/up (silu(gate) * up -> bf16 by TMA store).  Output blocks are staged in shared memory
 // in the 128-byte-swizzled layout the tensor maps expect (conflict-free for one-row-per-thread writes).
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 #include "ptx.cuh"
@@ -271,18 +272,19 @@ struct UnitWalk {
   }
 };
 
-template <bool PAIR>
+// (one instantiation per mode: an epilogue does not pay with registers for the others)
+template <bool PAIR, int MODE>
 __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // Ring geometry.  Pairs: 6 stages of 32 KB.  Single blocks: a stage holds the A box (128 rows, or only 64 / 32
   // when the step is that small) and one or two 128-row B boxes, and the ring holds as many stages as fit (at
   // most kMaxStages): a block's streaming rate is stages in flight / memory latency, so the small stages of a
   // small step buy depth -- 8 or 9 stages instead of 4.
-  const bool b_two = p.mode == kGemmGateUp || (p.mode == kGemmResid ? p.bn : gemm_qkv_width(p)) > 128;
+  const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) > 128;
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
   const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * BH_BYTES;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
-  const bool fold_pair = PAIR && p.mode == kGemmResid && p.norm_gain != nullptr;
+  const bool fold_pair = PAIR && MODE == kGemmResid && p.norm_gain != nullptr;
   const int STAGES = PAIR ? Ring<true>::STAGES - (fold_pair ? 1 : 0)
                           : (RING_BYTES / STAGE_BYTES < kMaxStages ? RING_BYTES / STAGE_BYTES : kMaxStages);
   const int b_off = PAIR ? A_BYTES : a_bytes;     // B boxes follow the A box inside a stage
@@ -305,7 +307,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   const int worker = PAIR ? int(blockIdx.x >> 1) : int(blockIdx.x);
   const int n_workers = PAIR ? int(gridDim.x >> 1) : int(gridDim.x);
   // a single block that stands in for a pair (stream-K form at sm_budget 1) walks the pair's 256-row tiles
-  const bool emulate_pair = !PAIR && p.pair && p.mode == kGemmResid && p.stream_k_slots > 0;
+  const bool emulate_pair = !PAIR && p.pair && MODE == kGemmResid && p.stream_k_slots > 0;
   const int n_m_tiles = PAIR || emulate_pair ? (p.M + 2 * BM - 1) / (2 * BM) : (p.M + BM - 1) / BM;
   const int n_n_tiles = gemm_n_tiles(p);
   const int n_tiles = n_m_tiles * n_n_tiles;
@@ -331,7 +333,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     fence_barrier_init();
     tma_prefetch_desc(&p.tm_a);
     tma_prefetch_desc(&p.tm_b[0]);
-    tma_prefetch_desc(p.mode == kGemmResid ? &p.tm_out : p.mode == kGemmQkv ? &p.tm_q : &p.tm_act);
+    tma_prefetch_desc(MODE == kGemmResid ? &p.tm_out : MODE == kGemmQkv ? &p.tm_q : &p.tm_act);
   }
   if (warp == 1) {
     if (PAIR) {
@@ -419,7 +421,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
-                                                 PAIR ? BN : p.mode == kGemmResid ? p.bn : p.mode == kGemmQkv ? gemm_qkv_width(p) : BN) &
+                                                 PAIR ? BN : MODE == kGemmResid ? p.bn : MODE == kGemmQkv ? gemm_qkv_width(p) : BN) &
                              (p.ab_f16 ? ~(63u << 7) : ~0u);
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
@@ -479,7 +481,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       const int row_base = m * BM + quarter * 32;          // first row of this warp's 32
       // folded RMSNorm, consuming side: r of this thread's row, requested before the wait for the accumulator
       float rs = 1.f;
-      if (p.in_row_rs != nullptr && p.mode != kGemmResid && row_ok) rs = __ldcg(p.in_row_rs + row);
+      if (p.in_row_rs != nullptr && MODE != kGemmResid && row_ok) rs = __ldcg(p.in_row_rs + row);
       // folded RMSNorm, producing side: the first two blocks of this warp's rows of y are on their way before the
       // tile's products are complete
       const bool fold_now = fold_pair && un.last;
@@ -511,7 +513,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       float v0[32], v1[32];
 
 
-      if (p.mode == kGemmResid) {
+      if (MODE == kGemmResid) {
         // Ordered split-K: the partial sums of a tile are added into the output in split order, so the
         // result is the same fixed sum whatever block computed which split.  This warp owns 32 rows of the
         // tile; it waits until the previous split's add of those rows has been performed.
@@ -692,7 +694,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           __threadfence();
           st_release(turn, un.last ? 0 : ks + 1);   // the last segment leaves the word at zero
         }
-      } else if (p.mode == kGemmGateUp) {
+      } else if (MODE == kGemmGateUp) {
         for (int c = 0; c < 4; ++c) {
           const int col0 = n * 128 + c * 32;
           if (col0 >= p.N) break;
@@ -825,21 +827,34 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   }
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
-  gemm_body<false>(p);
+  gemm_body<false, MODE>(p);
 }
 // Two blocks per cluster, one 256 x 256 tile per pair.
+template <int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ GemmParams p) {
-  gemm_body<true>(p);
+  gemm_body<true, MODE>(p);
+}
+
+template <typename F>
+auto by_mode(int mode, F f) {
+  return mode == kGemmResid ? f(std::integral_constant<int, kGemmResid>()) : mode == kGemmQkv ? f(std::integral_constant<int, kGemmQkv>())
+                                                                                             : f(std::integral_constant<int, kGemmGateUp>());
 }
 
 }  // namespace
 
 cudaError_t gemm_set_attributes() {
-  cudaError_t e = set_kernel_smem(gemm_pair_kernel, GEMM_SMEM);
-  if (e != cudaSuccess) return e;
-  return set_kernel_smem(gemm_kernel, GEMM_SMEM);
+  for (const int mode : {kGemmResid, kGemmQkv, kGemmGateUp}) {
+    const cudaError_t e = by_mode(mode, [](auto m) {
+      const cudaError_t e1 = set_kernel_smem(gemm_pair_kernel<decltype(m)::value>, GEMM_SMEM);
+      return e1 != cudaSuccess ? e1 : set_kernel_smem(gemm_kernel<decltype(m)::value>, GEMM_SMEM);
+    });
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 int gemm_pick_bn(int M, int N, int sm_count) {
@@ -960,10 +975,14 @@ cudaError_t launch_gemm(const GemmParams& p, int sm_budget, cudaStream_t stream)
     const int pairs = p.mode == kGemmResid && p.stream_k_slots > 0 ? p.stream_k_slots
                       : p.mode == kGemmResid && p.part_rows > 0 && p.ksplit > 1 ? pair_tiles * p.ksplit : pair_tiles;
     const int grid = 2 * (pairs < sm_budget / 2 ? pairs : sm_budget / 2);
-    return launch_step_kernel(gemm_pair_kernel, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
+    return by_mode(p.mode, [&](auto m) {
+      return launch_step_kernel(gemm_pair_kernel<decltype(m)::value>, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
+    });
   }
   const int grid = n_tiles < sm_budget ? n_tiles : sm_budget;
-  return launch_step_kernel(gemm_kernel, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
+  return by_mode(p.mode, [&](auto m) {
+    return launch_step_kernel(gemm_kernel<decltype(m)::value>, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
+  });
 }
 
 }  // namespace hs
