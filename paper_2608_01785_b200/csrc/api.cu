@@ -1109,7 +1109,7 @@ size_t head_status_offset(const hs_head_config_t& c) { return align_up(size_t(c.
 
 size_t hs_head_workspace_bytes(const hs_head_config_t* cfg) {
   if (!cfg || !head_config_ok(*cfg)) return 0;
-  return head_status_offset(*cfg) + 1024;
+  return head_status_offset(*cfg) + 4096;      // status words, sampling keys of at most 128 rows, their counter
 }
 
 hs_status_t hs_head_create(const hs_head_config_t* cfg, const void* g_final, const void* w_vocab, void* workspace_dev,
@@ -1138,7 +1138,7 @@ hs_status_t hs_head_create(const hs_head_config_t* cfg, const void* g_final, con
   if (!encode_2d(&h->tm_h, h->ws_dev, cfg->max_rows, cfg->d_model, 128) ||
       !encode_2d(&h->tm_w, w_vocab, cfg->vocab, cfg->d_model, 128))
     return HS_ERR_CUDA;
-  if (cudaMemset(h->ws_dev + h->off_status, 0, 256) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+  if (cudaMemset(h->ws_dev + h->off_status, 0, 4096) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
     return HS_ERR_CUDA;
   *out = h.release();
   return HS_OK;
@@ -1165,6 +1165,8 @@ hs_status_t hs_head_step(hs_head_t* h, const float* y, const int32_t* rows, int3
   np.row_index = rows;
   np.sm_count = h->sm_count;
   np.status = status;
+  const int overlap = sm_budget == h->sm_count ? kOverlapEarly : kOverlapLate;
+  np.overlap = overlap;
   cudaError_t e = launch_rmsnorm(np, sm_budget, stream);
   if (e != cudaSuccess) return cuda_fail("head rmsnorm", e);
 
@@ -1179,16 +1181,13 @@ hs_status_t hs_head_step(hs_head_t* h, const float* y, const int32_t* rows, int3
   g.bn = gemm_pick_bn(n, V, h->sm_count);
   g.ksplit = 1;
   g.status = status;
+  g.overlap = overlap;
+  // greedy sampling in the epilogue: a kernel of its own read the logits once more (65 rows: 22 us of 237)
+  g.argmax_key = reinterpret_cast<unsigned long long*>(h->ws_dev + h->off_status + 1024);
+  g.argmax_done = reinterpret_cast<int*>(h->ws_dev + h->off_status + 2048);
+  g.argmax_token = tokens;
   e = launch_gemm(g, sm_budget, stream);
-  if (e != cudaSuccess) return cuda_fail("head gemm", e);
-
-  ArgmaxParams a{};
-  a.logits = logits;
-  a.tokens = tokens;
-  a.n = n;
-  a.vocab = V;
-  e = launch_argmax(a, sm_budget, stream);
-  return e == cudaSuccess ? HS_OK : cuda_fail("head argmax", e);
+  return e == cudaSuccess ? HS_OK : cuda_fail("head gemm", e);
 }
 
 hs_status_t hs_head_status(hs_head_t* h) {

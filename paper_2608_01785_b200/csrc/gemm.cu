@@ -655,7 +655,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           if (lane == 0) bulk_wait_read<0>();         // the staging blocks go back to the alternating use below
           __syncwarp();
           epi_sel = 0;
-        } else
+        } else {
+        float best_v = -INFINITY;              // greedy sampling: this thread's row over the tile
+        int best_c = 0x7fffffff;
         for (int c = 0; c < p.bn / 32; ++c) {
           const int col0 = n * p.bn + c * 32;
           if (col0 >= p.N) break;
@@ -676,6 +678,19 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
               r0[4 * e + 3] = __float_as_uint(__uint_as_float(r0[4 * e + 3]) * gv[e].w);
             }
           }
+          if (!PAIR && p.argmax_key != nullptr) {
+            // (N is a multiple of 8; a NaN is never the maximum; columns ascend, so the first maximum stays)
+            float mx = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+              if (col0 + (e & ~7) < p.N) mx = fmaxf(mx, __uint_as_float(r0[e]));
+            if (mx > best_v || best_c == 0x7fffffff) {
+#pragma unroll
+              for (int e = 31; e >= 0; --e)
+                if (col0 + (e & ~7) < p.N && __uint_as_float(r0[e]) == mx) best_c = col0 + e;
+              best_v = mx;
+            }
+          }
           if (lane == 0) bulk_wait_read<1>();     // the block staged two chunks ago has been read
           __syncwarp();
           uint8_t* buf = epi_buf + epi_sel * EPI_BUF_BYTES;
@@ -688,6 +703,13 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
             bulk_commit();
           }
           epi_sel ^= 1;
+        }
+        if (!PAIR && p.argmax_key != nullptr && row_ok) {
+          const uint32_t u = __float_as_uint(best_v + 0.f);                       // (-0 and +0 are the same value)
+          const uint32_t ord = u & 0x80000000u ? ~u : u | 0x80000000u;
+          atomicMax(p.argmax_key + row, (static_cast<unsigned long long>(ord) << 32) | (0xffffffffu - uint32_t(best_c)));
+          __threadfence();
+        }
         }
         if (ordered && !(ks == 0 && un.last) && lane == 0) {    // a tile with a single segment needs no turn
           bulk_wait<0>();                     // this segment's adds have been performed
@@ -819,6 +841,20 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   if (*abort_flag) drain_after_abort();
   tc_fence_before_sync();
   __syncthreads();
+  if (!PAIR && MODE == kGemmResid && p.argmax_key != nullptr && warp == 2) {   // the last block to leave turns the keys into tokens
+    int last = 0;
+    if (lane == 0) {
+      __threadfence();
+      last = atomicAdd(p.argmax_done, 1) == int(gridDim.x) - 1;
+    }
+    if (__shfl_sync(0xffffffffu, last, 0)) {
+      __threadfence();
+      for (int r = lane; r < p.M; r += 32) {
+        p.argmax_token[r] = int32_t(0xffffffffu - uint32_t(atomicExch(p.argmax_key + r, 0ull)));
+      }
+      if (lane == 0) *p.argmax_done = 0;
+    }
+  }
   if (PAIR) cluster_sync_all();               // neither block leaves while the other may still reach into it
   if (warp == 1) {
     tc_fence_after_sync();

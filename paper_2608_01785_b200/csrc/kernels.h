@@ -40,6 +40,12 @@ struct GemmParams {
   int bn;                    // tile width of this launch (gemm_pick_bn); 256 when unused
   int ksplit;                // K splits per output tile, added in split order (gemm_pick_ksplit); 0/1 = none
   int stream_k_slots;        // pairs only: > 0 = cut the tiles' K blocks into this many equal runs (gemm_pick_stream_k)
+  // Resid in store mode on single blocks, optional: greedy sampling of every row (argmax_key non-null).  The tile's epilogue, which holds the
+  // values in registers, maximises the row's key -- order-preserving bits of the value above the complement of the
+  // column, so that the first maximum wins whatever the order -- and the block that leaves last turns the keys into tokens.
+  unsigned long long* argmax_key;   // [M], zero at entry and at exit
+  int* argmax_done;          // one counter, zero at entry and at exit
+  int32_t* argmax_token;     // [M]: lowest column of the row's maximum
   int part_rows;             // > 0: partial sums -- K split ks of the tile goes, unadded, to rows ks * part_rows ... of
                              // tm_out (a scratch [ksplit * part_rows, N] fp32 matrix; part_rows a multiple of 32, at
                              // least M), in equal splits; the RMSNorm behind the GEMM adds them (NormParams::part)
@@ -205,7 +211,7 @@ struct NormParams {
 cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stream);
 constexpr int kNormRowMaxD = 512 * 8 * 4;    // widest row of the kernel that adds partial sums
 
-// Embedding lookup and greedy sampling (head.cu).
+// Embedding lookup (head.cu).
 struct EmbedParams {
   const int32_t* tokens;           // device [n]
   const __nv_bfloat16* table;      // [vocab, d]
@@ -213,14 +219,8 @@ struct EmbedParams {
   int n, vocab, d;
   int* status;                     // receives HS_ERR_INVALID_ARG for an id outside the table
 };
-struct ArgmaxParams {
-  const float* logits;             // [n, vocab]
-  int32_t* tokens;                 // [n]: lowest index of each row's maximum
-  int n, vocab;
-};
 cudaError_t head_set_attributes();
 cudaError_t launch_embed(const EmbedParams& p, int sm_budget, cudaStream_t stream);
-cudaError_t launch_argmax(const ArgmaxParams& p, int sm_budget, cudaStream_t stream);
 // dst[i] = fp16(src[i]) for n bf16 values (n a multiple of 8, both 16-byte aligned); used once per weight
 // matrix when a stage is created
 cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_t stream);

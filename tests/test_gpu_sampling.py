@@ -1,0 +1,40 @@
+"""Greedy sampling in the vocabulary GEMM's epilogue: the token is the first maximum of the logits the call wrote, at the
+edges of its column tiles and row boxes, in call after call, and for rows without a maximum."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_01785_b200 import binding as B
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("V,n", [(8, 1), (264, 33), (1032, 65), (40008, 128)])
+def test_tokens_are_the_first_maximum_of_the_logits(V, n):
+    dev = torch.device("cuda:0")
+    d = 256
+    g = torch.Generator().manual_seed(V + n)
+    gain = torch.ones(d, dtype=torch.bfloat16, device=dev)
+    w = (0.02 * torch.randn(V, d, generator=g)).to(torch.bfloat16)
+    w[V // 2:V // 2 + 2] = w[:2]                      # exact ties
+    w = w.to(dev)
+    cfg = B.make_head_config(d, V, 1e-6, 128)
+    ws = torch.empty(B.hs_head_workspace_bytes(cfg), dtype=torch.uint8, device=dev)
+    head = B.hs_head_create(cfg, gain.data_ptr(), w.data_ptr(), ws.data_ptr())
+    try:
+        rows = torch.arange(n, dtype=torch.int32, device=dev)
+        for rep, budget in enumerate((148, 148, 5, 1)):
+            y = torch.randn(n, d, generator=g)
+            if rep == 1:
+                y[n - 1] = float("inf")               # its logits are NaN: no maximum, and no trace in the next call
+            y = y.to(dev)
+            logits = torch.empty(n, V, device=dev)
+            tokens = torch.full((n,), -7, dtype=torch.int32, device=dev)
+            B.hs_head_step(head, y.data_ptr(), rows.data_ptr(), n, logits.data_ptr(), tokens.data_ptr(), budget)
+            torch.cuda.synchronize()
+            want = np.argmax(logits.cpu().numpy(), axis=1).astype(np.int32)
+            if rep == 1:
+                assert bool(torch.isnan(logits[n - 1]).all())
+                want[n - 1] = 0x7fffffff
+            assert np.array_equal(tokens.cpu().numpy(), want)
+    finally:
+        B.hs_head_destroy(head)
