@@ -26,7 +26,6 @@ namespace hs {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLazyMax = 8.f;         // the softmax reference moves when a score exceeds it by this much (log2 units)
 
 template <int DH>
 struct Geom {
@@ -292,12 +291,13 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
 
     // A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
     // bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs per key
-    // half, the V fragments are fetched while the scores are on their way, and the exponentials are taken against a reference that follows the running maximum only when a score exceeds it by more than 8 in
-    // log2 units (the sum uses the same reference, so O / l is the same quotient): no shuffles and no rescale for most
-    // pages.  Against a loop with one chain of MMAs, a running maximum moved on every page (four shuffles, exp2f) and V
-    // fetched behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker
-    // step of 16 rows 300.5 -> 287.6 us, of 11 rows on 52 SMs 471 -> 448; at config-3 dimensions 9 rows, 4 layers 493 ->
-    // 482 us, 29 rows on 96 SMs 796 -> 779, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.15 ms.
+    // half, the V fragments are fetched while the scores are on their way, and a page on which no row's maximum moves --
+    // most of them, after the first few -- needs a vote, but no shuffles and no rescale.  (A reference that follows the
+    // maximum only beyond a factor of 256 is another 1 - 2 % faster, but leaves the largest weight rounded: error against
+    // 64 bits up to 6 % larger.)  Against a loop with one chain of MMAs, shuffles and exp2f on every page and V fetched
+    // behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker step of 16
+    // rows 300.5 -> 289 us, of 11 rows on 52 SMs 471 -> 457; at config-3 dimensions 9 rows, 4 layers 493 -> 483 us, 29 rows
+    // on 96 SMs 796 -> 782, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.16 ms.
     for (int pi = 0; pi < n_pages; ++pi) {
       // the slot read in the previous iteration is free: keep DC_STAGES - 1 pages in flight
       const int page_ahead = __shfl_sync(0xffffffffu, my_page, (pi + DC_STAGES - 1) & 31);
@@ -345,7 +345,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
       }
       const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
       const float mx_b = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2;
-      if (__any_sync(0xffffffffu, mx_a > m_a + kLazyMax || mx_b > m_b + kLazyMax)) {
+      if (__any_sync(0xffffffffu, mx_a > m_a || mx_b > m_b)) {
         const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = fmaxf(m_b, quad_max(mx_b));
         const float al_a = fast_exp2(m_a - mn_a), al_b = fast_exp2(m_b - mn_b);
         m_a = mn_a;
