@@ -167,6 +167,16 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
     const int sms = sm_count > 0 ? sm_count : 148;
     if (groups == 0 || groups > sms || longest > kDecodeWarps * 32 * kPage) group_mode = false;
   }
+  // Tokens per prefill item: two Q tiles that share their key blocks, or one where that gives every item an SM of its own
+  // (an item's tiles are independent rows, so the results are the same).  Measured on B200: denoising stage (64 items of
+  // two tiles, 128 of one) 1009 -> 998 us, a chunk of 394 tokens with 7 decode rows (52 and 104 items) 1091 -> 1082 us.
+  int item_tokens = 2 * Mt;
+  {
+    int singles = 0;
+    for (int s = 0; s < b.n_seqs; ++s)
+      if (b.q_len[s] > 1) singles += ceil_div(b.q_len[s], Mt) * c.n_kv_heads;
+    if (singles <= (sm_count > 0 ? sm_count : 148)) item_tokens = Mt;
+  }
   StepPlan p;
   p.n_tokens = b.n_tokens;
   p.n_seqs = b.n_seqs;
@@ -232,10 +242,10 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
       p.decode_kv_bytes += int64_t(keys) * 2 * c.n_kv_heads * c.head_dim * 2;
       ++n_dec_rows;
     } else {
-      // a prefill item covers two Q tiles of Mt tokens each (the second one may be short or absent)
-      for (int t0 = 0; t0 < n; t0 += 2 * Mt)
+      // a prefill item covers one or two Q tiles of Mt tokens each (the last one may be short)
+      for (int t0 = 0; t0 < n; t0 += item_tokens)
         for (int hk = 0; hk < c.n_kv_heads; ++hk) {
-          const int nt = std::min(2 * Mt, n - t0);
+          const int nt = std::min(item_tokens, n - t0);
           pre.push_back(Item{{s, hk, t0, nt, ctx, t, n, 0}, ctx + t0 + nt});
           const int keys_item = (c.flags & HS_FLAG_BIDIRECTIONAL) ? ctx + n : ctx + t0 + nt;
           const int blocks = ceil_div(keys_item, 64);
