@@ -1165,8 +1165,11 @@ hs_status_t hs_head_step(hs_head_t* h, const float* y, const int32_t* rows, int3
   np.row_index = rows;
   np.sm_count = h->sm_count;
   np.status = status;
+  // The norm reads the gains in front of its wait, and what is in front of it is the caller's: an update of the gains in
+  // place has to be behind it.  (In a stage step the copy of the metadata stands between; the vocabulary GEMM is behind a
+  // norm all of whose blocks have waited.)
   const int overlap = sm_budget == h->sm_count ? kOverlapEarly : kOverlapLate;
-  np.overlap = overlap;
+  np.overlap = overlap == kOverlapEarly ? kOverlapFirst : kOverlapNone;
   cudaError_t e = launch_rmsnorm(np, sm_budget, stream);
   if (e != cudaSuccess) return cuda_fail("head rmsnorm", e);
 

@@ -415,7 +415,7 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
     if (p.n_parts > 0 || (p.sm_count > 0 && blocks <= sms)) {
       const int grid = blocks < sm_budget ? blocks : sm_budget, V = (d4 + tpr - 1) / tpr;
       auto kernel = V <= 1 ? rmsnorm_row_kernel<1> : V <= 2 ? rmsnorm_row_kernel<2> : V <= 4 ? rmsnorm_row_kernel<4> : rmsnorm_row_kernel<8>;
-      return launch_step_kernel(kernel, grid, ROW_THREADS, kMinSmemBytes, stream, p.overlap != 0, p, tpr);
+      return launch_step_kernel(kernel, grid, ROW_THREADS, kMinSmemBytes, stream, launches_ahead(p.overlap), p, tpr);
     }
   }
   // bulk-staged variant: as many warps as have room for two fp32 rows each (a function of d alone, never of
@@ -428,12 +428,12 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
     const int grid = blocks < sm_budget ? blocks : sm_budget;
     const size_t smem = 512 + size_t(warps) * pair_bytes + gain_bytes;
     const size_t bytes = smem < size_t(kMinSmemBytes) ? size_t(kMinSmemBytes) : smem;
-    if (p.mod) return launch_step_kernel(rmsnorm_bulk_kernel<true>, grid, warps * 32, bytes, stream, p.overlap != 0, p);
-    return launch_step_kernel(rmsnorm_bulk_kernel<false>, grid, warps * 32, bytes, stream, p.overlap != 0, p);
+    if (p.mod) return launch_step_kernel(rmsnorm_bulk_kernel<true>, grid, warps * 32, bytes, stream, launches_ahead(p.overlap), p);
+    return launch_step_kernel(rmsnorm_bulk_kernel<false>, grid, warps * 32, bytes, stream, launches_ahead(p.overlap), p);
   }
   const int blocks = (p.T + NORM_WARPS - 1) / NORM_WARPS;
   const int grid = blocks < sm_budget ? blocks : sm_budget;
-  return launch_step_kernel(rmsnorm_kernel, grid, NORM_THREADS, NORM_SMEM, stream, p.overlap != 0, p);
+  return launch_step_kernel(rmsnorm_kernel, grid, NORM_THREADS, NORM_SMEM, stream, launches_ahead(p.overlap), p);
 }
 
 }  // namespace hs

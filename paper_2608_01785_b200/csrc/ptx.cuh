@@ -362,12 +362,16 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
 //                  when the last block of this kernel has left its SM (and wait for the flush of its writes).  Never
 //                  more than sm_budget SMs are in use, and the launch latency is no longer part of the gap between two
 //                  kernels.  For partial budgets.
+//   kOverlapFirst  launched the ordinary way, triggers as kOverlapEarly: for the first kernel of a call, where it reads
+//                  weights in front of griddep_wait().  Its predecessor is the caller's kernel, which may be the one that
+//                  writes those weights; an ordinary launch starts behind its writes.
 // Measured on B200, step of 29 decode rows at config-3 dimensions, 4 layers, 96 SMs: 865 us with launches that wait for the
 // completed kernel in front, 809 us with kOverlapLate (29 launches: 1.9 us each).
-enum OverlapMode : int { kOverlapNone = 0, kOverlapEarly = 1, kOverlapLate = 2 };
+enum OverlapMode : int { kOverlapNone = 0, kOverlapEarly = 1, kOverlapLate = 2, kOverlapFirst = 3 };
+inline bool launches_ahead(int overlap) { return overlap == kOverlapEarly || overlap == kOverlapLate; }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents(int overlap) {
-  if (overlap == kOverlapEarly) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (overlap == kOverlapEarly || overlap == kOverlapFirst) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Host side: launches `kernel`; with `overlap` set, the launch carries the programmatic-stream-serialisation

@@ -38,3 +38,38 @@ def test_tokens_are_the_first_maximum_of_the_logits(V, n):
             assert np.array_equal(tokens.cpu().numpy(), want)
     finally:
         B.hs_head_destroy(head)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("budget", [148, 52])
+def test_a_step_sees_gains_written_right_in_front_of_it(budget):
+    """The gains are borrowed, not constant: a caller's kernel that rewrites them on the stream is ordered before the
+    step, with no synchronisation between them."""
+    dev = torch.device("cuda:0")
+    d, V, n = 3584, 2048, 65
+    g = torch.Generator(device=dev).manual_seed(3)
+    w = torch.empty(V, d, dtype=torch.bfloat16, device=dev).normal_(0.0, 0.02, generator=g)
+    gains = [torch.full((d,), float(v), dtype=torch.bfloat16, device=dev) for v in (1, 2, 4, 8)]     # exact factors
+    gain = gains[0].clone()
+    y = torch.randn(n, d, generator=g, device=dev)
+    rows = torch.arange(n, dtype=torch.int32, device=dev)
+    cfg = B.make_head_config(d, V, 1e-6, 128)
+    ws = torch.empty(B.hs_head_workspace_bytes(cfg), dtype=torch.uint8, device=dev)
+    head = B.hs_head_create(cfg, gain.data_ptr(), w.data_ptr(), ws.data_ptr())
+    try:
+        tokens = torch.empty(n, dtype=torch.int32, device=dev)
+        logits = torch.empty(17, n, V, device=dev)
+        scratch = torch.empty(1 << 24, device=dev)
+        torch.cuda.synchronize()
+        stream = torch.cuda.Stream(device=dev)
+        with torch.cuda.stream(stream):
+            for i in range(17):
+                scratch.fill_(float(i))              # the device is busy when the update is enqueued
+                gain.copy_(gains[i % 4])
+                B.hs_head_step(head, y.data_ptr(), rows.data_ptr(), n, logits[i].data_ptr(), tokens.data_ptr(), budget,
+                               stream.cuda_stream)
+        torch.cuda.synchronize()
+        for i in range(17):                          # powers of two: every rounding of the step scales with the gain
+            assert torch.equal(logits[i], logits[0] * float(gains[i % 4][0])), i
+    finally:
+        B.hs_head_destroy(head)
