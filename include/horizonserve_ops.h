@@ -152,6 +152,14 @@ hs_status_t hs_stage_plan_attention(hs_stage_t *stage, const hs_batch_t *batch, 
                                     int32_t prefill_cap, int32_t *n_prefill_items);
 
 /*
+ * Host-only: the number of K splits whose partial sums the residual GEMM of M rows, width N and contraction length K
+ * leaves to the RMSNorm behind it, in a step with separate norm kernels on a device of 148 SMs; 0 where the GEMM adds into
+ * the residual stream itself.  Depends on the shape only, never on the SM budget.  Returns -1 for M < 1, or N or K below
+ * 64 or not a multiple of 8.
+ */
+int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K);
+
+/*
  * Host-only: the K block (of 64) at which split i (0 .. ks; i = ks gives k_blocks) of a small step's residual GEMM
  * begins when its k_blocks are cut into ks splits.  Each split is ten K blocks longer than the one before it (the
  * splits add their sums one after the other, and a link of that chain takes about as long as ten K blocks take to

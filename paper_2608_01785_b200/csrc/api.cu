@@ -34,6 +34,37 @@ size_t weight_elems(const hs_stage_config_t& c, int i) {
   return n[i];
 }
 
+// Rows of d floats kept for the partial sums of K-split residual GEMMs: at most ten splits and 40 MB.
+int part_rows_cap(int T, int d) {
+  return int(std::min(size_t(10) * align_up(T, 32), (size_t(40) << 20) / (size_t(d) * 4)));
+}
+
+// More than one 128-row tile of tokens: a GEMM runs on pairs of SMs (256 x 256 tiles), unless such tiles would
+// occupy less than half of the device's pairs AND its 128-row tiles for single blocks fit one wave: then single
+// blocks occupy more SMs (and a residual GEMM may split K).  A choice by shape, never by budget; the two
+// kernels give the same bits.  Measured at config-3 dimensions, one prefill chunk + decodes (ms per step, all
+// pairs -> this rule): 220 rows 7.41 -> 5.60, 440 rows 9.23 -> 8.63; at 650 rows and more (pair tiles on 57 %
+// of the pairs and up) pairs are the faster form again, a pair tile moving two thirds of the operand bytes of
+// two single tiles.
+bool on_pairs(int T, int n_cols, int single_bn, int sm_count) {
+  if (T <= 128) return false;
+  const bool few_pair_tiles = ceil_div(T, 256) * ceil_div(n_cols, 256) < sm_count / 4;
+  const bool singles_fit = ceil_div(T, 128) * ceil_div(n_cols, single_bn) <= sm_count;
+  return !(few_pair_tiles && singles_fit);
+}
+
+// Residual GEMM (K -> d) of a step with separate norm kernels: its K splits leave their partial sums in scratch and the norm
+// kernel behind it adds them (the last layer's: a launch of the same kernel without a norm).  Nothing waits for its turn
+// and all splits are equally long, so every SM streams weights until the end.  Where that is expected to be the faster
+// form (gemm_plan_parts); a choice by shape and stage, never by budget.  A row too wide for the norm kernel, a scratch
+// that does not fit and the small-step fold keep the GEMM without it, and so does a GEMM that fills pairs of SMs, which
+// needs no splits: conditioned steps at 7B dimensions with its partial sums (2 layers) 600 rows 620 -> 640 us, 1450
+// rows 1133 -> 1280.
+ResidPlan plan_parts(int T, int d, int K, int sm_count, int part_rows, bool skinny) {
+  if (d > kNormRowMaxD || (T <= 16 && skinny) || on_pairs(T, d, gemm_pick_bn(T, d, sm_count), sm_count)) return ResidPlan{0, 0, 0};
+  return gemm_plan_parts(T, d, K, sm_count, part_rows, skinny);
+}
+
 WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   WsLayout w{};
   size_t off = 0;
@@ -58,8 +89,7 @@ WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   w.row_ss = take(std::max(T * kRowSsStride, size_t(64) * size_t(c.d_model / 32 + 1)) * 4);
   w.row_rs = take(T * 4);                            // r of every token
   w.row_done = take((T / 32 + 2) * 4);               // tile columns delivered per group of 32 token rows
-  // partial sums of the K-split residual GEMMs of small and middling steps (gemm_plan_parts): at most ten splits and 40 MB
-  w.part_rows = int(std::min(size_t(10) * align_up(T, 32), (size_t(40) << 20) / (size_t(c.d_model) * 4)));
+  w.part_rows = part_rows_cap(c.max_tokens, c.d_model);      // (plan_parts)
   w.gemm_part = take(size_t(w.part_rows) * c.d_model * 4);
   // fp16 copies of the seven weight matrices of every layer (absent with HS_FLAG_BF16_ACTIVATIONS);
   // within a layer: w_q, w_k, w_v, w_o, w_gate, w_up, w_down, each 1024-byte aligned
@@ -469,6 +499,12 @@ hs_status_t hs_stage_plan_attention(hs_stage_t* s, const hs_batch_t* b, int32_t*
   return HS_OK;
 }
 
+int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K) {
+  constexpr int kSms = 148;
+  if (M < 1 || N < 64 || K < 64 || N % 8 != 0 || K % 8 != 0) return -1;
+  return plan_parts(M, N, K, kSms, part_rows_cap(M, N), gemm_skinny_wins(M, K, N, kGemmResid, 0, kSms)).ks;
+}
+
 int32_t hs_op_gemm_split_begin(int32_t k_blocks, int32_t ks, int32_t i) {
   if (k_blocks < 1 || ks < 1 || i < 0 || i > ks) return -1;
   return gemm_split_begin(k_blocks, ks, i);
@@ -527,20 +563,8 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const size_t layer_kv_elems = size_t(c.num_pages) * c.n_kv_heads * kPage * Dh;
   cudaError_t e = cudaSuccess;
   const char* where = "";
-  // More than one 128-row tile of tokens: a GEMM runs on pairs of SMs (256 x 256 tiles), unless such tiles would
-  // occupy less than half of the device's pairs AND its 128-row tiles for single blocks fit one wave: then single
-  // blocks occupy more SMs (and a residual GEMM may split K).  A choice by shape, never by budget; the two
-  // kernels give the same bits.  Measured at config-3 dimensions, one prefill chunk + decodes (ms per step, all
-  // pairs -> this rule): 220 rows 7.41 -> 5.60, 440 rows 9.23 -> 8.63; at 650 rows and more (pair tiles on 57 %
-  // of the pairs and up) pairs are the faster form again, a pair tile moving two thirds of the operand bytes of
-  // two single tiles.
   const bool use_pair = T > 128;
-  auto pair_for = [&](int n_cols, int single_bn) {
-    if (!use_pair) return false;
-    const bool few_pair_tiles = ceil_div(T, 256) * ceil_div(n_cols, 256) < s->sm_count / 4;
-    const bool singles_fit = ceil_div(T, 128) * ceil_div(n_cols, single_bn) <= s->sm_count;
-    return !(few_pair_tiles && singles_fit);
-  };
+  auto pair_for = [&](int n_cols, int single_bn) { return on_pairs(T, n_cols, single_bn, s->sm_count); };
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
@@ -573,20 +597,12 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const bool fold_norm = !s->modulation && n_ss_tiles <= kRowSsStride && !skinny(d, q_dim + 2 * kv_dim, kGemmQkv) &&
                          !skinny(q_dim, d, kGemmResid) && !skinny(d, F, kGemmGateUp) && !skinny(F, d, kGemmResid) &&
                          pair_d && pair_qkv && pair_gu;
-  // A step with separate norm kernels: the K splits of a residual GEMM leave their partial sums in scratch and the norm
-  // kernel behind it adds them (the last layer's: a launch of the same kernel without a norm).  Nothing waits for its
-  // turn and all splits are equally long, so every SM streams weights until the end.  A choice by shape and stage, never
-  // by budget; a width or a scratch that does not fit keeps the ordered chain.  Measured on B200 against that chain
-  // and the norm kernel of one warp per row: 64 decode rows at config-3 dimensions 5.14 -> 4.96 ms, 29 rows on 96 SMs (4
-  // layers) 780 -> 714 us, a chunk of 394 tokens with 7 decode rows (4 layers) 1239 -> 1127 us, denoising 1125 -> 1034 us.
-  const bool parts_ok = !fold_norm && d <= kNormRowMaxD;
-  auto plan_parts = [&](int K) {
-    ResidPlan r{0, 0, 0, 0.0};
-    if (parts_ok && !(T <= 16 && skinny(K, d, kGemmResid))) r = gemm_plan_parts(T, d, K, s->sm_count, s->ws.part_rows);
-    if (r.ks > 0 && skinny(K, d, kGemmResid) && gemm_skinny_cost_us(T, K, d, kGemmResid, s->sm_count) < r.us) r.ks = 0;
-    return r;
+  // A step with separate norm kernels leaves the partial sums of its residual GEMMs' K splits to the norms where that is
+  // the faster form
+  auto parts_of = [&](int K) {
+    return fold_norm ? ResidPlan{0, 0, 0} : plan_parts(T, d, K, s->sm_count, s->ws.part_rows, skinny(K, d, kGemmResid));
   };
-  const ResidPlan parts_out = plan_parts(q_dim), parts_down = plan_parts(F);
+  const ResidPlan parts_out = parts_of(q_dim), parts_down = parts_of(F);
   const int part_rows = ceil_div(T, 32) * 32;
   auto use_parts = [&](GemmParams& gp, const ResidPlan& r) {
     gp.pair = r.pair;

@@ -937,49 +937,77 @@ int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count) {
   return best;
 }
 
-ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows) {
-  // A block (pair) works K blocks of a tile at the slowest of five rates, measured on B200: issue and tensor core (0.20 us per
-  // K block 128 columns wide, 0.27 for 256 and for pairs), what one SM takes in (120 KB/us) and what of it can be weights
-  // from the HBM (68 KB/us: latency against the ring's bytes in flight), what the L2 hands out to all SMs (14.5 MB/us) and
-  // what the HBM delivers (6.2 MB/us of weights, which the row tiles of a column share).  Rounds of one unit per worker,
-  // 2.5 us of start and end, 1.2 us per further round, and the partial sums are read once more (12 MB/us).
-  // What the choice minimises is the time on the whole device plus 0.15 of those on 13/16, 3/4, 13/20 and 1/2 of it, so that
-  // a stage with a neighbour is not left with a short last round.  Measured on B200, K = 18944, N = 3584, by splits x width
-  // (us per launch, events around it): 64 rows on 148 SMs 3 x 128 36.6, 5 x 128 33.7, 10 x 128 34.2, 10 x 256 34.9; 29
-  // rows on 96 SMs 36.5 / 42.3 / 36.9 / 39.1.
+namespace {
+// Time (us) of a residual GEMM's launch on `sms` SMs, its longest unit `kb` K blocks of 64.  A block (pair) works a K block
+// at the slowest of five rates, measured on B200: issue and tensor core (0.20 us per K block 128 columns wide, 0.27 for
+// 256 and for pairs), what one SM takes in (120 KB/us) and what of it can be weights from the HBM (68 KB/us: latency
+// against the ring's bytes in flight), what the L2 hands out to all SMs (14.5 MB/us) and what the HBM delivers (6.2 MB/us
+// of weights, which the row tiles of a column share).  Rounds of one unit per worker, 2.5 us of start and end, 1.2 us per
+// further round.
+double resid_launch_us(int M, int N, bool pair, int bn, int ks, int kb, int sms) {
+  const int W = pair ? sms / 2 : sms;
+  if (W < 1) return 0.0;
+  const int m_tiles = pair ? (M + 2 * BM - 1) / (2 * BM) : (M + BM - 1) / BM, units = m_tiles * ((N + bn - 1) / bn) * ks;
+  const double a_bytes = (!pair && M <= 32 ? 32 : !pair && M <= 64 ? 64 : 128) * BK * 2;
+  const double b_bytes = (pair || bn <= 128 ? 128 : 256) * BK * 2;
+  auto round_us = [&](int n) {
+    const double sm = pair ? 2.0 * n : n;
+    double t = pair || bn > 128 ? 0.27 : 0.20;
+    t = std::max(t, (a_bytes + b_bytes) / 120e3);
+    t = std::max(t, b_bytes / m_tiles / 68e3);
+    t = std::max(t, sm * (a_bytes + b_bytes) / 14.5e6);
+    t = std::max(t, sm * b_bytes / m_tiles / 6.2e6);
+    return kb * t;
+  };
+  const int full = units / W, rest = units - full * W;
+  return full * round_us(W) + (rest ? round_us(rest) : 0.0) + 2.5 + 1.2 * (full + (rest ? 1 : 0) - 1);
+}
+// Time on the whole device and, with a weight of 0.15 each, on 13/16, 3/4, 13/20 and 1/2 of it (120, 111, 96 and 74 of 148
+// SMs, budgets a stage with a neighbour is given), so that such a stage is not left with a short last round.
+template <typename F>
+double over_budgets(int sm_count, F us) {
+  double sum = us(sm_count);
+  for (const int eightieths : {65, 60, 52, 40}) sum += 0.15 * us(std::max(1, sm_count * eightieths / 80));
+  return sum / 1.6;
+}
+}  // namespace
+
+ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows, bool skinny) {
+  // The best form with partial sums, read back at 12 MB/us, against the one the GEMM has without them (weight-streaming
+  // kernel, or single blocks whose splits add in order), both by the times above.  Against that one the partial sums
+  // count 3 MB/us where the norm kernel's threads hold eight groups each or its rows need a second round (pair of norms,
+  // 1024 x 1024 with 21 MB +4 us, 1280 x 1024 with 26 MB +10, 600 x 2048 with 25 MB +11), and 3 us that no rate explains
+  // (17 rows of d = 1024: out-projection +2.1 us, norm +1.7, whatever K).  Measured on B200, kernel by kernel, at 17 ..
+  // 4096 rows of d = 1024 / 2048 / 3584 with K = d and 2.75 .. 5.3 d, on 148 and 74 SMs.  In steps, without -> with partial
+  // sums: 128 rows of d = 1024 713 -> 574 us, 401 rows at 7B dimensions (2 layers) 501 -> 464; but 17 rows of d = 1024
+  // 369 -> 426, 1280 rows 1114 -> 1209, which is why the two are compared.
+  // Splits x width at 7B dimensions, down-projection (us per launch): 64 rows on 148 SMs 3 x 128 36.6, 5 x 128 33.7, 10 x
+  // 128 34.2, 10 x 256 34.9; 29 rows on 96 SMs 36.5 / 42.3 / 36.9 / 39.1.
   const int k_blocks = (K + BK - 1) / BK, part_rows = (M + 31) / 32 * 32;
-  ResidPlan best{0, 0, 0, 1e30};
+  const double part_bytes = double(part_rows) * N * 4.0;
+  ResidPlan best{0, 0, 0};
+  double best_us = 1e30;
   for (int form = 0; form < 3; ++form) {                     // single blocks 128 and 256 columns wide, pairs
     const bool pair = form == 2;
     if (pair && M <= BM) continue;
     const int bn = form == 0 ? 128 : 256;
-    const int m_tiles = pair ? (M + 2 * BM - 1) / (2 * BM) : (M + BM - 1) / BM, tiles = m_tiles * ((N + bn - 1) / bn);
-    const double a_bytes = (!pair && M <= 32 ? 32 : !pair && M <= 64 ? 64 : 128) * BK * 2, b_bytes = (pair ? 128 : bn) * BK * 2;
-    for (int ks = 1; ks <= 10 && ks <= k_blocks && ks * part_rows <= part_cap_rows; ++ks) {
-      const int units = tiles * ks, kb = (k_blocks + ks - 1) / ks;
-      double cost = 0.0;
-      for (const int eightieths : {80, 65, 60, 52, 40}) {
-        const int sms = sm_count * eightieths / 80, W = pair ? sms / 2 : sms;
-        if (W < 1) continue;
-        auto round_us = [&](int n) {
-          const double sm = pair ? 2.0 * n : n;
-          double t = pair || bn == 256 ? 0.27 : 0.20;
-          t = std::max(t, (a_bytes + b_bytes) / 120e3);
-          t = std::max(t, b_bytes / m_tiles / 68e3);
-          t = std::max(t, sm * (a_bytes + b_bytes) / 14.5e6);
-          t = std::max(t, sm * b_bytes / m_tiles / 6.2e6);
-          return kb * t;
-        };
-        const int full = units / W, rest = units - full * W;
-        const double us = full * round_us(W) + (rest ? round_us(rest) : 0.0) + 2.5 + 1.2 * (full + (rest ? 1 : 0) - 1) +
-                          double(ks) * part_rows * N * 4.0 / 12e6;
-        cost += eightieths == 80 ? us : 0.15 * us;
-      }
-      if (cost < best.us - 1e-9) best = ResidPlan{pair ? 1 : 0, bn, ks, cost};
+    for (int ks = 2; ks <= 10 && ks <= k_blocks && ks * part_rows <= part_cap_rows; ++ks) {
+      const double us = over_budgets(sm_count, [&](int sms) {
+        return resid_launch_us(M, N, pair, bn, ks, (k_blocks + ks - 1) / ks, sms);
+      }) + ks * part_bytes / 12e6;
+      if (us < best_us - 1e-9) { best_us = us; best = ResidPlan{pair ? 1 : 0, bn, ks}; }
     }
   }
-  best.us /= 1.6;
-  return best;
+  const int tpr = norm_row_threads(M, N, sm_count), rows_per_block = kNormRowThreads / tpr;
+  const bool wide = ((N >> 2) + tpr - 1) / tpr > 4 || (M + rows_per_block - 1) / rows_per_block > sm_count;
+  if (wide) best_us += best.ks * part_bytes * (1 / 3e6 - 1 / 12e6);
+  const int bn = gemm_pick_bn(M, N, sm_count), ks = gemm_pick_ksplit(M, N, K, bn, sm_count);
+  const int longest = k_blocks - gemm_split_begin(k_blocks, ks, ks - 1);
+  const double without = over_budgets(sm_count, [&](int sms) {
+    if (skinny) return (((N >> 5) + sms - 1) / sms) * (1.5 + double(32 + M) * K * 2 / 70e3);
+    return resid_launch_us(M, N, false, bn, ks, longest, sms) + gemm_chain_us(k_blocks, ks);
+  });
+  return best_us + 3.0 < without ? best : ResidPlan{0, 0, 0};
 }
 
 int gemm_pick_stream_k(int M, int N, int K, int sm_count) {

@@ -598,16 +598,12 @@ bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim) {
 // all projections tiled -> this rule): 16 rows 4.39 -> 3.49, 5.42 -> 5.14, 5.74 -> 5.27; 32 rows 4.91 -> 4.36,
 // 5.99 -> 5.80, 6.34 -> 6.15; 64 rows 5.72 -> 5.38, 7.21 -> 7.43, 8.06 -> 8.32 (with its unit count just below
 // the SM count this kernel needs a second round as soon as the budget drops, which at 64 rows costs 3 %).
-double gemm_skinny_cost_us(int T, int K, int N, int mode, int sm_count) {
+bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count) {
+  if (!gemm_skinny_supports(T, K, N, mode, head_dim)) return false;
   const int mt = T <= 16 ? 1 : T <= 32 ? 2 : 4;
   const int units = mode == kGemmGateUp ? N / 16 : N / 32;
   const int rounds = (units + sm_count - 1) / sm_count;
-  return rounds * (1.5 + double(32 + 16 * mt) * K * 2 / 70e3);
-}
-
-bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count) {
-  if (!gemm_skinny_supports(T, K, N, mode, head_dim)) return false;
-  const double mine = gemm_skinny_cost_us(T, K, N, mode, sm_count);
+  const double mine = rounds * (1.5 + double(32 + 16 * mt) * K * 2 / 70e3);
   const int k_blocks = (K + 63) / 64;
   double tiled;
   if (mode == kGemmResid) {

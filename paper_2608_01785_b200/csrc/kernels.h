@@ -108,21 +108,26 @@ __host__ __device__ inline int gemm_split_begin(int k_blocks, int ks, int i) {
   }
   return i * ((k_blocks - tri) / ks) + kSplitSkew * i * (i - 1) / 2;
 }
+// What of the chain of adds is not hidden behind the longest split's stream (us).
+inline double gemm_chain_us(int k_blocks, int ks) {
+  const bool skewed = gemm_split_begin(k_blocks, ks, 1) != (k_blocks + ks - 1) / ks || ks == 1;
+  return ks > 1 ? (skewed ? 3.5 : (ks - 1) * 3.5) : 0.0;
+}
 // Modelled time (us) of a K-split residual GEMM of `waves` rounds on single blocks: the longest split's stream and
 // what of the chain of adds is not hidden behind it.
 inline double gemm_ksplit_cost_us(int k_blocks, int ks, int waves) {
   const int last = k_blocks - gemm_split_begin(k_blocks, ks, ks - 1);
-  const bool skewed = gemm_split_begin(k_blocks, ks, 1) != (k_blocks + ks - 1) / ks || ks == 1;
-  return double(waves) * last * 0.36 + (ks > 1 ? (skewed ? 3.5 : (ks - 1) * 3.5) : 0.0);
+  return double(waves) * last * 0.36 + gemm_chain_us(k_blocks, ks);
 }
 // Runs for the stream-K form of a Resid-mode GEMM on pairs (one per pair of the device), or 0 when whole tiles
 // already fill their waves well enough (budget independent).
 int gemm_pick_stream_k(int M, int N, int K, int sm_count);
 // Form of a residual GEMM whose K splits leave partial sums for the RMSNorm behind it (GemmParams::part_rows): tile width,
-// pairs or single blocks, and the number of splits, or ks = 0 when no form fits `part_cap_rows` rows of scratch.  `us` is
-// the modelled time with the extra reading of the partials.  A function of the shape and the device's SM count only.
-struct ResidPlan { int pair, bn, ks; double us; };
-ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows);
+// pairs or single blocks, and the number of splits, or ks = 0 where no such form fits `part_cap_rows` rows of scratch or
+// is expected to be faster, with the reading of the partial sums, than the form on single blocks -- on the weight-streaming
+// kernel with `skinny` -- that it replaces.  A function of the shape and the device's SM count only.
+struct ResidPlan { int pair, bn, ks; };
+ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows, bool skinny);
 // The same three GEMMs for steps of at most 64 rows (gemm_skinny.cu): weight streaming on plain loads and
 // warp-level MMAs, one block per 32 output columns and the whole K range, no K split across blocks.
 struct SkinnyParams {
@@ -169,7 +174,6 @@ struct SkinnyParams {
 };
 // True when the skinny kernel covers this shape (few rows, K a multiple of 32, widths it can tile).
 bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim);
-double gemm_skinny_cost_us(int T, int K, int N, int mode, int sm_count);
 // True when it is also expected to be faster than the tiled kernel for this shape (budget independent).
 bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count);
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream);
@@ -209,7 +213,16 @@ struct NormParams {
   int* smid_log;             // nullable: SM census slots of this launch
 };
 cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stream);
-constexpr int kNormRowMaxD = 512 * 8 * 4;    // widest row of the kernel that adds partial sums
+constexpr int kNormRowThreads = 512;
+constexpr int kNormRowMaxD = kNormRowThreads * 8 * 4;    // widest row of the kernel that adds partial sums
+// Threads per row of that kernel: as many as leave one round of rows on the device, with at most eight groups of four
+// columns each.
+inline int norm_row_threads(int T, int d, int sms) {
+  int tpr = kNormRowThreads;
+  while (tpr > 32 && (T + kNormRowThreads / tpr - 1) / (kNormRowThreads / tpr) > sms && ((d >> 2) + tpr / 2 - 1) / (tpr / 2) <= 8)
+    tpr >>= 1;
+  return tpr;
+}
 
 // Embedding lookup (head.cu).
 struct EmbedParams {

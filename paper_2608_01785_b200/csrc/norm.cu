@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
 // that latency: one warp per row (the kernel above) took 8.2 us per launch at 64 x 3584 and 9.3 us at 1024 x 1024
 // (conditioned), this one 5.4 us with three partial sums to add and 9.5-10 with two (ncu).  Sums: a thread's groups in order, a butterfly per warp, the warps in
 // order -- a function of the shape and the device's SM count, never of the budget.
-constexpr int ROW_THREADS = 512;
+constexpr int ROW_THREADS = kNormRowThreads;
 
 template <int V>
 __global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormParams p, int tpr) {
@@ -408,9 +408,7 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
   if (p.T <= 0) return cudaSuccess;
   // few rows (one round of them on the whole device), or partial sums to add: many threads per row
   if (p.d <= kNormRowMaxD) {
-    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2;
-    int tpr = ROW_THREADS;
-    while (tpr > 32 && (p.T + ROW_THREADS / tpr - 1) / (ROW_THREADS / tpr) > sms && (d4 + tpr / 2 - 1) / (tpr / 2) <= 8) tpr >>= 1;
+    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, tpr = norm_row_threads(p.T, p.d, sms);
     const int rows_per_block = ROW_THREADS / tpr, blocks = (p.T + rows_per_block - 1) / rows_per_block;
     if (p.n_parts > 0 || (p.sm_count > 0 && blocks <= sms)) {
       const int grid = blocks < sm_budget ? blocks : sm_budget, V = (d4 + tpr - 1) / tpr;
