@@ -142,7 +142,7 @@ hs_status_t hs_op_decode_attention_noalloc_status(int32_t *status_out);
  *                  partial slot, items of the group | index within the group << 16}; in group mode (*decode_group = 1:
  *                  a small batch, every (sequence, KV head) group worked by one block) eight page slices per group,
  *                  group-major, some possibly empty (first key = end key), the last two words unused.
- *   prefill_items  [prefill_cap][8] int32, longest first: {sequence, KV head, first new token, tokens (at most two Q
+ *   prefill_items  [prefill_cap][8] int32, as for a budget of all SMs, longest first: {sequence, KV head, first new token, tokens (at most two Q
  *                  tiles), cached tokens, token row of the sequence's first new token, new tokens of the sequence, 0}.
  * Any pointer may be NULL; counts are always written when their pointer is given; at most cap records are copied.
  * Errors: INVALID_ARG, BAD_BLOCK_TABLE.
@@ -150,6 +150,18 @@ hs_status_t hs_op_decode_attention_noalloc_status(int32_t *status_out);
 hs_status_t hs_stage_plan_attention(hs_stage_t *stage, const hs_batch_t *batch, int32_t *decode_items, int32_t decode_cap,
                                     int32_t *n_decode_items, int32_t *decode_group, int32_t *prefill_items,
                                     int32_t prefill_cap, int32_t *n_prefill_items);
+
+/*
+ * Host-only diagnosis: how hs_stage_step would share sm_budget out for the attention of `batch` (validated as by
+ * hs_stage_plan; a stage without a device plans for 148 SMs).
+ *   *n_prefill_items   prefill work items, of one Q tile each where every item then has an SM of the prefill kernel's share
+ *                      to itself and that is expected to be the faster form, else of two.  The results are the same bits.
+ *   *decode_sms        SMs of the budget for the decode kernel while the prefill kernel runs beside it on the rest; 0 when
+ *                      the two run one after the other on the whole budget, or only one of them has work.
+ * Either pointer may be NULL.  Errors: INVALID_ARG, INVALID_BUDGET, BAD_BLOCK_TABLE.
+ */
+hs_status_t hs_stage_plan_shares(hs_stage_t *stage, const hs_batch_t *batch, int32_t sm_budget, int32_t *n_prefill_items,
+                                 int32_t *decode_sms);
 
 /*
  * Host-only: the number of K splits whose partial sums the residual GEMM of M rows, width N and contraction length K

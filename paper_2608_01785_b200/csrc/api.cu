@@ -470,11 +470,13 @@ int32_t hs_kv_free_pages(const hs_stage_t* s) { return s ? s->alloc->free_pages(
 
 int32_t hs_stage_sm_count(const hs_stage_t* s) { return s ? s->sm_count : 0; }
 
+static int plan_sms(const hs_stage_t* s) { return s->sm_count > 0 ? s->sm_count : 148; }    // (a stage without a device)
+
 hs_status_t hs_stage_plan(hs_stage_t* s, const hs_batch_t* b, int32_t* tok_seq, int32_t* tok_pos, int32_t* tok_slot) {
   if (!s || !b) return HS_ERR_INVALID_ARG;
   std::vector<int32_t> meta(s->ml.total);
   StepPlan plan;
-  const hs_status_t st = plan_step(s->cfg, s->ml, *b, s->sm_count, s->page_stamp, ++s->stamp, meta.data(), tok_seq, &plan);
+  const hs_status_t st = plan_step(s->cfg, s->ml, *b, s->sm_count, plan_sms(s), true, s->page_stamp, ++s->stamp, meta.data(), tok_seq, &plan);
   if (st != HS_OK) return st;
   if (tok_pos) memcpy(tok_pos, meta.data() + s->ml.tok_pos, size_t(plan.n_tokens) * 4);
   if (tok_slot) memcpy(tok_slot, meta.data() + s->ml.tok_slot, size_t(plan.n_tokens) * 4);
@@ -487,7 +489,7 @@ hs_status_t hs_stage_plan_attention(hs_stage_t* s, const hs_batch_t* b, int32_t*
   if (!s || !b || decode_cap < 0 || prefill_cap < 0) return HS_ERR_INVALID_ARG;
   std::vector<int32_t> meta(s->ml.total);
   StepPlan plan;
-  const hs_status_t st = plan_step(s->cfg, s->ml, *b, s->sm_count, s->page_stamp, ++s->stamp, meta.data(), nullptr, &plan);
+  const hs_status_t st = plan_step(s->cfg, s->ml, *b, s->sm_count, plan_sms(s), true, s->page_stamp, ++s->stamp, meta.data(), nullptr, &plan);
   if (st != HS_OK) return st;
   if (n_decode_items) *n_decode_items = plan.n_decode_items;
   if (decode_group) *decode_group = plan.decode_group;
@@ -496,6 +498,18 @@ hs_status_t hs_stage_plan_attention(hs_stage_t* s, const hs_batch_t* b, int32_t*
     memcpy(decode_items, meta.data() + s->ml.decode_items, size_t(std::min(decode_cap, plan.n_decode_items)) * 32);
   if (prefill_items)
     memcpy(prefill_items, meta.data() + s->ml.prefill_items, size_t(std::min(prefill_cap, plan.n_prefill_items)) * 32);
+  return HS_OK;
+}
+
+hs_status_t hs_stage_plan_shares(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget, int32_t* n_prefill_items,
+                                 int32_t* decode_sms) {
+  if (!s || !b) return HS_ERR_INVALID_ARG;
+  if (sm_budget < 1 || sm_budget > plan_sms(s)) return HS_ERR_INVALID_BUDGET;
+  StepPlan plan;
+  const hs_status_t st = plan_step(s->cfg, s->ml, *b, s->sm_count, sm_budget, true, s->page_stamp, ++s->stamp, nullptr, nullptr, &plan);
+  if (st != HS_OK) return st;
+  if (n_prefill_items) *n_prefill_items = plan.n_prefill_items;
+  if (decode_sms) *decode_sms = plan.decode_sms;
   return HS_OK;
 }
 
@@ -528,7 +542,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     s->ev_pending[slot] = false;
   }
   StepPlan plan;
-  hs_status_t st = plan_step(c, s->ml, *b, s->sm_count, s->page_stamp, ++s->stamp, s->pinned[slot], nullptr, &plan);
+  hs_status_t st = plan_step(c, s->ml, *b, s->sm_count, sm_budget, !s->profile, s->page_stamp, ++s->stamp, s->pinned[slot], nullptr, &plan);
   if (st != HS_OK) return st;
   s->ring_pos = (slot + 1) % kRing;
 
@@ -669,22 +683,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     return HS_ERR_CUDA;
   auto slots = [&](int cls) { return census ? census + cls * kSmidSlots : nullptr; };
 
-  // Split of the SM budget between the two attention kernels when a step has both kinds of work (0 = one after the
-  // other).  The decode kernel is bound by the K / V bytes it streams, the prefill kernel by its key blocks; with the
-  // rates measured on B200 (about 42 GB/s per SM up to 5.5 TB/s; 1.15 us per block of an item; 12 us per launch)
-  //   t_decode(b) = 12 + bytes / min(5.5e6, 42e3 b)    t_prefill(b) = 12 + 1.15 max(longest item, blocks / b)   [us]
-  // and the split is the one with the smallest larger time, taken only if that beats running them in turn by 8 %.
-  // It moves work between SMs, never between results: both kernels give the same bits at any grid size.
-  int decode_sms = 0;
-  if (plan.n_prefill_items > 0 && plan.n_decode_items > 0 && sm_budget >= 16 && !s->profile) {   // (per-kernel timing keeps them apart)
-    auto t_dec = [&](int b) { return 12.0 + double(plan.decode_kv_bytes) / std::min(5.5e6, 42e3 * b); };
-    auto t_pre = [&](int b) { return 12.0 + 1.15 * std::max(double(plan.prefill_longest), double(plan.prefill_blocks) / b); };
-    double best = 0.92 * (t_dec(sm_budget) + t_pre(sm_budget));
-    for (int b = 4; b <= sm_budget - 4; ++b) {
-      const double t = std::max(t_dec(b), t_pre(sm_budget - b));
-      if (t < best) { best = t; decode_sms = b; }
-    }
-  }
+  const int decode_sms = plan.decode_sms;     // (per-kernel timing keeps the two attention kernels apart: 0)
 
   auto make_attn = [&](int l) {
     AttnParams a{};

@@ -1,7 +1,8 @@
 // Causal GQA attention for prefill chunks on the 5th-generation tensor cores.
 //
 //   work item   (sequence, KV head, up to 2 Mt consecutive tokens), Mt = 128 / G rounded down to a multiple of 8.
-//               The item is two Q tiles: tile A holds its first Mt tokens, tile B the rest.  In a tile the G query
+//               The item is two Q tiles: tile A holds its first Mt tokens, tile B the rest (absent where the planner makes
+//               items of one tile, the same bits).  In a tile the G query
 //               heads that share the KV head are stacked head-major as rows of a 128-row tile (row = head * Mt +
 //               token).  Both tiles read the same K / V blocks, which are staged once for the two of them.
 //   per block   of 64 keys and per tile:  S = Q K^T (tcgen05.mma, M128 N64, fp32 in tensor memory)  ->  the tile's
@@ -111,7 +112,9 @@ __device__ __forceinline__ ItemView view_item(const AttnParams& p, const int4& i
   v.n_tok_t[0] = min(v.n_tok, Mt);
   v.n_tok_t[1] = v.n_tok - v.n_tok_t[0];
   const int all = v.ctx + sq.z;
-  v.n_keys = p.bidirectional ? all : v.pos0 + v.n_tok;
+  // (an item of one tile counts the keys that the item of two tiles it belongs to would: what a masked key's V row holds --
+  // its values, or zeros -- is then the same in both, also where it is not finite)
+  v.n_keys = p.bidirectional ? all : min(v.ctx + (v.tok_begin / (2 * Mt) + 1) * (2 * Mt), all);
   const int keys_a = p.bidirectional ? all : v.pos0 + v.n_tok_t[0];
   v.nblk_t[0] = (keys_a + PF_KEYS - 1) / PF_KEYS;
   v.nblk_t[1] = v.n_tok_t[1] > 0 ? (v.n_keys + PF_KEYS - 1) / PF_KEYS : 0;

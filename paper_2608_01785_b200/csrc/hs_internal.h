@@ -70,23 +70,22 @@ struct StepPlan {
   int n_tokens = 0, n_seqs = 0;
   int n_prefill_items = 0, n_decode_items = 0, n_decode_rows = 0;
   int decode_group = 0;           // 1: decode items are eight page slices per (sequence, KV head), group-major (see plan_step)
-  // work estimates of the two attention kernels (for the split of the SM budget when they run side by side)
-  int64_t prefill_blocks = 0;     // 64-key blocks over all prefill items (an item's two tiles share a block)
-  int prefill_longest = 0;        // blocks of the longest prefill item
+  int decode_sms = 0;             // SMs of the budget for the decode kernel beside the prefill kernel; 0: one after the other
   int64_t decode_kv_bytes = 0;    // K and V bytes the decode items read, one layer
 };
 
 // Validates `b` against `c` and, when `meta` is non-NULL, fills the metadata block (layout `ml`).
 // `page_stamp` is scratch of num_pages entries used to detect a page named by two sequences; `stamp`
 // must be a value not used by an earlier call.  tok_seq (nullable) receives the owning sequence of each
-// token.  Returns HS_OK, HS_ERR_INVALID_ARG or HS_ERR_BAD_BLOCK_TABLE.
+// token.  `sm_budget` (and whether the two attention kernels may run side by side) decides the shape of the prefill items
+// and StepPlan::decode_sms, nothing that a result depends on.  Returns HS_OK, HS_ERR_INVALID_ARG or HS_ERR_BAD_BLOCK_TABLE.
 // Keys per decode work item for this batch: 128, 256, 384 or 512, whichever lets the device's warps finish the items
 // in the fewest, shortest rounds (among the sizes whose item count fits max_items).  A function of the batch and of
 // the device's SM count only (never of the budget).
 int pick_decode_split(const hs_stage_config_t& c, const hs_batch_t& b, int sm_count, int max_items);
-hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs_batch_t& b, int sm_count,
-                      std::vector<int32_t>& page_stamp, int32_t stamp, int32_t* meta, int32_t* tok_seq,
-                      StepPlan* plan);
+hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs_batch_t& b, int sm_count, int sm_budget,
+                      bool side_by_side, std::vector<int32_t>& page_stamp, int32_t stamp, int32_t* meta,
+                      int32_t* tok_seq, StepPlan* plan);
 
 hs_status_t validate_config(const hs_stage_config_t& c);
 

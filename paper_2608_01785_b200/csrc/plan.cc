@@ -1,6 +1,7 @@
 // Host-only logic of the stage: configuration checks, the page allocator, and the per-step planner
-// that turns a batch descriptor into the integer metadata the kernels consume.  Nothing here depends
-// on the SM budget, which is what keeps results identical across budgets.
+// that turns a batch descriptor into the integer metadata the kernels consume.  Nothing that a result depends on
+// depends on the SM budget, which is what keeps results identical across budgets; only how many (independent) Q tiles a
+// prefill item carries and the two attention kernels' shares of the budget do.
 #include <algorithm>
 #include <numeric>
 
@@ -127,9 +128,54 @@ int pick_decode_split(const hs_stage_config_t& c, const hs_batch_t& b, int sm_co
   return best;
 }
 
-hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs_batch_t& b, int sm_count,
-                      std::vector<int32_t>& page_stamp, int32_t stamp, int32_t* meta, int32_t* tok_seq,
-                      StepPlan* plan) {
+namespace {
+// Work of the prefill attention with one or two Q tiles per item: items, 64-key blocks over all of them, longest item.
+struct PrefillWork { int64_t items = 0, blocks = 0; int longest = 0; };
+PrefillWork prefill_work(const hs_stage_config_t& c, const hs_batch_t& b, int item_tokens) {
+  PrefillWork w;
+  for (int s = 0; s < b.n_seqs; ++s) {
+    const int n = b.q_len[s], ctx = b.ctx_len[s];
+    if (n < 2) continue;
+    for (int t0 = 0; t0 < n; t0 += item_tokens) {
+      const int keys = (c.flags & HS_FLAG_BIDIRECTIONAL) ? ctx + n : ctx + std::min(t0 + item_tokens, n), blocks = ceil_div(keys, 64);
+      w.items += c.n_kv_heads;
+      w.blocks += int64_t(c.n_kv_heads) * blocks;
+      w.longest = std::max(w.longest, blocks);
+    }
+  }
+  return w;
+}
+
+// Split of the SM budget between the two attention kernels when a step has both kinds of work (decode_sms = 0: one after
+// the other).  The decode kernel is bound by the K / V bytes it streams, the prefill kernel by its key blocks; with the
+// rates measured on B200 (about 42 GB/s per SM up to 5.5 TB/s; 1.15 us per block of an item; 12 us per launch)
+//   t_decode(b) = 12 + bytes / min(5.5e6, 42e3 b)    t_prefill(b) = 12 + 1.15 max(longest item, blocks / b)   [us]
+// and the split is the one with the smallest larger time, taken only if that beats running them in turn by 8 %.
+// Items of one tile (`singles`) take 2 us less but load their key blocks for one tile only, so they are taken only where
+// every one has an SM of the kernel's share to itself.
+// It moves work between SMs, never between results: both kernels give the same bits at any grid size.
+struct AttnSplit { int decode_sms; double us; };
+AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_bytes, int budget, bool side_by_side) {
+  auto t_dec = [&](int b) { return decode_kv_bytes > 0 ? 12.0 + double(decode_kv_bytes) / std::min(5.5e6, 42e3 * b) : 0.0; };
+  auto t_pre = [&](int b) {
+    if (singles) return w.items <= b ? 10.0 + 1.15 * w.longest : 1e30;
+    return 12.0 + 1.15 * std::max(double(w.longest), double(w.blocks) / b);
+  };
+  const double in_turn = t_dec(budget) + t_pre(budget);
+  AttnSplit r{0, in_turn};
+  if (decode_kv_bytes == 0 || w.items == 0 || budget < 16 || !side_by_side) return r;
+  double best = 0.92 * in_turn;
+  for (int b = 4; b <= budget - 4; ++b) {
+    const double t = std::max(t_dec(b), t_pre(budget - b));
+    if (t < best) { best = t; r = AttnSplit{b, t}; }
+  }
+  return r;
+}
+}  // namespace
+
+hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs_batch_t& b, int sm_count, int sm_budget,
+                      bool side_by_side, std::vector<int32_t>& page_stamp, int32_t stamp, int32_t* meta,
+                      int32_t* tok_seq, StepPlan* plan) {
   if (!b.q_len || !b.ctx_len || !b.block_tables) return HS_ERR_INVALID_ARG;
   if (b.n_seqs < 1 || b.n_seqs > c.max_seqs || b.n_tokens < 1 || b.n_tokens > c.max_tokens) return HS_ERR_INVALID_ARG;
   const int mpps = c.max_pages_per_seq;
@@ -167,19 +213,25 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
     const int sms = sm_count > 0 ? sm_count : 148;
     if (groups == 0 || groups > sms || longest > kDecodeWarps * 32 * kPage) group_mode = false;
   }
-  // Tokens per prefill item: two Q tiles that share their key blocks, or one where that gives every item an SM of its own
-  // (an item's tiles are independent rows, so the results are the same).  Measured on B200: denoising stage (64 items of
-  // two tiles, 128 of one) 1009 -> 998 us, a chunk of 394 tokens with 7 decode rows (52 and 104 items) 1091 -> 1082 us.
-  int item_tokens = 2 * Mt;
-  {
-    int singles = 0;
-    for (int s = 0; s < b.n_seqs; ++s)
-      if (b.q_len[s] > 1) singles += ceil_div(b.q_len[s], Mt) * c.n_kv_heads;
-    if (singles <= (sm_count > 0 ? sm_count : 148)) item_tokens = Mt;
-  }
   StepPlan p;
   p.n_tokens = b.n_tokens;
   p.n_seqs = b.n_seqs;
+  // Tokens per prefill item: two Q tiles that share their key blocks, or one.  An item's tiles are independent rows, so the
+  // results are the same bits (every budget sweep of the GPU tests crosses the line) and the choice may look at the
+  // budget: it is the form whose attention is expected to end first with the SMs the prefill kernel gets.  Measured on
+  // B200, two tiles -> one (us per step): denoising stage, 12 layers, 128 items of one tile, on 148 SMs 1009 -> 998, on 96
+  // 1140 -> 1167, on 37 1870 -> 1925; at 7B dimensions, 2 layers, 7 decode rows beside a chunk of 394 tokens (100 items) on
+  // 148 SMs 470 -> 466, on 96 662 -> 687, beside one of 100 tokens (28 items) on 148 304 -> 298, on 48 492 -> 519.
+  int item_tokens = 2 * Mt;
+  {
+    for (int s = 0; s < b.n_seqs; ++s)
+      if (b.q_len[s] == 1) p.decode_kv_bytes += int64_t(b.ctx_len[s] + 1) * 2 * c.n_kv_heads * c.head_dim * 2;
+    const PrefillWork one = prefill_work(c, b, Mt), two = prefill_work(c, b, 2 * Mt);
+    const AttnSplit with_one = split_attention(one, true, p.decode_kv_bytes, sm_budget, side_by_side);
+    const AttnSplit with_two = split_attention(two, false, p.decode_kv_bytes, sm_budget, side_by_side);
+    if (with_one.us < with_two.us) item_tokens = Mt;
+    p.decode_sms = item_tokens == Mt ? with_one.decode_sms : with_two.decode_sms;
+  }
 
   struct Item { int32_t v[8]; int32_t cost; };
   std::vector<Item> pre;
@@ -218,7 +270,6 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
           dec.push_back(DecItem{{n_dec_rows, hk, k0, k1, s, t, 0, 1}, 0});
         }
       n_dec_items += c.n_kv_heads * kDecodeWarps;
-      p.decode_kv_bytes += int64_t(keys) * 2 * c.n_kv_heads * c.head_dim * 2;
       ++n_dec_rows;
     } else if (n == 1) {
       // decode: keys 0..ctx cut into whole runs of `split` keys and the rest into pieces of kDecodeTail keys; the items
@@ -239,7 +290,6 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
           dec.push_back(DecItem{{n_dec_rows, hk, k0, k1, s, t, n_dec_items + hk * splits, splits | (j << 16)}, k1 - k0});
         }
       n_dec_items += c.n_kv_heads * splits;
-      p.decode_kv_bytes += int64_t(keys) * 2 * c.n_kv_heads * c.head_dim * 2;
       ++n_dec_rows;
     } else {
       // a prefill item covers one or two Q tiles of Mt tokens each (the last one may be short)
@@ -247,10 +297,6 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
         for (int hk = 0; hk < c.n_kv_heads; ++hk) {
           const int nt = std::min(item_tokens, n - t0);
           pre.push_back(Item{{s, hk, t0, nt, ctx, t, n, 0}, ctx + t0 + nt});
-          const int keys_item = (c.flags & HS_FLAG_BIDIRECTIONAL) ? ctx + n : ctx + t0 + nt;
-          const int blocks = ceil_div(keys_item, 64);
-          p.prefill_blocks += blocks;
-          p.prefill_longest = std::max(p.prefill_longest, blocks);
         }
     }
     t += n;

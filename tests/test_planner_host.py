@@ -144,3 +144,37 @@ def test_partial_sums_at_the_edges_of_their_range():
     assert B.hs_op_gemm_part_splits(9, 3584, 3584) == 0              # the small-step fold
     assert B.hs_op_gemm_part_splits(0, 1024, 1024) == -1 and B.hs_op_gemm_part_splits(8, 1020, 1024) == -1
     assert B.hs_op_gemm_part_splits(8, 1024, 40) == -1
+
+
+# dims, prefill chunks, cached tokens of the chunks, decode contexts -> items at budget, from the forms that measured faster
+SHARES = {
+    "denoise_2": ("c6_dit", [256] * 2, [0] * 2, [], {148: 64, 74: 64, 52: 32, 37: 32}),
+    "denoise_4": ("c6_dit", [256] * 4, [0] * 4, [], {148: 128, 96: 64, 37: 64}),
+    "denoise_5": ("c6_dit", [256] * 5, [0] * 5, [], {148: 80}),
+    "chunk_100": ("c3_7b", [100], [1000], [300, 700, 1500, 2200, 2600, 2900, 999], {148: 28, 96: 28, 48: 16}),
+    "chunk_394": ("c3_7b", [394], [1000], [300, 700, 1500, 2200, 2600, 2900, 999], {148: 100, 96: 52, 48: 52}),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SHARES))
+def test_prefill_items_of_one_tile_only_where_each_has_an_sm_of_the_kernels_share(name):
+    wname, q, c, dec, want = SHARES[name]
+    dims = wl.DIMS[wname]
+    stage, batch_c, batch = _stage_and_batch(dims, q + [1] * len(dec), c + dec)
+    mt = max(8, (128 // (dims.n_q_heads // dims.n_kv_heads)) & ~7)
+    singles = sum(-(-n // mt) for n in q) * dims.n_kv_heads
+    doubles = sum(-(-n // (2 * mt)) for n in q) * dims.n_kv_heads
+    try:
+        for budget in sorted({1, 2, 15, 16, 17, 147} | set(want)):
+            n, sms = B.hs_stage_plan_shares(stage, batch_c, budget)
+            assert n in (singles, doubles)
+            assert sms == 0 or (dec and 4 <= sms <= budget - 4 and budget >= 16)
+            if n == singles != doubles:
+                assert n <= budget - sms
+            if budget in want:
+                assert n == want[budget], (budget, n)
+        for budget in (0, 149):
+            with pytest.raises(B.HsError):
+                B.hs_stage_plan_shares(stage, batch_c, budget)
+    finally:
+        B.hs_stage_destroy(stage)
