@@ -73,3 +73,44 @@ def test_a_step_sees_gains_written_right_in_front_of_it(budget):
             assert torch.equal(logits[i], logits[0] * float(gains[i % 4][0])), i
     finally:
         B.hs_head_destroy(head)
+
+
+@pytest.mark.gpu
+def test_the_first_maximum_of_rows_of_infinities_and_zeros():
+    """Infinite logits of either sign, beside NaN ones too (never the maximum), and rows that underflow to zeros."""
+    dev = torch.device("cuda:0")
+    d, V, n = 256, 1032, 6
+    g = torch.Generator().manual_seed(8)
+    w = (0.02 * torch.randn(V, d, generator=g)).to(torch.bfloat16)
+    w[:, 0] = 0.0
+    w[700:, 0] = float("-inf")                    # logits -inf or +inf by the sign of the row's first element, NaN where it is 0
+    y = torch.randn(n, d, generator=g)
+    y[0, 0], y[1, 0], y[2, 0] = 1.0, -1.0, 0.0
+    for budget, everywhere, scale in ((148, False, 1.0), (5, True, 1.0), (148, False, 2.0 ** -120)):
+        if everywhere:
+            w[:, 0] = float("-inf")
+        if scale != 1.0:                          # gain and weights so small that every product underflows
+            w = (torch.randn(V, d, generator=g) * scale).to(torch.bfloat16)
+        wd, yd = w.to(dev), y.to(dev)
+        gain = torch.full((d,), scale, dtype=torch.bfloat16, device=dev)
+        cfg = B.make_head_config(d, V, 1e-6, 128)
+        ws = torch.empty(B.hs_head_workspace_bytes(cfg), dtype=torch.uint8, device=dev)
+        head = B.hs_head_create(cfg, gain.data_ptr(), wd.data_ptr(), ws.data_ptr())
+        try:
+            rows = torch.arange(n, dtype=torch.int32, device=dev)
+            logits = torch.empty(n, V, device=dev)
+            tokens = torch.full((n,), -7, dtype=torch.int32, device=dev)
+            B.hs_head_step(head, yd.data_ptr(), rows.data_ptr(), n, logits.data_ptr(), tokens.data_ptr(), budget)
+            torch.cuda.synchronize()
+            lg, got = logits.cpu().numpy(), tokens.cpu().numpy()
+            for r in range(n):
+                if np.isnan(lg[r]).all():
+                    assert got[r] == 0x7fffffff
+                else:
+                    assert got[r] == int(np.flatnonzero(lg[r] == np.nanmax(lg[r]))[0]), r
+            if scale != 1.0:
+                assert not lg.any() and not got.any()
+            elif everywhere:
+                assert np.isneginf(lg[0]).all() and np.isposinf(lg[1]).all() and got[0] == 0 and got[1] == 0
+        finally:
+            B.hs_head_destroy(head)
