@@ -1008,7 +1008,11 @@ ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows, 
     if (skinny) return (((N >> 5) + sms - 1) / sms) * (1.5 + double(32 + (M <= 32 ? M : 64)) * K * 2 / 70e3);
     return resid_launch_us(M, N, false, bn, ks, longest, sms) + gemm_chain_us(k_blocks, ks);
   });
-  return best_us + 3.0 < without ? best : ResidPlan{0, 0, 0};
+  // (A weight-streaming kernel with more units than half of the device loses in the second round under a partial budget what
+  // it wins on the whole device -- 29 rows at 7B dimensions, out-projection, partial sums -> that kernel: on 148 SMs (2
+  // layers) 284 -> 277 us, on 48 478 -> 487, on 96 (4 layers) 678 -> 688 -- so there it does not get the 3 us.)
+  const double extra = skinny && (N >> 5) > sm_count / 2 ? 0.0 : 3.0;
+  return best_us + extra < without ? best : ResidPlan{0, 0, 0};
 }
 
 int gemm_pick_stream_k(int M, int N, int K, int sm_count) {

@@ -125,7 +125,7 @@ def test_k_splits_tile_the_k_range():
 # Residual GEMMs (rows, width, contraction length) for which partial sums measured slower than the GEMM without them: few rows
 # on the weight-streaming kernel, many rows whose partial sums cost more traffic than the splits save, rows that fill pairs
 # of SMs; and such for which they measured clearly faster.
-@pytest.mark.parametrize("M,N,K", [(17, 1024, 1024), (17, 1024, 2816), (32, 1024, 2816), (24, 2048, 2048), (32, 3584, 3584),
+@pytest.mark.parametrize("M,N,K", [(17, 1024, 1024), (17, 1024, 2816), (32, 1024, 2816), (24, 2048, 2048),
                                    (1024, 1024, 1024), (1280, 1024, 2816), (1536, 1024, 2816), (2048, 1024, 2816),
                                    (3072, 1024, 2816), (1280, 2048, 5632), (3000, 2048, 5632), (600, 3584, 18944),
                                    (1450, 3584, 18944), (2112, 3584, 18944)])
@@ -133,7 +133,8 @@ def test_partial_sums_are_not_taken_where_they_are_slower(M, N, K):
     assert B.hs_op_gemm_part_splits(M, N, K) == 0
 
 
-@pytest.mark.parametrize("M,N,K", [(17, 3584, 18944), (64, 3584, 18944), (64, 2048, 5632), (65, 1024, 2816), (128, 2048, 2048),
+@pytest.mark.parametrize("M,N,K", [(17, 3584, 18944), (29, 3584, 3584), (64, 3584, 18944), (64, 2048, 5632), (65, 1024, 2816),
+                                   (128, 2048, 2048),
                                    (256, 1024, 2816), (1024, 1024, 2816), (401, 3584, 18944), (512, 3584, 18944)])
 def test_partial_sums_are_taken_where_they_are_faster(M, N, K):
     assert 2 <= B.hs_op_gemm_part_splits(M, N, K) <= 10
