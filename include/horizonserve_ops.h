@@ -65,7 +65,9 @@ hs_status_t hs_stage_debug_buffer(hs_stage_t *stage, const char *name, void **de
  * and decode attention kernels of a layer, which otherwise run side by side on two shares of the budget, run one
  * after the other on the whole budget), so the per-class times add up to more than an unprofiled step takes.
  * A residual GEMM that folds the RMSNorm behind it is timed with that work (classes 5 and 7); class 0 then counts
- * the one norm launch a step keeps.
+ * the one norm launch a step keeps.  Where a residual GEMM leaves partial sums, the norm that adds them is timed with
+ * that work (class 0); the last layer's, which no norm follows, are added by a launch that is timed with class 7 and
+ * has no entry in the SM census.
  * Classes: 0 rmsnorm, 1 qkv gemm, 2 prefill attention, 3 decode attention (with the merge of its split
  * partials), 4 unused (always zero; kept so that the class numbers stay what they were),
  * 5 out-proj gemm, 6 gate/up gemm, 7 down gemm.

@@ -720,8 +720,11 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   // folded, under a partial budget: after the first norm, ONE cooperative launch does all layers (launch_small_step);
   // the same device functions on the same units and items, so the same bits as the launches below (which is why this
   // choice may look at the budget).  At the full budget the separate launches overlap each other's set-up and are the
-  // faster form (talker step 0.40 ms against 0.52); below it they run strictly one after the other (0.58 / 0.60 /
-  // 0.75 ms at 112 / 74 / 37 SMs against 0.52 / 0.54 / 0.69 in one launch).  Not while the per-kernel timers run.
+  // faster form.  Below it the one launch was the faster one while separate launches waited for the completed kernel in
+  // front (talker step at 112 / 74 / 37 SMs 0.52 / 0.54 / 0.69 ms against 0.58 / 0.60 / 0.75).  Against launches that are
+  // placed while that kernel leaves (kOverlapLate) it no longer is: 0.41 / 0.43 / 0.58 in one launch, 0.37 / 0.39 / 0.53
+  // separate; beside a backbone on 96 SMs, on the other 52, 0.69 and 0.58.  The rule has not been changed for that yet.
+  // Not while the per-kernel timers run.
   const bool one_launch = sk_fold_mlp && sk_fold_attn && skinny(d, q_dim + 2 * kv_dim, kGemmQkv) && skinny(d, F, kGemmGateUp) &&
                           plan.n_prefill_items == 0 && plan.n_decode_items > 0 && !s->profile && sm_budget < s->sm_count;
   for (int l = 0; l < c.n_layers && e == cudaSuccess; ++l) {
@@ -928,7 +931,8 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
       LaunchTimer t(s, 7, stream); where = "down gemm"; e = launch_gemm_skinny(k, sm_budget, stream);
     } else {
       LaunchTimer t(s, 7, stream); where = "down gemm"; e = launch_gemm(gd, sm_budget, stream);
-      if (e == cudaSuccess && parts_down.ks > 0 && l + 1 == c.n_layers) {     // no norm follows: the sum alone
+      if (e == cudaSuccess && parts_down.ks > 0 && l + 1 == c.n_layers) {     // no norm follows: the sum alone (class 7)
+        np.smid_log = nullptr;                                                // (the census keeps the last norm's slots)
         np.h = nullptr;
         np.n_parts = 0;
         np.gate_which = 0;
