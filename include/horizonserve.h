@@ -139,8 +139,8 @@ typedef struct {
  *  KV pool: bf16 [n_layers][2 (K,V)][num_pages][n_kv_heads][16][head_dim]; K is stored after RoPE.
  *           One (page, head) block is 16*head_dim*2 contiguous bytes.  Must be 256-byte aligned (what cudaMalloc gives).
  *  Workspace: private scratch of the stage (activations, RoPE table, step metadata, attention
- *           partials and, unless HS_FLAG_BF16_ACTIVATIONS is set, fp16 copies of all projection weights, i.e.
- *           as many bytes again as those weights).  Must be 256-byte aligned (what cudaMalloc gives).  Its
+ *           partials, up to 40 MB of partial sums of the residual projections and, unless HS_FLAG_BF16_ACTIVATIONS is
+ *           set, fp16 copies of all projection weights, i.e. as many bytes again as those weights).  Must be 256-byte aligned (what cudaMalloc gives).  Its
  *           contents are meaningless to the caller.
  * Both return 0 for an invalid configuration.
  */
@@ -189,9 +189,9 @@ hs_status_t hs_stage_plan(hs_stage_t *stage, const hs_batch_t *batch, int32_t *t
  * ctx_len .. ctx_len + q_len - 1; their K/V are written to the cache pages named by the block table and
  * every new token attends causally to positions 0..p.  y_out receives all n_tokens rows.  Re-running
  * the same step rewrites the same slots with the same values.  The caller advances ctx_len itself.
- * With sm_budget < the device's SM count every kernel of the step starts only after the previous one has
- * ended, so that no block of the step ever sits on an SM outside the budget; with sm_budget == SM count
- * (no co-running neighbour) each kernel's set-up overlaps the previous kernel's drain.  A decode-only step of at
+ * With sm_budget < the device's SM count every kernel of the step is placed only when the last block of the
+ * previous one has left, so that no block of the step ever sits on an SM outside the budget; with sm_budget == SM
+ * count (no co-running neighbour) each kernel's set-up overlaps the previous kernel's drain.  A decode-only step of at
  * most 16 rows under a partial budget runs, after its first RMSNorm, as one cooperative launch of at most sm_budget
  * blocks whose phases are the same kernels' bodies separated by bounded grid-wide barriers (same results; the
  * separate launches are used instead where the device refuses a cooperative launch).  With both prefill and decode

@@ -171,8 +171,9 @@ constexpr int dc_smem_bytes() {
 // followed by one int (the abort flag) in shared memory outside that area.  The calling thread block is number
 // `block` of `n_blocks` working on the launch's items; it may have more than DC_WARPS warps (the others only take
 // part in the two block barriers).  `layer` and `counters` (this layer's two queue heads) stand in for the fields of
-// the same names in `p`, which holds the tensor map and therefore cannot be copied per layer.  `wait` is called once by every thread, after the set-up and the requests that do
-// not depend on the previous kernel or phase, and must return when that predecessor's writes are visible.
+// the same names in `p`, which holds the tensor map and therefore cannot be copied per layer.  `wait` is called once by
+// every thread, after the set-up and the requests that do not depend on the previous kernel or phase, and must return
+// when that predecessor's writes are visible.
 template <int DH, typename Wait>
 __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer, int32_t* counters, uint8_t* smem,
                                                  uint64_t* full_all, int block, int n_blocks, Wait wait) {

@@ -21,8 +21,8 @@
 //               end is exact whatever reference was used; values stay far inside the range of bf16 and fp32.
 //   pipeline    two tiles x two S buffers: while one tile's warp group exponentiates, the tensor core works on the
 //               other tile's products.  The tensor core runs its instructions in issue order, which is what makes
-//               the overlay safe: S of block j + 2 is issued after the P V product of block j, whose P it replaces.  K and V blocks arrive by TMA in two rings of their own
-//               ([half][page][16][64] tiles with the 128-byte swizzle, the K tile being a K-major and the V tile an
+//               the overlay safe: S of block j + 2 is issued after the P V product of block j, whose P it replaces.
+//               K and V blocks arrive by TMA in two rings of their own ([half][page][16][64] tiles with the 128-byte swizzle, the K tile being a K-major and the V tile an
 //               MN-major operand): a K slot is free again as soon as the block's scores are computed, a V slot
 //               after its P V products.  The producers own the work queue and run ahead across items.
 //   roles       warps 0..3 softmax of tile A, warps 4..7 softmax of tile B (thread = row = TMEM lane), warp 8 and

@@ -656,60 +656,61 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           __syncwarp();
           epi_sel = 0;
         } else {
-        float best_v = -INFINITY;              // greedy sampling: this thread's row over the tile
-        int best_c = 0x7fffffff;
-        for (int c = 0; c < p.bn / 32; ++c) {
-          const int col0 = n * p.bn + c * 32;
-          if (col0 >= p.N) break;
-          tmem_ld32(taddr + c * 32, r0);
-          float4 gv[8];
-          const int nv = p.N - col0 >= 32 ? 8 : (p.N - col0) >> 2;          // float4s of the chunk inside the row
-          if (gate) {                              // requested while the accumulator chunk is on its way
+          float best_v = -INFINITY;              // greedy sampling: this thread's row over the tile
+          int best_c = 0x7fffffff;
+          for (int c = 0; c < p.bn / 32; ++c) {
+            const int col0 = n * p.bn + c * 32;
+            if (col0 >= p.N) break;
+            tmem_ld32(taddr + c * 32, r0);
+            float4 gv[8];
+            const int nv = p.N - col0 >= 32 ? 8 : (p.N - col0) >> 2;          // float4s of the chunk inside the row
+            if (gate) {                              // requested while the accumulator chunk is on its way
 #pragma unroll
-            for (int e = 0; e < 8; ++e) gv[e] = e < nv ? __ldg(reinterpret_cast<const float4*>(gate + col0) + e) : make_float4(1.f, 1.f, 1.f, 1.f);
-          }
-          tmem_ld_wait();
-          if (gate) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              r0[4 * e] = __float_as_uint(__uint_as_float(r0[4 * e]) * gv[e].x);
-              r0[4 * e + 1] = __float_as_uint(__uint_as_float(r0[4 * e + 1]) * gv[e].y);
-              r0[4 * e + 2] = __float_as_uint(__uint_as_float(r0[4 * e + 2]) * gv[e].z);
-              r0[4 * e + 3] = __float_as_uint(__uint_as_float(r0[4 * e + 3]) * gv[e].w);
+              for (int e = 0; e < 8; ++e)
+                gv[e] = e < nv ? __ldg(reinterpret_cast<const float4*>(gate + col0) + e) : make_float4(1.f, 1.f, 1.f, 1.f);
             }
-          }
-          if (!PAIR && p.argmax_key != nullptr) {
-            // (N is a multiple of 8; a NaN is never the maximum; columns ascend, so the first maximum stays)
-            float mx = -INFINITY;
+            tmem_ld_wait();
+            if (gate) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (col0 + (e & ~7) < p.N) mx = fmaxf(mx, __uint_as_float(r0[e]));
-            if (mx > best_v || best_c == 0x7fffffff) {
-#pragma unroll
-              for (int e = 31; e >= 0; --e)
-                if (col0 + (e & ~7) < p.N && __uint_as_float(r0[e]) == mx) best_c = col0 + e;
-              best_v = mx;
+              for (int e = 0; e < 8; ++e) {
+                r0[4 * e] = __float_as_uint(__uint_as_float(r0[4 * e]) * gv[e].x);
+                r0[4 * e + 1] = __float_as_uint(__uint_as_float(r0[4 * e + 1]) * gv[e].y);
+                r0[4 * e + 2] = __float_as_uint(__uint_as_float(r0[4 * e + 2]) * gv[e].z);
+                r0[4 * e + 3] = __float_as_uint(__uint_as_float(r0[4 * e + 3]) * gv[e].w);
+              }
             }
+            if (!PAIR && p.argmax_key != nullptr) {
+              // (N is a multiple of 8; a NaN is never the maximum; columns ascend, so the first maximum stays)
+              float mx = -INFINITY;
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (col0 + (e & ~7) < p.N) mx = fmaxf(mx, __uint_as_float(r0[e]));
+              if (mx > best_v || best_c == 0x7fffffff) {
+#pragma unroll
+                for (int e = 31; e >= 0; --e)
+                  if (col0 + (e & ~7) < p.N && __uint_as_float(r0[e]) == mx) best_c = col0 + e;
+                best_v = mx;
+              }
+            }
+            if (lane == 0) bulk_wait_read<1>();     // the block staged two chunks ago has been read
+            __syncwarp();
+            uint8_t* buf = epi_buf + epi_sel * EPI_BUF_BYTES;
+            stage_f32x32(buf, lane, r0);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+              if (add) tma_reduce_add_2d(&p.tm_out, buf, col0, row_base);
+              else if (store_ok) tma_store_2d(&p.tm_out, buf, col0, out_row);
+              bulk_commit();
+            }
+            epi_sel ^= 1;
           }
-          if (lane == 0) bulk_wait_read<1>();     // the block staged two chunks ago has been read
-          __syncwarp();
-          uint8_t* buf = epi_buf + epi_sel * EPI_BUF_BYTES;
-          stage_f32x32(buf, lane, r0);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) {
-            if (add) tma_reduce_add_2d(&p.tm_out, buf, col0, row_base);
-            else if (store_ok) tma_store_2d(&p.tm_out, buf, col0, out_row);
-            bulk_commit();
+          if (!PAIR && p.argmax_key != nullptr && row_ok) {
+            const uint32_t u = __float_as_uint(best_v + 0.f);                       // (-0 and +0 are the same value)
+            const uint32_t ord = u & 0x80000000u ? ~u : u | 0x80000000u;
+            atomicMax(p.argmax_key + row, (static_cast<unsigned long long>(ord) << 32) | (0xffffffffu - uint32_t(best_c)));
+            __threadfence();
           }
-          epi_sel ^= 1;
-        }
-        if (!PAIR && p.argmax_key != nullptr && row_ok) {
-          const uint32_t u = __float_as_uint(best_v + 0.f);                       // (-0 and +0 are the same value)
-          const uint32_t ord = u & 0x80000000u ? ~u : u | 0x80000000u;
-          atomicMax(p.argmax_key + row, (static_cast<unsigned long long>(ord) << 32) | (0xffffffffu - uint32_t(best_c)));
-          __threadfence();
-        }
         }
         if (ordered && !(ks == 0 && un.last) && lane == 0) {    // a tile with a single segment needs no turn
           bulk_wait<0>();                     // this segment's adds have been performed

@@ -40,9 +40,10 @@ struct GemmParams {
   int bn;                    // tile width of this launch (gemm_pick_bn); 256 when unused
   int ksplit;                // K splits per output tile, added in split order (gemm_pick_ksplit); 0/1 = none
   int stream_k_slots;        // pairs only: > 0 = cut the tiles' K blocks into this many equal runs (gemm_pick_stream_k)
-  // Resid in store mode on single blocks, optional: greedy sampling of every row (argmax_key non-null).  The tile's epilogue, which holds the
-  // values in registers, maximises the row's key -- order-preserving bits of the value above the complement of the
-  // column, so that the first maximum wins whatever the order -- and the block that leaves last turns the keys into tokens.
+  // Resid in store mode on single blocks, optional: greedy sampling of every row (argmax_key non-null).  The tile's
+  // epilogue, which holds the values in registers, maximises the row's key -- order-preserving bits of the value above
+  // the complement of the column, so that the first maximum wins whatever the order -- and the block that leaves last
+  // turns the keys into tokens.
   unsigned long long* argmax_key;   // [M], zero at entry and at exit
   int* argmax_done;          // one counter, zero at entry and at exit
   int32_t* argmax_token;     // [M]: lowest column of the row's maximum

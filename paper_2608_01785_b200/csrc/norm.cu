@@ -263,7 +263,8 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
 // threads work on a row (as many as leave one round of rows on the device, at most 512), each holds its V groups of
 // four columns in registers, so a launch is one round trip to memory, one reduction and one write.  What bounds it is
 // that latency: one warp per row (the kernel above) took 8.2 us per launch at 64 x 3584 and 9.3 us at 1024 x 1024
-// (conditioned), this one 5.4 us with three partial sums to add and 9.5-10 with two (ncu).  Sums: a thread's groups in order, a butterfly per warp, the warps in
+// (conditioned); this one takes 5.4 with three partial sums to add and 7.7 with ten, and 7.5 without any and 10.1 with
+// three (single launches under the profiler, each).  Sums: a thread's groups in order, a butterfly per warp, the warps in
 // order -- a function of the shape and the device's SM count, never of the budget.
 constexpr int ROW_THREADS = kNormRowThreads;
 

@@ -196,7 +196,7 @@ EDGE = {
     "long_prefill_dh128": (wl.StageDims(1, 256, 8, 1, 128, 640), [700, 1], [0, 1500]),
     "many_sequences": (wl.StageDims(1, 256, 4, 2, 64, 688), [1] * 40 + [3] * 10, list(range(0, 400, 10)) + [5] * 10),
     "two_layers_talker_like": (wl.StageDims(2, 1024, 16, 4, 64, 2816), [1] * 16, [128 + 57 * i for i in range(16)]),
-    # few tokens against a long K: the QKV and gate/up GEMMs split K four ways through the scratch tile
+    # few tokens against a long K
     "small_step_split_k": (wl.StageDims(1, 2048, 8, 2, 128, 1024), [20, 1, 1], [0, 300, 17]),
     # the RoPE base of long-context checkpoints, positions up to 3000
     "rope_base_1e6": (wl.StageDims(1, 256, 4, 2, 64, 688, rope_base=1.0e6), [90, 1, 1], [0, 2999, 1500]),
@@ -637,7 +637,7 @@ def test_small_step_takes_the_norms_into_its_projections(orc, n_rows, flags):
 GUARDED = {
     # all four projections on SM pairs, both norms folded, stream-K residual GEMMs, both attention kernels side by side
     "pairs_folded": (wl.StageDims(2, 1024, 16, 4, 64, 2048), [1400, 1100] + [1] * 40, [0, 200] + [57 + 13 * i for i in range(40)]),
-    # single blocks with a K split, ragged row tile
+    # single blocks, residual GEMMs with partial sums, ragged row tile
     "single_blocks": (wl.StageDims(2, 512, 8, 2, 64, 1408), [100, 21, 1], [0, 40, 300]),
     # weight-streaming kernel with the small-step fold
     "small_step": (wl.StageDims(2, 1024, 16, 2, 64, 3072), [1] * 11, [33 + 29 * i for i in range(11)]),
@@ -648,8 +648,8 @@ GUARDED = {
 @pytest.mark.parametrize("name", sorted(GUARDED))
 def test_a_step_writes_nothing_outside_its_buffers(name):
     """Guard bytes in front of and behind the workspace, the KV pool, x_in and y_out keep their pattern through steps
-    at several budgets (the step forms differ: SM pairs with folded norms and stream-K, single blocks with a K split,
-    the weight-streaming kernel); y_out is written completely."""
+    at several budgets (the step forms differ: SM pairs with folded norms and stream-K, single blocks with partial
+    sums, the weight-streaming kernel); y_out is written completely."""
     dims, q_len, ctx_len = GUARDED[name]
     batch = wl.BatchSpec(list(q_len), list(ctx_len))
     case = make_case(dims, batch, seed=5, kv_fill=True)
