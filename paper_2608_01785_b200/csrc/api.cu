@@ -193,7 +193,6 @@ hs_status_t ensure_attributes(int device) {
   if ((e = attention_set_attributes()) != cudaSuccess) return cuda_fail("attention attributes", e);
   if ((e = head_set_attributes()) != cudaSuccess) return cuda_fail("head attributes", e);
   if ((e = gemm_skinny_set_attributes()) != cudaSuccess) return cuda_fail("small-step gemm attributes", e);
-  if ((e = small_step_set_attributes()) != cudaSuccess) return cuda_fail("one-launch small step attributes", e);
   if (device >= 0 && device < 64) g_attrs_set[device] = true;
   return HS_OK;
 }
@@ -546,17 +545,6 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   if (st != HS_OK) return st;
   s->ring_pos = (slot + 1) % kRing;
 
-  {  // the layers' constants for the one-launch small step travel with the metadata (biases may change between steps)
-    static_assert(sizeof(SmallLayer) == 24 * 4, "MetaLayout::small_layers holds 24 words per layer");
-    SmallLayer* sl = reinterpret_cast<SmallLayer*>(s->pinned[slot] + s->ml.small_layers);
-    for (int l = 0; l < c.n_layers; ++l) {
-      const hs_layer_weights_t& wo = s->operands[l];
-      sl[l] = SmallLayer{wo.w_q, wo.w_k, wo.w_v, wo.w_o, wo.w_gate, wo.w_up, wo.w_down,
-                         static_cast<const __nv_bfloat16*>(s->layers[l].g_attn),
-                         static_cast<const __nv_bfloat16*>(s->layers[l].g_mlp),
-                         {s->qkv_bias[l].b[0], s->qkv_bias[l].b[1], s->qkv_bias[l].b[2]}};
-    }
-  }
   int32_t* meta = reinterpret_cast<int32_t*>(s->ws_dev + s->ws.meta);
   if (cudaMemcpyAsync(meta, s->pinned[slot], size_t(s->ml.total) * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(s->ev[slot], stream) != cudaSuccess)
@@ -716,17 +704,6 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     a.smid_log = slots(2);       // prefill in class 2, decode in class 3 (the next slots)
     return a;
   };
-  // A decode-only step of at most 16 rows whose projections all run on the weight-streaming kernel with the norms
-  // folded, under a partial budget: after the first norm, ONE cooperative launch does all layers (launch_small_step);
-  // the same device functions on the same units and items, so the same bits as the launches below (which is why this
-  // choice may look at the budget).  At the full budget the separate launches overlap each other's set-up and are the
-  // faster form.  Below it the one launch was the faster one while separate launches waited for the completed kernel in
-  // front (talker step at 112 / 74 / 37 SMs 0.52 / 0.54 / 0.69 ms against 0.58 / 0.60 / 0.75).  Against launches that are
-  // placed while that kernel leaves (kOverlapLate) it no longer is: 0.41 / 0.43 / 0.58 in one launch, 0.37 / 0.39 / 0.53
-  // separate; beside a backbone on 96 SMs, on the other 52, 0.69 and 0.58.  The rule has not been changed for that yet.
-  // Not while the per-kernel timers run.
-  const bool one_launch = sk_fold_mlp && sk_fold_attn && skinny(d, q_dim + 2 * kv_dim, kGemmQkv) && skinny(d, F, kGemmGateUp) &&
-                          plan.n_prefill_items == 0 && plan.n_decode_items > 0 && !s->profile && sm_budget < s->sm_count;
   for (int l = 0; l < c.n_layers && e == cudaSuccess; ++l) {
     const hs_layer_weights_t& w = s->layers[l];
     const LayerMaps& m = s->maps[l];
@@ -754,32 +731,6 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     const bool folded_attn_norm = (fold_norm || sk_fold_attn) && l > 0;   // the previous layer's down-projection produced h and the sums
     if (!folded_attn_norm) { LaunchTimer t(s, 0, stream); where = "rmsnorm"; e = launch_rmsnorm(np, sm_budget, stream); }
     if (e != cudaSuccess) break;
-    if (one_launch) {
-      SmallStepParams sp{};
-      sp.attn = make_attn(0);
-      sp.attn.smid_log = nullptr;
-      sp.layers = reinterpret_cast<const SmallLayer*>(meta + s->ml.small_layers);
-      sp.n_layers = c.n_layers; sp.T = T; sp.d = d; sp.F = F; sp.f16 = f16;
-      sp.q_dim = q_dim; sp.kv_dim = kv_dim; sp.head_dim = Dh; sp.n_kv_heads = c.n_kv_heads;
-      sp.x = x; sp.h = h; sp.q = q; sp.o = o;
-      sp.act = reinterpret_cast<__nv_bfloat16*>(s->ws_dev + s->ws.act);
-      sp.kv_pool = s->kv_pool; sp.layer_kv_elems = layer_kv_elems;
-      sp.tok_pos = meta + s->ml.tok_pos; sp.tok_slot = meta + s->ml.tok_slot;
-      sp.rope = reinterpret_cast<const float2*>(s->ws_dev + s->ws.rope);
-      sp.counters = meta + s->ml.counters;
-      sp.row_ss = reinterpret_cast<float*>(s->ws_dev + s->ws.row_ss);
-      sp.eps = c.rms_eps;
-      sp.grid_bar = meta + s->ml.grid_bar;
-      sp.status = status;
-      sp.smid_log = slots(1);
-      where = "small step"; e = launch_small_step(sp, sm_budget, stream);
-      // a device or context that cannot hold the grid resident at once (or knows no cooperative launch) takes the
-      // separate launches below: the same results
-      if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) break;
-      cudaGetLastError();
-      e = cudaSuccess;
-    }
-
     GemmParams g{};
     g.tm_a = a_rows == 128 ? s->tm_h : s->tm_h_s[a_sel];
     g.a_box_rows = a_rows;

@@ -10,10 +10,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) attn_decode_kernel(const __grid
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full_all = reinterpret_cast<uint64_t*>(smem + DC_WARPS * DC_STAGES * 2 * Geom<DH>::PAGE_BYTES);
   log_smid(p.smid_log ? p.smid_log + kSmidSlots : nullptr);
-  attn_decode_body<DH>(p, p.layer, p.counters, smem, full_all, int(blockIdx.x), int(gridDim.x), [&] {
-    griddep_wait();
-    griddep_launch_dependents(p.overlap);
-  });
+  attn_decode_body<DH>(p, smem, full_all);
 }
 
 template <typename K>

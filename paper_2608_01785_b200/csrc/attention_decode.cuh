@@ -40,8 +40,8 @@ __device__ __forceinline__ int kv_off(int kk, int cc) {
 }
 // Requests the K and the V block of (layer, page, KV head) with one copy: [K | V][half][16 keys][128 B].
 template <int DH>
-__device__ __forceinline__ void load_page(const AttnParams& p, int layer, uint8_t* dst, uint64_t* bar, int page, int hk) {
-  tma_load_4d(dst, &p.tm_kv_page, bar, 0, (page * p.n_kv_heads + hk) * 16, 0, layer * 2);
+__device__ __forceinline__ void load_page(const AttnParams& p, uint8_t* dst, uint64_t* bar, int page, int hk) {
+  tma_load_4d(dst, &p.tm_kv_page, bar, 0, (page * p.n_kv_heads + hk) * 16, 0, p.layer * 2);
 }
 __device__ __forceinline__ float quad_max(float v) {
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -166,23 +166,16 @@ constexpr int dc_smem_bytes() {
   return b > kMinSmemBytes ? b : kMinSmemBytes;
 }
 
-// The body of the decode kernel as a device function, so that the kernel of its own and the one-launch small step
-// share it.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS * DC_STAGES mbarriers
-// followed by one int (the abort flag) in shared memory outside that area.  The calling thread block is number
-// `block` of `n_blocks` working on the launch's items; it may have more than DC_WARPS warps (the others only take
-// part in the two block barriers).  `layer` and `counters` (this layer's two queue heads) stand in for the fields of
-// the same names in `p`, which holds the tensor map and therefore cannot be copied per layer.  `wait` is called once by
-// every thread, after the set-up and the requests that do not depend on the previous kernel or phase, and must return
-// when that predecessor's writes are visible.
-template <int DH, typename Wait>
-__device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer, int32_t* counters, uint8_t* smem,
-                                                 uint64_t* full_all, int block, int n_blocks, Wait wait) {
+// The body of the decode kernel.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS *
+// DC_STAGES mbarriers followed by one int (the abort flag) in shared memory outside that area.
+template <int DH>
+__device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* smem, uint64_t* full_all) {
   using G_ = Geom<DH>;
   constexpr int SLOT_BYTES = 2 * G_::PAGE_BYTES;    // K page then V page
   volatile int* abort_flag = reinterpret_cast<volatile int*>(full_all + DC_WARPS * DC_STAGES);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool worker = warp < DC_WARPS;
+  const int block = int(blockIdx.x), n_blocks = int(gridDim.x);
   const int G = p.n_q_heads / p.n_kv_heads;
   const int q_dim = p.n_q_heads * DH;
   const float scale_log2 = kLog2e / sqrtf(float(DH));
@@ -195,14 +188,14 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
   }
   __syncthreads();
 
-  uint8_t* slots = smem + (worker ? warp : 0) * DC_STAGES * SLOT_BYTES;
-  uint64_t* full = full_all + (worker ? warp : 0) * DC_STAGES;
+  uint8_t* slots = smem + warp * DC_STAGES * SLOT_BYTES;
+  uint64_t* full = full_all + warp * DC_STAGES;
   int fill = 0;                           // ring slot of the next page to request, over all items of this warp
   int cur = 0;                            // ring slot of the next page to read, and its phase
   uint32_t cur_phase = 0;
   auto issue = [&](int page, int hk) {      // lane 0: request one page of an item
     mbar_expect_tx(&full[fill], SLOT_BYTES);
-    load_page<DH>(p, layer, slots + fill * SLOT_BYTES, &full[fill], page, hk);
+    load_page<DH>(p, slots + fill * SLOT_BYTES, &full[fill], page, hk);
     if (++fill == DC_STAGES) fill = 0;
   };
 
@@ -210,7 +203,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
   // the queue hands out the items after those.  The first item's record, its page ids and those of its first pages
   // that lie wholly inside the cached context are fetched before the wait for the previous kernel: the step's
   // metadata was copied before any kernel of the step started, and this step writes K / V at positions >= ctx only.
-  int item = worker ? block * DC_WARPS + warp : p.n_decode_items;
+  int item = block * DC_WARPS + warp;
   int4 it = make_int4(0, 0, 0, 0), dr = it;
   int my_page = 0, ahead = 0;             // ahead: pages of the current item already requested
   if (item < p.n_decode_items) {
@@ -229,7 +222,8 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
       }
     }
   }
-  wait();
+  griddep_wait();
+  griddep_launch_dependents(p.overlap);
 
   // Group mode (p.decode_group, a batch whose items would not fill the device's warps): item 8 g + w is the w-th
   // eighth of the pages of group g = (sequence, KV head); a block takes whole groups -- g = block, block + n_blocks,
@@ -240,9 +234,9 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
   for (int round = 0;; ++round) {
     if (!first_round) {
       if (group_mode) {
-        item = worker ? (block + round * n_blocks) * DC_WARPS + warp : p.n_decode_items;
+        item = (block + round * n_blocks) * DC_WARPS + warp;
       } else {
-        if (lane == 0) item = n_blocks * DC_WARPS + atomicAdd(counters + 1, 1);
+        if (lane == 0) item = n_blocks * DC_WARPS + atomicAdd(p.counters + 1, 1);
         item = __shfl_sync(0xffffffffu, item, 0);
       }
     }
@@ -278,7 +272,6 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
 #pragma unroll
     for (int ks = 0; ks < DH / 16; ++ks) {
       const int c = ks * 16 + 2 * (lane & 3);
-      // (read through the L2: in the one-launch small step another block of the same launch wrote q)
       qf[ks][0] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + ra * DH + c)) : 0u;
       qf[ks][1] = rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + rb * DH + c)) : 0u;
       qf[ks][2] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + ra * DH + c + 8)) : 0u;
@@ -404,7 +397,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, int layer,
       if (!failed) {
         // the eight partials are merged in slice order by the whole block: a thread per pair of output columns
         const bool f16 = p.o_f16 != 0;
-        for (int e = threadIdx.x; e < G * (DH / 2); e += blockDim.x) {
+        for (int e = threadIdx.x; e < G * (DH / 2); e += DC_THREADS) {
           const int g = e / (DH / 2), col = 2 * (e - g * (DH / 2));
           float mm = -INFINITY;
 #pragma unroll
