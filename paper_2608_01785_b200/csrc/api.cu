@@ -85,7 +85,7 @@ WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   w.status = take(256);
   w.turn = take(kGemmTurnWords * 4);
   w.smid = take(size_t(HS_PROFILE_CLASSES) * kSmidSlots * 4);
-  // partial sums of x^2 per (token, tile column) of a folded RMSNorm; steps of at most 64 rows keep one per 32 columns
+  // partial sums of x^2 per (token, tile column) of a folded RMSNorm; steps of at most 16 rows keep one per 16 columns
   w.row_ss = take(std::max(T * kRowSsStride, size_t(64) * size_t(c.d_model / 32 + 1)) * 4);
   w.row_rs = take(T * 4);                            // r of every token
   w.row_done = take((T / 32 + 2) * 4);               // tile columns delivered per group of 32 token rows
@@ -640,7 +640,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     k.norm_h = h;
     k.norm_h_f16 = f16;
     k.row_ss = reinterpret_cast<float*>(s->ws_dev + s->ws.row_ss);
-    k.ss_stride = d / 32;
+    k.ss_stride = d / 16;
     if (!consumer_is_skinny) {
       k.row_rs = reinterpret_cast<float*>(s->ws_dev + s->ws.row_rs);
       k.units_done = reinterpret_cast<int*>(s->ws_dev + s->ws.row_done);

@@ -2,17 +2,19 @@
 // weight-streaming problem, and what counts is how many SMs pull weights and how directly.  The tcgen05 kernel
 // of gemm.cu feeds 128-row tiles through TMA boxes of 128-byte pieces and needs a K split with an ordered
 // chain of adds to occupy the GPU; this kernel does the opposite:
-//   * one block per unit of 32 output columns and the WHOLE K range: no K split across blocks, no chain;
-//   * inside the block the K range is dealt over 8 warps; every warp streams its K steps of the unit's 32 weight
-//     rows with 16-byte cp.async copies into a private ring of shared memory (every lane reads back exactly the
+//   * one block per unit of 16 .. 112 weight rows and the WHOLE K range: no K split across blocks, no chain;
+//   * inside the block the K range is dealt over 8 warps; every warp streams its K steps of the unit's
+//     weight rows with 16-byte cp.async copies into a private ring of shared memory (every lane reads back exactly the
 //     16 bytes it copied, so the ring needs no barrier at all), the matching slice of the activations the same
 //     way, and feeds mma.sync m16n8k16 fragments from the ring -- no TMA, no TMEM, no mbarrier;
 //   * the 8 partial accumulators meet in shared memory and are summed in warp order, then the epilogue of the
 //     mode runs: residual add, RoPE + cache write + q store, or SwiGLU.
 // Units are listed independently of the SM budget and a unit's arithmetic is one fixed sequence, so the results
-// do not depend on the budget.  A unit's 32 columns are chosen per mode so that the epilogue finds its partner
-// columns in the same thread: Qkv units take columns c .. c+15 and c + Dh/2 .. c + Dh/2 + 15 of one head (the
-// rotation pairs), GateUp units 16 gate columns and the same 16 up columns.
+// do not depend on the budget -- nor on the width of a unit: an output element's sum is its own, and a folded norm's
+// partial sums of squares are kept per 16 columns.  So the width may be chosen by the budget (pick_width).  A unit's
+// columns are chosen per mode so that the epilogue finds its partner columns in the same thread: with P pairs of
+// 8-column tiles, Qkv units take columns c .. c + 8 P - 1 and the same of the head's other half (the rotation pairs),
+// GateUp units 8 P gate columns and the same 8 P up columns.
 //
 // Fragment trick: a lane loads 8 consecutive K elements (16 bytes) of its weight row and of its two
 // activation rows; the two MMAs of a 32-wide K step use elements 0..3 and 4..7 of those.  That is a
@@ -34,11 +36,11 @@ template <bool F16>
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1) {
   if (F16)
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
   else
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
@@ -52,10 +54,58 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-__device__ __forceinline__ uint4 lds16(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-  return v;
+// N values with the widest accesses: N * 4 bytes (N * 2 where 16-bit values are stored), aligned to their size or to 16.
+template <int N>
+__device__ __forceinline__ void lds_f32(float* v, const float* src) {
+  if constexpr (N == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(src);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    const float4 t = *reinterpret_cast<const float4*>(src);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void ldcg_f32(float (&v)[N], const float* src) {      // through the L2
+#pragma unroll
+  for (int i = 0; i < N; i += 4) {
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(src + i));
+    v[i] = t.x; v[i + 1] = t.y; v[i + 2] = t.z; v[i + 3] = t.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void ldg_f32(float (&v)[N], const float* src) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(src + i));
+    v[i] = t.x; v[i + 1] = t.y; v[i + 2] = t.z; v[i + 3] = t.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void ldg_u32(uint32_t (&v)[N], const __nv_bfloat16* src) {
+  if constexpr (N == 1) {
+    v[0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+  } else if constexpr (N == 2) {
+    const uint2 t = __ldg(reinterpret_cast<const uint2*>(src));
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    const uint4 t = __ldg(reinterpret_cast<const uint4*>(src));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  }
+}
+template <int N>
+__device__ __forceinline__ void stg_f32(float* dst, const float (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+}
+template <int N>
+__device__ __forceinline__ void stg_act(__nv_bfloat16* dst, const float* v, bool f16) {
+  uint32_t w[N / 2];
+#pragma unroll
+  for (int e = 0; e < N / 2; ++e) w[e] = pack_act(v[2 * e], v[2 * e + 1], f16);
+  if constexpr (N == 2) *reinterpret_cast<uint32_t*>(dst) = w[0];
+  else if constexpr (N == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+  else *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // First element of (slot, kv head) in one layer's K or V pages: [page][kv_head][16][Dh].
@@ -63,67 +113,78 @@ __device__ __forceinline__ __nv_bfloat16* cache_row(__nv_bfloat16* base, int slo
   return base + ((size_t(slot >> 4) * n_kv_heads + hk) * 16 + (slot & 15)) * Dh;
 }
 
-constexpr int NT = 4;                  // n8 tiles of a unit: 32 output columns
-constexpr int PART_STRIDE = 40;        // floats between rows of a warp's partial tile (32 + padding)
-
-// Where tile j (0..3), column g (0..7) of unit `unit` lives: the weight row to read.
+// Weight row that feeds column g (0..7) of tile j (0 .. 2 P - 1) of unit `unit`.  The last unit of a width that P does not
+// divide reads the last row again; its columns past the end are not stored.
+template <int P>
 __device__ __forceinline__ const uint8_t* unit_row(const SkinnyParams& p, int unit, int j, int g) {
   const size_t row_bytes = size_t(p.K) * 2;
-  if (p.mode == kGemmResid) return static_cast<const uint8_t*>(p.w[0]) + size_t(unit * 32 + j * 8 + g) * row_bytes;
-  if (p.mode == kGemmGateUp) {
-    const int r = unit * 16 + (j & 1) * 8 + g;                       // tiles 0,1 gate; 2,3 the same rows of up
-    return static_cast<const uint8_t*>(p.w[j >> 1]) + size_t(r) * row_bytes;
-  }
-  const int upr = p.head_dim >> 5;                                   // units per head
+  if (p.mode == kGemmResid) return static_cast<const uint8_t*>(p.w[0]) + size_t(min(unit * 16 * P + j * 8 + g, p.N - 1)) * row_bytes;
+  const int hi = j >= P ? 1 : 0, jj = j - hi * P;                    // tiles 0 .. P - 1 and their partners
+  if (p.mode == kGemmGateUp) return static_cast<const uint8_t*>(p.w[hi]) + size_t(min(unit * 8 * P + jj * 8 + g, p.N - 1)) * row_bytes;
+  const int upr = p.head_dim / (16 * P);                             // units per head
   const int head = unit / upr, sub = unit - head * upr;
-  int col = head * p.head_dim + sub * 16 + (j & 1) * 8 + g + (j >> 1) * (p.head_dim >> 1);
+  int col = head * p.head_dim + sub * 8 * P + jj * 8 + g + hi * (p.head_dim >> 1);
   int which = 0;
   if (col >= p.q_dim) { col -= p.q_dim; which = 1; }
   if (which == 1 && col >= p.kv_dim) { col -= p.kv_dim; which = 2; }
   return static_cast<const uint8_t*>(p.w[which]) + size_t(col) * row_bytes;
 }
+__host__ __device__ __forceinline__ int skinny_units(int N, int mode, int P) {
+  const int w = mode == kGemmGateUp ? 8 * P : 16 * P;
+  return (N + w - 1) / w;
+}
 
-
-// MT: 16-row tiles of activations (T <= 16 MT); DB: depth of a warp's ring of K steps.
-// FOLD: the instantiation that knows the folded RMSNorm (producing side in Resid mode, consuming side in the others);
-// the plain one carries none of its code.
-// r = rsqrt(mean(x^2) + eps) of row `row` from its n partial sums of squares (one per 32 columns): the four threads
-// of a row (threadIdx & 3) add every fourth partial each and then combine, a fixed order whoever calls.  Called by all
-// threads of a warp.
-__device__ __forceinline__ float row_norm_factor(const float* row_ss, int stride, int n, int row, int T, int width, float eps) {
-  const int q = threadIdx.x & 3;
+// Folded RMSNorm: r = rsqrt(mean(x^2) + eps) of row threadIdx / 16 (16 rows at most) from its n partial sums of squares, one
+// per 16 columns: the row's sixteen threads take every sixteenth partial each and then combine, a fixed order whoever
+// calls.  In two halves, so that the K loop runs while the partials travel.  Called by all threads of the block.
+constexpr int kSsPre = 16;             // partials a thread asks for ahead (all of them up to a width of 4096)
+__device__ __forceinline__ void row_norm_request(float (&v)[kSsPre], const float* row_ss, int stride, int n, int T) {
+  const int row = threadIdx.x >> 4, q = threadIdx.x & 15;
+#pragma unroll
+  for (int u = 0; u < kSsPre; ++u) v[u] = row < T && q + 16 * u < n ? __ldcg(row_ss + size_t(row) * stride + q + 16 * u) : 0.f;
+}
+__device__ __forceinline__ float row_norm_factor(const float (&v)[kSsPre], const float* row_ss, int stride, int n, int T, int width, float eps) {
+  const int row = threadIdx.x >> 4, q = threadIdx.x & 15;
   float sum = 0.f;
+#pragma unroll
+  for (int u = 0; u < kSsPre; ++u) sum += v[u];
   if (row < T)
-    for (int i0 = q; i0 < n; i0 += 4 * 8) {        // eight loads in flight at a time, added in order
-      float v[8];
+    for (int i = q + 16 * kSsPre; i < n; i += 16) sum += __ldcg(row_ss + size_t(row) * stride + i);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = i0 + 4 * u < n ? __ldcg(row_ss + size_t(row) * stride + i0 + 4 * u) : 0.f;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) sum += v[u];
-    }
-  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  for (int o = 1; o < 16; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   return rsqrtf(sum / float(width) + eps);
 }
 
-template <int MT, int DB, bool F16, bool FOLD>
+// What a launch takes once the kernel in front is done, in timestamps at the talker's dimensions (K = 1024): 1.1 us until the
+// activations are there, 0.4 in the K loop, 0.45 until the last warp's partial tile is, 0.6 in the epilogue.  So with a K range
+// that fits the rings there is one wait and no refills, the chains of MMAs are halved, an epilogue thread has four columns
+// instead of eight, and the divisions of the unit's geometry and the first look at the arguments stand in front of the wait:
+// talker step of one row 233 -> 223 us, of 16 rows 288 -> 276.
+// MT: 16-row tiles of activations (T <= 16 MT); P: pairs of 8-column tiles per unit; DB: depth of a warp's ring of K steps.
+// FOLD: the instantiation that knows the folded RMSNorm (producing side in Resid mode, consuming side in the others; steps
+// of at most 16 rows); the plain one carries none of its code.
+template <int MT, int P, int DB, bool F16, bool FOLD>
 __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const SkinnyParams p) {
   extern __shared__ __align__(16) uint8_t sk_smem[];
   log_smid(p.smid_log);
   const int block = int(blockIdx.x), n_blocks = int(gridDim.x);
-  constexpr int STAGE_BYTES = (NT + 2 * MT) * 512;          // per warp and K step: 4 weight tiles, 2 MT row groups
+  static_assert(!FOLD || MT == 1, "the folded norm's rows are those of one row tile");
+  constexpr int NT = 2 * P;                                 // n8 tiles of a unit
+  constexpr int PART_STRIDE = 8 * NT + 8;                   // floats between rows of a warp's partial tile
+  constexpr int STAGE_BYTES = (NT + 2 * MT) * 512;          // per warp and K step: the weight tiles, 2 MT row groups
   constexpr int RING_BYTES = DB * STAGE_BYTES;              // per warp
   constexpr int PART_FLOATS = MT * 16 * PART_STRIDE;        // per warp
   // The partial tiles of the reduction get their own shared memory when it fits; else they reuse the rings.
   constexpr bool ALIAS = SK_WARPS * (RING_BYTES + PART_FLOATS * 4) > 227 * 1024;
   static_assert(!ALIAS || PART_FLOATS * 4 <= RING_BYTES, "a warp's partial tile must fit its own ring");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const uint32_t ring = smem_u32(sk_smem) + warp * RING_BYTES + lane * 16;
+  const uint8_t* ring_at = sk_smem + warp * RING_BYTES + lane * 16;
+  const uint32_t ring = smem_u32(ring_at);
   float* part_all = reinterpret_cast<float*>(sk_smem + (ALIAS ? 0 : SK_WARPS * RING_BYTES));
   constexpr int PART_PITCH = ALIAS ? RING_BYTES / 4 : PART_FLOATS;   // floats between two warps' partial tiles
   float* part = part_all + warp * PART_PITCH;
 
-  const int units = p.mode == kGemmGateUp ? p.N >> 4 : p.N >> 5;
+  const int units = skinny_units(p.N, p.mode, P);
   // 32-wide K steps, dealt to the warps in turn: warp w takes steps w, w + 8, ...  The eight warps move through
   // the K range together, so at any moment the block reads 512 contiguous bytes of each weight row -- a run long
   // enough for the DRAM pages it opens.  (Contiguous per-warp K slices would make 8 x 32 separate 64-byte streams.)
@@ -131,11 +192,14 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
   const int n = (steps - warp + SK_WARPS - 1) / SK_WARPS;
   const size_t k_off = (size_t(warp) * 32 + t * 8) * 2;     // byte offset of this lane's first 16 bytes in a row
   constexpr int STEP_BYTES = SK_WARPS * 64;                 // from one of the warp's steps to its next
+  // A K range that fits the rings is copied whole: one wait, no refills.  Otherwise DB - 1 steps are kept in flight.
+  const bool whole = steps <= SK_WARPS * DB;
+  const int n_first = whole ? n : min(n, DB - 1);
 
   const uint8_t* wrow[NT];
   auto set_rows = [&](int unit) {
 #pragma unroll
-    for (int j = 0; j < NT; ++j) wrow[j] = unit_row(p, unit, j, g) + k_off;
+    for (int j = 0; j < NT; ++j) wrow[j] = unit_row<P>(p, unit, j, g) + k_off;
   };
   // Activation rows of this lane: rows 16 i + g and 16 i + g + 8.  Rows past the step are not copied: whatever their
   // ring bytes hold reaches only accumulator rows that no epilogue stores.  (Copying the last row in their place made
@@ -156,225 +220,256 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
       for (int h = 0; h < 2; ++h)
         if (16 * i + 8 * h + g < p.T) cp_async16(ring + slot * STAGE_BYTES + (NT + 2 * i + h) * 512, arow[i][h] + size_t(s) * STEP_BYTES);
   };
-  auto prologue = [&]() {
+  // (groups: one per step, or with a whole range a single one, the others empty)
+  auto first_b = [&]() {
 #pragma unroll
-    for (int s = 0; s < DB - 1; ++s) {
-      if (s < n) {
-        issue_b(s, s);
-        issue_a(s, s);
-      }
-      cp_async_commit();
+    for (int s = 0; s < DB; ++s)
+      if (s < n_first) issue_b(s, s);
+  };
+  auto first_a = [&]() {
+#pragma unroll
+    for (int s = 0; s < DB; ++s) {
+      if (s < n_first) issue_a(s, s);
+      if (s < DB - 1) cp_async_commit();
+    }
+    if (whole) cp_async_commit();
+  };
+  // Unit geometry of the Qkv mode: head, and first rotation pair inside it (the divisions stay in front of the wait)
+  int u_head = 0, u_pair = 0;
+  auto set_unit = [&](int unit) {
+    set_rows(unit);
+    if (p.mode == kGemmQkv) {
+      const int upr = p.head_dim / (16 * P);
+      u_head = unit / upr;
+      u_pair = (unit - u_head * upr) * 8 * P;
     }
   };
 
   int unit = block;
   if (unit < units) {                                       // weights never change: fetch them before the wait
-    set_rows(unit);
-#pragma unroll
-    for (int s = 0; s < DB - 1; ++s)
-      if (s < n) issue_b(s, s);
+    set_unit(unit);
+    first_b();
   }
-  // the epilogue row of this thread and what it needs from the step's metadata (written before the step's first kernel)
-  const int e_row = threadIdx.x >> 2, e_jq = (threadIdx.x & 3) * 4;
+  // This thread's part of the epilogue -- its row, and in Resid mode 2 Q consecutive columns, else Q columns of the first
+  // half and their partners -- and what it needs from the step's metadata (written before the step's first kernel).
+  constexpr int Q = MT == 1 && P <= 4 ? 2 : 4, TPR = 16 * P / (2 * Q);  // threads of a row
+  static_assert(MT * 16 * TPR <= SK_THREADS, "one epilogue task per thread");
+  const int e_row = threadIdx.x / TPR, e_q = threadIdx.x - e_row * TPR;
   const bool e_ok = e_row < MT * 16 && e_row < p.T;
   int e_pos = 0, e_slot = 0;
   if (p.mode == kGemmQkv && e_ok) {
     e_pos = p.tok_pos[e_row];
     e_slot = p.tok_slot[e_row];
   }
+  const int n_q_heads = p.mode == kGemmQkv ? p.q_dim / p.head_dim : 0;
+  // (the arguments the epilogue will read: their first use brings their lines of the constant bank)
+  asm volatile("" ::"l"(p.y), "l"(p.q_out), "l"(p.act), "l"(p.norm_gain), "l"(p.row_ss), "l"(p.in_row_ss), "l"(p.rope), "l"(p.qkv_bias[0]),
+               "l"(p.k_cache), "l"(p.status), "l"(p.gate_mod));
   griddep_wait();
   griddep_launch_dependents(p.overlap);
-  if (unit < units) {
-#pragma unroll
-    for (int s = 0; s < DB - 1; ++s) {
-      if (s < n) issue_a(s, s);
-      cp_async_commit();
-    }
-  }
-  // folded RMSNorm, consuming side: r of this thread's epilogue row, on its way while the first unit streams
+  // folded RMSNorm, consuming side: r of this thread's epilogue row, or the partial sums it is made of, which travel with the
+  // activations of the first unit
   float rs_in = 1.f;
-  if (FOLD && p.in_row_rs != nullptr && int(threadIdx.x >> 2) < p.T) rs_in = __ldcg(p.in_row_rs + (threadIdx.x >> 2));
-  if (FOLD && p.in_row_ss != nullptr) rs_in = row_norm_factor(p.in_row_ss, p.K >> 5, p.K >> 5, int(threadIdx.x >> 2), p.T, p.K, p.norm_eps);
-  int* last_unit = reinterpret_cast<int*>(part_all + SK_WARPS * PART_PITCH);   // FOLD: one word behind the partial tiles
+  const bool sums_in = FOLD && p.in_row_ss != nullptr;
+  float* row_r = part_all + SK_WARPS * PART_PITCH;          // FOLD: r of 16 rows behind the partial tiles, and one word
+  int* last_unit = reinterpret_cast<int*>(row_r + 16);
+  float ss_pre[kSsPre];
+  if (unit < units) first_a();
+  if (sums_in) row_norm_request(ss_pre, p.in_row_ss, p.K >> 4, p.K >> 4, p.T);
+  if (FOLD && p.in_row_rs != nullptr && e_ok) rs_in = __ldcg(p.in_row_rs + e_row);
+  bool first = true;
 
   for (; unit < units; unit += n_blocks) {
     // What the epilogue will read from memory is requested now, so that it has arrived when the K loop ends: the
     // output block to add to, the gains of a folded norm, the rotation of the row's position.
-    float4 y_pre_lo = make_float4(0.f, 0.f, 0.f, 0.f), y_pre_hi = y_pre_lo, cs0 = y_pre_lo, cs1 = y_pre_lo;
-    uint2 ng_lo = make_uint2(0u, 0u), ng_hi = ng_lo;
-    if (e_ok) {
-      if (p.mode == kGemmResid) {
-        if (p.accumulate) {
-          const float4* y_lo = reinterpret_cast<const float4*>(p.y + size_t(e_row) * p.N + unit * 32 + e_jq);
-          y_pre_lo = __ldcg(y_lo);
-          y_pre_hi = __ldcg(y_lo + 4);
-        }
-        if (FOLD && p.norm_gain != nullptr) {
-          ng_lo = __ldg(reinterpret_cast<const uint2*>(p.norm_gain + unit * 32 + e_jq));
-          ng_hi = __ldg(reinterpret_cast<const uint2*>(p.norm_gain + unit * 32 + e_jq + 16));
-        }
-      } else if (p.mode == kGemmQkv) {
-        const int upr = p.head_dim >> 5, head = unit / upr, sub = unit - head * upr;
-        if (head < p.q_dim / p.head_dim + p.n_kv_heads) {
-          const float4* cs = reinterpret_cast<const float4*>(p.rope + size_t(e_pos) * (p.head_dim >> 1) + sub * 16 + e_jq);
-          cs0 = cs[0];
-          cs1 = cs[1];
-        }
+    float y_pre[2 * Q], cs[2 * Q];                            // (cs: cosine and sine of Q pairs)
+    uint32_t ng[Q];                                           // 2 Q gains
+    const int r_col = unit * 16 * P + e_q * 2 * Q;            // Resid: this thread's first column
+    const bool r_ok = e_ok && r_col < p.N;
+    const int head = u_head, i0 = u_pair + e_q * Q;           // Qkv: head and first rotation pair
+    if (p.mode == kGemmResid) {
+      if (r_ok) {
+        if (p.accumulate) ldcg_f32<2 * Q>(y_pre, p.y + size_t(e_row) * p.N + r_col);
+        if (FOLD && p.norm_gain != nullptr) ldg_u32<Q>(ng, p.norm_gain + r_col);
       }
+    } else if (p.mode == kGemmQkv) {
+      if (e_ok && head < n_q_heads + p.n_kv_heads) ldg_f32<2 * Q>(cs, reinterpret_cast<const float*>(p.rope + size_t(e_pos) * (p.head_dim >> 1) + i0));
     }
-    float acc[MT][NT][4];
+    // even and odd K steps of the warp in accumulators of their own (MT = 1: their chains of MMAs are what a short K range
+    // takes), added at the end
+    constexpr int NA = MT == 1 ? 2 : 1;
+    float acc[NA][MT][NT][4];
 #pragma unroll
-    for (int i = 0; i < MT; ++i)
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[a][i][j][e] = 0.f;
+    auto step = [&](float (&d)[MT][NT][4], int slot) {
+      const uint8_t* at = ring_at + slot * STAGE_BYTES;
+      uint4 b[NT];
+#pragma unroll
+      for (int j = 0; j < NT; ++j) b[j] = *reinterpret_cast<const uint4*>(at + j * 512);
+#pragma unroll
+      for (int i = 0; i < MT; ++i) {
+        const uint4 lo = *reinterpret_cast<const uint4*>(at + (NT + 2 * i) * 512), hi = *reinterpret_cast<const uint4*>(at + (NT + 2 * i + 1) * 512);
+        // the two MMAs on one accumulator are kept apart: independent ones run between them
+#pragma unroll
+        for (int j = 0; j < NT; ++j) mma_16816<F16>(d[i][j], lo.x, hi.x, lo.y, hi.y, b[j].x, b[j].y);
+#pragma unroll
+        for (int j = 0; j < NT; ++j) mma_16816<F16>(d[i][j], lo.z, hi.z, lo.w, hi.w, b[j].z, b[j].w);
+      }
+    };
+    if (whole) {
+      cp_async_wait<0>();
+#pragma unroll 2
+      for (int s = 0; s + NA <= n; s += NA) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) step(acc[a], s + a);
+      }
+      if (NA == 2 && (n & 1)) step(acc[0], n - 1);
+    } else {
+      int slot = 0, fill = DB - 1;                          // ring slot of step s / of step s + DB - 1
+      auto turn = [&](float (&d)[MT][NT][4], int s) {
+        if (s + DB - 1 < n) {
+          issue_b(s + DB - 1, fill);
+          issue_a(s + DB - 1, fill);
+        }
+        cp_async_commit();
+        cp_async_wait<DB - 1>();
+        step(d, slot);
+        slot = slot + 1 == DB ? 0 : slot + 1;
+        fill = fill + 1 == DB ? 0 : fill + 1;
+      };
+      for (int s = 0; s < n; s += NA) {
+        turn(acc[0], s);
+        if (NA == 2 && s + 1 < n) turn(acc[NA - 1], s + 1);
+      }
+      cp_async_wait<0>();
+    }
+    if (NA == 2)
 #pragma unroll
       for (int j = 0; j < NT; ++j)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-
-    int slot = 0, fill = DB - 1;                            // ring slot of step s / of step s + DB - 1
-    for (int s = 0; s < n; ++s) {
-      if (s + DB - 1 < n) {
-        issue_b(s + DB - 1, fill);
-        issue_a(s + DB - 1, fill);
-      }
-      cp_async_commit();
-      cp_async_wait<DB - 1>();
-      const uint32_t at = ring + slot * STAGE_BYTES;
-      uint4 b[NT];
-#pragma unroll
-      for (int j = 0; j < NT; ++j) b[j] = lds16(at + j * 512);
-#pragma unroll
-      for (int i = 0; i < MT; ++i) {
-        const uint4 lo = lds16(at + (NT + 2 * i) * 512), hi = lds16(at + (NT + 2 * i + 1) * 512);
-        // the two MMAs on one accumulator are kept apart: four independent ones run between them
-#pragma unroll
-        for (int j = 0; j < NT; ++j) mma_16816<F16>(acc[i][j], lo.x, hi.x, lo.y, hi.y, b[j].x, b[j].y);
-#pragma unroll
-        for (int j = 0; j < NT; ++j) mma_16816<F16>(acc[i][j], lo.z, hi.z, lo.w, hi.w, b[j].z, b[j].w);
-      }
-      slot = slot + 1 == DB ? 0 : slot + 1;
-      fill = fill + 1 == DB ? 0 : fill + 1;
-    }
-    cp_async_wait<0>();
+        for (int e = 0; e < 4; ++e) acc[0][0][j][e] += acc[NA - 1][0][j][e];
 
     // the next unit's first steps travel while this one is reduced and written (when the rings stay free)
     const int next = unit + n_blocks;
     if (!ALIAS && next < units) {
-      set_rows(next);
-      prologue();
+      set_unit(next);
+      first_b();
+      first_a();
     }
 
-    // partial tiles -> shared memory
+    // partial tiles -> shared memory (rows past the step are not read)
 #pragma unroll
     for (int i = 0; i < MT; ++i)
 #pragma unroll
       for (int j = 0; j < NT; ++j) {
         float* at = part + (16 * i + g) * PART_STRIDE + 8 * j + 2 * t;
-        *reinterpret_cast<float2*>(at) = make_float2(acc[i][j][0], acc[i][j][1]);
-        *reinterpret_cast<float2*>(at + 8 * PART_STRIDE) = make_float2(acc[i][j][2], acc[i][j][3]);
+        *reinterpret_cast<float2*>(at) = make_float2(acc[0][i][j][0], acc[0][i][j][1]);
+        if (MT > 1 || p.T > 8) *reinterpret_cast<float2*>(at + 8 * PART_STRIDE) = make_float2(acc[0][i][j][2], acc[0][i][j][3]);
       }
+    if (sums_in && first) {
+      const float r = row_norm_factor(ss_pre, p.in_row_ss, p.K >> 4, p.K >> 4, p.T, p.K, p.norm_eps);
+      if ((threadIdx.x & 15) == 0) row_r[threadIdx.x >> 4] = r;
+    }
     __syncthreads();
 
-    // sum of the 8 warps' partials in warp order, then the epilogue of the mode.  Thread -> row tid / 4 and the
-    // tile columns jq .. jq + 3 ("lo") and 16 + jq .. 16 + jq + 3 ("hi").
-    const int row = threadIdx.x >> 2, jq = (threadIdx.x & 3) * 4;
-    if (row < MT * 16 && row < p.T) {
-      const float* src = part_all + row * PART_STRIDE + jq;
-      float4 lo = *reinterpret_cast<const float4*>(src), hi = *reinterpret_cast<const float4*>(src + 16);
+    // sum of the 8 warps' partials in warp order, then the epilogue of the mode
+    if (sums_in && first && e_ok) rs_in = row_r[e_row];
+    first = false;
+    const int row = e_row;
+    if (p.mode == kGemmResid ? r_ok : e_ok) {
+      const float* src = part_all + row * PART_STRIDE + (p.mode == kGemmResid ? e_q * 2 * Q : e_q * Q);
+      const int to_hi = p.mode == kGemmResid ? Q : 8 * P;
+      float v[2 * Q];                                       // the Q first columns, then the Q others
+      lds_f32<Q>(v, src);
+      lds_f32<Q>(v + Q, src + to_hi);
 #pragma unroll
       for (int w = 1; w < SK_WARPS; ++w) {
-        const float4 l = *reinterpret_cast<const float4*>(src + w * PART_PITCH);
-        const float4 h = *reinterpret_cast<const float4*>(src + w * PART_PITCH + 16);
-        lo.x += l.x; lo.y += l.y; lo.z += l.z; lo.w += l.w;
-        hi.x += h.x; hi.y += h.y; hi.z += h.z; hi.w += h.w;
+        float u[2 * Q];
+        lds_f32<Q>(u, src + w * PART_PITCH);
+        lds_f32<Q>(u + Q, src + w * PART_PITCH + to_hi);
+#pragma unroll
+        for (int e = 0; e < 2 * Q; ++e) v[e] += u[e];
       }
-      if (FOLD && (p.in_row_rs != nullptr || p.in_row_ss != nullptr)) {
-        lo.x *= rs_in; lo.y *= rs_in; lo.z *= rs_in; lo.w *= rs_in;
-        hi.x *= rs_in; hi.y *= rs_in; hi.z *= rs_in; hi.w *= rs_in;
+      if (FOLD && (p.in_row_rs != nullptr || sums_in)) {
+#pragma unroll
+        for (int e = 0; e < 2 * Q; ++e) v[e] *= rs_in;
       }
       if (p.mode == kGemmResid) {
-        float4* y_lo = reinterpret_cast<float4*>(p.y + size_t(row) * p.N + unit * 32 + jq);
-        float4* y_hi = y_lo + 4;
         if (p.gate_mod) {                                    // conditioned block: gate vector of the row's sequence
-          const float4* gate = reinterpret_cast<const float4*>(p.gate_mod + (size_t(p.tok_seq[row]) * 6 + p.gate_which) * p.N +
-                                                               unit * 32 + jq);
-          const float4 g_lo = __ldg(gate), g_hi = __ldg(gate + 4);
-          lo.x *= g_lo.x; lo.y *= g_lo.y; lo.z *= g_lo.z; lo.w *= g_lo.w;
-          hi.x *= g_hi.x; hi.y *= g_hi.y; hi.z *= g_hi.z; hi.w *= g_hi.w;
+          float gt[2 * Q];
+          ldg_f32<2 * Q>(gt, p.gate_mod + (size_t(p.tok_seq[row]) * 6 + p.gate_which) * p.N + r_col);
+#pragma unroll
+          for (int e = 0; e < 2 * Q; ++e) v[e] *= gt[e];
         }
         if (p.accumulate) {
-          const float4 a = y_pre_lo, b = y_pre_hi;
-          lo.x += a.x; lo.y += a.y; lo.z += a.z; lo.w += a.w;
-          hi.x += b.x; hi.y += b.y; hi.z += b.z; hi.w += b.w;
+#pragma unroll
+          for (int e = 0; e < 2 * Q; ++e) v[e] += y_pre[e];
         }
-        *y_lo = lo;
-        *y_hi = hi;
+        stg_f32<2 * Q>(p.y + size_t(row) * p.N + r_col, v);
         if (FOLD && p.norm_gain != nullptr) {
-          // folded RMSNorm, producing side: the next GEMM's operand and this unit's share of the row's sum of squares
-          // (the four threads of a row are neighbours in a warp)
-          const uint2 g_lo = ng_lo, g_hi = ng_hi;
-          float v[8] = {lo.x * __uint_as_float(g_lo.x << 16), lo.y * __uint_as_float(g_lo.x & 0xffff0000u),
-                        lo.z * __uint_as_float(g_lo.y << 16), lo.w * __uint_as_float(g_lo.y & 0xffff0000u),
-                        hi.x * __uint_as_float(g_hi.x << 16), hi.y * __uint_as_float(g_hi.x & 0xffff0000u),
-                        hi.z * __uint_as_float(g_hi.y << 16), hi.w * __uint_as_float(g_hi.y & 0xffff0000u)};
-          if (p.norm_h_f16 && p.status) note_f16_saturation(v, p.status);
-          __nv_bfloat16* hrow = p.norm_h + size_t(row) * p.N + unit * 32 + jq;
-          *reinterpret_cast<uint2*>(hrow) = make_uint2(pack_act(v[0], v[1], p.norm_h_f16 != 0), pack_act(v[2], v[3], p.norm_h_f16 != 0));
-          *reinterpret_cast<uint2*>(hrow + 16) = make_uint2(pack_act(v[4], v[5], p.norm_h_f16 != 0), pack_act(v[6], v[7], p.norm_h_f16 != 0));
-          float ss = lo.x * lo.x + lo.y * lo.y + lo.z * lo.z + lo.w * lo.w + hi.x * hi.x + hi.y * hi.y + hi.z * hi.z + hi.w * hi.w;
-          ss += __shfl_xor_sync(0xfu << (lane & 28), ss, 1);
-          ss += __shfl_xor_sync(0xfu << (lane & 28), ss, 2);
-          if ((threadIdx.x & 3) == 0) p.row_ss[size_t(row) * p.ss_stride + unit] = ss;
+          // folded RMSNorm, producing side: the next GEMM's operand and the share of the row's sum of squares of these 16
+          // columns (neighbouring threads)
+          float h[2 * Q];
+#pragma unroll
+          for (int e = 0; e < Q; ++e) {
+            h[2 * e] = v[2 * e] * __uint_as_float(ng[e] << 16);
+            h[2 * e + 1] = v[2 * e + 1] * __uint_as_float(ng[e] & 0xffff0000u);
+          }
+          if (p.norm_h_f16 && p.status) note_f16_saturation(h, p.status);
+          stg_act<2 * Q>(p.norm_h + size_t(row) * p.N + r_col, h, p.norm_h_f16 != 0);
+          float ss = 0.f;
+#pragma unroll
+          for (int e = 0; e < 2 * Q; ++e) ss += v[e] * v[e];
+          constexpr int L = 8 / Q;                           // threads of 16 columns
+          const uint32_t mask = ((1u << L) - 1) << (lane & ~(L - 1));
+#pragma unroll
+          for (int o = 1; o < L; o <<= 1) ss += __shfl_xor_sync(mask, ss, o);
+          if ((e_q & (L - 1)) == 0) p.row_ss[size_t(row) * p.ss_stride + (r_col >> 4)] = ss;
         }
       } else if (p.mode == kGemmGateUp) {
-        const float gt[4] = {lo.x, lo.y, lo.z, lo.w}, up[4] = {hi.x, hi.y, hi.z, hi.w};
-        float v[4];
+        const int col = unit * 8 * P + e_q * Q;
+        float o[Q];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = __fdividef(gt[e] * up[e], 1.f + __expf(-gt[e]));   // silu(gate) * up
-        if (p.act_f16 && p.status) note_f16_saturation(v, p.status);
-        uint2 out;
-        out.x = pack_act(v[0], v[1], p.act_f16 != 0);
-        out.y = pack_act(v[2], v[3], p.act_f16 != 0);
-        *reinterpret_cast<uint2*>(p.act + size_t(row) * p.N + unit * 16 + jq) = out;
+        for (int e = 0; e < Q; ++e) o[e] = __fdividef(v[e] * v[Q + e], 1.f + __expf(-v[e]));   // silu(gate) * up
+        if (col < p.N) {
+          if (p.act_f16 && p.status) note_f16_saturation(o, p.status);
+          stg_act<Q>(p.act + size_t(row) * p.N + col, o, p.act_f16 != 0);
+        }
       } else {
-        const int Dh = p.head_dim, half = Dh >> 1, upr = Dh >> 5;
-        const int head = unit / upr, sub = unit - head * upr;
-        const int i0 = sub * 16 + jq;                        // first rotation pair / first element inside the head
-        const int n_q_heads = p.q_dim / Dh;
-        float a[4] = {lo.x, lo.y, lo.z, lo.w}, b[4] = {hi.x, hi.y, hi.z, hi.w};
+        const int Dh = p.head_dim, half = Dh >> 1;
         const int region = head < n_q_heads ? 0 : head < n_q_heads + p.n_kv_heads ? 1 : 2;
         if (p.qkv_bias[region]) {                            // the bias comes before the rotation
-          const int col = (head - (region == 0 ? 0 : region == 1 ? n_q_heads : n_q_heads + p.n_kv_heads)) * Dh + i0;
-          const uint2 wl = __ldg(reinterpret_cast<const uint2*>(p.qkv_bias[region] + col));
-          const uint2 wh = __ldg(reinterpret_cast<const uint2*>(p.qkv_bias[region] + col + half));
-          a[0] += __uint_as_float(wl.x << 16); a[1] += __uint_as_float(wl.x & 0xffff0000u);
-          a[2] += __uint_as_float(wl.y << 16); a[3] += __uint_as_float(wl.y & 0xffff0000u);
-          b[0] += __uint_as_float(wh.x << 16); b[1] += __uint_as_float(wh.x & 0xffff0000u);
-          b[2] += __uint_as_float(wh.y << 16); b[3] += __uint_as_float(wh.y & 0xffff0000u);
-        }
-        if (head < n_q_heads + p.n_kv_heads) {               // q and k heads are rotated
-          const float4 t0 = cs0, t1 = cs1;                   // (cos, sin) of pairs i0 .. i0 + 3, requested at the unit's start
-          const float c[4] = {t0.x, t0.z, t1.x, t1.z}, sn[4] = {t0.y, t0.w, t1.y, t1.w};
+          const __nv_bfloat16* bias = p.qkv_bias[region] + (head - (region == 0 ? 0 : region == 1 ? n_q_heads : n_q_heads + p.n_kv_heads)) * Dh + i0;
+          uint32_t wl[Q / 2], wh[Q / 2];
+          ldg_u32<Q / 2>(wl, bias);
+          ldg_u32<Q / 2>(wh, bias + half);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float x0 = a[e], x1 = b[e];
-            a[e] = x0 * c[e] - x1 * sn[e];
-            b[e] = x1 * c[e] + x0 * sn[e];
+          for (int e = 0; e < Q / 2; ++e) {
+            v[2 * e] += __uint_as_float(wl[e] << 16);
+            v[2 * e + 1] += __uint_as_float(wl[e] & 0xffff0000u);
+            v[Q + 2 * e] += __uint_as_float(wh[e] << 16);
+            v[Q + 2 * e + 1] += __uint_as_float(wh[e] & 0xffff0000u);
           }
         }
-        uint2 o_lo, o_hi;
-        o_lo.x = pack_act(a[0], a[1], false); o_lo.y = pack_act(a[2], a[3], false);
-        o_hi.x = pack_act(b[0], b[1], false); o_hi.y = pack_act(b[2], b[3], false);
-        __nv_bfloat16* dst;
-        if (head < n_q_heads) {
-          dst = p.q_out + size_t(row) * p.q_dim + head * Dh + i0;
-        } else {
-          const int hk = head - n_q_heads;
-          const int slot = e_slot;
-          dst = hk < p.n_kv_heads ? cache_row(p.k_cache, slot, hk, p.n_kv_heads, Dh) + i0
-                                  : cache_row(p.v_cache, slot, hk - p.n_kv_heads, p.n_kv_heads, Dh) + i0;
+        if (region != 2) {                                   // q and k heads are rotated
+#pragma unroll
+          for (int e = 0; e < Q; ++e) {
+            const float x0 = v[e], x1 = v[Q + e], c = cs[2 * e], sn = cs[2 * e + 1];
+            v[e] = x0 * c - x1 * sn;
+            v[Q + e] = x1 * c + x0 * sn;
+          }
         }
-        *reinterpret_cast<uint2*>(dst) = o_lo;
-        *reinterpret_cast<uint2*>(dst + half) = o_hi;
+        __nv_bfloat16* dst = region == 0 ? p.q_out + size_t(row) * p.q_dim + head * Dh + i0
+                                         : cache_row(region == 1 ? p.k_cache : p.v_cache, e_slot,
+                                                     head - n_q_heads - (region == 1 ? 0 : p.n_kv_heads), p.n_kv_heads, Dh) + i0;
+        stg_act<Q>(dst, v, false);
+        stg_act<Q>(dst + half, v + Q, false);
       }
     }
     __syncthreads();                                         // the partial tiles are free again
@@ -388,46 +483,75 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
       __syncthreads();
       if (*last_unit) {
         __threadfence();
-        const float r = row_norm_factor(p.row_ss, p.ss_stride, units, row, p.T, p.N, p.norm_eps);
-        if ((threadIdx.x & 3) == 0 && row < p.T) p.row_rs[row] = r;
+        float v[kSsPre];
+        row_norm_request(v, p.row_ss, p.ss_stride, p.N >> 4, p.T);
+        const float r = row_norm_factor(v, p.row_ss, p.ss_stride, p.N >> 4, p.T, p.N, p.norm_eps);
+        if ((threadIdx.x & 15) == 0 && int(threadIdx.x >> 4) < p.T) p.row_rs[threadIdx.x >> 4] = r;
         if (threadIdx.x == 0) *p.units_done = 0;             // ready for the next launch
       }
     }
     if (ALIAS && next < units) {
-      set_rows(next);
-      prologue();
+      set_unit(next);
+      first_b();
+      first_a();
     }
   }
 }
 
-template <int MT, int DB>
+template <int MT, int P, int DB>
 constexpr int skinny_smem() {
-  constexpr int rings = SK_WARPS * DB * (NT + 2 * MT) * 512, both = rings + SK_WARPS * MT * 16 * PART_STRIDE * 4;
-  return (both > 227 * 1024 ? rings : both) + 16;            // + the word of the folded norm's last-unit flag
+  constexpr int rings = SK_WARPS * DB * 2 * (P + MT) * 512, both = rings + SK_WARPS * MT * 16 * (16 * P + 8) * 4;
+  constexpr int bytes = (both > 227 * 1024 - 128 ? rings : both) + 16 * 4 + 16;      // + r of the folded norm's rows, its last-unit flag
+  return bytes < kMinSmemBytes ? kMinSmemBytes : bytes;
 }
-constexpr int DB1 = 8, DB2 = 6, DB4 = 4;                     // ring depths by row-tile count
-static_assert(skinny_smem<1, DB1>() <= 227 * 1024 && skinny_smem<2, DB2>() <= 227 * 1024 && skinny_smem<4, DB4>() <= 227 * 1024,
-              "rings and partial tiles must fit one SM");
+// Ring depth: what fits one SM, at least 96 KB of weights in flight.
+constexpr int ring_depth(int MT, int P) {
+  return MT == 1 ? (P == 1 ? 12 : P == 2 ? 8 : P == 3 ? 6 : P <= 6 ? 4 : 3) : MT == 2 ? (P == 1 ? 8 : P == 2 ? 6 : P == 3 ? 4 : 3) : 4;
+}
 
-template <int MT, int DB>
+template <int MT, int P>
 cudaError_t launch_one(const SkinnyParams& p, int grid, cudaStream_t stream) {
-  constexpr int smem = skinny_smem<MT, DB>() < kMinSmemBytes ? kMinSmemBytes : skinny_smem<MT, DB>();
-  const bool fold = p.norm_gain != nullptr || p.in_row_rs != nullptr || p.in_row_ss != nullptr;
-  if (p.ab_f16) {
-    if (fold) return launch_step_kernel(gemm_skinny_kernel<MT, DB, true, true>, grid, SK_THREADS, smem, stream, p.overlap != 0, p);
-    return launch_step_kernel(gemm_skinny_kernel<MT, DB, true, false>, grid, SK_THREADS, smem, stream, p.overlap != 0, p);
+  constexpr int DB = ring_depth(MT, P), smem = skinny_smem<MT, P, DB>();
+  const bool early = p.overlap != 0;
+  if constexpr (MT == 1) {
+    if (p.norm_gain != nullptr || p.in_row_rs != nullptr || p.in_row_ss != nullptr) {
+      if (p.ab_f16) return launch_step_kernel(gemm_skinny_kernel<MT, P, DB, true, true>, grid, SK_THREADS, smem, stream, early, p);
+      return launch_step_kernel(gemm_skinny_kernel<MT, P, DB, false, true>, grid, SK_THREADS, smem, stream, early, p);
+    }
   }
-  if (fold) return launch_step_kernel(gemm_skinny_kernel<MT, DB, false, true>, grid, SK_THREADS, smem, stream, p.overlap != 0, p);
-  return launch_step_kernel(gemm_skinny_kernel<MT, DB, false, false>, grid, SK_THREADS, smem, stream, p.overlap != 0, p);
+  if (p.ab_f16) return launch_step_kernel(gemm_skinny_kernel<MT, P, DB, true, false>, grid, SK_THREADS, smem, stream, early, p);
+  return launch_step_kernel(gemm_skinny_kernel<MT, P, DB, false, false>, grid, SK_THREADS, smem, stream, early, p);
 }
-template <int MT, int DB>
+template <int MT, int P>
 cudaError_t set_one() {
-  constexpr int smem = skinny_smem<MT, DB>() < kMinSmemBytes ? kMinSmemBytes : skinny_smem<MT, DB>();
-  cudaError_t e = set_kernel_smem(gemm_skinny_kernel<MT, DB, true, false>, smem);
-  if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, DB, false, false>, smem);
-  if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, DB, true, true>, smem);
-  if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, DB, false, true>, smem);
+  constexpr int DB = ring_depth(MT, P), smem = skinny_smem<MT, P, DB>();
+  static_assert(smem <= 227 * 1024, "rings and partial tiles must fit one SM");
+  cudaError_t e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, true, false>, smem);
+  if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, false, false>, smem);
+  if constexpr (MT == 1) {
+    if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, true, true>, smem);
+    if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, false, true>, smem);
+  }
   return e;
+}
+
+// Width of a launch's units.  A block takes in about 70 KB/us, weights and activations alike, with about 1.5 us per unit
+// beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
+// budget.  Units wider than 64 weight rows, for a gate/up projection on few SMs, keep eight columns per epilogue thread and
+// their partial tiles in the rings.  Measured on B200 against 32 rows throughout: talker step of 16 rows at 112 / 96 / 28 SMs
+// 352 -> 333, 351 -> 333, 683 -> 632 us, of 11 rows at 52 (51 units of 112 rows instead of 176 of 32) 395 -> 382; at 7B
+// dimensions 9 rows, 4 layers, at 96 / 74 / 37 SMs 606 -> 546, 594 -> 562, 963 -> 897.
+int pick_width(int T, int K, int N, int mode, int head_dim, int sms) {
+  const int max_p = T <= 16 && mode == kGemmGateUp ? 7 : T <= 32 ? 4 : 2;
+  int best = 2;
+  double best_us = 1e30;
+  for (int P = 1; P <= max_p; ++P) {
+    if (mode == kGemmQkv && (head_dim >> 4) % P != 0) continue;
+    const int units = skinny_units(N, mode, P), rounds = (units + sms - 1) / sms;
+    const double us = rounds * (1.5 + double(16 * P + (T <= 32 ? T : 64)) * K * 2 / 70e3);
+    if (us < best_us - 1e-9) { best_us = us; best = P; }
+  }
+  return best;
 }
 
 }  // namespace
@@ -472,19 +596,37 @@ bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count)
 }
 
 cudaError_t gemm_skinny_set_attributes() {
-  cudaError_t e = set_one<1, DB1>();
-  if (e == cudaSuccess) e = set_one<2, DB2>();
-  if (e == cudaSuccess) e = set_one<4, DB4>();
+  cudaError_t e = cudaSuccess;
+  for (const auto set : {set_one<1, 1>, set_one<1, 2>, set_one<1, 3>, set_one<1, 4>, set_one<1, 5>, set_one<1, 6>, set_one<1, 7>, set_one<2, 1>, set_one<2, 2>, set_one<2, 3>,
+                         set_one<2, 4>, set_one<4, 1>, set_one<4, 2>})
+    if (e == cudaSuccess) e = set();
   return e;
 }
 
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream) {
   if (p.T <= 0) return cudaSuccess;
-  const int units = p.mode == kGemmGateUp ? p.N / 16 : p.N / 32;
+  const int P = pick_width(p.T, p.K, p.N, p.mode, p.head_dim, sm_budget), units = skinny_units(p.N, p.mode, P);
   const int grid = units < sm_budget ? units : sm_budget;
-  if (p.T <= 16) return launch_one<1, DB1>(p, grid, stream);
-  if (p.T <= 32) return launch_one<2, DB2>(p, grid, stream);
-  return launch_one<4, DB4>(p, grid, stream);
+  if (p.T <= 16) {
+    switch (P) {
+      case 1: return launch_one<1, 1>(p, grid, stream);
+      case 2: return launch_one<1, 2>(p, grid, stream);
+      case 3: return launch_one<1, 3>(p, grid, stream);
+      case 4: return launch_one<1, 4>(p, grid, stream);
+      case 5: return launch_one<1, 5>(p, grid, stream);
+      case 6: return launch_one<1, 6>(p, grid, stream);
+      default: return launch_one<1, 7>(p, grid, stream);
+    }
+  }
+  if (p.T <= 32) {
+    switch (P) {
+      case 1: return launch_one<2, 1>(p, grid, stream);
+      case 2: return launch_one<2, 2>(p, grid, stream);
+      case 3: return launch_one<2, 3>(p, grid, stream);
+      default: return launch_one<2, 4>(p, grid, stream);
+    }
+  }
+  return P == 1 ? launch_one<4, 1>(p, grid, stream) : launch_one<4, 2>(p, grid, stream);
 }
 
 }  // namespace hs
