@@ -142,8 +142,9 @@ hs_status_t hs_op_decode_attention_noalloc_status(int32_t *status_out);
  *   decode_items   [decode_cap][8] int32, in the order the kernel's queue hands them out:
  *                  {decode row, KV head, first key, end key (exclusive), sequence, token row, the group's first
  *                  partial slot, items of the group | index within the group << 16}; in group mode (*decode_group = 1:
- *                  a small batch, every (sequence, KV head) group worked by one block) eight page slices per group,
- *                  group-major, some possibly empty (first key = end key), the last two words unused.
+ *                  a small batch) the items come in eights, group-major, some possibly empty (first key = end key): eight
+ *                  warps of one block share a slice of a (sequence, KV head) group's pages, and the last two words count
+ *                  slices {the group's first partial slot, slices of the group | index of the slice << 16}.
  *   prefill_items  [prefill_cap][8] int32, as for a budget of all SMs, longest first: {sequence, KV head, first new token, tokens (at most two Q
  *                  tiles), cached tokens, token row of the sequence's first new token, new tokens of the sequence, 0}.
  * Any pointer may be NULL; counts are always written when their pointer is given; at most cap records are copied.

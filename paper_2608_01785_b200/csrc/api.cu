@@ -546,7 +546,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   s->ring_pos = (slot + 1) % kRing;
 
   int32_t* meta = reinterpret_cast<int32_t*>(s->ws_dev + s->ws.meta);
-  if (cudaMemcpyAsync(meta, s->pinned[slot], size_t(s->ml.total) * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(meta, s->pinned[slot], size_t(plan.meta_words) * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
       cudaEventRecord(s->ev[slot], stream) != cudaSuccess)
     return HS_ERR_CUDA;
   s->ev_pending[slot] = true;

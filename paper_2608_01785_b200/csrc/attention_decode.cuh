@@ -167,12 +167,13 @@ constexpr int dc_smem_bytes() {
 }
 
 // The body of the decode kernel.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS *
-// DC_STAGES mbarriers followed by one int (the abort flag) in shared memory outside that area.
+// DC_STAGES mbarriers followed by two ints (the abort flag; a flag of the block's) in shared memory outside that area.
 template <int DH>
 __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* smem, uint64_t* full_all) {
   using G_ = Geom<DH>;
   constexpr int SLOT_BYTES = 2 * G_::PAGE_BYTES;    // K page then V page
   volatile int* abort_flag = reinterpret_cast<volatile int*>(full_all + DC_WARPS * DC_STAGES);
+  volatile int* block_flag = abort_flag + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int block = int(blockIdx.x), n_blocks = int(gridDim.x);
@@ -225,10 +226,11 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
   griddep_wait();
   griddep_launch_dependents(p.overlap);
 
-  // Group mode (p.decode_group, a batch whose items would not fill the device's warps): item 8 g + w is the w-th
-  // eighth of the pages of group g = (sequence, KV head); a block takes whole groups -- g = block, block + n_blocks,
-  // ... -- its eight warps one slice each, and their partial results meet in the block's shared memory instead of in
-  // global memory behind a counter.  Every warp of the block goes through the same barriers whatever happens to it.
+  // Group mode (p.decode_group, a batch small enough that one round of blocks reads all of it): a group = (sequence, KV
+  // head) is cut into slices of whole pages, item 8 i + w is the w-th eighth of slice i; a block takes whole slices -- i =
+  // block, block + n_blocks, ... -- and its eight warps' partial results meet in the block's shared memory.  A group of
+  // several slices leaves one partial result per slice in global memory, and the block that delivers the last one merges
+  // them in slice order.  Every warp of the block goes through the same barriers whatever happens to it.
   const bool group_mode = p.decode_group != 0;
   bool first_round = true;
   for (int round = 0;; ++round) {
@@ -395,8 +397,16 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
       }
       const bool failed = __syncthreads_or(!ok) != 0;      // the same answer in every warp of the block
       if (!failed) {
-        // the eight partials are merged in slice order by the whole block: a thread per pair of output columns
+        // the eight partials are merged in order by the whole block: a thread per pair of output columns
         const bool f16 = p.o_f16 != 0;
+        auto store = [&](int g, int col, float o0, float o1, float ll) {
+          const float inv = 1.f / ll;
+          if (f16) {
+            const float v2[2] = {o0, o1};
+            note_f16_saturation(v2, p.status, inv);
+          }
+          *reinterpret_cast<uint32_t*>(orow + g * DH + col) = pack_act(o0 * inv, o1 * inv, f16);
+        };
         for (int e = threadIdx.x; e < G * (DH / 2); e += DC_THREADS) {
           const int g = e / (DH / 2), col = 2 * (e - g * (DH / 2));
           float mm = -INFINITY;
@@ -414,12 +424,54 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
             o0 += f * v.x;
             o1 += f * v.y;
           }
-          const float inv = 1.f / ll;
-          if (f16) {
-            const float v2[2] = {o0, o1};
-            note_f16_saturation(v2, p.status, inv);
+          if (splits == 1) {
+            store(g, col, o0, o1, ll);
+          } else {
+            __stcg(reinterpret_cast<float2*>(p.part_o + (size_t(part) * 16 + g) * DH + col), make_float2(o0, o1));
+            if (col == 0) __stcg(reinterpret_cast<float2*>(p.part_ml) + size_t(part) * 16 + g, make_float2(mm, ll));
           }
-          *reinterpret_cast<uint32_t*>(orow + g * DH + col) = pack_act(o0 * inv, o1 * inv, f16);
+        }
+        if (splits > 1) {
+          // the block that delivers the group's last slice merges all of them, in slice order whoever it is
+          __threadfence();
+          __syncthreads();
+          int* done = p.group_done + drow * p.n_kv_heads + hk;
+          if (threadIdx.x == 0) *block_flag = atomicAdd(done, 1) == splits - 1;
+          __syncthreads();
+          if (*block_flag) {
+            __threadfence();
+            for (int e = threadIdx.x; e < G * (DH / 2); e += DC_THREADS) {
+              const int g = e / (DH / 2), col = 2 * (e - g * (DH / 2));
+              const float2* ml_g = reinterpret_cast<const float2*>(p.part_ml) + size_t(dr.z) * 16 + g;
+              const float* po_g = p.part_o + (size_t(dr.z) * 16 + g) * DH + col;
+              float mm = -INFINITY, ll = 0.f, o0 = 0.f, o1 = 0.f;
+              for (int j0 = 0; j0 < splits; j0 += 8) {       // eight slices on their way at a time
+                float2 ml[8], ov[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int j = min(j0 + u, splits - 1);
+                  ml[u] = __ldcg(ml_g + size_t(j) * 16);
+                  ov[u] = __ldcg(reinterpret_cast<const float2*>(po_g + size_t(j) * 16 * DH));
+                }
+                float pm = mm;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) pm = fmaxf(pm, ml[u].x);
+                const float sc = exp2f(mm - pm);             // 0 the first time (mm = -inf)
+                mm = pm;
+                ll *= sc; o0 *= sc; o1 *= sc;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                  if (j0 + u < splits) {
+                    const float f = exp2f(ml[u].x - mm);
+                    ll += f * ml[u].y;
+                    o0 += f * ov[u].x;
+                    o1 += f * ov[u].y;
+                  }
+              }
+              store(g, col, o0, o1, ll);
+            }
+            if (threadIdx.x == 0) *done = 0;                 // ready for the next launch
+          }
         }
       }
       // the rings go back to the copy engine: order these generic-proxy accesses before its next writes

@@ -15,6 +15,7 @@ constexpr int kDecodeWarps = 8;            // warps per block of the decode atte
 constexpr int kDecodeSplitMax = 512;     // largest number of keys per item the planner may choose
 constexpr int kDecodeTail = 128;         // keys per piece of a sequence's last, incomplete run (the items that end the kernel)
 static_assert(kDecodeSplit % 16 == 0 && kDecodeSplitMax / 16 <= 32, "the decode kernel keeps one page id per lane");
+constexpr int kMaxDecodeSlices = 160;     // slices (blocks) the decode attention's group mode may use
 constexpr int kPrefillRows = 128;        // (token, query head of one KV head) rows per prefill work item
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
@@ -51,14 +52,14 @@ struct MetaLayout {
   int tok_pos, tok_slot, tok_seq;    // [max_tokens]      absolute position / cache slot / sequence index of each new token
   int seq_tok0, seq_ctx, seq_qlen;   // [max_seqs]        first token row, cached tokens, new tokens
   int block_tables;                  // [max_seqs * max_pages_per_seq]
+  int decode_rows;                   // [max_seqs * 4]           {seq, token row, first item, splits}
+  int counters;                      // [n_layers * 2]           work-queue heads, zero at step start
+  int group_done;                    // [max_seqs * n_kv_heads]  finished decode splits per group, zero
   int prefill_items;                 // [max_prefill_items * 8]  {seq, kv_head, first token, tokens (at most two tiles),
                                      //                           cached tokens, first token row and new tokens of the sequence, 0}
   int decode_items;                  // [max_decode_items * 8]   {decode row, kv_head, first key, end key,
                                      //                           seq, token row, first partial slot of the group,
                                      //                           splits | index within the group << 16}
-  int decode_rows;                   // [max_seqs * 4]           {seq, token row, first item, splits}
-  int counters;                      // [n_layers * 2]           work-queue heads, zero at step start
-  int group_done;                    // [max_seqs * n_kv_heads]  finished decode splits per group, zero
   int total;                         // int32 words in the block
   int max_prefill_items, max_decode_items;
 };
@@ -67,8 +68,9 @@ MetaLayout make_meta_layout(const hs_stage_config_t& c);
 struct StepPlan {
   int n_tokens = 0, n_seqs = 0;
   int n_prefill_items = 0, n_decode_items = 0, n_decode_rows = 0;
-  int decode_group = 0;           // 1: decode items are eight page slices per (sequence, KV head), group-major (see plan_step)
+  int decode_group = 0;           // 1: decode items come in eights, a block's eight warps sharing a slice of a (sequence, KV head)'s pages (see plan_step)
   int decode_sms = 0;             // SMs of the budget for the decode kernel beside the prefill kernel; 0: one after the other
+  int meta_words = 0;             // int32 words of the metadata block in use: the work lists are at its end
   int64_t decode_kv_bytes = 0;    // K and V bytes the decode items read, one layer
 };
 

@@ -63,9 +63,11 @@ MetaLayout make_meta_layout(const hs_stage_config_t& c) {
   const int G = c.n_q_heads / c.n_kv_heads;
   m.max_prefill_items = c.n_kv_heads * (c.max_tokens / prefill_tokens_per_item(G) + c.max_seqs);
   // a decode sequence of n keys has at most n / kDecodeSplit whole runs and kDecodeSplitMax / kDecodeTail pieces of a
-  // last, incomplete one; cached keys are bounded by the pool
-  m.max_decode_items = c.n_kv_heads * (c.max_seqs * 2 * (kDecodeSplitMax / kDecodeTail) +
-                                       int((int64_t(c.num_pages) * kPage) / kDecodeSplit) + 1);
+  // last, incomplete one; cached keys are bounded by the pool.  (At least eight items for each SM of the device, so that a
+  // small batch may be cut finely.)
+  m.max_decode_items = std::max(kMaxDecodeSlices * kDecodeWarps,
+                                c.n_kv_heads * (c.max_seqs * 2 * (kDecodeSplitMax / kDecodeTail) +
+                                                int((int64_t(c.num_pages) * kPage) / kDecodeSplit) + 1));
   int off = 0;
   auto take = [&](int n) {
     int o = off;
@@ -79,11 +81,11 @@ MetaLayout make_meta_layout(const hs_stage_config_t& c) {
   m.seq_ctx = take(c.max_seqs);
   m.seq_qlen = take(c.max_seqs);
   m.block_tables = take(c.max_seqs * c.max_pages_per_seq);
-  m.prefill_items = take(m.max_prefill_items * 8);
-  m.decode_items = take(m.max_decode_items * 8);
   m.decode_rows = take(c.max_seqs * 4);
   m.counters = take(c.n_layers * 2);
   m.group_done = take(c.max_seqs * c.n_kv_heads);
+  m.prefill_items = take(m.max_prefill_items * 8);    // (last: only what a step has of them travels)
+  m.decode_items = take(m.max_decode_items * 8);
   m.total = off;
   return m;
 }
@@ -169,6 +171,39 @@ AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_
   }
   return r;
 }
+// Pages per slice of the decode attention's group mode, 0 = items of single warps instead.  One slice per group where every
+// group has a block of its own and 128-key items would leave warps idle; in a decode-only step more, all with a block of
+// their own on the device, where that is expected to be faster.  Modelled time of a launch: rounds of one slice per SM, each
+// 3.5 us and a step per page of a warp -- 0.45 us, or what eight pages take at an SM's intake and share of the HBM -- and
+// 2.5 us where a group's slices are merged; on the whole device and, with a weight of 0.15 each, on 13/16, 3/4, 13/20,
+// 1/2 and 7/20 of it, since the results depend on the cut and it must not depend on the budget; a cut has to gain a tenth.  Measured on B200: nine sequences of
+// 761 .. 3888 keys at 7B dimensions 23.8 -> 15.7 us per launch (with 256-key items for single warps, whose partial results
+// one warp merges, before); eleven of 216 .. 1463 keys of the talker, cut for the whole device, 9.1 -> 17 us on 52 SMs,
+// which is why the other budgets count.  Never for sequences longer than eight warps' 32 pages.
+int pick_decode_slice(const hs_stage_config_t& c, const hs_batch_t& b, int sm_count, int split) {
+  const int sms = std::min(sm_count > 0 ? sm_count : 148, kMaxDecodeSlices);
+  int longest = 0, rows = 0;
+  for (int s = 0; s < b.n_seqs; ++s)
+    if (b.q_len[s] == 1) { ++rows; longest = std::max(longest, ceil_div(b.ctx_len[s] + 1, kPage)); }
+  if (split != kDecodeTail || rows == 0 || rows * c.n_kv_heads > sms || longest > kDecodeWarps * 32) return 0;
+  int best = longest;
+  double best_us = 1e30;
+  for (int cuts = 1; cuts <= (rows < b.n_seqs ? 1 : 8); ++cuts) {
+    const int pages = ceil_div(longest, cuts);
+    int n = 0;
+    for (int s = 0; s < b.n_seqs; ++s)
+      if (b.q_len[s] == 1) n += c.n_kv_heads * ceil_div(ceil_div(b.ctx_len[s] + 1, kPage), pages);
+    if (n > sms) break;
+    double us = 0.0;
+    for (const int eightieths : {80, 65, 60, 52, 40, 28}) {
+      const int on = std::max(1, sms * eightieths / 80), rounds = ceil_div(n, on);
+      const double page_us = std::max(0.45, kDecodeWarps * 64.0 * c.head_dim / std::min(70e3, 6.2e6 / std::min(n, on)));
+      us += (eightieths == 80 ? 1.0 : 0.15) * rounds * (3.5 + ceil_div(pages, kDecodeWarps) * page_us + (cuts > 1 ? 2.5 : 0.0));
+    }
+    if (us < best_us * (cuts > 1 ? 0.9 : 1.0)) { best_us = us; best = pages; }
+  }
+  return best;
+}
 }  // namespace
 
 hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs_batch_t& b, int sm_count, int sm_budget,
@@ -199,18 +234,12 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
   const int G = c.n_q_heads / c.n_kv_heads;
   const int Mt = prefill_tokens_per_item(G);
   const int split = pick_decode_split(c, b, sm_count, ml.max_decode_items);
-  // Group mode of the decode attention: when even the smallest run length leaves warps idle (the batch is small) and
-  // every (sequence, KV head) group can have a block of its own, a group's pages are dealt evenly to the eight warps
-  // of one block, whose partial results then meet in shared memory -- no partials in global memory, no counter, no
-  // merging warp.  A function of the batch and the device's SM count, never of the budget.
-  bool group_mode = split == kDecodeTail;
-  {
-    int groups = 0, longest = 0;
-    for (int s = 0; s < b.n_seqs; ++s)
-      if (b.q_len[s] == 1) { groups += c.n_kv_heads; longest = std::max(longest, b.ctx_len[s] + 1); }
-    const int sms = sm_count > 0 ? sm_count : 148;
-    if (groups == 0 || groups > sms || longest > kDecodeWarps * 32 * kPage) group_mode = false;
-  }
+  // Group mode of the decode attention: in a batch small enough, every group = (sequence, KV head) is cut into equal
+  // slices of whole pages such that all slices have a block of their own on the device; a block's eight warps share a
+  // slice, and the block that delivers a group's last slice merges the group's (attention_decode.cuh).  A function of the
+  // batch and the device's SM count, never of the budget.
+  const int slice_pages = pick_decode_slice(c, b, sm_count, split);
+  const bool group_mode = slice_pages > 0;
   StepPlan p;
   p.n_tokens = b.n_tokens;
   p.n_seqs = b.n_seqs;
@@ -256,18 +285,22 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
       if (tok_seq) tok_seq[t + j] = s;
     }
     if (n == 1 && group_mode) {
-      // decode, group mode: eight slices of the sequence's pages per KV head (the last ones may be empty)
-      const int keys = ctx + 1, pages = ceil_div(keys, kPage), per = ceil_div(pages, kDecodeWarps) * kPage;
+      // decode, group mode: per KV head `slices` slices of the sequence's pages, each dealt evenly to eight warps (the last
+      // of which may have none)
+      const int keys = ctx + 1, pages = ceil_div(keys, kPage), slices = ceil_div(pages, slice_pages);
       if (meta) {
         int32_t* row = meta + ml.decode_rows + n_dec_rows * 4;
-        row[0] = s; row[1] = t; row[2] = n_dec_items; row[3] = kDecodeWarps;
+        row[0] = s; row[1] = t; row[2] = n_dec_items; row[3] = slices * kDecodeWarps;
       }
       for (int hk = 0; hk < c.n_kv_heads; ++hk)
-        for (int w = 0; w < kDecodeWarps; ++w) {
-          const int k0 = std::min(keys, w * per), k1 = std::min(keys, (w + 1) * per);
-          dec.push_back(DecItem{{n_dec_rows, hk, k0, k1, s, t, 0, 1}, 0});
+        for (int i = 0; i < slices; ++i) {
+          const int p0 = pages * i / slices, p1 = pages * (i + 1) / slices, per = ceil_div(p1 - p0, kDecodeWarps);
+          for (int w = 0; w < kDecodeWarps; ++w) {
+            const int k0 = std::min(keys, std::min(p1, p0 + w * per) * kPage), k1 = std::min(keys, std::min(p1, p0 + (w + 1) * per) * kPage);
+            dec.push_back(DecItem{{n_dec_rows, hk, k0, k1, s, t, n_dec_items / kDecodeWarps + hk * slices, slices | (i << 16)}, 0});
+          }
         }
-      n_dec_items += c.n_kv_heads * kDecodeWarps;
+      n_dec_items += c.n_kv_heads * slices * kDecodeWarps;
       ++n_dec_rows;
     } else if (n == 1) {
       // decode: keys 0..ctx cut into whole runs of `split` keys and the rest into pieces of kDecodeTail keys; the items
@@ -316,6 +349,7 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
   p.n_decode_items = n_dec_items;
   p.decode_group = group_mode && n_dec_items > 0 ? 1 : 0;
   p.n_decode_rows = n_dec_rows;
+  p.meta_words = n_dec_items > 0 ? ml.decode_items + n_dec_items * 8 : ml.prefill_items + int(pre.size()) * 8;
   if (plan) *plan = p;
   return HS_OK;
 }
