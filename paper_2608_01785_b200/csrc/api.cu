@@ -169,7 +169,7 @@ hs_status_t fail(const char* what) {
 // K splits for a residual GEMM, or 1 when the whose-turn array could not hold its tiles.
 int pick_ksplit(int M, int N, int K, int bn, int sm_count) {
   const int tiles = ceil_div(M, 128) * ceil_div(N, bn);
-  if (tiles * 4 > kGemmTurnWords) return 1;
+  if (tiles * 8 > kGemmTurnWords) return 1;
   return gemm_pick_ksplit(M, N, K, bn, sm_count);
 }
 
@@ -221,7 +221,7 @@ struct hs_stage {
   std::vector<LayerMaps> maps;
   CUtensorMap tm_h, tm_o, tm_act, tm_kv, tm_kv_page;   // operand loads
   CUtensorMap tm_h_s[2], tm_o_s[2], tm_act_s[2];   // the same A operands with 64- and 32-row boxes (small steps)
-  CUtensorMap tm_q_st, tm_act_st, tm_h_st; // epilogue stores (box 64 x 32)
+  CUtensorMap tm_act_st, tm_h_st;          // epilogue stores (box 64 x 32)
   CUtensorMap tm_part;                     // partial sums of the K-split residual GEMMs (box 32 x 32 fp32)
   CUtensorMap tm_q_attn;                   // Q tiles of the prefill attention (box 64 x tokens per item)
   int32_t* pinned[kRing] = {};
@@ -365,8 +365,7 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
     ok = encode_2d(&s->tm_h_s[i], s->ws_dev + s->ws.h, T, d, rows) && encode_2d(&s->tm_o_s[i], s->ws_dev + s->ws.o, T, q_dim, rows) &&
          encode_2d(&s->tm_act_s[i], s->ws_dev + s->ws.act, T, F, rows);
   }
-  ok = ok && encode_2d(&s->tm_q_st, s->ws_dev + s->ws.q, T, q_dim, 32) &&
-       encode_2d(&s->tm_act_st, s->ws_dev + s->ws.act, T, F, 32) && encode_2d(&s->tm_h_st, s->ws_dev + s->ws.h, T, d, 32);
+  ok = ok && encode_2d(&s->tm_act_st, s->ws_dev + s->ws.act, T, F, 32) && encode_2d(&s->tm_h_st, s->ws_dev + s->ws.h, T, d, 32);
   ok = ok && encode_2d(&s->tm_q_attn, s->ws_dev + s->ws.q, T, q_dim,
                        prefill_tokens_per_item(cfg->n_q_heads / cfg->n_kv_heads));
   if (s->ws.part_rows > 0) ok = ok && encode_2d(&s->tm_part, s->ws_dev + s->ws.gemm_part, s->ws.part_rows, d, 32, true);
@@ -742,7 +741,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     g.pair = pair_qkv;
     g.bn = pair_qkv ? 256 : 128;     // small steps: 128-column tiles, twice as many SMs stream the weights
     g.q_dim = q_dim; g.kv_dim = kv_dim; g.head_dim = Dh; g.n_kv_heads = c.n_kv_heads;
-    g.tm_q = s->tm_q_st;
+    g.q_out = q;
     g.k_cache = s->kv_pool + (size_t(l) * 2 + 0) * layer_kv_elems;
     g.v_cache = s->kv_pool + (size_t(l) * 2 + 1) * layer_kv_elems;
     g.tok_pos = meta + s->ml.tok_pos;

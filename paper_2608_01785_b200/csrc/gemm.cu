@@ -10,18 +10,18 @@
 //               small token counts, for sm_budget 1 and for the K-split path; both produce the same bits.
 //   operands    TMA (128-byte swizzle) -> shared-memory ring -> tcgen05.mma, fp32 accumulators in tensor
 //               memory, two accumulator buffers so the epilogue of tile i overlaps the main loop of i+1
-//   roles       warp 0: TMA producer, warp 1: MMA issuer (one thread, leader block only), warps 2..5:
-//               epilogue.  Cross-block signalling in a pair: both blocks' TMA bytes are counted on the
-//               leader's "full" barrier; the leader's tcgen05.commit arrives on the "empty" and
-//               "accumulator full" barriers of both blocks; epilogue warps of both blocks arrive on the
+//   roles       warp 0: TMA producer, warp 1: MMA issuer (one thread, leader block only), warps 2..9:
+//               epilogue, two per 32 rows of the accumulator.  Cross-block signalling in a pair: both blocks'
+//               TMA bytes are counted on the leader's "full" barrier; the leader's tcgen05.commit arrives on the
+//               "empty" and "accumulator full" barriers of both blocks; epilogue warps of both blocks arrive on the
 //               leader's "accumulator empty" barrier.
 //   schedule    unit = worker + i * workers, workers <= sm_budget (pairs: sm_budget / 2), one block per
 //               SM.  Each output tile is produced by one block (pair) with a fixed K order, so results do
 //               not depend on the budget.
 //
 // Epilogues: residual add (the fp32 tile is ADDED into the residual stream by a TMA reduction, so the
-// stream is never read by the SM), QKV (rotate-half RoPE; bf16 q by TMA store; k, v scattered into the
-// paged cache), gate/up (silu(gate) * up -> bf16 by TMA store).  Output blocks are staged in shared memory
+// stream is never read by the SM), QKV (rotate-half RoPE; a row's 64 contiguous bytes of q, k or v from the
+// registers, k and v into the paged cache), gate/up (silu(gate) * up -> bf16 by TMA store).  Output blocks are staged in shared memory
 // in the 128-byte-swizzled layout the tensor maps expect (conflict-free for one-row-per-thread writes).
 #include <algorithm>
 #include <type_traits>
@@ -44,11 +44,11 @@ template <bool PAIR> struct Ring {
 constexpr int RING_BYTES = 4 * (A_BYTES + 2 * BH_BYTES);
 static_assert(Ring<true>::STAGES * Ring<true>::STAGE_BYTES == RING_BYTES, "both rings fill the same space");
 constexpr int kMaxStages = 12;                  // barrier slots; the ring holds fewer when stages are large
-constexpr int GEMM_THREADS = 192;
+constexpr int EPI_WARPS = 8, GEMM_THREADS = 64 + EPI_WARPS * 32;
 constexpr int TMEM_COLS = 512;                  // two 128 x 256 fp32 accumulators
 constexpr int EPI_BUF_BYTES = 4096;             // 32 rows x 128 B: a 32 x 32 fp32 or 32 x 64 bf16 output block
-constexpr int EPI_WARP_BYTES = 2 * EPI_BUF_BYTES;   // two blocks per epilogue warp, filled alternately
-constexpr int GEMM_SMEM = 1024 + RING_BYTES + 4 * EPI_WARP_BYTES + 384;
+constexpr int EPI_BYTES = EPI_WARPS * EPI_BUF_BYTES;   // one block per epilogue warp
+constexpr int GEMM_SMEM = 1024 + RING_BYTES + EPI_BYTES + 384;
 static_assert(GEMM_SMEM <= 227 * 1024, "fits one SM");
 static_assert(GEMM_SMEM >= kMinSmemBytes, "one block per SM");
 
@@ -78,17 +78,19 @@ __device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-__device__ __forceinline__ void store_bf16x32(__nv_bfloat16* dst, const float (&v)[32], int n_valid) {
+__device__ __forceinline__ void st_global_32b(void* dst, const uint32_t (&w)[8]) {      // a lane's whole sector
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+               "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+// 32 fp32 values (raw bits) of one row -> 64 contiguous bytes of bf16, 32-byte aligned.
+__device__ __forceinline__ void store_bf16x32(__nv_bfloat16* dst, const uint32_t (&r)[32]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    if (i * 8 < n_valid) {
-      uint4 w;
-      w.x = pack_bf16(v[i * 8 + 0], v[i * 8 + 1]);
-      w.y = pack_bf16(v[i * 8 + 2], v[i * 8 + 3]);
-      w.z = pack_bf16(v[i * 8 + 4], v[i * 8 + 5]);
-      w.w = pack_bf16(v[i * 8 + 6], v[i * 8 + 7]);
-      *reinterpret_cast<uint4*>(dst + i * 8) = w;
-    }
+  for (int i = 0; i < 2; ++i) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = pack_bf16(__uint_as_float(r[i * 16 + 2 * e]), __uint_as_float(r[i * 16 + 2 * e + 1]));
+    st_global_32b(dst + 16 * i, w);
   }
 }
 
@@ -111,6 +113,12 @@ __device__ __forceinline__ void stage_bf16x32(uint8_t* buf, int lane, int u0, co
     w.w = pack_act(v[i * 8 + 6], v[i * 8 + 7], f16);
     *reinterpret_cast<uint4*>(buf + lane * 128 + (((u0 + i) ^ (lane & 7)) << 4)) = w;
   }
+}
+
+__device__ __forceinline__ void ldg_f32x8(float (&t)[8], const float2* src) {      // 32 bytes, 32-byte aligned, read-only data
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3]), "=f"(t[4]), "=f"(t[5]), "=f"(t[6]), "=f"(t[7])
+               : "l"(src));
 }
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
@@ -291,15 +299,19 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* epi_smem = smem + RING_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + 4 * EPI_WARP_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + EPI_BYTES);
   uint64_t* empty = full + kMaxStages;
   uint64_t* tfull = empty + kMaxStages;
   uint64_t* tempty = tfull + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  uint64_t* xbar = reinterpret_cast<uint64_t*>(epi_smem + 4 * EPI_WARP_BYTES + 256);   // [4 warps][4] landing-block barriers (three used)
+  uint64_t* xbar = reinterpret_cast<uint64_t*>(epi_smem + EPI_BYTES + 256);   // [4 warps][4] landing-block barriers (three used)
 
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
+  // Residual GEMMs on pairs, and those that fold the norm, leave the second warps of the quarters idle: their epilogue is bound by
+  // the residual stream's way through shared memory, and the idle warps' staging blocks serve the first (both at work with a
+  // block each: out and down at 7B dimensions, 2112 rows, 224 -> 230 us on average, partial sums of 401 rows 49.0 -> 49.8).
+  const bool solo = MODE == kGemmResid && (PAIR || p.norm_gain != nullptr);
   log_smid(p.smid_log);
   // In pair mode the two blocks of a cluster share every work unit: a unit's tile is 256 rows tall and
   // block `rank` owns rows 128 * rank .. 128 * rank + 127 of it.
@@ -319,21 +331,23 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   const bool ordered = !walk.parts && (walk.stream_k || walk.ksplit > 1);
   Unit un;
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
+  // (a lane per barrier: a block that starts when its predecessor's leaves has its set-up, 2 us of it, on the critical path)
+  if (warp == 0) {
+    if (lane < STAGES) {
+      mbar_init(&full[lane], 1);
+      mbar_init(&empty[lane], 1);
+    } else if (lane >= 16 && lane < 18) {
+      mbar_init(&tfull[lane - 16], 1);
+      mbar_init(&tempty[lane - 16], (PAIR ? 2 : 1) * (solo ? EPI_WARPS / 2 : EPI_WARPS));   // one arrival per epilogue warp (of both blocks)
+    } else if (lane == 18) {
+      *abort_flag = 0;
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], PAIR ? 8 : 4);      // one arrival per epilogue warp (of both blocks)
-    }
-    for (int i = 0; i < 16; ++i) mbar_init(&xbar[i], 1);
-    *abort_flag = 0;
+    if (lane >= 16) mbar_init(&xbar[lane - 16], 1);
     fence_barrier_init();
-    tma_prefetch_desc(&p.tm_a);
-    tma_prefetch_desc(&p.tm_b[0]);
-    tma_prefetch_desc(MODE == kGemmResid ? &p.tm_out : MODE == kGemmQkv ? &p.tm_q : &p.tm_act);
+  } else if (warp == 2) {
+    if (lane == 0) tma_prefetch_desc(&p.tm_a);
+    if (lane == 1) tma_prefetch_desc(&p.tm_b[0]);
+    if (lane == 2 && MODE != kGemmQkv) tma_prefetch_desc(MODE == kGemmResid ? &p.tm_out : &p.tm_act);
   }
   if (warp == 1) {
     if (PAIR) {
@@ -464,14 +478,19 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     }
   } else {
     // ----------------------------------------------------------- epilogue --
+    // Two warps per quarter, each with half of the tile's columns: an epilogue is a chain of latencies (tensor memory,
+    // shared memory, stores) of one warp per scheduler otherwise, and where a GEMM has a tile or two per SM it is exposed.
+    // Measured on B200, 1024 conditioned rows of d = 1024, per launch: QKV 18.7 -> 15.5 us, with 32-byte loads of the rotation
+    // and 32-byte stores (a lane's whole sector: its row is its own), out-projection 11.9 -> 10.7; step 984 -> 933 us.
     const int quarter = warp & 3;             // the TMEM lane quarter this warp may read
+    const int cg = (warp - 2) >> 2;           // its half of the columns
     int acc = 0;
     uint32_t acc_ph = 0;
     const int Dh = p.head_dim;
-    uint8_t* epi_buf = epi_smem + quarter * EPI_WARP_BYTES;
-    int epi_sel = 0;                          // staging block to fill next
+    uint8_t* epi_buf = epi_smem + (quarter + 4 * cg) * EPI_BUF_BYTES;
+    int epi_sel = 0;                          // staging block to fill next, of the two that a lone warp has
     uint32_t xph = 0;                         // phase bits of this warp's landing-block barriers
-    while (walk.next(un)) {
+    while (!(solo && cg == 1) && walk.next(un)) {
       const int tile = un.tile, ks = un.seg;
       const int m = PAIR ? 2 * (tile % n_m_tiles) + int(rank)
                          : emulate_pair ? 2 * (tile % n_m_tiles) + un.half : tile % n_m_tiles,
@@ -482,17 +501,30 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // folded RMSNorm, consuming side: r of this thread's row, requested before the wait for the accumulator
       float rs = 1.f;
       if (p.in_row_rs != nullptr && MODE != kGemmResid && row_ok) rs = __ldcg(p.in_row_rs + row);
+      // QKV: the row's position and cache slot, and its rotation's cosines and sines on their way into the L1
+      int pos = 0, slot = 0;
+      if (MODE == kGemmQkv) {
+        if (row_ok) {
+          pos = p.tok_pos[row];
+          slot = p.tok_slot[row];
+        }
+        const float2* cs = p.rope + size_t(pos) * (Dh >> 1) + (Dh == 128 ? 32 * cg : 0);
+        asm volatile("prefetch.global.L1 [%0];\n\tprefetch.global.L1 [%0 + 128];" ::"l"(cs));
+      }
       // folded RMSNorm, producing side: the first two blocks of this warp's rows of y are on their way before the
       // tile's products are complete
       const bool fold_now = fold_pair && un.last;
-      // three landing blocks per warp: two in the ring's unused last stage, the third is the warp's second staging block
+      // three landing blocks per warp that folds: two in the ring's unused last stage, the third is its idle neighbour's
+      // staging block
       uint8_t* xb_stage = smem + (Ring<true>::STAGES - 1) * Ring<true>::STAGE_BYTES + quarter * 2 * EPI_BUF_BYTES;
-      auto landing = [&](int i) -> uint8_t* { return i < 2 ? xb_stage + i * EPI_BUF_BYTES : epi_buf + EPI_BUF_BYTES; };
+      auto landing = [&](int i) -> uint8_t* { return i < 2 ? xb_stage + i * EPI_BUF_BYTES : epi_buf + 4 * EPI_BUF_BYTES; };
       uint64_t* xb_bar = xbar + quarter * 4;
-      const int n_chunks = min(p.bn / 32, (p.N - n * p.bn + 31) / 32);
+      // this warp's 32-column chunks of the tile: c_lo .. c_hi - 1
+      const int n_chunks = min(p.bn / 32, (p.N - n * p.bn + 31) / 32), c_mid = solo ? n_chunks : min((p.bn / 32 + 1) / 2, n_chunks);
+      const int c_lo = cg ? c_mid : 0, c_hi = cg ? n_chunks : c_mid;
       if (fold_now) {
         if (ordered && ks > 0) {              // every earlier segment of the tile must be in y before y is read
-          int* turn = p.tile_turn + (tile * 2 + int(rank)) * 4 + quarter;
+          int* turn = p.tile_turn + (tile * 2 + int(rank)) * EPI_WARPS + quarter + 4 * cg;
           bool go = true;
           if (lane == 0) go = spin_until_equal(turn, ks, abort_flag, p.status);
           if (!__shfl_sync(0xffffffffu, go, 0)) break;
@@ -510,14 +542,13 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       tc_fence_after_sync();
       const uint32_t taddr = tmem_base + acc * BN + (uint32_t(quarter * 32) << 16);
       uint32_t r0[32], r1[32];
-      float v0[32], v1[32];
-
+      float v0[32];
 
       if (MODE == kGemmResid) {
         // Ordered split-K: the partial sums of a tile are added into the output in split order, so the
-        // result is the same fixed sum whatever block computed which split.  This warp owns 32 rows of the
-        // tile; it waits until the previous split's add of those rows has been performed.
-        int* turn = p.tile_turn + (PAIR ? tile * 2 + int(rank) : emulate_pair ? tile * 2 + un.half : tile) * 4 + quarter;
+        // result is the same fixed sum whatever block computed which split.  This warp owns 32 rows of half the
+        // tile's columns; it waits until the previous split's add of those has been performed.
+        int* turn = p.tile_turn + (PAIR ? tile * 2 + int(rank) : emulate_pair ? tile * 2 + un.half : tile) * EPI_WARPS + quarter + 4 * cg;
         if (ordered && ks > 0 && !fold_now) {
           bool go = true;
           if (lane == 0) go = spin_until_equal(turn, ks, abort_flag, p.status);
@@ -606,7 +637,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           const bool h16 = p.norm_h_f16 != 0;
           float ss = 0.f;
           uint8_t* buf_x = epi_buf;                       // fp32 block of this chunk
-          uint8_t* buf_h = epi_buf + EPI_BUF_BYTES;       // 16-bit block of a pair of chunks
+          uint8_t* buf_h = epi_buf + 4 * EPI_BUF_BYTES;       // 16-bit block of a pair of chunks
           for (int c = 0; c < p.bn / 32; ++c) {
             const int col0 = n * p.bn + c * 32;
             if (col0 >= p.N) break;
@@ -658,9 +689,8 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
         } else {
           float best_v = -INFINITY;              // greedy sampling: this thread's row over the tile
           int best_c = 0x7fffffff;
-          for (int c = 0; c < p.bn / 32; ++c) {
+          for (int c = c_lo; c < c_hi; ++c) {
             const int col0 = n * p.bn + c * 32;
-            if (col0 >= p.N) break;
             tmem_ld32(taddr + c * 32, r0);
             float4 gv[8];
             const int nv = p.N - col0 >= 32 ? 8 : (p.N - col0) >> 2;          // float4s of the chunk inside the row
@@ -692,9 +722,12 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
                 best_v = mx;
               }
             }
-            if (lane == 0) bulk_wait_read<1>();     // the block staged two chunks ago has been read
+            if (lane == 0) {                        // the staging block has been read by its last store
+              if (solo) bulk_wait_read<1>();
+              else bulk_wait_read<0>();
+            }
             __syncwarp();
-            uint8_t* buf = epi_buf + epi_sel * EPI_BUF_BYTES;
+            uint8_t* buf = epi_buf + epi_sel * 4 * EPI_BUF_BYTES;
             stage_f32x32(buf, lane, r0);
             fence_proxy_async();
             __syncwarp();
@@ -703,7 +736,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
               else if (store_ok) tma_store_2d(&p.tm_out, buf, col0, out_row);
               bulk_commit();
             }
-            epi_sel ^= 1;
+            if (solo) epi_sel ^= 1;
           }
           if (!PAIR && p.argmax_key != nullptr && row_ok) {
             const uint32_t u = __float_as_uint(best_v + 0.f);                       // (-0 and +0 are the same value)
@@ -718,7 +751,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           st_release(turn, un.last ? 0 : ks + 1);   // the last segment leaves the word at zero
         }
       } else if (MODE == kGemmGateUp) {
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 2 * cg; c < 2 * cg + 2; ++c) {        // (this warp's 64 columns are one block of the output map)
           const int col0 = n * 128 + c * 32;
           if (col0 >= p.N) break;
           tmem_ld32(taddr + c * 32, r0);          // gate
@@ -730,26 +763,21 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
             v0[e] = __fdividef(g * u, 1.f + __expf(-g));   // silu(g) * u
           }
           if (p.act_f16) note_f16_saturation(v0, p.status);
-          uint8_t* buf = epi_buf + epi_sel * EPI_BUF_BYTES;
           if ((c & 1) == 0) {
-            if (lane == 0) bulk_wait_read<1>();
+            if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
           }
-          stage_bf16x32(buf, lane, (c & 1) * 4, v0, p.act_f16 != 0);
-          const bool block_done = (c & 1) || col0 + 32 >= p.N;
-          if (block_done) {                       // 64 columns staged (or the ragged end of the row)
+          stage_bf16x32(epi_buf, lane, (c & 1) * 4, v0, p.act_f16 != 0);
+          if ((c & 1) || col0 + 32 >= p.N) {      // 64 columns staged (or the ragged end of the row)
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
-              tma_store_2d(&p.tm_act, buf, n * 128 + (c >> 1) * 64, row_base);
+              tma_store_2d(&p.tm_act, epi_buf, n * 128 + cg * 64, row_base);
               bulk_commit();
             }
-            epi_sel ^= 1;
           }
         }
       } else {
-        const int pos = row_ok ? p.tok_pos[row] : 0;
-        const int slot = row_ok ? p.tok_slot[row] : 0;
         const int half_dh = Dh >> 1;
         const int qkv_w = gemm_qkv_width(p);
         for (int half = 0; half < qkv_w / 128; ++half) {
@@ -759,67 +787,43 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           if (vcol >= p.q_dim) { region = 1; vcol -= p.q_dim; }
           if (region == 1 && vcol >= p.kv_dim) { region = 2; vcol -= p.kv_dim; }
           const __nv_bfloat16* bias = p.qkv_bias[region];      // of this region's projection, or null
-          if (region == 2) {
-            for (int c = 0; c < 4; ++c) {
-              tmem_ld32(taddr + half * 128 + c * 32, r0);
-              tmem_ld_wait();
-              if (p.in_row_rs) scale32(r0, rs);
-              if (bias) add_bias32(r0, bias + vcol + c * 32);
-              if (row_ok) {
+          // this warp's two 32-column chunks of the half: rotation partners (q and k heads; the same pairs in both halves)
+          const int lo = Dh == 128 ? cg : 2 * cg, hi = lo + (Dh == 128 ? 2 : 1);
+          tmem_ld32(taddr + half * 128 + lo * 32, r0);
+          tmem_ld32(taddr + half * 128 + hi * 32, r1);
+          tmem_ld_wait();
+          if (p.in_row_rs) {
+            scale32(r0, rs);
+            scale32(r1, rs);
+          }
+          if (bias) {                                          // the bias comes before the rotation
+            add_bias32(r0, bias + vcol + lo * 32);
+            add_bias32(r1, bias + vcol + hi * 32);
+          }
+          if (region != 2) {
+            const float2* cs = p.rope + size_t(pos) * half_dh + (Dh == 128 ? 32 * cg : 0);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) v0[e] = __uint_as_float(r0[e]);
-                const int col = vcol + c * 32;
-                store_bf16x32(cache_ptr(p.v_cache, slot, col / Dh, p.n_kv_heads, Dh, col % Dh), v0, 32);
-              }
-            }
-          } else {
-            if (region == 0) {                    // both staging blocks are about to be refilled
-              if (lane == 0) bulk_wait_read<0>();
-              __syncwarp();
-            }
-            for (int j = 0; j < 2; ++j) {
-              const int lo = Dh == 128 ? j : 2 * j, hi = lo + (Dh == 128 ? 2 : 1);
-              const int i0 = Dh == 128 ? 32 * j : 0;       // index of the first rotation pair
-              tmem_ld32(taddr + half * 128 + lo * 32, r0);
-              tmem_ld32(taddr + half * 128 + hi * 32, r1);
-              tmem_ld_wait();
-              if (p.in_row_rs) {
-                scale32(r0, rs);
-                scale32(r1, rs);
-              }
-              if (bias) {                                        // the bias comes before the rotation
-                add_bias32(r0, bias + vcol + lo * 32);
-                add_bias32(r1, bias + vcol + hi * 32);
-              }
-              const float2* cs = p.rope + size_t(pos) * half_dh + i0;
+            for (int e = 0; e < 32; e += 4) {
+              float t[8];                                      // cos, sin of pairs e .. e + 3
+              ldg_f32x8(t, cs + e);
 #pragma unroll
-              for (int e = 0; e < 32; e += 2) {
-                const float4 t = *reinterpret_cast<const float4*>(cs + e);   // cos,sin of pairs e, e+1
-                const float a0 = __uint_as_float(r0[e]), b0 = __uint_as_float(r1[e]);
-                const float a1 = __uint_as_float(r0[e + 1]), b1 = __uint_as_float(r1[e + 1]);
-                v0[e] = a0 * t.x - b0 * t.y;
-                v1[e] = b0 * t.x + a0 * t.y;
-                v0[e + 1] = a1 * t.z - b1 * t.w;
-                v1[e + 1] = b1 * t.z + a1 * t.w;
-              }
-              if (region == 0) {
-                // chunk ch of the half belongs to 64-column block ch / 2, units 4 (ch % 2) ..
-                stage_bf16x32(epi_buf + (lo >> 1) * EPI_BUF_BYTES, lane, (lo & 1) * 4, v0);
-                stage_bf16x32(epi_buf + (hi >> 1) * EPI_BUF_BYTES, lane, (hi & 1) * 4, v1);
-              } else if (row_ok) {
-                const int col_lo = vcol + lo * 32, col_hi = vcol + hi * 32;
-                store_bf16x32(cache_ptr(p.k_cache, slot, col_lo / Dh, p.n_kv_heads, Dh, col_lo % Dh), v0, 32);
-                store_bf16x32(cache_ptr(p.k_cache, slot, col_hi / Dh, p.n_kv_heads, Dh, col_hi % Dh), v1, 32);
+              for (int u = 0; u < 4; ++u) {
+                const float a = __uint_as_float(r0[e + u]), b = __uint_as_float(r1[e + u]);
+                r0[e + u] = __float_as_uint(a * t[2 * u] - b * t[2 * u + 1]);
+                r1[e + u] = __float_as_uint(b * t[2 * u] + a * t[2 * u + 1]);
               }
             }
+          }
+          if (row_ok) {
+            const int col_lo = vcol + lo * 32, col_hi = vcol + hi * 32;
             if (region == 0) {
-              fence_proxy_async();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_2d(&p.tm_q, epi_buf, vcol, row_base);
-                tma_store_2d(&p.tm_q, epi_buf + EPI_BUF_BYTES, vcol + 64, row_base);
-                bulk_commit();
-              }
+              __nv_bfloat16* qrow = p.q_out + size_t(row) * p.q_dim;
+              store_bf16x32(qrow + col_lo, r0);
+              store_bf16x32(qrow + col_hi, r1);
+            } else {
+              __nv_bfloat16* cache = region == 1 ? p.k_cache : p.v_cache;
+              store_bf16x32(cache_ptr(cache, slot, col_lo / Dh, p.n_kv_heads, Dh, col_lo % Dh), r0);
+              store_bf16x32(cache_ptr(cache, slot, col_hi / Dh, p.n_kv_heads, Dh, col_hi % Dh), r1);
             }
           }
         }
@@ -1028,7 +1032,7 @@ int gemm_pick_stream_k(int M, int N, int K, int sm_count) {
   const int W = sm_count / 2;
   const int tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
   const int k_blocks = (K + BK - 1) / BK;
-  if (W < 1 || tiles * 8 > kGemmTurnWords || k_blocks < 64) return 0;
+  if (W < 1 || tiles * 2 * EPI_WARPS > kGemmTurnWords || k_blocks < 64) return 0;
   if (tiles * 2 < W) return 0;                       // few tiles: single blocks with a K split serve better
   const int rounds = (tiles + W - 1) / W;
   return double(tiles) / W < 0.92 * rounds ? W : 0;

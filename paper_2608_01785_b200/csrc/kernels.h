@@ -50,10 +50,10 @@ struct GemmParams {
   int part_rows;             // > 0: partial sums -- K split ks of the tile goes, unadded, to rows ks * part_rows ... of
                              // tm_out (a scratch [ksplit * part_rows, N] fp32 matrix; part_rows a multiple of 32, at
                              // least M), in equal splits; the RMSNorm behind the GEMM adds them (NormParams::part)
-  int* tile_turn;            // [tiles * 4] ([tiles * 8] on pairs) whose-turn words for the ordered adds; zero at entry and at exit
+  int* tile_turn;            // [tiles * 8] ([tiles * 16] on pairs) whose-turn words for the ordered adds; zero at entry and at exit
   // Qkv
   int q_dim, kv_dim, head_dim, n_kv_heads;
-  CUtensorMap tm_q;          // bf16 q [M, q_dim], box 64 x 32, 128-byte swizzle
+  __nv_bfloat16* q_out;      // bf16 q [M, q_dim]
   __nv_bfloat16* k_cache;    // this layer's K pages: [page][kv_head][16][Dh]
   __nv_bfloat16* v_cache;
   const int32_t* tok_pos;    // [M]
@@ -179,7 +179,7 @@ bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim);
 bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count);
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream);
 cudaError_t gemm_skinny_set_attributes();
-constexpr int kGemmTurnWords = 4096;   // capacity of the whose-turn array: splits are used only when tiles * 4 fits
+constexpr int kGemmTurnWords = 8192;   // capacity of the whose-turn array: splits are used only when tiles * 8 fits
 
 // ---------------------------------------------------------------- RMSNorm --
 // h[t,:] = bf16(x[t,:] * rsqrt(mean(x[t,:]^2) + eps) * g).  x comes either as bf16 (x_bf16, first layer;
