@@ -568,6 +568,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   auto pair_for = [&](int n_cols, int single_bn) { return on_pairs(T, n_cols, single_bn, s->sm_count); };
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
+  const int gu_width = gemm_pick_gu_width(T, F, sm_budget);      // (the results do not depend on it)
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
   // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next
@@ -839,6 +840,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     gu.act_f16 = f16;
     gu.pair = pair_gu;
     gu.tm_act = s->tm_act_st;
+    gu.act = reinterpret_cast<__nv_bfloat16*>(s->ws_dev + s->ws.act);
     gu.status = status;
     gu.smid_log = slots(6);
     if (fold_norm || sk_fold_mlp) fold_in(gu);
@@ -850,7 +852,13 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
       if (sk_fold_mlp) sk_fold_in(k);
       else k.in_row_rs = gu.in_row_rs;
       LaunchTimer t(s, 6, stream); where = "gate/up gemm"; e = launch_gemm_skinny(k, sm_budget, stream);
-    } else { LaunchTimer t(s, 6, stream); where = "gate/up gemm"; e = launch_gemm(gu, sm_budget, stream); }
+    } else {
+      if (!pair_gu && gu_width != 128) {
+        gu.gu_width = gu_width;
+        if (!encode_2d(&gu.tm_b[0], wo.w_gate, F, d, gu_width) || !encode_2d(&gu.tm_b[1], wo.w_up, F, d, gu_width)) return HS_ERR_CUDA;
+      }
+      LaunchTimer t(s, 6, stream); where = "gate/up gemm"; e = launch_gemm(gu, sm_budget, stream);
+    }
     if (e != cudaSuccess) break;
 
     GemmParams gd{};

@@ -57,10 +57,14 @@ static_assert(GEMM_SMEM >= kMinSmemBytes, "one block per SM");
 // tile never straddles q | k | v (their widths are multiples of 128) and holds whole heads.
 __host__ __device__ __forceinline__ int gemm_qkv_width(const GemmParams& p) { return p.bn == 128 && !p.pair ? 128 : BN; }
 
+// GateUp mode: activation columns of a tile, 128, or on single blocks p.gu_width.
+__host__ __device__ __forceinline__ int gemm_gu_width(const GemmParams& p) { return p.gu_width > 0 && !p.pair ? p.gu_width : 128; }
+
 // Output-tile width: 256 virtual columns, except in Resid mode where the launcher picks p.bn (a multiple
-// of 32 in [128, 256]) from the problem shape so that the tile count fills whole waves of SMs.
+// of 32 in [128, 256]) from the problem shape so that the tile count fills whole waves of SMs, and in GateUp mode on
+// single blocks.
 __host__ __device__ __forceinline__ int gemm_n_tiles(const GemmParams& p) {
-  if (p.mode == kGemmGateUp) return (p.N + 127) / 128;
+  if (p.mode == kGemmGateUp) return (p.N + gemm_gu_width(p) - 1) / gemm_gu_width(p);
   const int bn = p.mode == kGemmResid ? p.bn : gemm_qkv_width(p);
   return (p.N + bn - 1) / bn;
 }
@@ -68,7 +72,7 @@ __host__ __device__ __forceinline__ int gemm_n_tiles(const GemmParams& p) {
 struct BSource { int map, row; };
 __device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int half) {
   if (p.mode == kGemmResid) return {0, n_tile * p.bn + half * 128};
-  if (p.mode == kGemmGateUp) return {half, n_tile * 128};
+  if (p.mode == kGemmGateUp) return {half, n_tile * gemm_gu_width(p)};
   int v = n_tile * gemm_qkv_width(p) + half * 128;
   if (v < p.q_dim) return {0, v};
   v -= p.q_dim;
@@ -82,6 +86,21 @@ __device__ __forceinline__ void st_global_32b(void* dst, const uint32_t (&w)[8])
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
                "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                : "memory");
+}
+// n_valid (a multiple of 8) of 32 values of one row -> 16-bit values at dst: 32-byte stores where dst is aligned to that.
+__device__ __forceinline__ void store_act32(__nv_bfloat16* dst, const float (&v)[32], bool f16, int n_valid) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = pack_act(v[i * 16 + 2 * e], v[i * 16 + 2 * e + 1], f16);
+    if (16 * i + 16 <= n_valid && (reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
+      st_global_32b(dst + 16 * i, w);
+    } else {
+      if (16 * i + 8 <= n_valid) *reinterpret_cast<uint4*>(dst + 16 * i) = make_uint4(w[0], w[1], w[2], w[3]);
+      if (16 * i + 16 <= n_valid) *reinterpret_cast<uint4*>(dst + 16 * i + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+  }
 }
 // 32 fp32 values (raw bits) of one row -> 64 contiguous bytes of bf16, 32-byte aligned.
 __device__ __forceinline__ void store_bf16x32(__nv_bfloat16* dst, const uint32_t (&r)[32]) {
@@ -289,7 +308,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // small step buy depth -- 8 or 9 stages instead of 4.
   const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) > 128;
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
-  const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * BH_BYTES;
+  // (a narrow GateUp tile: its gate rows, and right behind them its up rows, one operand of 2 gu_w rows)
+  const int gu_w = MODE == kGemmGateUp && !PAIR ? gemm_gu_width(p) : 128, bh_bytes = gu_w * BK * 2;
+  const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * bh_bytes;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
   const bool fold_pair = PAIR && MODE == kGemmResid && p.norm_gain != nullptr;
@@ -375,9 +396,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
       tma_load_2d_pair(st + b_off, &p.tm_b[b0.map], mapa_u32(smem_u32(&full[s]), 0), kb * BK, b0.row);
     } else {
-      mbar_expect_tx(&full[s], a_bytes + (two_halves ? 2 * BH_BYTES : BH_BYTES));
+      mbar_expect_tx(&full[s], a_bytes + (two_halves ? 2 * bh_bytes : bh_bytes));
       tma_load_2d(st + b_off, &p.tm_b[b0.map], &full[s], kb * BK, b0.row);
-      if (two_halves) tma_load_2d(st + b_off + BH_BYTES, &p.tm_b[b1.map], &full[s], kb * BK, b1.row);
+      if (two_halves) tma_load_2d(st + b_off + bh_bytes, &p.tm_b[b1.map], &full[s], kb * BK, b1.row);
     }
   };
   auto load_a = [&](int s, int kb, int m, int half) {
@@ -435,7 +456,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
-                                                 PAIR ? BN : MODE == kGemmResid ? p.bn : MODE == kGemmQkv ? gemm_qkv_width(p) : BN) &
+                                                 PAIR ? BN : MODE == kGemmResid ? p.bn : MODE == kGemmQkv ? gemm_qkv_width(p) : 2 * gu_w) &
                              (p.ab_f16 ? ~(63u << 7) : ~0u);
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
@@ -752,15 +773,26 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
         }
       } else if (MODE == kGemmGateUp) {
         for (int c = 2 * cg; c < 2 * cg + 2; ++c) {        // (this warp's 64 columns are one block of the output map)
-          const int col0 = n * 128 + c * 32;
-          if (col0 >= p.N) break;
+          const int col0 = n * gu_w + c * 32;
+          if (col0 >= p.N || c * 32 >= gu_w) break;
           tmem_ld32(taddr + c * 32, r0);          // gate
-          tmem_ld32(taddr + 128 + c * 32, r1);    // up
+          tmem_ld32(taddr + gu_w + c * 32, r1);   // up
           tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 32; ++e) {
             const float g = __uint_as_float(r0[e]) * rs, u = __uint_as_float(r1[e]) * rs;
             v0[e] = __fdividef(g * u, 1.f + __expf(-g));   // silu(g) * u
+          }
+          if (gu_w < 128) {                       // a narrow tile: straight from the registers
+            const int nv = min(min(32, gu_w - c * 32), p.N - col0);
+            if (nv < 32)
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v0[e] = e < nv ? v0[e] : 0.f;        // (what follows the tile's columns is not act)
+            if (row_ok) {
+              if (p.act_f16) note_f16_saturation(v0, p.status);
+              store_act32(p.act + size_t(row) * p.N + col0, v0, p.act_f16 != 0, nv);
+            }
+            continue;
           }
           if (p.act_f16) note_f16_saturation(v0, p.status);
           if ((c & 1) == 0) {
@@ -1036,6 +1068,29 @@ int gemm_pick_stream_k(int M, int N, int K, int sm_count) {
   if (tiles * 2 < W) return 0;                       // few tiles: single blocks with a K split serve better
   const int rounds = (tiles + W - 1) / W;
   return double(tiles) / W < 0.92 * rounds ? W : 0;
+}
+
+// Activation columns of a GateUp tile on single blocks, from the SMs the launch gets: an output element's sum is the same
+// whatever the tile's width, so this choice may look at the budget.  Tiles of 128 columns at 7B dimensions, 148 of them, are
+// one round on the whole device but two on 96 to 147 SMs.  Time per K block by the rates of resid_launch_us, 0.02 us of it
+// for a further round.  Measured on B200, 29 rows on 96 SMs: 112 columns 50.7 us per launch, 128 columns 53.8; step of 4
+// layers 669 -> 657 us.
+int gemm_pick_gu_width(int M, int N, int sms) {
+  if (M > BM) return 128;
+  const double a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2;
+  int best = 128;
+  double best_us = 1e30;
+  for (int w = 128; w >= 48; w -= 16) {
+    const int tiles = (N + w - 1) / w, rounds = (tiles + sms - 1) / sms;
+    const double b_bytes = 2.0 * w * BK * 2;
+    auto round_us = [&](int n) {
+      return std::max(std::max(0.27 * (0.4 + 0.6 * w / 128), (a_bytes + b_bytes) / 120e3), std::max(b_bytes / 68e3, n * b_bytes / 6.2e6));
+    };
+    const int rest = tiles - (rounds - 1) * sms;
+    const double us = (rounds - 1) * (round_us(sms) + 0.02) + round_us(rest);     // per K block; 1.2 us per further round
+    if (us < best_us * 0.97) { best_us = us; best = w; }
+  }
+  return best;
 }
 
 cudaError_t launch_gemm(const GemmParams& p, int sm_budget, cudaStream_t stream) {
