@@ -155,7 +155,13 @@ PrefillWork prefill_work(const hs_stage_config_t& c, const hs_batch_t& b, int it
 // every one has an SM of the kernel's share to itself.
 // It moves work between SMs, never between results: both kernels give the same bits at any grid size.
 struct AttnSplit { int decode_sms; double us; };
-AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_bytes, int budget, bool side_by_side) {
+// Two-tile items: the choice between side by side and in turn stands, but the SMs are then shared out by what the kernels
+// take beyond that -- the prefill kernel 5.6 us an item beside its 1.13 us a block; the decode kernel in group mode
+// (`groups` blocks) whole rounds of its longest group, 0.85 us per page of a warp.  A batch too large for group mode comes with
+// a step that runs into the power cap: 1.3 of the prefill kernel's time at full clocks.  Measured on B200: 2048 new tokens
+// beside 64 decode rows at 7B dimensions, 90 SMs for the decode kernel: 86 us, the prefill kernel 137.
+AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_bytes, int budget, bool side_by_side, int groups,
+                          int longest_pages) {
   auto t_dec = [&](int b) { return decode_kv_bytes > 0 ? 12.0 + double(decode_kv_bytes) / std::min(5.5e6, 42e3 * b) : 0.0; };
   auto t_pre = [&](int b) {
     if (singles) return w.items <= b ? 10.0 + 1.15 * w.longest : 1e30;
@@ -168,6 +174,14 @@ AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_
   for (int b = 4; b <= budget - 4; ++b) {
     const double t = std::max(t_dec(b), t_pre(budget - b));
     if (t < best) { best = t; r = AttnSplit{b, t}; }
+  }
+  if (r.decode_sms > 0 && !singles) {
+    best = 1e30;
+    for (int b = 4; b <= budget - 4; ++b) {
+      const double pre = 9.0 + (groups ? 1.0 : 1.3) * std::max(5.6 + 1.13 * w.longest, (5.6 * double(w.items) + 1.13 * double(w.blocks)) / (budget - b));
+      const double dec = groups ? 4.0 + ceil_div(groups, b) * (2.0 + 0.85 * ceil_div(longest_pages, kDecodeWarps)) : t_dec(b);
+      if (std::max(pre, dec) < best - 1e-9) { best = std::max(pre, dec); r.decode_sms = b; }
+    }
   }
   return r;
 }
@@ -254,8 +268,10 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
     for (int s = 0; s < b.n_seqs; ++s)
       if (b.q_len[s] == 1) p.decode_kv_bytes += int64_t(b.ctx_len[s] + 1) * 2 * c.n_kv_heads * c.head_dim * 2;
     const PrefillWork one = prefill_work(c, b, Mt), two = prefill_work(c, b, 2 * Mt);
-    const AttnSplit with_one = split_attention(one, true, p.decode_kv_bytes, sm_budget, side_by_side);
-    const AttnSplit with_two = split_attention(two, false, p.decode_kv_bytes, sm_budget, side_by_side);
+    const AttnSplit with_one = split_attention(one, true, p.decode_kv_bytes, sm_budget, side_by_side, 0, 0);
+    int groups = 0;                                   // (beside prefill work a group is one slice)
+    for (int s = 0; s < b.n_seqs; ++s) groups += group_mode && b.q_len[s] == 1 ? c.n_kv_heads : 0;
+    const AttnSplit with_two = split_attention(two, false, p.decode_kv_bytes, sm_budget, side_by_side, groups, slice_pages);
     if (with_one.us < with_two.us) item_tokens = Mt;
     p.decode_sms = item_tokens == Mt ? with_one.decode_sms : with_two.decode_sms;
   }
