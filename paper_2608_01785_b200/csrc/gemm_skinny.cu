@@ -569,7 +569,7 @@ bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim) {
 // The tiled kernel streams a 64-wide K block in about 0.36 us (0.8 us with two weight boxes per stage, gate/up)
 // and pays 3.5 us per link of a K-split chain.  So this kernel wins where the tiled one has too few tiles to
 // occupy the device or needs a long chain (QKV, out-projection, down at few rows), and loses where there are
-// tiles enough (gate/up of a wide FFN), because here every 32 columns re-read the activations.
+// tiles enough (gate/up of a wide FFN), because here every unit re-reads the activations.
 // Depends on the shape and the device only, never on the SM budget: the two kernels round differently, and a
 // step's result must not depend on its budget.  Rounds and waves are counted for the whole device.  Measured
 // against the alternatives over budgets 148 / 111 / 74 at config-3 dimensions (ms per 28-layer decode-only step,

@@ -3,6 +3,8 @@
 // does not depend on how many blocks run.  HBM-bound: reads the row once (it is kept in shared memory for
 // the scaling pass), writes the bf16 normalised row (and, for the first layer, the fp32 copy that starts
 // the residual stream).
+#include <algorithm>
+
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
 }
 
 // The same operation for steps of few rows, and the one that adds the partial sums of a K-split residual GEMM first: TPR
-// threads work on a row (as many as leave one round of rows on the device, at most 512), each holds its V groups of
+// threads work on a row (as many as leave one round of rows on the device, at most 512, a multiple of 32), each holds its V groups of
 // four columns in registers, so a launch is one round trip to memory, one reduction and one write.  What bounds it is
 // that latency: one warp per row (the kernel above) took 8.2 us per launch at 64 x 3584 and 9.3 us at 1024 x 1024
 // (conditioned); this one takes 5.4 with three partial sums to add and 7.7 with ten, and 7.5 without any and 10.1 with
@@ -270,7 +272,7 @@ constexpr int ROW_THREADS = kNormRowThreads;
 
 template <int V>
 __global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormParams p, int tpr) {
-  constexpr int PB = V >= 8 ? 2 : V >= 4 ? 4 : 8;      // partial sums requested at a time (V * PB groups in flight)
+  constexpr int PB = V >= 6 ? 2 : V >= 4 ? 4 : 8;      // partial sums requested at a time (V * PB groups in flight)
   extern __shared__ uint8_t row_unused_smem[];
   __shared__ float red[2][ROW_THREADS / 32];
   log_smid(p.smid_log);
@@ -400,6 +402,7 @@ cudaError_t norm_set_attributes() {
   if ((e = set_kernel_smem(rmsnorm_row_kernel<1>, kMinSmemBytes)) != cudaSuccess) return e;
   if ((e = set_kernel_smem(rmsnorm_row_kernel<2>, kMinSmemBytes)) != cudaSuccess) return e;
   if ((e = set_kernel_smem(rmsnorm_row_kernel<4>, kMinSmemBytes)) != cudaSuccess) return e;
+  if ((e = set_kernel_smem(rmsnorm_row_kernel<6>, kMinSmemBytes)) != cudaSuccess) return e;
   if ((e = set_kernel_smem(rmsnorm_row_kernel<8>, kMinSmemBytes)) != cudaSuccess) return e;
   if ((e = set_kernel_smem(rmsnorm_bulk_kernel<false>, 512 + BULK_SMEM_BUDGET)) != cudaSuccess) return e;
   return set_kernel_smem(rmsnorm_bulk_kernel<true>, 512 + BULK_SMEM_BUDGET);
@@ -409,12 +412,16 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
   if (p.T <= 0) return cudaSuccess;
   // few rows (one round of them on the whole device), or partial sums to add: many threads per row
   if (p.d <= kNormRowMaxD) {
-    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, tpr = norm_row_threads(p.T, p.d, sms);
+    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, rows = (p.T + sms - 1) / sms;
+    // Where that leaves SMs without rows, more threads per row, no power of two.  Measured on B200, 401 rows of d = 3584 with the
+    // partial sums of four to six splits: 128 threads each on 101 SMs 10.2 us per launch, 160 on 134 7.3.
+    int tpr = norm_row_threads(p.T, p.d, sms);
+    if (rows <= ROW_THREADS / 32) tpr = std::max(tpr, ROW_THREADS / rows / 32 * 32);
     const int rows_per_block = ROW_THREADS / tpr, blocks = (p.T + rows_per_block - 1) / rows_per_block;
     if (p.n_parts > 0 || (p.sm_count > 0 && blocks <= sms)) {
       const int grid = blocks < sm_budget ? blocks : sm_budget, V = (d4 + tpr - 1) / tpr;
-      auto kernel = V <= 1 ? rmsnorm_row_kernel<1> : V <= 2 ? rmsnorm_row_kernel<2> : V <= 4 ? rmsnorm_row_kernel<4> : rmsnorm_row_kernel<8>;
-      return launch_step_kernel(kernel, grid, ROW_THREADS, kMinSmemBytes, stream, launches_ahead(p.overlap), p, tpr);
+      auto kernel = V <= 1 ? rmsnorm_row_kernel<1> : V <= 2 ? rmsnorm_row_kernel<2> : V <= 4 ? rmsnorm_row_kernel<4> : V <= 6 ? rmsnorm_row_kernel<6> : rmsnorm_row_kernel<8>;
+      return launch_step_kernel(kernel, grid, rows_per_block * tpr, kMinSmemBytes, stream, launches_ahead(p.overlap), p, tpr);
     }
   }
   // bulk-staged variant: as many warps as have room for two fp32 rows each (a function of d alone, never of
