@@ -840,9 +840,10 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
               ldg_f32x8(t, cs + e);
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
-                const float a = __uint_as_float(r0[e + u]), b = __uint_as_float(r1[e + u]);
-                r0[e + u] = __float_as_uint(a * t[2 * u] - b * t[2 * u + 1]);
-                r1[e + u] = __float_as_uint(b * t[2 * u] + a * t[2 * u + 1]);
+                float a = __uint_as_float(r0[e + u]), b = __uint_as_float(r1[e + u]);
+                rotate_pair(a, b, t[2 * u], t[2 * u + 1]);
+                r0[e + u] = __float_as_uint(a);
+                r1[e + u] = __float_as_uint(b);
               }
             }
           }

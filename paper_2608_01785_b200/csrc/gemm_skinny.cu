@@ -459,11 +459,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
         }
         if (region != 2) {                                   // q and k heads are rotated
 #pragma unroll
-          for (int e = 0; e < Q; ++e) {
-            const float x0 = v[e], x1 = v[Q + e], c = cs[2 * e], sn = cs[2 * e + 1];
-            v[e] = x0 * c - x1 * sn;
-            v[Q + e] = x1 * c + x0 * sn;
-          }
+          for (int e = 0; e < Q; ++e) rotate_pair(v[e], v[Q + e], cs[2 * e], cs[2 * e + 1]);
         }
         __nv_bfloat16* dst = region == 0 ? p.q_out + size_t(row) * p.q_dim + head * Dh + i0
                                          : cache_row(region == 1 ? p.k_cache : p.v_cache, e_slot,

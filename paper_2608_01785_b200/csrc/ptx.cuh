@@ -310,6 +310,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// Rotation of the pair (a, b) by an angle's cosine and sine.  The fused multiply-adds are written out: from a * c - b * s the
+// compiler fuses either product, as the code around it has it, and every kernel that rotates must round alike.
+__device__ __forceinline__ void rotate_pair(float& a, float& b, float c, float s) {
+  const float lo = fmaf(a, c, -(b * s)), hi = fmaf(a, s, b * c);
+  a = lo;
+  b = hi;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);   // round-to-nearest-even; .x = lo (low 16 bits)
   return *reinterpret_cast<uint32_t*>(&v);
