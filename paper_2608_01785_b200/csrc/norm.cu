@@ -266,14 +266,19 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
 // four columns in registers, so a launch is one round trip to memory, one reduction and one write.  What bounds it is
 // that latency: one warp per row (the kernel above) took 8.2 us per launch at 64 x 3584 and 9.3 us at 1024 x 1024
 // (conditioned); this one takes 5.4 with three partial sums to add and 7.7 with ten, and 7.5 without any and 10.1 with
-// three (single launches under the profiler, each).  Sums: a thread's groups in order, a butterfly per warp, the warps in
-// order -- a function of the shape and the device's SM count, never of the budget.
+// three (single launches under the profiler, each).  Sums of squares: groups i, i + sum_tpr, ... of the row in order, for i =
+// 0 .. sum_tpr - 1, a butterfly per 32 of them, those in order -- a function of the shape and the device's SM count, never of
+// the budget nor of how many threads do the rest: where those are not sum_tpr, the groups' sums pass through shared memory.
 constexpr int ROW_THREADS = kNormRowThreads;
 
-template <int V>
-__global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormParams p, int tpr) {
+// (written out: what the compiler fuses here would follow the code around it)
+__device__ __forceinline__ float square_sum(const float4& a) { return fmaf(a.x, a.x, a.y * a.y) + fmaf(a.z, a.z, a.w * a.w); }
+
+// OTHER: tpr is not sum_tpr.
+template <int V, bool OTHER>
+__global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormParams p, int tpr, int sum_tpr) {
   constexpr int PB = V >= 6 ? 2 : V >= 4 ? 4 : 8;      // partial sums requested at a time (V * PB groups in flight)
-  extern __shared__ uint8_t row_unused_smem[];
+  extern __shared__ float row_squares[];               // [rows of the block][d / 4], at most ROW_THREADS * V
   __shared__ float red[2][ROW_THREADS / 32];
   log_smid(p.smid_log);
   const int rows_per_block = ROW_THREADS / tpr, group = threadIdx.x / tpr, tid = threadIdx.x - group * tpr;
@@ -343,14 +348,24 @@ __global__ void __launch_bounds__(ROW_THREADS, 1) rmsnorm_row_kernel(const NormP
     }
     if (!p.h) continue;
     float ss = 0.f;
+    if (!OTHER) {
 #pragma unroll
-    for (int v = 0; v < V; ++v) ss += (a[v].x * a[v].x + a[v].y * a[v].y) + (a[v].z * a[v].z + a[v].w * a[v].w);
+      for (int v = 0; v < V; ++v) ss += square_sum(a[v]);
+    } else {
+      float* sq = row_squares + group * d4;
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (tid + v * tpr < d4) sq[tid + v * tpr] = square_sum(a[v]);
+      named_barrier_sync(1 + group, tpr);
+      if (tid < sum_tpr)
+        for (int i = tid; i < d4; i += sum_tpr) ss += sq[i];
+    }
     ss = warp_sum(ss);
     if (warps_per_row > 1) {                           // (the row's warps meet in shared memory; two buffers, one barrier)
       if (lane == 0) red[phase][warp] = ss;
       named_barrier_sync(1 + group, tpr);
       ss = 0.f;
-      for (int w = 0; w < warps_per_row; ++w) ss += red[phase][first_warp + w];
+      for (int w = 0; w < (OTHER ? sum_tpr >> 5 : warps_per_row); ++w) ss += red[phase][first_warp + w];
     }
     const float r = rsqrtf(ss / float(p.d) + p.eps);
     uint2* hdst = reinterpret_cast<uint2*>(p.h + size_t(row) * p.d);
@@ -387,6 +402,12 @@ __global__ void __launch_bounds__(256) bf16_to_f16_kernel(const uint4* __restric
 
 }  // namespace
 
+using RowKernel = void (*)(NormParams, int, int);
+template <bool OTHER>
+static RowKernel row_kernel(int V) {
+  return V <= 1 ? rmsnorm_row_kernel<1, OTHER> : V <= 2 ? rmsnorm_row_kernel<2, OTHER> : V <= 4 ? rmsnorm_row_kernel<4, OTHER> : V <= 6 ? rmsnorm_row_kernel<6, OTHER> : rmsnorm_row_kernel<8, OTHER>;
+}
+
 cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_t stream) {
   const size_t n8 = n / 8;
   if (n8 == 0) return cudaSuccess;
@@ -399,11 +420,10 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_
 cudaError_t norm_set_attributes() {
   cudaError_t e = set_kernel_smem(rmsnorm_kernel, NORM_SMEM);
   if (e != cudaSuccess) return e;
-  if ((e = set_kernel_smem(rmsnorm_row_kernel<1>, kMinSmemBytes)) != cudaSuccess) return e;
-  if ((e = set_kernel_smem(rmsnorm_row_kernel<2>, kMinSmemBytes)) != cudaSuccess) return e;
-  if ((e = set_kernel_smem(rmsnorm_row_kernel<4>, kMinSmemBytes)) != cudaSuccess) return e;
-  if ((e = set_kernel_smem(rmsnorm_row_kernel<6>, kMinSmemBytes)) != cudaSuccess) return e;
-  if ((e = set_kernel_smem(rmsnorm_row_kernel<8>, kMinSmemBytes)) != cudaSuccess) return e;
+  for (const int V : {1, 2, 4, 6, 8}) {
+    if ((e = set_kernel_smem(row_kernel<false>(V), kMinSmemBytes)) != cudaSuccess) return e;
+    if ((e = set_kernel_smem(row_kernel<true>(V), kMinSmemBytes)) != cudaSuccess) return e;
+  }
   if ((e = set_kernel_smem(rmsnorm_bulk_kernel<false>, 512 + BULK_SMEM_BUDGET)) != cudaSuccess) return e;
   return set_kernel_smem(rmsnorm_bulk_kernel<true>, 512 + BULK_SMEM_BUDGET);
 }
@@ -413,15 +433,16 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
   // few rows (one round of them on the whole device), or partial sums to add: many threads per row
   if (p.d <= kNormRowMaxD) {
     const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, rows = (p.T + sms - 1) / sms;
-    // Where that leaves SMs without rows, more threads per row, no power of two.  Measured on B200, 401 rows of d = 3584 with the
-    // partial sums of four to six splits: 128 threads each on 101 SMs 10.2 us per launch, 160 on 134 7.3.
-    int tpr = norm_row_threads(p.T, p.d, sms);
-    if (rows <= ROW_THREADS / 32) tpr = std::max(tpr, ROW_THREADS / rows / 32 * 32);
+    // Where that leaves SMs without rows, more threads per row, no power of two (the row's sum keeps its order).  Measured on
+    // B200, 401 rows of d = 3584 with the partial sums of four to six splits: 128 threads each on 101 SMs 10.2 us per launch,
+    // 160 on 134 7.3.
+    const int sum_tpr = norm_row_threads(p.T, p.d, sms);
+    const int tpr = rows <= ROW_THREADS / 32 ? std::max(sum_tpr, ROW_THREADS / rows / 32 * 32) : sum_tpr;
     const int rows_per_block = ROW_THREADS / tpr, blocks = (p.T + rows_per_block - 1) / rows_per_block;
     if (p.n_parts > 0 || (p.sm_count > 0 && blocks <= sms)) {
       const int grid = blocks < sm_budget ? blocks : sm_budget, V = (d4 + tpr - 1) / tpr;
-      auto kernel = V <= 1 ? rmsnorm_row_kernel<1> : V <= 2 ? rmsnorm_row_kernel<2> : V <= 4 ? rmsnorm_row_kernel<4> : V <= 6 ? rmsnorm_row_kernel<6> : rmsnorm_row_kernel<8>;
-      return launch_step_kernel(kernel, grid, rows_per_block * tpr, kMinSmemBytes, stream, launches_ahead(p.overlap), p, tpr);
+      const auto kernel = tpr != sum_tpr ? row_kernel<true>(V) : row_kernel<false>(V);
+      return launch_step_kernel(kernel, grid, rows_per_block * tpr, kMinSmemBytes, stream, launches_ahead(p.overlap), p, tpr, sum_tpr);
     }
   }
   // bulk-staged variant: as many warps as have room for two fp32 rows each (a function of d alone, never of

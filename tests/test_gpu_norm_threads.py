@@ -40,3 +40,22 @@ def test_norm_with_any_multiple_of_32_threads_per_row(name, conditioned):
         assert rel_err(first[0], y_ref) <= 2e-2        # the rule of every parity test (16-bit operands)
     finally:
         st.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,T", [(2568, 297), (3208, 444), (1032, 297)])
+def test_a_rows_sum_does_not_depend_on_the_threads_that_work_on_it(d, T):
+    """T rows leave three to a block, 160 threads each; 592 leave four, 128 each: the keys and values of the first T, made from
+    the norm of the same input, are the same bits (QKV's sums are, whatever the number of rows)."""
+    dims = wl.StageDims(1, d, 8, 2, 64, 512)
+    x = wl.make_x(592, d, 89)
+    pools = []
+    for n in (T, 592):
+        case = make_case(dims, wl.BatchSpec([n], [0]), seed=89, mpps=37, num_pages=40)
+        st = make_stage(case)
+        try:
+            pool = run_step(st, case, st.sm_count, x_t=x[:n])[1].reshape(2, 40, 2, 16, 64)[:, case.block_tables[0][: -(-n // 16)]]
+            pools.append(pool.transpose(0, 1, 3, 2, 4).reshape(2, -1, 2, 64)[:, :T])
+        finally:
+            st.close()
+    assert np.array_equal(pools[0], pools[1])
