@@ -188,12 +188,15 @@ AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_
 // Pages per slice of the decode attention's group mode, 0 = items of single warps instead.  One slice per group where every
 // group has a block of its own and 128-key items would leave warps idle; in a decode-only step more, all with a block of
 // their own on the device, where that is expected to be faster.  Modelled time of a launch: rounds of one slice per SM, each
-// 3.5 us and a step per page of a warp -- 0.45 us, or what eight pages take at an SM's intake and share of the HBM -- and
-// 2.5 us where a group's slices are merged; on the whole device and, with a weight of 0.15 each, on 13/16, 3/4, 13/20,
-// 1/2 and 7/20 of it, since the results depend on the cut and it must not depend on the budget; a cut has to gain a tenth.  Measured on B200: nine sequences of
-// 761 .. 3888 keys at 7B dimensions 23.8 -> 15.7 us per launch (with 256-key items for single warps, whose partial results
-// one warp merges, before); eleven of 216 .. 1463 keys of the talker, cut for the whole device, 9.1 -> 17 us on 52 SMs,
-// which is why the other budgets count.  Never for sequences longer than eight warps' 32 pages.
+// Dh / 16 - 2 us, a step of Dh / 272 us per page of a warp and 1.9 us where a group's slices are merged (fitted to steps of 1 to
+// 32 rows of three stages, 1 to 8 cuts, 28 to 148 SMs); on the whole device and, with a weight of 0.1 each, on 13/16, 3/4,
+// 13/20, 1/2, 7/20 and 1/4 of it, since the results depend on the cut and it must not depend on the budget; a cut has to gain a
+// twenty-fifth.  Measured on B200, us per step on 148 / 74 / 37 SMs, one slice -> the cut taken: a row of 4000 keys at 7B
+// dimensions, 2 layers, 242 -> 220, 289 -> 266, 425 -> 402; five of up to 3142 241 -> 232, 289 -> 279, 424 -> 434; nine of up to
+// 3747 252 -> 241, 301 -> 314, 440 -> 472 (the one step of these where the whole device has the better of it); on a small
+// backbone eight of up to 1931 192 -> 183, 248 -> 235, 357 -> 343, cut four times 180, 232 and 377; 32 of them stay whole (cut in
+// two 258 for 257, 370 for 332, 509 for 481).  Never for sequences longer than eight warps' 32 pages: those are so many keys
+// that items of single warps fill the device.
 int pick_decode_slice(const hs_stage_config_t& c, const hs_batch_t& b, int sm_count, int split) {
   const int sms = std::min(sm_count > 0 ? sm_count : 148, kMaxDecodeSlices);
   int longest = 0, rows = 0;
@@ -209,12 +212,10 @@ int pick_decode_slice(const hs_stage_config_t& c, const hs_batch_t& b, int sm_co
       if (b.q_len[s] == 1) n += c.n_kv_heads * ceil_div(ceil_div(b.ctx_len[s] + 1, kPage), pages);
     if (n > sms) break;
     double us = 0.0;
-    for (const int eightieths : {80, 65, 60, 52, 40, 28}) {
-      const int on = std::max(1, sms * eightieths / 80), rounds = ceil_div(n, on);
-      const double page_us = std::max(0.45, kDecodeWarps * 64.0 * c.head_dim / std::min(70e3, 6.2e6 / std::min(n, on)));
-      us += (eightieths == 80 ? 1.0 : 0.15) * rounds * (3.5 + ceil_div(pages, kDecodeWarps) * page_us + (cuts > 1 ? 2.5 : 0.0));
-    }
-    if (us < best_us * (cuts > 1 ? 0.9 : 1.0)) { best_us = us; best = pages; }
+    const double round_us = c.head_dim / 16.0 - 2.0 + ceil_div(pages, kDecodeWarps) * c.head_dim / 272.0 + (cuts > 1 ? 1.9 : 0.0);
+    for (const int eightieths : {80, 65, 60, 52, 40, 28, 20})
+      us += (eightieths == 80 ? 1.0 : 0.1) * ceil_div(n, std::max(1, sms * eightieths / 80)) * round_us;
+    if (us < best_us * (cuts > 1 ? 0.96 : 1.0)) { best_us = us; best = pages; }
   }
   return best;
 }

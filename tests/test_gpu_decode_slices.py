@@ -61,6 +61,18 @@ def test_short_batches_and_batches_with_prefill_keep_one_slice_per_group():
     assert group and len(items) == 8 * 2 * dims.n_kv_heads
 
 
+# Batches (stage, rows, cached tokens from .. to) that measured faster with one slice per group, over the budgets or on most of
+# them, and such that measured faster cut, at every budget: slices of the longest group, at least .. at most.
+@pytest.mark.parametrize("name,rows,lo,hi,least,most", [
+    ("c2_shared", 32, 256, 2048, 1, 1), ("c2_shared", 16, 256, 2048, 1, 2), ("c2_shared", 8, 256, 2048, 2, 3), ("c3_7b", 14, 512, 4096, 1, 2),
+    ("c4_talker", 4, 128, 1024, 1, 1), ("c4_talker", 11, 128, 1500, 1, 1), ("c3_7b", 1, 4000, 4001, 5, 8), ("c3_7b", 3, 512, 4096, 3, 6),
+    ("c2_shared", 1, 1500, 1501, 4, 8)])
+def test_groups_are_cut_where_that_measured_faster(name, rows, lo, hi, least, most):
+    ctx_len = np.random.default_rng(rows * 1000 + hi).integers(lo, hi, rows).tolist()
+    items, group, _ = _plan(wl.DIMS[name], ctx_len)
+    assert group and least <= max(int(r[7]) & 0xffff for r in items) <= most
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("flags", [0, B.HS_FLAG_BF16_ACTIVATIONS])
 @pytest.mark.parametrize("name", sorted(CASES))
