@@ -157,9 +157,12 @@ PrefillWork prefill_work(const hs_stage_config_t& c, const hs_batch_t& b, int it
 struct AttnSplit { int decode_sms; double us; };
 // Two-tile items: the choice between side by side and in turn stands, but the SMs are then shared out by what the kernels
 // take beyond that -- the prefill kernel 5.6 us an item beside its 1.13 us a block; the decode kernel in group mode
-// (`groups` blocks) whole rounds of its longest group, 0.85 us per page of a warp.  A batch too large for group mode comes with
-// a step that runs into the power cap: 1.3 of the prefill kernel's time at full clocks.  Measured on B200: 2048 new tokens
-// beside 64 decode rows at 7B dimensions, 90 SMs for the decode kernel: 86 us, the prefill kernel 137.
+// (`groups` blocks) whole rounds of its longest group, 0.85 us per page of a warp.  Beside items of single warps that stream
+// more than 150 MB a layer, and so from the HBM for as long as they run, not from the L2, the prefill kernel takes 1.3 of that.
+// Measured on B200, us per step without -> with the 1.3: 302 MB (64 decode rows at 7B dimensions, 4 layers) beside 2048 new
+// tokens on 148 / 120 SMs 3568 -> 3472, 4745 -> 4642, beside 1024 on 112 / 74 2855 -> 2816, 3163 -> 3093; 188 MB (40 rows) beside
+// 394 on 148 / 74 1078 -> 1074, 1620 -> 1609; 123 MB (80 rows of a small backbone) beside 5600 on 112 2485 -> 2519; 12 MB (8 rows,
+// one of them of 4200 keys) beside 600 on 112 626 -> 644.
 AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_bytes, int budget, bool side_by_side, int groups,
                           int longest_pages) {
   auto t_dec = [&](int b) { return decode_kv_bytes > 0 ? 12.0 + double(decode_kv_bytes) / std::min(5.5e6, 42e3 * b) : 0.0; };
@@ -176,9 +179,10 @@ AttnSplit split_attention(const PrefillWork& w, bool singles, int64_t decode_kv_
     if (t < best) { best = t; r = AttnSplit{b, t}; }
   }
   if (r.decode_sms > 0 && !singles) {
+    const double beside = groups == 0 && decode_kv_bytes > int64_t(150) * 1000000 ? 1.3 : 1.0;
     best = 1e30;
     for (int b = 4; b <= budget - 4; ++b) {
-      const double pre = 9.0 + (groups ? 1.0 : 1.3) * std::max(5.6 + 1.13 * w.longest, (5.6 * double(w.items) + 1.13 * double(w.blocks)) / (budget - b));
+      const double pre = 9.0 + beside * std::max(5.6 + 1.13 * w.longest, (5.6 * double(w.items) + 1.13 * double(w.blocks)) / (budget - b));
       const double dec = groups ? 4.0 + ceil_div(groups, b) * (2.0 + 0.85 * ceil_div(longest_pages, kDecodeWarps)) : t_dec(b);
       if (std::max(pre, dec) < best - 1e-9) { best = std::max(pre, dec); r.decode_sms = b; }
     }

@@ -36,3 +36,24 @@ def test_the_decode_kernel_gets_whole_rounds_of_its_blocks(rows, longest):
     for n, (items, sms) in _shares(dims, [700] * 8 + [1] * rows, [0] * 8 + [longest - 3 * i for i in range(rows)], (148, 112, 74)).items():
         assert items == 8 * 22 * dims.n_kv_heads and 4 <= sms <= n - 4
         assert sms == 4 or -(-groups // (sms - 1)) > -(-groups // sms), (n, sms)
+
+
+# Batches on items of single warps (more than 148 groups, or a sequence beyond 4096 keys) -> what the prefill kernel takes
+# beside them, of its time alone.
+@pytest.mark.parametrize("name,q,c,dec,beside", [
+    ("c2_shared", [300] * 2, [0] * 2, [900] * 7 + [4200], 1.0), ("c2_shared", [700] * 8, [0] * 8, [1500] * 80, 1.0),
+    ("c3_7b", [394], [1000], [900] * 6 + [4200], 1.0), ("c3_7b", [1024], [0], [2500] * 64, 1.3), ("c3_7b", [2048], [0], [1999] * 40, 1.3)])
+def test_the_shares_of_a_batch_without_groups_follow_the_bytes_it_streams(name, q, c, dec, beside):
+    """The balance written out: 9 + beside * (5.6 us an item + 1.13 us a block) against 12 us + bytes at 42 GB/s per SM, at most
+    5.5 TB/s; the smallest share of the least larger time."""
+    dims = wl.DIMS[name]
+    tokens = 2 * max(8, (128 // (dims.n_q_heads // dims.n_kv_heads)) & ~7)
+    blocks = [-(-(x + min(t + tokens, n)) // 64) for n, x in zip(q, c) for t in range(0, n, tokens)]
+    n_items, n_blocks, longest = len(blocks) * dims.n_kv_heads, sum(blocks) * dims.n_kv_heads, max(blocks)
+    kv = sum(k + 1 for k in dec) * 4 * dims.kv_dim
+    for n, (items, sms) in _shares(dims, q + [1] * len(dec), c + dec, (148, 112, 96)).items():
+        if items != n_items or sms == 0:                # one-tile items, or the two in turn
+            continue
+        def us(b):
+            return max(9 + beside * max(5.6 + 1.13 * longest, (5.6 * n_items + 1.13 * n_blocks) / (n - b)), 12 + kv / min(5.5e6, 42e3 * b))
+        assert us(sms) <= min(us(b) for b in range(4, n - 3)) + 1e-6, (n, sms)
