@@ -138,6 +138,7 @@ bool encode_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, u
 
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, wgate, wup, wdown;
+  CUtensorMap gu_narrow[kGuNarrow][2];     // gate and up weights in boxes of kGuMinWidth + 16 i rows
 };
 
 struct DeviceGuard {
@@ -395,6 +396,8 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
          encode_2d(&m.wv, w.w_v, kv_dim, d, 128) && encode_2d(&m.wo, w.w_o, d, q_dim, 128) &&
          encode_2d(&m.wgate, w.w_gate, F, d, 128) && encode_2d(&m.wup, w.w_up, F, d, 128) &&
          encode_2d(&m.wdown, w.w_down, d, F, 128);
+    for (int i = 0; i < kGuNarrow && ok; ++i)
+      ok = encode_2d(&m.gu_narrow[i][0], w.w_gate, F, d, kGuMinWidth + 16 * i) && encode_2d(&m.gu_narrow[i][1], w.w_up, F, d, kGuMinWidth + 16 * i);
   }
   if (!ok)
     return fail("hs_stage_create: fp16 weight copy or tensor-map encoding failed (cuTensorMapEncodeTiled unavailable, or "
@@ -855,7 +858,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     } else {
       if (!pair_gu && gu_width != 128) {
         gu.gu_width = gu_width;
-        if (!encode_2d(&gu.tm_b[0], wo.w_gate, F, d, gu_width) || !encode_2d(&gu.tm_b[1], wo.w_up, F, d, gu_width)) return HS_ERR_CUDA;
+        for (int i = 0; i < 2; ++i) gu.tm_b[i] = m.gu_narrow[(gu_width - kGuMinWidth) / 16][i];
       }
       LaunchTimer t(s, 6, stream); where = "gate/up gemm"; e = launch_gemm(gu, sm_budget, stream);
     }

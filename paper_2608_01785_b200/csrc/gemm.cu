@@ -32,6 +32,8 @@
 namespace hs {
 namespace {
 
+static_assert(kGuMinWidth + 16 * kGuNarrow == 128, "a step of 16 columns from one width to the next");
+
 constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;            // 16 KB
 constexpr int BH_BYTES = 128 * BK * 2;          // one 128-row half of the B tile, 16 KB
@@ -1081,7 +1083,7 @@ int gemm_pick_gu_width(int M, int N, int sms) {
   const double a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2;
   int best = 128;
   double best_us = 1e30;
-  for (int w = 128; w >= 48; w -= 16) {
+  for (int w = 128; w >= kGuMinWidth; w -= 16) {
     const int tiles = (N + w - 1) / w, rounds = (tiles + sms - 1) / sms;
     const double b_bytes = 2.0 * w * BK * 2;
     auto round_us = [&](int n) {

@@ -97,7 +97,8 @@ cudaError_t gemm_set_attributes();
 // Tile width for a Resid-mode GEMM of this shape on a device with sm_count SMs (budget independent).
 int gemm_pick_bn(int M, int N, int sm_count);
 int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count);
-// Activation columns per tile of a GateUp GEMM on single blocks with `sms` SMs: a multiple of 16, 48 .. 128.
+// Activation columns per tile of a GateUp GEMM on single blocks with `sms` SMs: 128, or kGuMinWidth + 16 i, i < kGuNarrow.
+constexpr int kGuMinWidth = 48, kGuNarrow = 5;
 int gemm_pick_gu_width(int M, int N, int sms);
 // Where split i (0 .. ks) of a tile's k_blocks begins.  The splits add their sums one after the other, a link of that
 // chain costing about as long as kSplitSkew K blocks take to stream; so each split is that much longer than the one
