@@ -155,6 +155,22 @@ __device__ __forceinline__ float row_norm_factor(const float (&v)[kSsPre], const
   return rsqrtf(sum / float(width) + eps);
 }
 
+// Shared memory of an instantiation: the warps' rings, the partial tiles of the reduction -- of their own where all fits, else
+// in the rings -- and a tail: r of a folded norm's 16 rows and its last-unit flag.
+template <int MT, int P, int DB>
+struct SkinnySmem {
+  static constexpr int STAGE_BYTES = (2 * P + 2 * MT) * 512;        // per warp and K step: 2 P weight tiles, 2 MT row groups
+  static constexpr int RING_BYTES = DB * STAGE_BYTES;               // per warp
+  static constexpr int PART_STRIDE = 16 * P + 8;                    // floats between rows of a warp's partial tile
+  static constexpr int PART_FLOATS = MT * 16 * PART_STRIDE;         // per warp
+  static constexpr int TAIL_BYTES = 16 * 4 + 16, MAX_BYTES = 227 * 1024;
+  static constexpr bool ALIAS = SK_WARPS * (RING_BYTES + PART_FLOATS * 4) + TAIL_BYTES > MAX_BYTES;
+  static constexpr int TAIL_AT = SK_WARPS * (RING_BYTES + (ALIAS ? 0 : PART_FLOATS * 4));
+  static constexpr int BYTES = TAIL_AT + TAIL_BYTES < kMinSmemBytes ? kMinSmemBytes : TAIL_AT + TAIL_BYTES;
+  static_assert(!ALIAS || PART_FLOATS * 4 <= RING_BYTES, "a warp's partial tile must fit its own ring");
+  static_assert(BYTES <= MAX_BYTES, "rings and partial tiles must fit one SM");
+};
+
 // What a launch takes once the kernel in front is done, in timestamps at the talker's dimensions (K = 1024): 1.1 us until the
 // activations are there, 0.4 in the K loop, 0.45 until the last warp's partial tile is, 0.6 in the epilogue.  So with a K range
 // that fits the rings there is one wait and no refills, the chains of MMAs are halved, an epilogue thread has four columns
@@ -170,13 +186,9 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
   const int block = int(blockIdx.x), n_blocks = int(gridDim.x);
   static_assert(!FOLD || MT == 1, "the folded norm's rows are those of one row tile");
   constexpr int NT = 2 * P;                                 // n8 tiles of a unit
-  constexpr int PART_STRIDE = 8 * NT + 8;                   // floats between rows of a warp's partial tile
-  constexpr int STAGE_BYTES = (NT + 2 * MT) * 512;          // per warp and K step: the weight tiles, 2 MT row groups
-  constexpr int RING_BYTES = DB * STAGE_BYTES;              // per warp
-  constexpr int PART_FLOATS = MT * 16 * PART_STRIDE;        // per warp
-  // The partial tiles of the reduction get their own shared memory when it fits; else they reuse the rings.
-  constexpr bool ALIAS = SK_WARPS * (RING_BYTES + PART_FLOATS * 4) > 227 * 1024;
-  static_assert(!ALIAS || PART_FLOATS * 4 <= RING_BYTES, "a warp's partial tile must fit its own ring");
+  using Smem = SkinnySmem<MT, P, DB>;
+  constexpr int PART_STRIDE = Smem::PART_STRIDE, STAGE_BYTES = Smem::STAGE_BYTES, RING_BYTES = Smem::RING_BYTES, PART_FLOATS = Smem::PART_FLOATS;
+  constexpr bool ALIAS = Smem::ALIAS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const uint8_t* ring_at = sk_smem + warp * RING_BYTES + lane * 16;
   const uint32_t ring = smem_u32(ring_at);
@@ -271,7 +283,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
   // activations of the first unit
   float rs_in = 1.f;
   const bool sums_in = FOLD && p.in_row_ss != nullptr;
-  float* row_r = part_all + SK_WARPS * PART_PITCH;          // FOLD: r of 16 rows behind the partial tiles, and one word
+  float* row_r = reinterpret_cast<float*>(sk_smem + Smem::TAIL_AT);         // FOLD: r of 16 rows, and one word
   int* last_unit = reinterpret_cast<int*>(row_r + 16);
   float ss_pre[kSsPre];
   if (unit < units) first_a();
@@ -494,20 +506,15 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
   }
 }
 
-template <int MT, int P, int DB>
-constexpr int skinny_smem() {
-  constexpr int rings = SK_WARPS * DB * 2 * (P + MT) * 512, both = rings + SK_WARPS * MT * 16 * (16 * P + 8) * 4;
-  constexpr int bytes = (both > 227 * 1024 - 128 ? rings : both) + 16 * 4 + 16;      // + r of the folded norm's rows, its last-unit flag
-  return bytes < kMinSmemBytes ? kMinSmemBytes : bytes;
-}
-// Ring depth: what fits one SM, at least 96 KB of weights in flight.
+// Ring depth: what fits one SM beside the activations.  Weights in the rings of a block: 96 .. 192 KB with one row tile, 64
+// (P = 1) and 96 KB with two, 32 P KB with four; of a K range that does not fit them, one step of each warp less is in flight.
 constexpr int ring_depth(int MT, int P) {
   return MT == 1 ? (P == 1 ? 12 : P == 2 ? 8 : P == 3 ? 6 : P <= 6 ? 4 : 3) : MT == 2 ? (P == 1 ? 8 : P == 2 ? 6 : P == 3 ? 4 : 3) : 4;
 }
 
 template <int MT, int P>
 cudaError_t launch_one(const SkinnyParams& p, int grid, cudaStream_t stream) {
-  constexpr int DB = ring_depth(MT, P), smem = skinny_smem<MT, P, DB>();
+  constexpr int DB = ring_depth(MT, P), smem = SkinnySmem<MT, P, DB>::BYTES;
   const bool early = p.overlap != 0;
   if constexpr (MT == 1) {
     if (p.norm_gain != nullptr || p.in_row_rs != nullptr || p.in_row_ss != nullptr) {
@@ -520,8 +527,7 @@ cudaError_t launch_one(const SkinnyParams& p, int grid, cudaStream_t stream) {
 }
 template <int MT, int P>
 cudaError_t set_one() {
-  constexpr int DB = ring_depth(MT, P), smem = skinny_smem<MT, P, DB>();
-  static_assert(smem <= 227 * 1024, "rings and partial tiles must fit one SM");
+  constexpr int DB = ring_depth(MT, P), smem = SkinnySmem<MT, P, DB>::BYTES;
   cudaError_t e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, true, false>, smem);
   if (e == cudaSuccess) e = set_kernel_smem(gemm_skinny_kernel<MT, P, DB, false, false>, smem);
   if constexpr (MT == 1) {
