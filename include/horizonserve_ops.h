@@ -175,6 +175,13 @@ hs_status_t hs_stage_plan_shares(hs_stage_t *stage, const hs_batch_t *batch, int
 int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K);
 
 /*
+ * Host-only: activation columns per tile (48 .. 128, a multiple of 16) of the gate/up GEMM of M rows, d_ffn N and contraction
+ * length K when it runs on the tensor-memory kernel's single blocks on sm_budget SMs.  The results do not depend on it.
+ * Returns -1 for M, K or sm_budget < 1, or N < 64.
+ */
+int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
+
+/*
  * Host-only: the K block (of 64) at which split i (0 .. ks; i = ks gives k_blocks) of a small step's residual GEMM
  * begins when its k_blocks are cut into ks splits.  Each split is ten K blocks longer than the one before it (the
  * splits add their sums one after the other, and a link of that chain takes about as long as ten K blocks take to

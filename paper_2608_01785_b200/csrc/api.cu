@@ -520,6 +520,10 @@ int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K) {
   return plan_parts(M, N, K, kSms, part_rows_cap(M, N), gemm_skinny_wins(M, K, N, kGemmResid, 0, kSms)).ks;
 }
 
+int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
+  return M < 1 || N < 64 || K < 1 || sm_budget < 1 ? -1 : gemm_pick_gu_width(M, N, K, sm_budget);
+}
+
 int32_t hs_op_gemm_split_begin(int32_t k_blocks, int32_t ks, int32_t i) {
   if (k_blocks < 1 || ks < 1 || i < 0 || i > ks) return -1;
   return gemm_split_begin(k_blocks, ks, i);
@@ -571,7 +575,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   auto pair_for = [&](int n_cols, int single_bn) { return on_pairs(T, n_cols, single_bn, s->sm_count); };
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
-  const int gu_width = gemm_pick_gu_width(T, F, sm_budget);      // (the results do not depend on it)
+  const int gu_width = gemm_pick_gu_width(T, F, d, sm_budget);      // (the results do not depend on it)
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
   // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next

@@ -1075,22 +1075,24 @@ int gemm_pick_stream_k(int M, int N, int K, int sm_count) {
 
 // Activation columns of a GateUp tile on single blocks, from the SMs the launch gets: an output element's sum is the same
 // whatever the tile's width, so this choice may look at the budget.  Tiles of 128 columns at 7B dimensions, 148 of them, are
-// one round on the whole device but two on 96 to 147 SMs.  Time per K block by the rates of resid_launch_us, 0.02 us of it
-// for a further round.  Measured on B200, 29 rows on 96 SMs: 112 columns 50.7 us per launch, 128 columns 53.8; step of 4
-// layers 669 -> 657 us.
-int gemm_pick_gu_width(int M, int N, int sms) {
+// one round on the whole device but two on 96 to 147 SMs.  Time per K block: the larger of issue, shared memory, an SM's intake
+// -- 80 KB/us of the weights and 4.5 KB more, which is what narrow boxes pay -- and its share of the HBM; 1.1 us per further
+// round.  Measured on B200, us per launch at 7B dimensions, 128 columns -> the width taken: 29 rows on 96 SMs 53.8 -> 50.7 (112
+// columns); steps of 2 layers, 5 rows on 64 SMs 297 -> 283 (112), on 112 245 -> 233 (96), on 120 249 -> 232 (80), on 28 475 (128; 80
+// columns, which the bytes alone would have, 509).
+int gemm_pick_gu_width(int M, int N, int K, int sms) {
   if (M > BM) return 128;
-  const double a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2;
+  const double a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2, k_blocks = (K + BK - 1) / BK;
   int best = 128;
   double best_us = 1e30;
   for (int w = 128; w >= kGuMinWidth; w -= 16) {
     const int tiles = (N + w - 1) / w, rounds = (tiles + sms - 1) / sms;
     const double b_bytes = 2.0 * w * BK * 2;
-    auto round_us = [&](int n) {
-      return std::max(std::max(0.27 * (0.4 + 0.6 * w / 128), (a_bytes + b_bytes) / 120e3), std::max(b_bytes / 68e3, n * b_bytes / 6.2e6));
+    auto k_block_us = [&](int n) {
+      return std::max(std::max(0.27 * (0.4 + 0.6 * w / 128), (a_bytes + b_bytes) / 120e3), std::max((b_bytes + 4608) / 80e3, n * b_bytes / 6.2e6));
     };
     const int rest = tiles - (rounds - 1) * sms;
-    const double us = (rounds - 1) * (round_us(sms) + 0.02) + round_us(rest);     // per K block; 1.2 us per further round
+    const double us = k_blocks * ((rounds - 1) * k_block_us(sms) + k_block_us(rest)) + (rounds - 1) * 1.1;
     if (us < best_us * 0.97) { best_us = us; best = w; }
   }
   return best;

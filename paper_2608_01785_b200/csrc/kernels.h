@@ -99,7 +99,7 @@ int gemm_pick_bn(int M, int N, int sm_count);
 int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count);
 // Activation columns per tile of a GateUp GEMM on single blocks with `sms` SMs: 128, or kGuMinWidth + 16 i, i < kGuNarrow.
 constexpr int kGuMinWidth = 48, kGuNarrow = 5;
-int gemm_pick_gu_width(int M, int N, int sms);
+int gemm_pick_gu_width(int M, int N, int K, int sms);
 // Where split i (0 .. ks) of a tile's k_blocks begins.  The splits add their sums one after the other, a link of that
 // chain costing about as long as kSplitSkew K blocks take to stream; so each split is that much longer than the one
 // before it and finishes just when its turn comes, instead of all finishing together and then queueing.  Equal

@@ -147,6 +147,27 @@ def test_partial_sums_at_the_edges_of_their_range():
     assert B.hs_op_gemm_part_splits(8, 1024, 40) == -1
 
 
+# Gate/up projections (rows, width, contraction length, SMs) -> the tile width whose step measured fastest, or within a
+# hundredth of it.
+@pytest.mark.parametrize("M,N,K,sms,widths", [
+    (5, 18944, 3584, 24, (112, 128)), (24, 18944, 3584, 28, (112, 128)), (5, 18944, 3584, 64, (112,)), (29, 18944, 3584, 96, (96, 112)),
+    (24, 18944, 3584, 120, (80,)), (100, 18944, 3584, 130, (80,)), (5, 18944, 3584, 148, (128,)), (24, 5632, 2048, 148, (48,))])
+def test_width_of_the_gate_up_tiles(M, N, K, sms, widths):
+    assert B.hs_op_gate_up_width(M, N, K, sms) in widths
+
+
+def test_width_of_the_gate_up_tiles_at_the_edges():
+    # a further round costs what it does whatever the length of K: the shorter K, the fewer rounds are worth having
+    assert B.hs_op_gate_up_width(32, 2816, 1024, 20) > 48
+    rounds = [-(-2816 // B.hs_op_gate_up_width(32, 2816, k, 20)) for k in (64, 256, 1024, 4096)]
+    assert rounds == sorted(rounds)
+    assert B.hs_op_gate_up_width(129, 18944, 3584, 96) == 128
+    assert all(B.hs_op_gate_up_width(m, n, k, s) == -1 for m, n, k, s in ((0, 1024, 64, 1), (1, 56, 64, 1), (1, 1024, 0, 1), (1, 1024, 64, 0)))
+    for sms in range(1, 149):
+        w = B.hs_op_gate_up_width(64, 18944, 3584, sms)
+        assert w % 16 == 0 and 48 <= w <= 128
+
+
 # dims, prefill chunks, cached tokens of the chunks, decode contexts -> items at budget, from the forms that measured faster
 SHARES = {
     "denoise_2": ("c6_dit", [256] * 2, [0] * 2, [], {148: 64, 74: 64, 52: 32, 37: 32}),
