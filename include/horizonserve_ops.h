@@ -182,6 +182,12 @@ int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K);
 int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
 
 /*
+ * Host-only: weight rows per block of the weight-streaming kernel for a residual GEMM of M rows, width N and contraction length
+ * K on sm_budget SMs.  The results do not depend on it.  Returns -1 for a shape that kernel does not take or sm_budget < 1.
+ */
+int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
+
+/*
  * Host-only: the K block (of 64) at which split i (0 .. ks; i = ks gives k_blocks) of a small step's residual GEMM
  * begins when its k_blocks are cut into ks splits.  Each split is ten K blocks longer than the one before it (the
  * splits add their sums one after the other, and a link of that chain takes about as long as ten K blocks take to

@@ -30,7 +30,8 @@ EXPORTS = ("hs_status_str", "hs_kv_pool_bytes", "hs_workspace_bytes", "hs_stage_
            "hs_head_destroy", "hs_op_embed", "hs_temporal_create", "hs_temporal_step", "hs_temporal_destroy",
            "hs_stage_set_qkv_bias", "hs_stage_set_modulation", "hs_stage_saturation_count", "hs_op_wait_probe",
            "hs_op_decode_attention_noalloc_status", "hs_stage_plan_attention", "hs_op_gemm_split_begin",
-           "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width")
+           "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width",
+           "hs_op_weight_streaming_rows")
 PROFILE_CLASSES = ("rmsnorm", "gemm_qkv", "attn_prefill", "attn_decode", "attn_combine", "gemm_out", "gemm_gateup",
                    "gemm_down")
 
@@ -119,6 +120,8 @@ def lib() -> C.CDLL:
         l.hs_op_gemm_part_splits.restype = C.c_int32
         l.hs_op_gate_up_width.argtypes = [C.c_int32] * 4
         l.hs_op_gate_up_width.restype = C.c_int32
+        l.hs_op_weight_streaming_rows.argtypes = [C.c_int32] * 4
+        l.hs_op_weight_streaming_rows.restype = C.c_int32
         l.hs_stage_plan_shares.argtypes = [C.c_void_p, C.POINTER(hs_batch_t), C.c_int32, C.c_void_p, C.c_void_p]
         l.hs_stage_plan_shares.restype = C.c_int
         l.hs_stage_step.argtypes = [C.c_void_p, C.POINTER(hs_batch_t), C.c_int32, C.c_void_p]
@@ -278,6 +281,10 @@ def hs_op_gemm_part_splits(M: int, N: int, K: int) -> int:
 
 def hs_op_gate_up_width(M: int, N: int, K: int, sm_budget: int) -> int:
     return int(lib().hs_op_gate_up_width(M, N, K, sm_budget))
+
+
+def hs_op_weight_streaming_rows(M: int, N: int, K: int, sm_budget: int) -> int:
+    return int(lib().hs_op_weight_streaming_rows(M, N, K, sm_budget))
 
 
 def hs_op_gemm_split_begin(k_blocks: int, ks: int, i: int) -> int:

@@ -524,6 +524,10 @@ int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget) 
   return M < 1 || N < 64 || K < 1 || sm_budget < 1 ? -1 : gemm_pick_gu_width(M, N, K, sm_budget);
 }
 
+int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
+  return sm_budget < 1 || !gemm_skinny_supports(M, K, N, kGemmResid, 0) ? -1 : gemm_skinny_rows(M, K, N, kGemmResid, 0, sm_budget);
+}
+
 int32_t hs_op_gemm_split_begin(int32_t k_blocks, int32_t ks, int32_t i) {
   if (k_blocks < 1 || ks < 1 || i < 0 || i > ks) return -1;
   return gemm_split_begin(k_blocks, ks, i);

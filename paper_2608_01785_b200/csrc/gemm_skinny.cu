@@ -537,12 +537,13 @@ cudaError_t set_one() {
   return e;
 }
 
-// Width of a launch's units.  A block takes in about 70 KB/us, weights and activations alike, with about 1.5 us per unit
-// beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
+// Width of a launch's units.  A block takes in about 70 KB/us, weights and activations alike -- 56 with units of 16 weight
+// rows -- with about 1.5 us per unit beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
 // budget.  Units wider than 64 weight rows, for a gate/up projection on few SMs, keep eight columns per epilogue thread and
 // their partial tiles in the rings.  Measured on B200 against 32 rows throughout: talker step of 16 rows at 112 / 96 / 28 SMs
 // 352 -> 333, 351 -> 333, 683 -> 632 us, of 11 rows at 52 (51 units of 112 rows instead of 176 of 32) 395 -> 382; at 7B
-// dimensions 9 rows, 4 layers, at 96 / 74 / 37 SMs 606 -> 546, 594 -> 562, 963 -> 897.
+// dimensions 9 rows, 4 layers, at 96 / 74 / 37 SMs 606 -> 546, 594 -> 562, 963 -> 897; one row, 2 layers, at 52 SMs 344 -> 331 (two
+// rounds of 48 rows; five rounds of 16, which 70 KB/us would have, 370).
 int pick_width(int T, int K, int N, int mode, int head_dim, int sms) {
   const int max_p = T <= 16 && mode == kGemmGateUp ? 7 : T <= 32 ? 4 : 2;
   int best = 2;
@@ -550,7 +551,7 @@ int pick_width(int T, int K, int N, int mode, int head_dim, int sms) {
   for (int P = 1; P <= max_p; ++P) {
     if (mode == kGemmQkv && (head_dim >> 4) % P != 0) continue;
     const int units = skinny_units(N, mode, P), rounds = (units + sms - 1) / sms;
-    const double us = rounds * (1.5 + double(16 * P + (T <= 32 ? T : 64)) * K * 2 / 70e3);
+    const double us = rounds * (1.5 + double(16 * P + (T <= 32 ? T : 64)) * K * 2 / (P == 1 ? 56e3 : 70e3));
     if (us < best_us - 1e-9) { best_us = us; best = P; }
   }
   return best;
@@ -604,6 +605,8 @@ cudaError_t gemm_skinny_set_attributes() {
     if (e == cudaSuccess) e = set();
   return e;
 }
+
+int gemm_skinny_rows(int T, int K, int N, int mode, int head_dim, int sms) { return 16 * pick_width(T, K, N, mode, head_dim, sms); }
 
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream) {
   if (p.T <= 0) return cudaSuccess;

@@ -182,6 +182,8 @@ struct SkinnyParams {
 bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim);
 // True when it is also expected to be faster than the tiled kernel for this shape (budget independent).
 bool gemm_skinny_wins(int T, int K, int N, int mode, int head_dim, int sm_count);
+// Weight rows of a block's unit on `sms` SMs (the results do not depend on it).
+int gemm_skinny_rows(int T, int K, int N, int mode, int head_dim, int sms);
 cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_t stream);
 cudaError_t gemm_skinny_set_attributes();
 constexpr int kGemmTurnWords = 8192;   // capacity of the whose-turn array: splits are used only when tiles * 8 fits

@@ -156,6 +156,16 @@ def test_width_of_the_gate_up_tiles(M, N, K, sms, widths):
     assert B.hs_op_gate_up_width(M, N, K, sms) in widths
 
 
+# Residual projections (rows, width, contraction length, SMs) -> weight rows per block whose step measured fastest: units of 16
+# rows where they are one round or all that occupies the device, not five rounds of them.
+@pytest.mark.parametrize("M,N,K,sms,rows", [
+    (1, 3584, 18944, 52, (48,)), (2, 3584, 18944, 52, (48,)), (5, 3584, 18944, 52, (48,)), (1, 3584, 18944, 148, (32,)),
+    (1, 1024, 2816, 148, (16,)), (16, 1024, 1024, 96, (16,)), (8, 1024, 2816, 52, (32,))])
+def test_weight_rows_of_a_weight_streaming_block(M, N, K, sms, rows):
+    assert B.hs_op_weight_streaming_rows(M, N, K, sms) in rows
+    assert B.hs_op_weight_streaming_rows(65, N, K, sms) == B.hs_op_weight_streaming_rows(M, N + 8, K, sms) == -1
+
+
 def test_width_of_the_gate_up_tiles_at_the_edges():
     # a further round costs what it does whatever the length of K: the shorter K, the fewer rounds are worth having
     assert B.hs_op_gate_up_width(32, 2816, 1024, 20) > 48
