@@ -168,7 +168,9 @@ constexpr int dc_smem_bytes() {
 
 // The body of the decode kernel.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS *
 // DC_STAGES mbarriers followed by two ints (the abort flag; a flag of the block's) in shared memory outside that area.
-template <int DH>
+// SLICED: group mode with groups of several slices (the merge of those is no part of the other instantiation: it was 2 us of the
+// talker step of 16 rows, twelve launches, that has none).
+template <int DH, bool SLICED>
 __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* smem, uint64_t* full_all) {
   using G_ = Geom<DH>;
   constexpr int SLOT_BYTES = 2 * G_::PAGE_BYTES;    // K page then V page
@@ -424,14 +426,14 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
             o0 += f * v.x;
             o1 += f * v.y;
           }
-          if (splits == 1) {
+          if (!SLICED || splits == 1) {
             store(g, col, o0, o1, ll);
           } else {
             __stcg(reinterpret_cast<float2*>(p.part_o + (size_t(part) * 16 + g) * DH + col), make_float2(o0, o1));
             if (col == 0) __stcg(reinterpret_cast<float2*>(p.part_ml) + size_t(part) * 16 + g, make_float2(mm, ll));
           }
         }
-        if (splits > 1) {
+        if (SLICED && splits > 1) {
           // the block that delivers the group's last slice merges all of them, in slice order whoever it is
           __threadfence();
           __syncthreads();

@@ -69,6 +69,7 @@ struct StepPlan {
   int n_tokens = 0, n_seqs = 0;
   int n_prefill_items = 0, n_decode_items = 0, n_decode_rows = 0;
   int decode_group = 0;           // 1: decode items come in eights, a block's eight warps sharing a slice of a (sequence, KV head)'s pages (see plan_step)
+  int decode_sliced = 0;          // 1: group mode, and a group has more than one slice
   int decode_sms = 0;             // SMs of the budget for the decode kernel beside the prefill kernel; 0: one after the other
   int meta_words = 0;             // int32 words of the metadata block in use: the work lists are at its end
   int64_t decode_kv_bytes = 0;    // K and V bytes the decode items read, one layer

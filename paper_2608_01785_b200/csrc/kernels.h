@@ -289,6 +289,7 @@ struct AttnParams {
   int decode_group;                // 1: the items come in eights: a block's eight warps share a slice of a (sequence, KV
                                    //    head)'s pages and meet in shared memory (small batches); first item and splits of
                                    //    the record then count slices
+  int decode_sliced;               // 1: group mode, and a group has more than one slice
   const int32_t* decode_rows;      // int4 per decode sequence
   int n_decode_rows;
   float* part_o;                   // [max_decode_items][16][Dh] unnormalised partial outputs

@@ -322,6 +322,7 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
           }
         }
       n_dec_items += c.n_kv_heads * slices * kDecodeWarps;
+      if (slices > 1) p.decode_sliced = 1;
       ++n_dec_rows;
     } else if (n == 1) {
       // decode: keys 0..ctx cut into whole runs of `split` keys and the rest into pieces of kDecodeTail keys; the items
