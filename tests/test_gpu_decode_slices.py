@@ -19,8 +19,8 @@ CASES = {
 }
 
 
-def _plan(dims, ctx_len):
-    batch = wl.BatchSpec([1] * len(ctx_len), list(ctx_len))
+def _plan(dims, ctx_len, q_len=None):
+    batch = wl.BatchSpec([1] * len(ctx_len) if q_len is None else list(q_len), list(ctx_len))
     mpps = max(-(-t // 16) for t in batch.total_len())
     cfg = B.make_config(dims, wl.pages_needed(batch) + 4, batch.n_tokens, batch.n_seqs, mpps, max(batch.total_len()), device=-1)
     stage = B.hs_stage_create(cfg, None, 0, 0)
@@ -59,6 +59,21 @@ def test_short_batches_and_batches_with_prefill_keep_one_slice_per_group():
     dims = wl.DIMS["c4_talker"]
     items, group, _ = _plan(dims, [100, 50])
     assert group and len(items) == 8 * 2 * dims.n_kv_heads
+    for name in ("one_long", "nine"):                  # cut alone (above), whole beside a chunk
+        dims, ctx_len = CASES[name]
+        items, group, chunk = _plan(dims, [0] + ctx_len, [40] + [1] * len(ctx_len))
+        assert group and len(chunk) and len(items) == 8 * len(ctx_len) * dims.n_kv_heads
+        assert all(int(r[7]) == 1 for r in items)
+
+
+def test_sequences_beyond_4096_keys_are_items_of_single_warps():
+    """A warp keeps a page id per lane, so eight warps hold 256 pages: the longest slice of a group that is not cut."""
+    dims = wl.DIMS["c3_7b"]
+    for ctx, want in ((4094, True), (4095, True), (4096, False), (4097, False)):
+        items, group, _ = _plan(dims, [ctx, 700])
+        keys = sum(int(r[3]) - int(r[2]) for r in items if int(r[4]) == 0)
+        assert group == want and keys == dims.n_kv_heads * (ctx + 1)
+        assert all(int(r[3]) - int(r[2]) <= 512 for r in items)
 
 
 # Batches (stage, rows, cached tokens from .. to) that measured faster with one slice per group, over the budgets or on most of
@@ -91,5 +106,29 @@ def test_slices_match_the_oracle_at_every_budget(name, flags):
                 first = out if first is None else first
                 assert np.array_equal(out[0], first[0]) and np.array_equal(out[1], first[1]), budget
         assert rel_err(first[0], y_ref) <= 2e-2        # the rule of every parity test (16-bit operands)
+    finally:
+        st.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("scale", [1, -1])
+def test_saturated_outputs_of_merged_slices_are_counted_once(scale):
+    """Values beyond fp16's range in the cache: every element of a long sequence's attention output is clamped and counted by the
+    block that merges the group's slices, none of a sequence whose values are ordinary."""
+    dims, ctx_len = wl.StageDims(1, 256, 8, 2, 64, 512), [3001, 2500, 40]
+    items, group, _ = _plan(dims, ctx_len)
+    assert group and max(int(r[7]) & 0xffff for r in items) > 1
+    case = make_case(dims, wl.BatchSpec([1] * 3, ctx_len), seed=67, kv_fill=True)
+    pool = wl.bits_to_bf16_tensor(case.kv_pool).view(wl.kv_pool_shape(dims, case.cfg.num_pages))
+    for s in (0, 1):
+        for page in case.block_tables[s][: -(-(ctx_len[s] + 1) // 16)]:
+            pool[0, 1, int(page)] = scale * 1.0e5
+    st = make_stage(case, weights=[dict(lw, w_o=lw["w_o"] * 0) for lw in case.weights_t])      # (nothing behind it leaves the range)
+    try:
+        for i, budget in enumerate((148, 60, 1)):
+            st.kv_pool.copy_(pool.reshape(-1))
+            run_step(st, case, budget, expect_saturation=True)
+            assert st.saturation_count() == (i + 1) * 2 * dims.q_dim, budget
+            assert bool((st.debug_tensor("o")[:2].float() == scale * 65504).all())
     finally:
         st.close()

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from oracle.oracle import Oracle
+from paper_2608_01785_b200 import binding as B
 from paper_2608_01785_b200 import workloads as wl
 from paper_2608_01785_b200.stage import Stage
 from tests.gpu_helpers import make_stage, run_step
@@ -21,12 +22,14 @@ CASES = {
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, B.HS_FLAG_BF16_ACTIVATIONS])
 @pytest.mark.parametrize("name", sorted(CASES))
-def test_tile_width_does_not_reach_the_output(name):
+def test_tile_width_does_not_reach_the_output(name, flags):
     dims, q_len, ctx_len = CASES[name]
+    assert len({B.hs_op_gate_up_width(sum(q_len), dims.d_ffn, dims.d_model, n) for n in BUDGETS}) > (2 if dims.d_ffn > 128 else 0)
     case = make_case(dims, wl.BatchSpec(q_len, ctx_len), seed=71, kv_fill=True)
     y_ref = Oracle("f32").step(case.cfg, case.weights, case.kv_pool.copy(), q_len, ctx_len, case.block_tables, case.x)
-    st = make_stage(case)
+    st = make_stage(case, flags=flags)
     try:
         first = None
         for budget in BUDGETS:
@@ -35,6 +38,31 @@ def test_tile_width_does_not_reach_the_output(name):
             first = out if first is None else first
             assert np.array_equal(out[0], first[0]) and np.array_equal(out[1], first[1]), budget
         assert rel_err(first[0], y_ref) <= 2e-2        # the rule of every parity test (16-bit operands)
+    finally:
+        st.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["100_rows", "128_rows_ragged"])
+def test_saturated_values_are_counted_once_at_every_width(name):
+    """Gate and up weights scaled such that some of the products leave fp16's range: a tile's last chunk of 32 columns has columns
+    of the up projection behind the tile's own, which are as large and must not count."""
+    dims, q_len, ctx_len = CASES[name]
+    case = make_case(dims, wl.BatchSpec(q_len, ctx_len), seed=73, kv_fill=True)
+    weights = [dict(lw, w_gate=lw["w_gate"] * 512, w_up=lw["w_up"] * 512) for lw in case.weights_t]
+    st = make_stage(case, weights=weights)
+    try:
+        first, counts, before = None, [], 0
+        for budget in BUDGETS:
+            st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
+            out = run_step(st, case, budget, expect_saturation=True)
+            first = out if first is None else first
+            assert np.array_equal(out[0], first[0]), budget
+            counts.append(st.saturation_count() - before)
+            before += counts[-1]
+        assert len(set(counts)) == 1 and counts[0] > 0
+        if dims.n_layers == 1:                         # (the count is of all layers; 65504 is also what some smaller values round to)
+            assert counts[0] <= int((st.debug_tensor("act")[: sum(q_len)].float().abs() == 65504).sum())
     finally:
         st.close()
 
