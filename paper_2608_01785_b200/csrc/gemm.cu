@@ -1044,7 +1044,8 @@ ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows, 
   const int bn = gemm_pick_bn(M, N, sm_count), ks = gemm_pick_ksplit(M, N, K, bn, sm_count);
   const int longest = k_blocks - gemm_split_begin(k_blocks, ks, ks - 1);
   const double without = over_budgets(sm_count, [&](int sms) {
-    // (rows past the step are not copied; from 33 rows on the MMAs of 64 rows take as long as 64 rows' copies)
+    // (units of 32 weight rows, though a launch may take others; rows past the step are not copied; from 33 rows on the MMAs of
+    // 64 rows take as long as 64 rows' copies)
     if (skinny) return (((N >> 5) + sms - 1) / sms) * (1.5 + double(32 + (M <= 32 ? M : 64)) * K * 2 / 70e3);
     return resid_launch_us(M, N, false, bn, ks, longest, sms) + gemm_chain_us(k_blocks, ks);
   });

@@ -175,7 +175,7 @@ struct SkinnySmem {
 // activations are there, 0.4 in the K loop, 0.45 until the last warp's partial tile is, 0.6 in the epilogue.  So with a K range
 // that fits the rings there is one wait and no refills, the chains of MMAs are halved, an epilogue thread has four columns
 // instead of eight, and the divisions of the unit's geometry and the first look at the arguments stand in front of the wait:
-// talker step of one row 233 -> 223 us, of 16 rows 288 -> 276.
+// talker step of one row 232 -> 225 us, of 16 rows 288 -> 276, all of it together.
 // MT: 16-row tiles of activations (T <= 16 MT); P: pairs of 8-column tiles per unit; DB: depth of a warp's ring of K steps.
 // FOLD: the instantiation that knows the folded RMSNorm (producing side in Resid mode, consuming side in the others; steps
 // of at most 16 rows); the plain one carries none of its code.
@@ -540,7 +540,8 @@ cudaError_t set_one() {
 // Width of a launch's units.  A block takes in about 70 KB/us, weights and activations alike -- 56 with units of 16 weight
 // rows -- with about 1.5 us per unit beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
 // budget.  Units wider than 64 weight rows, for a gate/up projection on few SMs, keep eight columns per epilogue thread and
-// their partial tiles in the rings.  Measured on B200 against 32 rows throughout: talker step of 16 rows at 112 / 96 / 28 SMs
+// their partial tiles in the rings: steps of a small backbone (4 layers, d_ffn 5632), next best width -> this one, 80 rows: one
+// row on 74 SMs 210 -> 201 us, 96: nine rows on 120 188 -> 183, 112: nine rows on 112 192 -> 184.  Measured on B200 against 32 rows throughout: talker step of 16 rows at 112 / 96 / 28 SMs
 // 352 -> 333, 351 -> 333, 683 -> 632 us, of 11 rows at 52 (51 units of 112 rows instead of 176 of 32) 395 -> 382; at 7B
 // dimensions 9 rows, 4 layers, at 96 / 74 / 37 SMs 606 -> 546, 594 -> 562, 963 -> 897; one row, 2 layers, at 52 SMs 344 -> 331 (two
 // rounds of 48 rows; five rounds of 16, which 70 KB/us would have, 370).
@@ -567,8 +568,10 @@ bool gemm_skinny_supports(int T, int K, int N, int mode, int head_dim) {
 }
 
 // Which kernel is faster for this shape, from measurements on B200 (config-3 and talker dimensions, 8 .. 64 rows).
-// A block of this kernel takes in about 70 KB/us and reads, per unit, 32 weight rows plus all (16 MT) activation
-// rows of width K, with about 1.5 us per unit for set-up, reduction and epilogue; units run in rounds of one per SM.
+// The rule counts this kernel as it was when they were taken: units of 32 weight rows in rounds of one per SM, 70 KB/us of
+// those and of 16 MT activation rows of width K, 1.5 us per unit for set-up, reduction and epilogue.  A launch today takes
+// 16 .. 112 weight rows (pick_width) and copies the step's rows alone, so where units of 32 rows are several rounds -- gate/up
+// of a wide FFN above all -- the rule holds this kernel for slower than it is.
 // The tiled kernel streams a 64-wide K block in about 0.36 us (0.8 us with two weight boxes per stage, gate/up)
 // and pays 3.5 us per link of a K-split chain.  So this kernel wins where the tiled one has too few tiles to
 // occupy the device or needs a long chain (QKV, out-projection, down at few rows), and loses where there are

@@ -135,7 +135,7 @@ int gemm_pick_stream_k(int M, int N, int K, int sm_count);
 struct ResidPlan { int pair, bn, ks; };
 ResidPlan gemm_plan_parts(int M, int N, int K, int sm_count, int part_cap_rows, bool skinny);
 // The same three GEMMs for steps of at most 64 rows (gemm_skinny.cu): weight streaming on plain loads and
-// warp-level MMAs, one block per 16 .. 64 weight rows and the whole K range, no K split across blocks.
+// warp-level MMAs, one block per 16 .. 112 weight rows and the whole K range, no K split across blocks.
 struct SkinnyParams {
   const void* a;             // activations [rows >= T, K], 16-bit (fp16 or bf16 as ab_f16 says), row-major
   const void* w[3];          // Resid {W}, Qkv {Wq, Wk, Wv}, GateUp {Wgate, Wup}; 16-bit [out, K] row-major

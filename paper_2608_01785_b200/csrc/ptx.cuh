@@ -1,6 +1,7 @@
 // Thin wrappers over the sm_100a instructions the kernels use: mbarrier, bulk tensor copies (TMA),
 // tcgen05 (5th-generation tensor cores with tensor-memory accumulators), ldmatrix / mma.sync for the
-// warp-level attention tiles.  No instruction here carries a cluster-multicast qualifier.
+// warp-level attention tiles.  No load here carries a cluster-multicast qualifier (a commit of the pair GEMM does: it signals both
+// blocks' barriers).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
