@@ -62,6 +62,7 @@ struct MetaLayout {
                                      //                           splits | index within the group << 16}
   int total;                         // int32 words in the block
   int max_prefill_items, max_decode_items;
+  int max_warp_items;                // of the decode items, those a step may use for items of single warps
 };
 MetaLayout make_meta_layout(const hs_stage_config_t& c);
 

@@ -64,10 +64,11 @@ MetaLayout make_meta_layout(const hs_stage_config_t& c) {
   m.max_prefill_items = c.n_kv_heads * (c.max_tokens / prefill_tokens_per_item(G) + c.max_seqs);
   // a decode sequence of n keys has at most n / kDecodeSplit whole runs and kDecodeSplitMax / kDecodeTail pieces of a
   // last, incomplete one; cached keys are bounded by the pool.  (At least eight items for each SM of the device, so that a
-  // small batch may be cut finely.)
-  m.max_decode_items = std::max(kMaxDecodeSlices * kDecodeWarps,
-                                c.n_kv_heads * (c.max_seqs * 2 * (kDecodeSplitMax / kDecodeTail) +
-                                                int((int64_t(c.num_pages) * kPage) / kDecodeSplit) + 1));
+  // small batch may be cut into slices finely; not into items of single warps, whose partial results one warp merges, 0.4 us
+  // each: with that room a few sequences beyond 4096 keys were runs of 128 keys instead of 256, at 7B dimensions, 2 layers, one
+  // of 8000 keys 257 -> 274 us per step, of 32000 351 -> 458.)
+  m.max_warp_items = c.n_kv_heads * (c.max_seqs * 2 * (kDecodeSplitMax / kDecodeTail) + int((int64_t(c.num_pages) * kPage) / kDecodeSplit) + 1);
+  m.max_decode_items = std::max(kMaxDecodeSlices * kDecodeWarps, m.max_warp_items);
   int off = 0;
   auto take = [&](int n) {
     int o = off;
@@ -252,13 +253,14 @@ hs_status_t plan_step(const hs_stage_config_t& c, const MetaLayout& ml, const hs
 
   const int G = c.n_q_heads / c.n_kv_heads;
   const int Mt = prefill_tokens_per_item(G);
-  const int split = pick_decode_split(c, b, sm_count, ml.max_decode_items);
+  int split = pick_decode_split(c, b, sm_count, ml.max_decode_items);
   // Group mode of the decode attention: in a batch small enough, every group = (sequence, KV head) is cut into equal
   // slices of whole pages such that all slices have a block of their own on the device; a block's eight warps share a
   // slice, and the block that delivers a group's last slice merges the group's (attention_decode.cuh).  A function of the
   // batch and the device's SM count, never of the budget.
   const int slice_pages = pick_decode_slice(c, b, sm_count, split);
   const bool group_mode = slice_pages > 0;
+  if (!group_mode) split = pick_decode_split(c, b, sm_count, ml.max_warp_items);
   StepPlan p;
   p.n_tokens = b.n_tokens;
   p.n_seqs = b.n_seqs;

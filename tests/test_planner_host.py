@@ -103,6 +103,19 @@ def test_attention_work_lists_cover_every_key_and_token_once(name):
         B.hs_stage_destroy(stage)
 
 
+@pytest.mark.parametrize("name,ctx,keys", [("c3_7b", [4096], 256), ("c3_7b", [16000], 256), ("c3_7b", [8000, 7963], 256), ("c2_shared", [6000], 256),
+                                           ("c4_talker", [7999, 7000, 6000, 5000], 256)])
+def test_items_of_long_sequences_are_no_finer_than_one_warp_can_merge(name, ctx, keys):
+    """A stage of the size of the batch: room for slices of small batches is not taken for items of single warps."""
+    stage, batch_c, batch = _stage_and_batch(wl.DIMS[name], [1] * len(ctx), ctx)
+    try:
+        items, group, _ = B.hs_stage_plan_attention(stage, batch_c)
+        _check_decode(wl.DIMS[name], batch, items, group)
+        assert not group and int((items[:, 3] - items[:, 2]).max()) == keys
+    finally:
+        B.hs_stage_destroy(stage)
+
+
 def test_k_splits_tile_the_k_range():
     for k_blocks in list(range(1, 70)) + [112, 148, 296, 1000]:
         for ks in range(1, 9):
