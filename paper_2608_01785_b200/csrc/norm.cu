@@ -432,10 +432,11 @@ cudaError_t launch_rmsnorm(const NormParams& p, int sm_budget, cudaStream_t stre
   if (p.T <= 0) return cudaSuccess;
   // few rows (one round of them on the whole device), or partial sums to add: many threads per row
   if (p.d <= kNormRowMaxD) {
-    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, rows = (p.T + sms - 1) / sms;
-    // Where that leaves SMs without rows, more threads per row, no power of two (the row's sum keeps its order).  Measured on
-    // B200, 401 rows of d = 3584 with the partial sums of four to six splits: 128 threads each on 101 SMs 10.2 us per launch,
-    // 160 on 134 7.3.
+    const int sms = p.sm_count > 0 ? p.sm_count : sm_budget, d4 = p.d >> 2, rows = (p.T + sm_budget - 1) / sm_budget;
+    // Where that leaves SMs without rows, more threads per row, no power of two (the row's sum keeps its order, so this may look
+    // at the budget: as many as leave one round of rows on it).  Measured on B200, 401 rows of d = 3584 with the partial sums of
+    // four to six splits: 128 threads each on 101 SMs 10.2 us per launch, 160 on 134 7.3; but 160 threads in two rounds on 112
+    // SMs, 408 rows on a small backbone, 478 us per step of 4 layers, 128 in one 445; 600 conditioned rows, 12 layers, 1020 and 933.
     const int sum_tpr = norm_row_threads(p.T, p.d, sms);
     const int tpr = rows <= ROW_THREADS / 32 ? std::max(sum_tpr, ROW_THREADS / rows / 32 * 32) : sum_tpr;
     const int rows_per_block = ROW_THREADS / tpr, blocks = (p.T + rows_per_block - 1) / rows_per_block;
