@@ -204,8 +204,11 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
   const int n = (steps - warp + SK_WARPS - 1) / SK_WARPS;
   const size_t k_off = (size_t(warp) * 32 + t * 8) * 2;     // byte offset of this lane's first 16 bytes in a row
   constexpr int STEP_BYTES = SK_WARPS * 64;                 // from one of the warp's steps to its next
-  // A K range that fits the rings is copied whole: one wait, no refills.  Otherwise DB - 1 steps are kept in flight.
-  const bool whole = steps <= SK_WARPS * DB;
+  // A K range that fits the rings is copied whole: one wait, no refills.  Otherwise DB - 1 steps are kept in flight.  (Not with
+  // four row tiles, whose MMAs take long enough to start on the first step that is there: 64 rows of the talker on 112 / 37 SMs
+  // 594 -> 556, 1023 -> 967 us with that and a step's weights and activations in one group, as below, for every unit but the
+  // first, whose weights go ahead of the wait; 16 .. 32 rows, several units a block, 370 for 404 on 112 SMs.)
+  const bool whole = MT < 4 && steps <= SK_WARPS * DB;
   const int n_first = whole ? n : min(n, DB - 1);
 
   const uint8_t* wrow[NT];
@@ -242,6 +245,17 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
 #pragma unroll
     for (int s = 0; s < DB; ++s) {
       if (s < n_first) issue_a(s, s);
+      if (s < DB - 1) cp_async_commit();
+    }
+    if (whole) cp_async_commit();
+  };
+  auto first_both = [&]() {                                 // both, a step's weights and activations in its own group
+#pragma unroll
+    for (int s = 0; s < DB; ++s) {
+      if (s < n_first) {
+        issue_b(s, s);
+        issue_a(s, s);
+      }
       if (s < DB - 1) cp_async_commit();
     }
     if (whole) cp_async_commit();
@@ -371,8 +385,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
     const int next = unit + n_blocks;
     if (!ALIAS && next < units) {
       set_unit(next);
-      first_b();
-      first_a();
+      first_both();
     }
 
     // partial tiles -> shared memory (rows past the step are not read)
@@ -500,8 +513,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
     }
     if (ALIAS && next < units) {
       set_unit(next);
-      first_b();
-      first_a();
+      first_both();
     }
   }
 }
@@ -538,7 +550,7 @@ cudaError_t set_one() {
 }
 
 // Width of a launch's units.  A block takes in about 70 KB/us, weights and activations alike -- 56 with units of 16 weight
-// rows -- with about 1.5 us per unit beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
+// rows beside at most 16 of activations -- with about 1.5 us per unit beside that, and units run in rounds of one per SM.  The results do not depend on the width, so the rule may look at the
 // budget.  Units wider than 64 weight rows, for a gate/up projection on few SMs, keep eight columns per epilogue thread and
 // their partial tiles in the rings: steps of a small backbone (4 layers, d_ffn 5632), next best width -> this one, 80 rows: one
 // row on 74 SMs 210 -> 201 us, 96: nine rows on 120 188 -> 183, 112: nine rows on 112 192 -> 184.  Measured on B200 against 32 rows throughout: talker step of 16 rows at 112 / 96 / 28 SMs
@@ -552,7 +564,7 @@ int pick_width(int T, int K, int N, int mode, int head_dim, int sms) {
   for (int P = 1; P <= max_p; ++P) {
     if (mode == kGemmQkv && (head_dim >> 4) % P != 0) continue;
     const int units = skinny_units(N, mode, P), rounds = (units + sms - 1) / sms;
-    const double us = rounds * (1.5 + double(16 * P + (T <= 32 ? T : 64)) * K * 2 / (P == 1 ? 56e3 : 70e3));
+    const double us = rounds * (1.5 + double(16 * P + (T <= 32 ? T : 64)) * K * 2 / (P == 1 && T <= 16 ? 56e3 : 70e3));
     if (us < best_us - 1e-9) { best_us = us; best = P; }
   }
   return best;
