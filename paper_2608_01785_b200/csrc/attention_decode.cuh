@@ -58,6 +58,105 @@ __device__ __forceinline__ uint32_t mask_v(uint32_t r, int k, int n_valid) {
   return r;
 }
 
+// Running state of one warp's attention: rows lane / 4 and lane / 4 + 8 of the G query heads, unnormalised output, maximum (log2
+// domain) and this lane's share of the sum.
+template <int DH>
+struct Attend {
+  float o[DH / 8][4], m_a, m_b, l_a, l_b;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < DH / 8; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+    m_a = m_b = -INFINITY;
+    l_a = l_b = 0.f;
+  }
+};
+// One page in shared memory, n_valid keys of which belong to the item (16 or more: all).
+// A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
+// bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs per key
+// half, the V fragments are fetched while the scores are on their way, and a page on which no row's maximum moves --
+// most of them, after the first few -- needs a vote, but no shuffles and no rescale.  (A reference that follows the
+// maximum only beyond a factor of 256 is another 1 - 2 % faster, but leaves the largest weight rounded: error against
+// 64 bits up to 6 % larger.)  Against a loop with one chain of MMAs, shuffles and exp2f on every page and V fetched
+// behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker step of 16
+// rows 300.5 -> 289 us, of 11 rows on 52 SMs 471 -> 457; at config-3 dimensions 9 rows, 4 layers 493 -> 483 us, 29 rows
+// on 96 SMs 796 -> 782, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.16 ms.
+// TWO: rows lane / 4 + 8 are in use (groups of more than eight heads).
+template <int DH, bool TWO = true>
+__device__ __forceinline__ void attend_page(Attend<DH>& at, const uint32_t (&qf)[DH / 16][4], uint32_t k_base, uint32_t v_base, int n_valid,
+                                            int lane, float scale_log2) {
+  float (&o)[DH / 8][4] = at.o;
+  float &m_a = at.m_a, &m_b = at.m_b, &l_a = at.l_a, &l_b = at.l_b;
+  float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+  float sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int ks = 0; ks < DH / 16; ks += 2) {
+    uint32_t kf[4], kg[4];
+    const int kk = (lane & 7) + (lane >> 4) * 8, cc = 2 * ks + ((lane >> 3) & 1);
+    ldmatrix_x4(kf, k_base + kv_off(kk, cc));
+    ldmatrix_x4(kg, k_base + kv_off(kk, cc + 2));
+    mma_bf16_16816(sc[0], qf[ks], kf[0], kf[1]);
+    mma_bf16_16816(sc[1], qf[ks], kf[2], kf[3]);
+    mma_bf16_16816(sd[0], qf[ks + 1], kg[0], kg[1]);
+    mma_bf16_16816(sd[1], qf[ks + 1], kg[2], kg[3]);
+  }
+  uint32_t vf[DH / 16][4];
+#pragma unroll
+  for (int dp = 0; dp < DH / 16; ++dp) {
+    const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
+    ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, cc));
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) sc[j][e] += sd[j][e];
+  if (n_valid < 16) {
+    const int k = 2 * (lane & 3);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (8 * j + k + (e & 1) >= n_valid) sc[j][e] = -INFINITY;
+#pragma unroll
+    for (int dp = 0; dp < DH / 16; ++dp)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], k + 8 * (e & 1), n_valid);
+  }
+  const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
+  const float mx_b = TWO ? fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2 : -INFINITY;
+  if (__any_sync(0xffffffffu, mx_a > m_a || (TWO && mx_b > m_b))) {
+    const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = TWO ? fmaxf(m_b, quad_max(mx_b)) : 0.f;
+    const float al_a = fast_exp2(m_a - mn_a), al_b = TWO ? fast_exp2(m_b - mn_b) : 0.f;
+    m_a = mn_a;
+    m_b = mn_b;
+    l_a *= al_a;
+    l_b *= al_b;
+#pragma unroll
+    for (int j = 0; j < DH / 8; ++j) {
+      o[j][0] *= al_a; o[j][1] *= al_a;
+      if (TWO) { o[j][2] *= al_b; o[j][3] *= al_b; }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    sc[j][0] = fast_exp2(fmaf(sc[j][0], scale_log2, -m_a));
+    sc[j][1] = fast_exp2(fmaf(sc[j][1], scale_log2, -m_a));
+    sc[j][2] = TWO ? fast_exp2(fmaf(sc[j][2], scale_log2, -m_b)) : 0.f;
+    sc[j][3] = TWO ? fast_exp2(fmaf(sc[j][3], scale_log2, -m_b)) : 0.f;
+  }
+  l_a += (sc[0][0] + sc[0][1]) + (sc[1][0] + sc[1][1]);
+  if (TWO) l_b += (sc[0][2] + sc[0][3]) + (sc[1][2] + sc[1][3]);
+  uint32_t pf[4];
+  pf[0] = pack_bf16(sc[0][0], sc[0][1]);
+  pf[1] = pack_bf16(sc[0][2], sc[0][3]);
+  pf[2] = pack_bf16(sc[1][0], sc[1][1]);
+  pf[3] = pack_bf16(sc[1][2], sc[1][3]);
+#pragma unroll
+  for (int dp = 0; dp < DH / 16; ++dp) {
+    mma_bf16_16816(o[2 * dp], pf, vf[dp][0], vf[dp][1]);
+    mma_bf16_16816(o[2 * dp + 1], pf, vf[dp][2], vf[dp][3]);
+  }
+}
+
 // Merges the partials of one (sequence, KV head) group -- items first .. first + splits - 1 -- in split
 // order and writes the normalised output rows.  LPH lanes share one query head, each owning DH / LPH
 // contiguous columns.  A lone warp does this at the tail of the kernel, so what counts is latency: the
@@ -164,6 +263,63 @@ template <int DH>
 constexpr int dc_smem_bytes() {
   int b = 1024 + DC_WARPS * DC_STAGES * 2 * Geom<DH>::PAGE_BYTES + 512;
   return b > kMinSmemBytes ? b : kMinSmemBytes;
+}
+
+// Group mode, a warp's part of a slice, into an area of its own: [ROWS][DH] unnormalised output, then [ROWS] (max, sum); ROWS is at
+// least G.
+template <int DH, int ROWS>
+__device__ __forceinline__ void slice_partial(uint8_t* slots, const float (&o)[DH / 8][4], float m_a, float m_b, float l_a, float l_b, int G,
+                                              int lane) {
+  const int ra = lane >> 2, rb = ra + 8;
+  float* po = reinterpret_cast<float*>(slots);
+  float2* pml = reinterpret_cast<float2*>(slots + ROWS * DH * 4);
+#pragma unroll
+  for (int j = 0; j < DH / 8; ++j) {
+    const int col = 8 * j + 2 * (lane & 3);
+    if (ra < G) *reinterpret_cast<float2*>(po + ra * DH + col) = make_float2(o[j][0], o[j][1]);
+    if (rb < G) *reinterpret_cast<float2*>(po + rb * DH + col) = make_float2(o[j][2], o[j][3]);
+  }
+  if ((lane & 3) == 0) {
+    if (ra < G) pml[ra] = make_float2(m_a, l_a);
+    if (rb < G) pml[rb] = make_float2(m_b, l_b);
+  }
+}
+// The eight warps' parts of a slice, PITCH bytes apart, merged in order: head g, columns col and col + 1, unnormalised, with the
+// maximum and the sum.
+template <int DH, int ROWS, int PITCH, int UNROLL = DC_WARPS>
+__device__ __forceinline__ void merge_eight(const uint8_t* parts, int g, int col, float& mm, float& ll, float& o0, float& o1) {
+  mm = -INFINITY;
+#pragma unroll UNROLL
+  for (int w = 0; w < DC_WARPS; ++w) mm = fmaxf(mm, reinterpret_cast<const float2*>(parts + w * PITCH + ROWS * DH * 4)[g].x);
+  ll = 0.f, o0 = 0.f, o1 = 0.f;
+#pragma unroll UNROLL
+  for (int w = 0; w < DC_WARPS; ++w) {
+    const uint8_t* base = parts + w * PITCH;
+    const float2 ml = reinterpret_cast<const float2*>(base + ROWS * DH * 4)[g];
+    const float f = exp2f(ml.x - mm);                 // 0 for an empty slice (max = -inf)
+    const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + g * DH + col);
+    ll += f * ml.y;
+    o0 += f * v.x;
+    o1 += f * v.y;
+  }
+}
+// The next eight (or `left`) slices of a group: their (max, sum) and two columns of their outputs into the running ones.
+__device__ __forceinline__ void merge_slices(const float2 (&ml)[8], const float2 (&ov)[8], int left, float& mm, float& ll, float& o0, float& o1) {
+  float pm = mm;
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (u < left) pm = fmaxf(pm, ml[u].x);
+  const float sc = exp2f(mm - pm);                 // 0 the first time (mm = -inf)
+  mm = pm;
+  ll *= sc; o0 *= sc; o1 *= sc;
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (u < left) {
+      const float f = exp2f(ml[u].x - mm);
+      ll += f * ml[u].y;
+      o0 += f * ov[u].x;
+      o1 += f * ov[u].y;
+    }
 }
 
 // The body of the decode kernel.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS *
@@ -281,21 +437,11 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
       qf[ks][2] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + ra * DH + c + 8)) : 0u;
       qf[ks][3] = rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + rb * DH + c + 8)) : 0u;
     }
-    float o_acc[DH / 8][4];
-#pragma unroll
-    for (int j = 0; j < DH / 8; ++j) o_acc[j][0] = o_acc[j][1] = o_acc[j][2] = o_acc[j][3] = 0.f;
-    float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
+    Attend<DH> at;
+    at.clear();
+    float (&o_acc)[DH / 8][4] = at.o;
     bool ok = true;
 
-    // A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
-    // bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs per key
-    // half, the V fragments are fetched while the scores are on their way, and a page on which no row's maximum moves --
-    // most of them, after the first few -- needs a vote, but no shuffles and no rescale.  (A reference that follows the
-    // maximum only beyond a factor of 256 is another 1 - 2 % faster, but leaves the largest weight rounded: error against
-    // 64 bits up to 6 % larger.)  Against a loop with one chain of MMAs, shuffles and exp2f on every page and V fetched
-    // behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker step of 16
-    // rows 300.5 -> 289 us, of 11 rows on 52 SMs 471 -> 457; at config-3 dimensions 9 rows, 4 layers 493 -> 483 us, 29 rows
-    // on 96 SMs 796 -> 782, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.16 ms.
     for (int pi = 0; pi < n_pages; ++pi) {
       // the slot read in the previous iteration is free: keep DC_STAGES - 1 pages in flight
       const int page_ahead = __shfl_sync(0xffffffffu, my_page, (pi + DC_STAGES - 1) & 31);
@@ -306,97 +452,15 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
       const uint32_t v_base = k_base + G_::PAGE_BYTES;
       if (++cur == DC_STAGES) { cur = 0; cur_phase ^= 1; }
       const int n_valid = k1 - (k0 + pi * 16);            // keys of this page that belong to the item
-      float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      float sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-      for (int ks = 0; ks < DH / 16; ks += 2) {
-        uint32_t kf[4], kg[4];
-        const int kk = (lane & 7) + (lane >> 4) * 8, cc = 2 * ks + ((lane >> 3) & 1);
-        ldmatrix_x4(kf, k_base + kv_off(kk, cc));
-        ldmatrix_x4(kg, k_base + kv_off(kk, cc + 2));
-        mma_bf16_16816(sc[0], qf[ks], kf[0], kf[1]);
-        mma_bf16_16816(sc[1], qf[ks], kf[2], kf[3]);
-        mma_bf16_16816(sd[0], qf[ks + 1], kg[0], kg[1]);
-        mma_bf16_16816(sd[1], qf[ks + 1], kg[2], kg[3]);
-      }
-      uint32_t vf[DH / 16][4];
-#pragma unroll
-      for (int dp = 0; dp < DH / 16; ++dp) {
-        const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
-        ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, cc));
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) sc[j][e] += sd[j][e];
-      if (n_valid < 16) {
-        const int k = 2 * (lane & 3);
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (8 * j + k + (e & 1) >= n_valid) sc[j][e] = -INFINITY;
-#pragma unroll
-        for (int dp = 0; dp < DH / 16; ++dp)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], k + 8 * (e & 1), n_valid);
-      }
-      const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
-      const float mx_b = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2;
-      if (__any_sync(0xffffffffu, mx_a > m_a || mx_b > m_b)) {
-        const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = fmaxf(m_b, quad_max(mx_b));
-        const float al_a = fast_exp2(m_a - mn_a), al_b = fast_exp2(m_b - mn_b);
-        m_a = mn_a;
-        m_b = mn_b;
-        l_a *= al_a;
-        l_b *= al_b;
-#pragma unroll
-        for (int j = 0; j < DH / 8; ++j) {
-          o_acc[j][0] *= al_a; o_acc[j][1] *= al_a;
-          o_acc[j][2] *= al_b; o_acc[j][3] *= al_b;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        sc[j][0] = fast_exp2(fmaf(sc[j][0], scale_log2, -m_a));
-        sc[j][1] = fast_exp2(fmaf(sc[j][1], scale_log2, -m_a));
-        sc[j][2] = fast_exp2(fmaf(sc[j][2], scale_log2, -m_b));
-        sc[j][3] = fast_exp2(fmaf(sc[j][3], scale_log2, -m_b));
-      }
-      l_a += (sc[0][0] + sc[0][1]) + (sc[1][0] + sc[1][1]);
-      l_b += (sc[0][2] + sc[0][3]) + (sc[1][2] + sc[1][3]);
-      uint32_t pf[4];
-      pf[0] = pack_bf16(sc[0][0], sc[0][1]);
-      pf[1] = pack_bf16(sc[0][2], sc[0][3]);
-      pf[2] = pack_bf16(sc[1][0], sc[1][1]);
-      pf[3] = pack_bf16(sc[1][2], sc[1][3]);
-#pragma unroll
-      for (int dp = 0; dp < DH / 16; ++dp) {
-        mma_bf16_16816(o_acc[2 * dp], pf, vf[dp][0], vf[dp][1]);
-        mma_bf16_16816(o_acc[2 * dp + 1], pf, vf[dp][2], vf[dp][3]);
-      }
+      attend_page<DH>(at, qf, k_base, v_base, n_valid, lane, scale_log2);
       __syncwarp();                         // every lane is done with this slot before lane 0 refills it
     }
     if (!ok && !group_mode) break;
 
-    l_a = quad_sum(l_a);
-    l_b = quad_sum(l_b);
+    const float m_a = at.m_a, m_b = at.m_b, l_a = quad_sum(at.l_a), l_b = quad_sum(at.l_b);
     __nv_bfloat16* orow = p.o + size_t(tok) * q_dim + size_t(hk) * G * DH;
     if (group_mode) {
-      // this slice's partial into the warp's own (now idle) page ring: [16 rows][DH] unnormalised output, then
-      // [16 rows] (max, sum)
-      float* po = reinterpret_cast<float*>(slots);
-      float2* pml = reinterpret_cast<float2*>(slots + 16 * DH * 4);
-#pragma unroll
-      for (int j = 0; j < DH / 8; ++j) {
-        const int col = 8 * j + 2 * (lane & 3);
-        if (ra < G) *reinterpret_cast<float2*>(po + ra * DH + col) = make_float2(o_acc[j][0], o_acc[j][1]);
-        if (rb < G) *reinterpret_cast<float2*>(po + rb * DH + col) = make_float2(o_acc[j][2], o_acc[j][3]);
-      }
-      if ((lane & 3) == 0) {
-        if (ra < G) pml[ra] = make_float2(m_a, l_a);
-        if (rb < G) pml[rb] = make_float2(m_b, l_b);
-      }
+      slice_partial<DH, 16>(slots, at.o, m_a, m_b, l_a, l_b, G, lane);
       const bool failed = __syncthreads_or(!ok) != 0;      // the same answer in every warp of the block
       if (!failed) {
         // the eight partials are merged in order by the whole block: a thread per pair of output columns
@@ -411,21 +475,8 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
         };
         for (int e = threadIdx.x; e < G * (DH / 2); e += DC_THREADS) {
           const int g = e / (DH / 2), col = 2 * (e - g * (DH / 2));
-          float mm = -INFINITY;
-#pragma unroll
-          for (int w = 0; w < DC_WARPS; ++w)
-            mm = fmaxf(mm, reinterpret_cast<const float2*>(smem + w * DC_STAGES * SLOT_BYTES + 16 * DH * 4)[g].x);
-          float ll = 0.f, o0 = 0.f, o1 = 0.f;
-#pragma unroll
-          for (int w = 0; w < DC_WARPS; ++w) {
-            const uint8_t* base = smem + w * DC_STAGES * SLOT_BYTES;
-            const float2 ml = reinterpret_cast<const float2*>(base + 16 * DH * 4)[g];
-            const float f = exp2f(ml.x - mm);                 // 0 for an empty slice (max = -inf)
-            const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + g * DH + col);
-            ll += f * ml.y;
-            o0 += f * v.x;
-            o1 += f * v.y;
-          }
+          float mm, ll, o0, o1;
+          merge_eight<DH, 16, DC_STAGES * SLOT_BYTES>(smem, g, col, mm, ll, o0, o1);
           if (!SLICED || splits == 1) {
             store(g, col, o0, o1, ll);
           } else {
@@ -455,20 +506,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
                   ml[u] = __ldcg(ml_g + size_t(j) * 16);
                   ov[u] = __ldcg(reinterpret_cast<const float2*>(po_g + size_t(j) * 16 * DH));
                 }
-                float pm = mm;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) pm = fmaxf(pm, ml[u].x);
-                const float sc = exp2f(mm - pm);             // 0 the first time (mm = -inf)
-                mm = pm;
-                ll *= sc; o0 *= sc; o1 *= sc;
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                  if (j0 + u < splits) {
-                    const float f = exp2f(ml[u].x - mm);
-                    ll += f * ml[u].y;
-                    o0 += f * ov[u].x;
-                    o1 += f * ov[u].y;
-                  }
+                merge_slices(ml, ov, splits - j0, mm, ll, o0, o1);
               }
               store(g, col, o0, o1, ll);
             }

@@ -17,11 +17,6 @@ constexpr int NORM_STAGE_FLOATS = 2048;   // per-warp row cache in shared memory
 constexpr int NORM_SMEM = NORM_WARPS * NORM_STAGE_FLOATS * 4 > kMinSmemBytes ? NORM_WARPS * NORM_STAGE_FLOATS * 4
                                                                               : kMinSmemBytes;
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
   const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -270,9 +265,6 @@ __global__ void __launch_bounds__(BULK_MAX_WARPS * 32, 1) rmsnorm_bulk_kernel(co
 // 0 .. sum_tpr - 1, a butterfly per 32 of them, those in order -- a function of the shape and the device's SM count, never of
 // the budget nor of how many threads do the rest: where those are not sum_tpr, the groups' sums pass through shared memory.
 constexpr int ROW_THREADS = kNormRowThreads;
-
-// (written out: what the compiler fuses here would follow the code around it)
-__device__ __forceinline__ float square_sum(const float4& a) { return fmaf(a.x, a.x, a.y * a.y) + fmaf(a.z, a.z, a.w * a.w); }
 
 // OTHER: tpr is not sum_tpr.
 template <int V, bool OTHER>

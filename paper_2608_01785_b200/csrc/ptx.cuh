@@ -318,6 +318,13 @@ __device__ __forceinline__ void rotate_pair(float& a, float& b, float c, float s
   a = lo;
   b = hi;
 }
+// Squares of a group of four columns, for RMSNorm (written out: what the compiler fuses here would follow the code around it).
+__device__ __forceinline__ float square_sum(const float4& a) { return fmaf(a.x, a.x, a.y * a.y) + fmaf(a.z, a.z, a.w * a.w); }
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);   // round-to-nearest-even; .x = lo (low 16 bits)
   return *reinterpret_cast<uint32_t*>(&v);
