@@ -188,6 +188,15 @@ int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
 
 /*
+ * Host-only: 1 if hs_stage_step runs a decode-only step of `rows` rows of an unconditioned stage of these dimensions as one
+ * cooperative launch on sm_budget SMs of a device of 148, provided that the attention takes its group mode
+ * (hs_stage_plan_attention), 0 if it is a chain of launches.  The results do not depend on it.  Steps that are profiled, or made
+ * after hs_stage_debug_buffer("smid") was asked for, are always the chain.  Returns -1 for a value below 1.
+ */
+int32_t hs_op_one_launch_step(int32_t rows, int32_t d_model, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int32_t d_ffn,
+                              int32_t n_layers, int32_t sm_budget);
+
+/*
  * Host-only: the K block (of 64) at which split i (0 .. ks; i = ks gives k_blocks) of a small step's residual GEMM
  * begins when its k_blocks are cut into ks splits.  Each split is ten K blocks longer than the one before it (the
  * splits add their sums one after the other, and a link of that chain takes about as long as ten K blocks take to

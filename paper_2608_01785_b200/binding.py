@@ -31,7 +31,7 @@ EXPORTS = ("hs_status_str", "hs_kv_pool_bytes", "hs_workspace_bytes", "hs_stage_
            "hs_stage_set_qkv_bias", "hs_stage_set_modulation", "hs_stage_saturation_count", "hs_op_wait_probe",
            "hs_op_decode_attention_noalloc_status", "hs_stage_plan_attention", "hs_op_gemm_split_begin",
            "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width",
-           "hs_op_weight_streaming_rows")
+           "hs_op_weight_streaming_rows", "hs_op_one_launch_step")
 PROFILE_CLASSES = ("rmsnorm", "gemm_qkv", "attn_prefill", "attn_decode", "attn_combine", "gemm_out", "gemm_gateup",
                    "gemm_down")
 
@@ -120,6 +120,8 @@ def lib() -> C.CDLL:
         l.hs_op_gemm_part_splits.restype = C.c_int32
         l.hs_op_gate_up_width.argtypes = [C.c_int32] * 4
         l.hs_op_gate_up_width.restype = C.c_int32
+        l.hs_op_one_launch_step.argtypes = [C.c_int32] * 8
+        l.hs_op_one_launch_step.restype = C.c_int32
         l.hs_op_weight_streaming_rows.argtypes = [C.c_int32] * 4
         l.hs_op_weight_streaming_rows.restype = C.c_int32
         l.hs_stage_plan_shares.argtypes = [C.c_void_p, C.POINTER(hs_batch_t), C.c_int32, C.c_void_p, C.c_void_p]
@@ -281,6 +283,11 @@ def hs_op_gemm_part_splits(M: int, N: int, K: int) -> int:
 
 def hs_op_gate_up_width(M: int, N: int, K: int, sm_budget: int) -> int:
     return int(lib().hs_op_gate_up_width(M, N, K, sm_budget))
+
+
+def hs_op_one_launch_step(rows: int, dims, sm_budget: int) -> int:
+    return int(lib().hs_op_one_launch_step(rows, dims.d_model, dims.n_q_heads, dims.n_kv_heads, dims.head_dim, dims.d_ffn, dims.n_layers,
+                                           sm_budget))
 
 
 def hs_op_weight_streaming_rows(M: int, N: int, K: int, sm_budget: int) -> int:

@@ -22,7 +22,7 @@ constexpr int kRing = 4;   // pinned staging slots for step metadata
 constexpr int kRowSsStride = 64;   // partial sums of x^2 kept per token: one per 128-column tile of d_model at most
 
 struct WsLayout {
-  size_t rope, h, q, o, act, meta, part_o, part_ml, status, turn, smid, row_ss, row_rs, row_done, gemm_part, w16, w16_layer, total;
+  size_t rope, h, q, o, act, meta, part_o, part_ml, status, turn, smid, row_ss, row_rs, row_done, gemm_part, exchange, small_maps, w16, w16_layer, total;
   int part_rows;             // rows of d_model floats in gemm_part
 };
 
@@ -65,6 +65,22 @@ ResidPlan plan_parts(int T, int d, int K, int sm_count, int part_rows, bool skin
   return gemm_plan_parts(T, d, K, sm_count, part_rows, skinny);
 }
 
+// A decode-only step of T rows may take the form of one launch (launch_small_step), as far as its sizes go.
+bool small_step_of(const hs_stage_config_t& c, int T) {
+  return small_step_supports(T, c.d_model, c.n_q_heads * c.head_dim, c.n_kv_heads * c.head_dim, c.d_ffn, c.head_dim, c.n_layers);
+}
+// A decode-only step of T rows whose attention is in group mode takes that form on sm_budget SMs: its projections all run on the
+// weight-streaming kernel, which folds the norms.
+bool one_launch(const hs_stage_config_t& c, int T, int sm_count, int sm_budget) {
+  const int d = c.d_model, F = c.d_ffn, Dh = c.head_dim, q_dim = c.n_q_heads * Dh, kv_dim = c.n_kv_heads * Dh;
+  return small_step_of(c, T) && sm_count >= T && small_step_wins(T, d, q_dim, sm_budget) && gemm_skinny_wins(T, d, q_dim + 2 * kv_dim, kGemmQkv, Dh, sm_count) &&
+         gemm_skinny_wins(T, q_dim, d, kGemmResid, Dh, sm_count) && gemm_skinny_wins(T, d, F, kGemmGateUp, Dh, sm_count) &&
+         gemm_skinny_wins(T, F, d, kGemmResid, Dh, sm_count);
+}
+SmallExchange exchange_of(const hs_stage_config_t& c) {
+  return small_exchange(c.d_model, c.n_q_heads * c.head_dim, c.n_kv_heads * c.head_dim, c.d_ffn, c.n_q_heads / c.n_kv_heads, kMaxDecodeSlices);
+}
+
 WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   WsLayout w{};
   size_t off = 0;
@@ -91,6 +107,10 @@ WsLayout make_ws_layout(const hs_stage_config_t& c, const MetaLayout& ml) {
   w.row_done = take((T / 32 + 2) * 4);               // tile columns delivered per group of 32 token rows
   w.part_rows = part_rows_cap(c.max_tokens, c.d_model);      // (plan_parts)
   w.gemm_part = take(size_t(w.part_rows) * c.d_model * 4);
+  w.exchange = off;                                  // the three buffers of a small step in one launch
+  if (small_step_of(c, 1)) take(3 * exchange_of(c).bytes);
+  w.small_maps = off;                                // and its tensor maps of the weights
+  if (small_step_of(c, 1)) take(size_t(c.n_layers) * 7 * sizeof(CUtensorMap));
   // fp16 copies of the seven weight matrices of every layer (absent with HS_FLAG_BF16_ACTIVATIONS);
   // within a layer: w_q, w_k, w_v, w_o, w_gate, w_up, w_down, each 1024-byte aligned
   w.w16 = off;
@@ -194,6 +214,7 @@ hs_status_t ensure_attributes(int device) {
   if ((e = attention_set_attributes()) != cudaSuccess) return cuda_fail("attention attributes", e);
   if ((e = head_set_attributes()) != cudaSuccess) return cuda_fail("head attributes", e);
   if ((e = gemm_skinny_set_attributes()) != cudaSuccess) return cuda_fail("small-step gemm attributes", e);
+  if ((e = small_step_set_attributes()) != cudaSuccess) return cuda_fail("one-launch step attributes", e);
   if (device >= 0 && device < 64) g_attrs_set[device] = true;
   return HS_OK;
 }
@@ -399,6 +420,17 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
     for (int i = 0; i < kGuNarrow && ok; ++i)
       ok = encode_2d(&m.gu_narrow[i][0], w.w_gate, F, d, kGuMinWidth + 16 * i) && encode_2d(&m.gu_narrow[i][1], w.w_up, F, d, kGuMinWidth + 16 * i);
   }
+  if (ok && small_step_of(*cfg, 1)) {
+    std::vector<CUtensorMap> small(size_t(cfg->n_layers) * 7);
+    for (int l = 0; l < cfg->n_layers && ok; ++l) {
+      const hs_layer_weights_t& w = s->operands[l];
+      const void* src[7] = {w.w_q, w.w_k, w.w_v, w.w_o, w.w_gate, w.w_up, w.w_down};
+      const uint64_t rows[7] = {q_dim, kv_dim, kv_dim, d, F, F, d}, cols[7] = {d, d, d, q_dim, d, d, F};
+      for (int i = 0; i < 7 && ok; ++i) ok = encode_small_weight(get_encode_fn(), &small[l * 7 + i], src[i], int(rows[i]), int(cols[i]));
+    }
+    if (ok && cudaMemcpy(s->ws_dev + s->ws.small_maps, small.data(), small.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess)
+      return cuda_fail("hs_stage_create: tensor maps of the weights", cudaGetLastError());
+  }
   if (!ok)
     return fail("hs_stage_create: fp16 weight copy or tensor-map encoding failed (cuTensorMapEncodeTiled unavailable, or "
                 "a matrix whose row pitch is not a multiple of 16 bytes)");
@@ -526,6 +558,14 @@ int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget) 
 
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
   return sm_budget < 1 || !gemm_skinny_supports(M, K, N, kGemmResid, 0) ? -1 : gemm_skinny_rows(M, K, N, kGemmResid, 0, sm_budget);
+}
+
+int32_t hs_op_one_launch_step(int32_t rows, int32_t d_model, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int32_t d_ffn,
+                              int32_t n_layers, int32_t sm_budget) {
+  if (rows < 1 || d_model < 1 || n_q_heads < 1 || n_kv_heads < 1 || head_dim < 1 || d_ffn < 1 || n_layers < 1 || sm_budget < 1) return -1;
+  hs_stage_config_t c{};
+  c.d_model = d_model; c.n_q_heads = n_q_heads; c.n_kv_heads = n_kv_heads; c.head_dim = head_dim; c.d_ffn = d_ffn; c.n_layers = n_layers;
+  return one_launch(c, rows, 148, sm_budget) ? 1 : 0;
 }
 
 int32_t hs_op_gemm_split_begin(int32_t k_blocks, int32_t ks, int32_t i) {
@@ -716,6 +756,38 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     a.smid_log = slots(2);       // prefill in class 2, decode in class 3 (the next slots)
     return a;
   };
+  // The whole step in one launch, with the bits of the launches below.  Not while those are timed or counted one by one, nor for a
+  // conditioned stage.
+  if (plan.n_prefill_items == 0 && plan.decode_group && !s->modulation && !s->profile && !s->census && one_launch(c, T, s->sm_count, sm_budget)) {
+    SmallStepParams k{};
+    k.tm_kv_page = s->tm_kv_page;
+    for (int l = 0; l < c.n_layers; ++l) {
+      k.layers[l] = SmallLayer{static_cast<const __nv_bfloat16*>(s->layers[l].g_attn), static_cast<const __nv_bfloat16*>(s->layers[l].g_mlp),
+                               {s->qkv_bias[l].b[0], s->qkv_bias[l].b[1], s->qkv_bias[l].b[2]}};
+    }
+    k.maps = reinterpret_cast<const CUtensorMap*>(s->ws_dev + s->ws.small_maps);
+    k.at = exchange_of(c);
+    k.exchange = s->ws_dev + s->ws.exchange;
+    k.n_layers = c.n_layers; k.T = T; k.d = d; k.F = F; k.q_dim = q_dim; k.kv_dim = kv_dim;
+    k.n_q_heads = c.n_q_heads; k.n_kv_heads = c.n_kv_heads; k.max_pages_per_seq = c.max_pages_per_seq;
+    k.n_slices = plan.n_decode_items / kDecodeWarps;
+    k.f16 = f16; k.eps = c.rms_eps;
+    k.x_in = static_cast<const __nv_bfloat16*>(b->x_in);
+    k.y = x; k.h = h; k.q = q; k.o = o;
+    k.act = reinterpret_cast<__nv_bfloat16*>(s->ws_dev + s->ws.act);
+    k.kv_pool = s->kv_pool; k.layer_kv_elems = layer_kv_elems;
+    k.tok_pos = meta + s->ml.tok_pos; k.tok_slot = meta + s->ml.tok_slot;
+    k.decode_items = meta + s->ml.decode_items; k.seq_ctx = meta + s->ml.seq_ctx; k.block_tables = meta + s->ml.block_tables;
+    k.rope = reinterpret_cast<const float2*>(s->ws_dev + s->ws.rope);
+    k.sync = meta + s->ml.counters;
+    k.status = status;
+    e = launch_small_step(k, sm_budget, stream);
+    if (e == cudaSuccess) return HS_OK;
+    // a context that does not hold so many blocks at once takes the separate launches
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return cuda_fail("small step", e);
+    cudaGetLastError();
+    e = cudaSuccess;
+  }
   for (int l = 0; l < c.n_layers && e == cudaSuccess; ++l) {
     const hs_layer_weights_t& w = s->layers[l];
     const LayerMaps& m = s->maps[l];

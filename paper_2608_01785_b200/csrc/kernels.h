@@ -188,6 +188,64 @@ cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_
 cudaError_t gemm_skinny_set_attributes();
 constexpr int kGemmTurnWords = 8192;   // capacity of the whose-turn array: splits are used only when tiles * 8 fits
 
+// ------------------------------------------------- a small step in one launch --
+// Decode-only step of at most 16 rows whose projections all stream weights past the rows, head_dim 64, at most eight query heads
+// per KV head, d_model and q_dim up to kSmallMaxModel, d_ffn up to kSmallMaxWidth, all three multiples of 256, as ONE cooperative
+// launch: every block goes through the phases of every layer, and what one phase leaves for the next travels through buffers in
+// which a value that is not there yet reads as a pattern that no value has (small_step.cu).  The same units, slices and orders as
+// the kernels of their own: the same bits.
+constexpr int kSmallMaxRows = 16, kSmallMaxModel = 2048, kSmallMaxWidth = 3072, kSmallMaxLayers = 32;
+struct SmallLayer {
+  const __nv_bfloat16 *g_attn, *g_mlp;
+  const __nv_bfloat16* bias[3];                                    // of q, k, v, or null
+};
+// Byte offsets inside one of the three exchange buffers of a stage: 16 rows of h in front of the attention and of the MLP, q, k,
+// v, o and act, the sums of squares that belong to the two h, and the partial results of `slices` slices of the attention.
+struct SmallExchange {
+  uint32_t h_attn, h_mlp, q, k, v, o, act, ss_attn, ss_mlp, slice_o, slice_ml, bytes;
+};
+SmallExchange small_exchange(int d, int q_dim, int kv_dim, int F, int heads_per_group, int slices);
+struct SmallStepParams {
+  CUtensorMap tm_kv_page;          // as in AttnParams
+  const CUtensorMap* maps;         // device, [n_layers][7]: w_q, w_k, w_v, w_o, w_gate, w_up, w_down (encode_small_weight)
+  SmallLayer layers[kSmallMaxLayers];
+  SmallExchange at;
+  uint8_t* exchange;               // three buffers of at.bytes
+  int n_layers, T, d, F, q_dim, kv_dim, n_q_heads, n_kv_heads, max_pages_per_seq;
+  int n_slices;                    // of the decode attention in group mode
+  int f16;                         // format of h, o and act
+  float eps;
+  const __nv_bfloat16* x_in;       // [T, d]
+  float* y;                        // [T, d]
+  __nv_bfloat16 *h, *q, *o, *act;  // the stage's own buffers, which hold the last layer's values after a step
+  __nv_bfloat16* kv_pool;
+  size_t layer_kv_elems;           // elements of one layer's K (or V) pages
+  const int32_t *tok_pos, *tok_slot, *decode_items, *seq_ctx, *block_tables;
+  const float2* rope;
+  int* sync;                       // two words, zero at entry: blocks that have arrived, and a flag of blocks that gave up
+  int* status;
+};
+// Tensor map of a 16-bit weight matrix [rows, K], K a multiple of 256, from which one copy brings eight rows of four consecutive
+// 256-column blocks as [block][eighth of it: one warp's 32 columns][row][64 bytes].
+template <typename Encode>
+inline bool encode_small_weight(Encode encode, CUtensorMap* m, const void* w, int rows, int K) {
+  cuuint64_t dims[4] = {32, cuuint64_t(rows), 8, cuuint64_t(K) / 256}, strides[3] = {cuuint64_t(K) * 2, 64, 512};
+  cuuint32_t box[4] = {32, 8, 8, 4}, estr[4] = {1, 1, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(w), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// The sizes of a stage and the rows of a step that the kernel takes.  Wider stages would fit, but their weights are long enough to
+// hide the launches: d_model = q_dim = 3072, 4 layers, one / eight rows on 148 SMs 146 -> 158, 146 -> 163 us (2048, 8 layers: 235 ->
+// 214, 228 -> 224, on 74 SMs 317 -> 233, 311 -> 238).
+bool small_step_supports(int T, int d, int q_dim, int kv_dim, int F, int head_dim, int n_layers);
+// Where it is the faster form.  Up to eight rows at every budget tried (2 .. 148 SMs).  With more, a block's load of the rows is
+// what a phase waits for, which wide rows and few blocks lengthen: 13 rows, d_model 2048, on 148 SMs 229 -> 255 us; the talker's 13 on
+// 28 / 8 / 2 540 -> 507, 1325 -> 1379, 4524 -> 5031; d_model 768 on 148 / 52 / 28 162 -> 161, 204 -> 187, 297 -> 273; 512 on 28 201 -> 209.
+// The results are the same bits, so the choice may look at the budget.
+bool small_step_wins(int T, int d, int q_dim, int sm_budget);
+cudaError_t launch_small_step(const SmallStepParams& p, int sm_budget, cudaStream_t stream);
+cudaError_t small_step_set_attributes();
+
 // ---------------------------------------------------------------- RMSNorm --
 // h[t,:] = bf16(x[t,:] * rsqrt(mean(x[t,:]^2) + eps) * g).  x comes either as bf16 (x_bf16, first layer;
 // x_f32_out then receives the widened copy that starts the fp32 residual stream) or as fp32 (x_f32).

@@ -1,0 +1,99 @@
+"""Small decode-only steps in one cooperative launch: against the oracle, and bit for bit -- outputs, cache and the stage's own
+buffers -- against the chain of launches that a profiled step is, at every budget."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.oracle import Oracle
+from paper_2608_01785_b200 import binding as B
+from paper_2608_01785_b200 import workloads as wl
+from tests.gpu_helpers import make_stage, run_step
+from tests.helpers import make_case, rel_err
+
+D = wl.StageDims
+# name: dims, cached tokens.  Two K steps per warp, a copy's four, one more, the most; heads per KV head from one to eight; rows of
+# one tile and of two, a tile full and one row more; new tokens at the first and the last place of a page; groups cut into
+# slices, more slices than blocks at the smaller budgets; one layer, and more than the three exchange buffers.
+CASES = {
+    "one_row": (D(4, 1024, 16, 4, 64, 2816), [300]),
+    "one_row_sliced": (D(2, 1024, 16, 4, 64, 2816), [4079]),
+    "first_token": (D(5, 512, 8, 2, 64, 512), [0]),
+    "page_edges": (D(3, 768, 12, 4, 64, 2048), [0, 14, 15, 16, 31, 32, 1023]),
+    "eight_heads_a_group": (D(3, 1024, 16, 2, 64, 1536), [700, 33, 255, 256, 1023, 5, 64, 300]),
+    "nine_rows": (D(4, 1024, 16, 2, 64, 3072), [31 * i + 2 for i in range(9)]),
+    "sixteen_rows": (D(2, 1024, 16, 4, 64, 2816), [61 * i + 15 for i in range(16)]),
+    "wide": (D(2, 2048, 32, 8, 64, 3072), [90, 17, 400]),
+    "one_head_a_group": (D(1, 1280, 20, 20, 64, 1280), [40, 200, 7]),
+}
+
+
+def _budgets(n, dims, sms):
+    return [b for b in (sms, 96, 52, 33, 5, 1) if B.hs_op_one_launch_step(n, dims, b) == 1]
+
+
+def _step(st, case, budget):
+    st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
+    y, pool = run_step(st, case, budget)
+    n = case.batch.n_seqs
+    return y, pool, *[st.debug_tensor(k)[:n].float().cpu().numpy() for k in ("h", "q", "o", "act")]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, B.HS_FLAG_BF16_ACTIVATIONS])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_one_launch_gives_the_bits_of_the_chain(name, flags):
+    dims, ctx = CASES[name]
+    case = make_case(dims, wl.BatchSpec([1] * len(ctx), ctx), seed=61, kv_fill=True)
+    st = make_stage(case, flags=flags)
+    try:
+        bias = [torch.randn(k, device=st.device).mul_(0.1).to(torch.bfloat16) for k in (dims.q_dim, dims.kv_dim, dims.kv_dim)]
+        budgets = _budgets(len(ctx), dims, st.sm_count)
+        assert budgets
+        for biased in (False, True):
+            if biased:
+                st.set_qkv_bias(dims.n_layers - 1, *bias)
+            B.hs_stage_profile_enable(st.handle, True)
+            want = _step(st, case, st.sm_count)
+            assert B.hs_stage_profile_read(st.handle)["gemm_qkv"][1] == dims.n_layers
+            B.hs_stage_profile_enable(st.handle, False)
+            for budget in budgets:
+                for a, b in zip(_step(st, case, budget), want):
+                    assert np.array_equal(a, b), (budget, biased)
+            if not biased:
+                y_ref = Oracle("f32").step(case.cfg, case.weights, case.kv_pool.copy(), case.batch.q_len, case.batch.ctx_len, case.block_tables, case.x)
+                assert rel_err(want[0], y_ref) <= 2e-2
+    finally:
+        st.close()
+
+
+@pytest.mark.gpu
+def test_steps_of_other_sizes_leave_nothing_behind_for_the_next():
+    """Rows come and go between steps of one stage, and NaN is a result like another: what a step finds in the exchange buffers
+    must not matter."""
+    dims = D(4, 1024, 16, 4, 64, 2816)
+    ctx = [100 + 37 * i for i in range(16)]
+    case = make_case(dims, wl.BatchSpec([1] * 16, ctx), seed=62, kv_fill=True)
+    st = make_stage(case)
+    try:
+        def step(n, x):
+            st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
+            return run_step(st, case, st.sm_count, [1] * n, ctx[:n], x[:n], case.block_tables[:n])[0]
+        first = {n: step(n, case.x_t) for n in (16, 3, 9, 1)}
+        bad = case.x_t.clone()
+        bad[0] = float("nan")
+        y = step(9, bad)
+        assert np.isnan(y[0]).all() and np.array_equal(y[1:], first[9][1:])
+        for n in (3, 16, 1, 9):
+            assert np.array_equal(step(n, case.x_t), first[n]), n
+    finally:
+        st.close()
+
+
+def test_the_rule_that_takes_the_one_launch():
+    t = wl.DIMS["c4_talker"]
+    assert [B.hs_op_one_launch_step(n, t, 148) for n in (1, 8, 9, 16, 17)] == [1, 1, 1, 1, 0]
+    assert [B.hs_op_one_launch_step(8, t, b) for b in (1, 52)] == [1, 1] and [B.hs_op_one_launch_step(9, t, b) for b in (31, 32)] == [0, 1]
+    for dims in (D(33, 1024, 16, 4, 64, 2816), D(2, 1024, 8, 4, 128, 2816), D(2, 1024, 16, 1, 64, 2816), D(2, 1088, 16, 4, 64, 2816),
+                 D(2, 1024, 16, 4, 64, 2832), D(2, 1024, 16, 4, 64, 3328), D(2, 2304, 16, 4, 64, 2816), wl.DIMS["c3_7b"], wl.DIMS["c2_shared"]):
+        assert B.hs_op_one_launch_step(4, dims, 148) == 0, dims
+    assert B.hs_op_one_launch_step(9, D(2, 1280, 16, 4, 64, 2816), 148) == 0 and B.hs_op_one_launch_step(0, t, 148) == -1
