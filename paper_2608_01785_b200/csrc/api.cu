@@ -214,6 +214,7 @@ hs_status_t ensure_attributes(int device) {
   if ((e = attention_set_attributes()) != cudaSuccess) return cuda_fail("attention attributes", e);
   if ((e = head_set_attributes()) != cudaSuccess) return cuda_fail("head attributes", e);
   if ((e = gemm_skinny_set_attributes()) != cudaSuccess) return cuda_fail("small-step gemm attributes", e);
+  if ((e = metadata_set_attributes()) != cudaSuccess) return cuda_fail("metadata attributes", e);
   if ((e = small_step_set_attributes()) != cudaSuccess) return cuda_fail("one-launch step attributes", e);
   if (device >= 0 && device < 64) g_attrs_set[device] = true;
   return HS_OK;
@@ -595,11 +596,22 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   if (st != HS_OK) return st;
   s->ring_pos = (slot + 1) % kRing;
 
+  // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
+  // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next
+  // kernel would wait on SMs outside the budget, so they are placed only when the last block in front has left (see
+  // OverlapMode).  (Not while the per-kernel timers run: an event between two kernels serialises them anyway.)
+  const int overlap = s->profile ? kOverlapNone : sm_budget == s->sm_count ? kOverlapEarly : kOverlapLate;
   int32_t* meta = reinterpret_cast<int32_t*>(s->ws_dev + s->ws.meta);
-  if (cudaMemcpyAsync(meta, s->pinned[slot], size_t(plan.meta_words) * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
-      cudaEventRecord(s->ev[slot], stream) != cudaSuccess)
-    return HS_ERR_CUDA;
-  s->ev_pending[slot] = true;
+  // the slot may be planned into again when the step is through (an event behind the first kernel would keep the second one's
+  // set-up from overlapping it)
+  struct SlotInUse {
+    hs_stage* s;
+    int slot;
+    cudaStream_t stream;
+    ~SlotInUse() { s->ev_pending[slot] = cudaEventRecord(s->ev[slot], stream) == cudaSuccess; }
+  } slot_in_use{s, slot, stream};
+  if (const cudaError_t fetched = launch_fetch_metadata(s->pinned[slot], meta, plan.meta_words, overlap, sm_budget, stream); fetched != cudaSuccess)
+    return cuda_fail("metadata", fetched);
 
   const int T = plan.n_tokens, d = c.d_model, F = c.d_ffn, Dh = c.head_dim;
   const int q_dim = c.n_q_heads * Dh, kv_dim = c.n_kv_heads * Dh;
@@ -621,11 +633,6 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
   const int gu_width = gemm_pick_gu_width(T, F, d, sm_budget);      // (the results do not depend on it)
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
-  // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
-  // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next
-  // kernel would wait on SMs outside the budget, so they are placed only when the last block in front has left (see
-  // OverlapMode).  (Not while the per-kernel timers run: an event between two kernels serialises them anyway.)
-  const int overlap = s->profile ? kOverlapNone : sm_budget == s->sm_count ? kOverlapEarly : kOverlapLate;
   // A operands of a small step are fetched with boxes of 64 or 32 rows instead of 128
   const int a_rows = use_pair ? 128 : (T <= 32 ? 32 : T <= 64 ? 64 : 128);
   const int a_sel = a_rows == 64 ? 0 : 1;

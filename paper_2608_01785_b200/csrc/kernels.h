@@ -188,6 +188,10 @@ cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_
 cudaError_t gemm_skinny_set_attributes();
 constexpr int kGemmTurnWords = 8192;   // capacity of the whose-turn array: splits are used only when tiles * 8 fits
 
+// The step's metadata from pinned host memory (a multiple of four words, 16-byte aligned).
+cudaError_t launch_fetch_metadata(const void* host, void* dev, int words, int overlap, int sm_budget, cudaStream_t stream);
+cudaError_t metadata_set_attributes();
+
 // ------------------------------------------------- a small step in one launch --
 // Decode-only step of at most 16 rows whose projections all stream weights past the rows, head_dim 64, at most eight query heads
 // per KV head, d_model and q_dim up to kSmallMaxModel, d_ffn up to kSmallMaxWidth, all three multiples of 256, as ONE cooperative
