@@ -19,6 +19,8 @@
 #pragma once
 #include <math.h>
 
+#include <type_traits>
+
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -51,6 +53,23 @@ __device__ __forceinline__ float quad_sum(float v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
+// The same over the eight lanes that share lane % 4.
+__device__ __forceinline__ float column_max(float v) {
+  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
+  v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
+  return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
+}
+__device__ __forceinline__ float column_sum(float v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 8);
+  return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+// Transposes an 8 x 8 matrix of 16-bit values of which lane l holds row l / 4, columns 2 (l % 4) and the next.
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t v) {
+  uint32_t t;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(t) : "r"(v));
+  return t;
+}
 // Zeroes the halves of a V fragment register whose keys (k, k + 1) are not below n_valid.
 __device__ __forceinline__ uint32_t mask_v(uint32_t r, int k, int n_valid) {
   if (k >= n_valid) return 0u;
@@ -58,10 +77,24 @@ __device__ __forceinline__ uint32_t mask_v(uint32_t r, int k, int n_valid) {
   return r;
 }
 
-// Running state of one warp's attention: rows lane / 4 and lane / 4 + 8 of the G query heads, unnormalised output, maximum (log2
-// domain) and this lane's share of the sum.
+// Running state of one warp's attention over the pages of an item: the group's queries, unnormalised outputs, maxima (log2 domain)
+// and sums.  page(): one page in shared memory, n_valid keys of which belong to the item (16 or more: all).  put(): what an item
+// leaves, output rows `pitch` floats apart and (max, sum) per head.  store(): the normalised output of an item that is a whole
+// sequence, with the saturation report of fp16 (see note_f16_saturation).
+// A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
+// bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs,
+// the V fragments are fetched while the scores are on their way, and a page on which no row's maximum moves --
+// most of them, after the first few -- needs a vote, but no shuffles and no rescale.  (A reference that follows the
+// maximum only beyond a factor of 256 is another 1 - 2 % faster, but leaves the largest weight rounded: error against
+// 64 bits up to 6 % larger.)  Against a loop with one chain of MMAs, shuffles and exp2f on every page and V fetched
+// behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker step of 16
+// rows 300.5 -> 289 us, of 11 rows on 52 SMs 471 -> 457; at config-3 dimensions 9 rows, 4 layers 493 -> 483 us, 29 rows
+// on 96 SMs 796 -> 782, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.16 ms.
+//
+// More than eight heads: the heads are the MMA's sixteen rows; this lane has rows lane / 4 and lane / 4 + 8.
 template <int DH>
-struct Attend {
+struct HeadsAsRows {
+  uint32_t qf[DH / 16][4];
   float o[DH / 8][4], m_a, m_b, l_a, l_b;
   __device__ __forceinline__ void clear() {
 #pragma unroll
@@ -69,93 +102,232 @@ struct Attend {
     m_a = m_b = -INFINITY;
     l_a = l_b = 0.f;
   }
-};
-// One page in shared memory, n_valid keys of which belong to the item (16 or more: all).
-// A page is a chain of dependent steps in one warp (two warps per scheduler): its latency, not the bytes, is what
-// bounds a batch that does not saturate the HBM.  So the scores of a page are two chains of DH / 32 MMAs per key
-// half, the V fragments are fetched while the scores are on their way, and a page on which no row's maximum moves --
-// most of them, after the first few -- needs a vote, but no shuffles and no rescale.  (A reference that follows the
-// maximum only beyond a factor of 256 is another 1 - 2 % faster, but leaves the largest weight rounded: error against
-// 64 bits up to 6 % larger.)  Against a loop with one chain of MMAs, shuffles and exp2f on every page and V fetched
-// behind the softmax (1250 cycles per page at head_dim 128 with the page already in shared memory): talker step of 16
-// rows 300.5 -> 289 us, of 11 rows on 52 SMs 471 -> 457; at config-3 dimensions 9 rows, 4 layers 493 -> 483 us, 29 rows
-// on 96 SMs 796 -> 782, 64 rows, 28 layers (HBM-bound) 5.20 -> 5.16 ms.
-// TWO: rows lane / 4 + 8 are in use (groups of more than eight heads).
-template <int DH, bool TWO = true>
-__device__ __forceinline__ void attend_page(Attend<DH>& at, const uint32_t (&qf)[DH / 16][4], uint32_t k_base, uint32_t v_base, int n_valid,
-                                            int lane, float scale_log2) {
-  float (&o)[DH / 8][4] = at.o;
-  float &m_a = at.m_a, &m_b = at.m_b, &l_a = at.l_a, &l_b = at.l_b;
-  float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  float sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+  __device__ __forceinline__ void load_q(const __nv_bfloat16* q, int G, int lane) {
+    const int ra = lane >> 2, rb = ra + 8;
 #pragma unroll
-  for (int ks = 0; ks < DH / 16; ks += 2) {
-    uint32_t kf[4], kg[4];
-    const int kk = (lane & 7) + (lane >> 4) * 8, cc = 2 * ks + ((lane >> 3) & 1);
-    ldmatrix_x4(kf, k_base + kv_off(kk, cc));
-    ldmatrix_x4(kg, k_base + kv_off(kk, cc + 2));
-    mma_bf16_16816(sc[0], qf[ks], kf[0], kf[1]);
-    mma_bf16_16816(sc[1], qf[ks], kf[2], kf[3]);
-    mma_bf16_16816(sd[0], qf[ks + 1], kg[0], kg[1]);
-    mma_bf16_16816(sd[1], qf[ks + 1], kg[2], kg[3]);
+    for (int ks = 0; ks < DH / 16; ++ks) {
+      const int c = ks * 16 + 2 * (lane & 3);
+      qf[ks][0] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(q + ra * DH + c)) : 0u;
+      qf[ks][1] = rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(q + rb * DH + c)) : 0u;
+      qf[ks][2] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(q + ra * DH + c + 8)) : 0u;
+      qf[ks][3] = rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(q + rb * DH + c + 8)) : 0u;
+    }
   }
-  uint32_t vf[DH / 16][4];
+  __device__ __forceinline__ void page(uint32_t k_base, uint32_t v_base, int n_valid, int lane, float scale_log2) {
+    float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    float sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-  for (int dp = 0; dp < DH / 16; ++dp) {
-    const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
-    ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, cc));
-  }
+    for (int ks = 0; ks < DH / 16; ks += 2) {
+      uint32_t kf[4], kg[4];
+      const int kk = (lane & 7) + (lane >> 4) * 8, cc = 2 * ks + ((lane >> 3) & 1);
+      ldmatrix_x4(kf, k_base + kv_off(kk, cc));
+      ldmatrix_x4(kg, k_base + kv_off(kk, cc + 2));
+      mma_bf16_16816(sc[0], qf[ks], kf[0], kf[1]);
+      mma_bf16_16816(sc[1], qf[ks], kf[2], kf[3]);
+      mma_bf16_16816(sd[0], qf[ks + 1], kg[0], kg[1]);
+      mma_bf16_16816(sd[1], qf[ks + 1], kg[2], kg[3]);
+    }
+    uint32_t vf[DH / 16][4];
 #pragma unroll
-  for (int j = 0; j < 2; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) sc[j][e] += sd[j][e];
-  if (n_valid < 16) {
-    const int k = 2 * (lane & 3);
+    for (int dp = 0; dp < DH / 16; ++dp) {
+      const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = 2 * dp + (lane >> 4);
+      ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, cc));
+    }
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (8 * j + k + (e & 1) >= n_valid) sc[j][e] = -INFINITY;
+      for (int e = 0; e < 4; ++e) sc[j][e] += sd[j][e];
+    if (n_valid < 16) {
+      const int k = 2 * (lane & 3);
 #pragma unroll
-    for (int dp = 0; dp < DH / 16; ++dp)
+      for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], k + 8 * (e & 1), n_valid);
-  }
-  const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
-  const float mx_b = TWO ? fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2 : -INFINITY;
-  if (__any_sync(0xffffffffu, mx_a > m_a || (TWO && mx_b > m_b))) {
-    const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = TWO ? fmaxf(m_b, quad_max(mx_b)) : 0.f;
-    const float al_a = fast_exp2(m_a - mn_a), al_b = TWO ? fast_exp2(m_b - mn_b) : 0.f;
-    m_a = mn_a;
-    m_b = mn_b;
-    l_a *= al_a;
-    l_b *= al_b;
+        for (int e = 0; e < 4; ++e)
+          if (8 * j + k + (e & 1) >= n_valid) sc[j][e] = -INFINITY;
 #pragma unroll
-    for (int j = 0; j < DH / 8; ++j) {
-      o[j][0] *= al_a; o[j][1] *= al_a;
-      if (TWO) { o[j][2] *= al_b; o[j][3] *= al_b; }
+      for (int dp = 0; dp < DH / 16; ++dp)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], k + 8 * (e & 1), n_valid);
+    }
+    const float mx_a = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1])) * scale_log2;
+    const float mx_b = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3])) * scale_log2;
+    if (__any_sync(0xffffffffu, mx_a > m_a || mx_b > m_b)) {
+      const float mn_a = fmaxf(m_a, quad_max(mx_a)), mn_b = fmaxf(m_b, quad_max(mx_b));
+      const float al_a = fast_exp2(m_a - mn_a), al_b = fast_exp2(m_b - mn_b);
+      m_a = mn_a;
+      m_b = mn_b;
+      l_a *= al_a;
+      l_b *= al_b;
+#pragma unroll
+      for (int j = 0; j < DH / 8; ++j) {
+        o[j][0] *= al_a; o[j][1] *= al_a;
+        o[j][2] *= al_b; o[j][3] *= al_b;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      sc[j][0] = fast_exp2(fmaf(sc[j][0], scale_log2, -m_a));
+      sc[j][1] = fast_exp2(fmaf(sc[j][1], scale_log2, -m_a));
+      sc[j][2] = fast_exp2(fmaf(sc[j][2], scale_log2, -m_b));
+      sc[j][3] = fast_exp2(fmaf(sc[j][3], scale_log2, -m_b));
+    }
+    l_a += (sc[0][0] + sc[0][1]) + (sc[1][0] + sc[1][1]);
+    l_b += (sc[0][2] + sc[0][3]) + (sc[1][2] + sc[1][3]);
+    uint32_t pf[4];
+    pf[0] = pack_bf16(sc[0][0], sc[0][1]);
+    pf[1] = pack_bf16(sc[0][2], sc[0][3]);
+    pf[2] = pack_bf16(sc[1][0], sc[1][1]);
+    pf[3] = pack_bf16(sc[1][2], sc[1][3]);
+#pragma unroll
+    for (int dp = 0; dp < DH / 16; ++dp) {
+      mma_bf16_16816(o[2 * dp], pf, vf[dp][0], vf[dp][1]);
+      mma_bf16_16816(o[2 * dp + 1], pf, vf[dp][2], vf[dp][3]);
     }
   }
+  __device__ __forceinline__ void put(float* po, int pitch, float2* pml, int G, int lane) {
+    const int ra = lane >> 2, rb = ra + 8;
+    l_a = quad_sum(l_a);
+    l_b = quad_sum(l_b);
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    sc[j][0] = fast_exp2(fmaf(sc[j][0], scale_log2, -m_a));
-    sc[j][1] = fast_exp2(fmaf(sc[j][1], scale_log2, -m_a));
-    sc[j][2] = TWO ? fast_exp2(fmaf(sc[j][2], scale_log2, -m_b)) : 0.f;
-    sc[j][3] = TWO ? fast_exp2(fmaf(sc[j][3], scale_log2, -m_b)) : 0.f;
+    for (int j = 0; j < DH / 8; ++j) {
+      const int col = 8 * j + 2 * (lane & 3);
+      if (ra < G) *reinterpret_cast<float2*>(po + ra * pitch + col) = make_float2(o[j][0], o[j][1]);
+      if (rb < G) *reinterpret_cast<float2*>(po + rb * pitch + col) = make_float2(o[j][2], o[j][3]);
+    }
+    if ((lane & 3) == 0) {
+      if (ra < G) pml[ra] = make_float2(m_a, l_a);
+      if (rb < G) pml[rb] = make_float2(m_b, l_b);
+    }
   }
-  l_a += (sc[0][0] + sc[0][1]) + (sc[1][0] + sc[1][1]);
-  if (TWO) l_b += (sc[0][2] + sc[0][3]) + (sc[1][2] + sc[1][3]);
-  uint32_t pf[4];
-  pf[0] = pack_bf16(sc[0][0], sc[0][1]);
-  pf[1] = pack_bf16(sc[0][2], sc[0][3]);
-  pf[2] = pack_bf16(sc[1][0], sc[1][1]);
-  pf[3] = pack_bf16(sc[1][2], sc[1][3]);
+  __device__ __forceinline__ void store(__nv_bfloat16* out, bool f16, int* status, int G, int lane) {
+    const int ra = lane >> 2, rb = ra + 8;
+    const float inv_a = 1.f / quad_sum(l_a), inv_b = 1.f / quad_sum(l_b);
 #pragma unroll
-  for (int dp = 0; dp < DH / 16; ++dp) {
-    mma_bf16_16816(o[2 * dp], pf, vf[dp][0], vf[dp][1]);
-    mma_bf16_16816(o[2 * dp + 1], pf, vf[dp][2], vf[dp][3]);
+    for (int j = 0; j < DH / 8; ++j) {
+      const int col = 8 * j + 2 * (lane & 3);
+      const float a[2] = {o[j][0], o[j][1]}, b[2] = {o[j][2], o[j][3]};
+      if (ra < G) {
+        if (f16) note_f16_saturation(a, status, inv_a);
+        *reinterpret_cast<uint32_t*>(out + ra * DH + col) = pack_act(a[0] * inv_a, a[1] * inv_a, f16);
+      }
+      if (rb < G) {
+        if (f16) note_f16_saturation(b, status, inv_b);
+        *reinterpret_cast<uint32_t*>(out + rb * DH + col) = pack_act(b[0] * inv_b, b[1] * inv_b, f16);
+      }
+    }
   }
-}
+};
+// At most eight: the keys are the rows of the scores' MMA and the head dimension those of the outputs', the heads their eight
+// columns, so that no half of a tile is padding: half the MMAs, and as an MMA takes its scheduler ten cycles, they were most of a
+// page (in shared memory, cycles at head_dim 128 / 64: 784 -> 597, 473 -> 392).  This lane has heads 2 (lane % 4) and the next one; keys, and
+// dimensions, lane / 4 and lane / 4 + 8.  The scores become the second product's operand by two 8 x 8 transpositions.
+// Steps, us: eleven rows of the talker on 52 SMs 368 -> 364, 16 on 148 260.2 -> 259.6; at 7B dimensions 29 rows on 96 SMs 642 -> 639, 64
+// rows 4801 -> 4787.
+template <int DH>
+struct HeadsAsColumns {
+  uint32_t qf[DH / 16][2];
+  float o[DH / 16][4], m[2], l[2];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < DH / 16; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+    m[0] = m[1] = -INFINITY;
+    l[0] = l[1] = 0.f;
+  }
+  __device__ __forceinline__ void load_q(const __nv_bfloat16* q, int G, int lane) {
+    const int h = lane >> 2;
+#pragma unroll
+    for (int ks = 0; ks < DH / 16; ++ks)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) qf[ks][e] = h < G ? __ldcg(reinterpret_cast<const uint32_t*>(q + h * DH + ks * 16 + 8 * e + 2 * (lane & 3))) : 0u;
+  }
+  __device__ __forceinline__ void page(uint32_t k_base, uint32_t v_base, int n_valid, int lane, float scale_log2) {
+    const int key = lane >> 2;
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+    {
+      const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = lane >> 4;
+#pragma unroll
+      for (int ks = 0; ks < DH / 16; ks += 2) {
+        uint32_t kf[4], kg[4];
+        ldmatrix_x4(kf, k_base + kv_off(kk, 2 * ks + cc));
+        ldmatrix_x4(kg, k_base + kv_off(kk, 2 * ks + 2 + cc));
+        mma_bf16_16816(s, kf, qf[ks][0], qf[ks][1]);
+        mma_bf16_16816(s2, kg, qf[ks + 1][0], qf[ks + 1][1]);
+      }
+    }
+    uint32_t vf[DH / 16][4];
+    {
+      const int kk = (lane & 7) + (lane >> 4) * 8, cc = (lane >> 3) & 1;
+#pragma unroll
+      for (int dp = 0; dp < DH / 16; ++dp) ldmatrix_x4_trans(vf[dp], v_base + kv_off(kk, 2 * dp + cc));
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] += s2[e];
+    if (n_valid < 16) {
+      if (key >= n_valid) s[0] = s[1] = -INFINITY;
+      if (key + 8 >= n_valid) s[2] = s[3] = -INFINITY;
+#pragma unroll
+      for (int dp = 0; dp < DH / 16; ++dp)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) vf[dp][e] = mask_v(vf[dp][e], 2 * (lane & 3) + 8 * (e >> 1), n_valid);
+    }
+    const float mx0 = fmaxf(s[0], s[2]) * scale_log2, mx1 = fmaxf(s[1], s[3]) * scale_log2;
+    if (__any_sync(0xffffffffu, mx0 > m[0] || mx1 > m[1])) {
+      const float mn0 = fmaxf(m[0], column_max(mx0)), mn1 = fmaxf(m[1], column_max(mx1));
+      const float al0 = fast_exp2(m[0] - mn0), al1 = fast_exp2(m[1] - mn1);
+      m[0] = mn0;
+      m[1] = mn1;
+      l[0] *= al0;
+      l[1] *= al1;
+#pragma unroll
+      for (int j = 0; j < DH / 16; ++j) {
+        o[j][0] *= al0; o[j][1] *= al1;
+        o[j][2] *= al0; o[j][3] *= al1;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] = fast_exp2(fmaf(s[e], scale_log2, -m[e & 1]));
+    l[0] += s[0] + s[2];
+    l[1] += s[1] + s[3];
+    const uint32_t p0 = transpose_8x8(pack_bf16(s[0], s[1])), p1 = transpose_8x8(pack_bf16(s[2], s[3]));
+#pragma unroll
+    for (int dp = 0; dp < DH / 16; ++dp) mma_bf16_16816(o[dp], vf[dp], p0, p1);
+  }
+  __device__ __forceinline__ void put(float* po, int pitch, float2* pml, int G, int lane) {
+    const int d = lane >> 2, h = 2 * (lane & 3);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      l[e] = column_sum(l[e]);
+      if (h + e < G) {
+#pragma unroll
+        for (int j = 0; j < DH / 16; ++j) {
+          po[(h + e) * pitch + 16 * j + d] = o[j][e];
+          po[(h + e) * pitch + 16 * j + d + 8] = o[j][e + 2];
+        }
+        if (d == 0) pml[h + e] = make_float2(m[e], l[e]);
+      }
+    }
+  }
+  __device__ __forceinline__ void store(__nv_bfloat16* out, bool f16, int* status, int G, int lane) {
+    const int d = lane >> 2, h = 2 * (lane & 3);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float inv = 1.f / column_sum(l[e]);
+      if (h + e < G) {
+#pragma unroll
+        for (int j = 0; j < DH / 16; ++j) {
+          const float v[2] = {o[j][e], o[j][e + 2]};
+          if (f16) note_f16_saturation(v, status, inv);
+          const uint32_t w = pack_act(v[0] * inv, v[1] * inv, f16);
+          uint16_t* at = reinterpret_cast<uint16_t*>(out) + (h + e) * DH + 16 * j + d;
+          at[0] = uint16_t(w);
+          at[8] = uint16_t(w >> 16);
+        }
+      }
+    }
+  }
+};
+template <int DH, bool TWO>
+using Heads = std::conditional_t<TWO, HeadsAsRows<DH>, HeadsAsColumns<DH>>;
 
 // Merges the partials of one (sequence, KV head) group -- items first .. first + splits - 1 -- in split
 // order and writes the normalised output rows.  LPH lanes share one query head, each owning DH / LPH
@@ -265,39 +437,23 @@ constexpr int dc_smem_bytes() {
   return b > kMinSmemBytes ? b : kMinSmemBytes;
 }
 
-// Group mode, a warp's part of a slice, into an area of its own: [ROWS][DH] unnormalised output, then [ROWS] (max, sum); ROWS is at
-// least G.
-template <int DH, int ROWS>
-__device__ __forceinline__ void slice_partial(uint8_t* slots, const float (&o)[DH / 8][4], float m_a, float m_b, float l_a, float l_b, int G,
-                                              int lane) {
-  const int ra = lane >> 2, rb = ra + 8;
-  float* po = reinterpret_cast<float*>(slots);
-  float2* pml = reinterpret_cast<float2*>(slots + ROWS * DH * 4);
-#pragma unroll
-  for (int j = 0; j < DH / 8; ++j) {
-    const int col = 8 * j + 2 * (lane & 3);
-    if (ra < G) *reinterpret_cast<float2*>(po + ra * DH + col) = make_float2(o[j][0], o[j][1]);
-    if (rb < G) *reinterpret_cast<float2*>(po + rb * DH + col) = make_float2(o[j][2], o[j][3]);
-  }
-  if ((lane & 3) == 0) {
-    if (ra < G) pml[ra] = make_float2(m_a, l_a);
-    if (rb < G) pml[rb] = make_float2(m_b, l_b);
-  }
-}
-// The eight warps' parts of a slice, PITCH bytes apart, merged in order: head g, columns col and col + 1, unnormalised, with the
+// Floats between the heads of a warp's part of a slice in shared memory (conflict-free for HeadsAsColumns::put).
+template <int DH>
+constexpr int kPartPitch = DH + 4;
+// The eight warps' parts of a slice, [ROWS][kPartPitch] output and [ROWS] (max, sum) each, PITCH bytes apart, merged in order: head g, columns col and col + 1, unnormalised, with the
 // maximum and the sum.
 template <int DH, int ROWS, int PITCH, int UNROLL = DC_WARPS>
 __device__ __forceinline__ void merge_eight(const uint8_t* parts, int g, int col, float& mm, float& ll, float& o0, float& o1) {
   mm = -INFINITY;
 #pragma unroll UNROLL
-  for (int w = 0; w < DC_WARPS; ++w) mm = fmaxf(mm, reinterpret_cast<const float2*>(parts + w * PITCH + ROWS * DH * 4)[g].x);
+  for (int w = 0; w < DC_WARPS; ++w) mm = fmaxf(mm, reinterpret_cast<const float2*>(parts + w * PITCH + ROWS * kPartPitch<DH> * 4)[g].x);
   ll = 0.f, o0 = 0.f, o1 = 0.f;
 #pragma unroll UNROLL
   for (int w = 0; w < DC_WARPS; ++w) {
     const uint8_t* base = parts + w * PITCH;
-    const float2 ml = reinterpret_cast<const float2*>(base + ROWS * DH * 4)[g];
+    const float2 ml = reinterpret_cast<const float2*>(base + ROWS * kPartPitch<DH> * 4)[g];
     const float f = exp2f(ml.x - mm);                 // 0 for an empty slice (max = -inf)
-    const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + g * DH + col);
+    const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + g * kPartPitch<DH> + col);
     ll += f * ml.y;
     o0 += f * v.x;
     o1 += f * v.y;
@@ -325,9 +481,7 @@ __device__ __forceinline__ void merge_slices(const float2 (&ml)[8], const float2
 // The body of the decode kernel.  `smem`: 1024-byte aligned, DC_WARPS * DC_STAGES * 2 pages; `full_all`: DC_WARPS *
 // DC_STAGES mbarriers followed by two ints (the abort flag; a flag of the block's) in shared memory outside that area.
 // SLICED: group mode with groups of several slices (the merge of those is no part of the other instantiation: it was 2 us of the
-// talker step of 16 rows, twelve launches, that has none).  TWO: groups of more than eight heads (attend_page); the others carry
-// none of the second eight rows' maxima, exponentials and stores: us per launch at 7B dimensions, 64 rows 61.8 -> 60.9, 29 on 96 SMs
-// 45.9 -> 44.5, nine 17.5 -> 16.8.
+// talker step of 16 rows, twelve launches, that has none).  TWO: groups of more than eight heads (Heads).
 template <int DH, bool SLICED, bool TWO>
 __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* smem, uint64_t* full_all) {
   using G_ = Geom<DH>;
@@ -340,6 +494,8 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
   const int G = TWO ? p.n_q_heads / p.n_kv_heads : min(p.n_q_heads / p.n_kv_heads, 8);     // (so that the compiler knows)
   const int q_dim = p.n_q_heads * DH;
   const float scale_log2 = kLog2e / sqrtf(float(DH));
+  constexpr int kRows = TWO ? 16 : 8;               // heads that a warp's part of a slice has room for
+  static_assert(kRows * kPartPitch<DH> * 4 + kRows * 8 <= DC_STAGES * SLOT_BYTES, "in the warp's ring");
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < DC_WARPS * DC_STAGES; ++i) mbar_init(&full_all[i], 1);
@@ -429,19 +585,9 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
 
     // Q fragments straight from global memory: rows = query heads hk*G .. hk*G + G - 1 of the new token
     const __nv_bfloat16* qrow = p.q + size_t(tok) * q_dim + size_t(hk) * G * DH;
-    const int ra = lane >> 2, rb = ra + 8;
-    uint32_t qf[DH / 16][4];
-#pragma unroll
-    for (int ks = 0; ks < DH / 16; ++ks) {
-      const int c = ks * 16 + 2 * (lane & 3);
-      qf[ks][0] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + ra * DH + c)) : 0u;
-      qf[ks][1] = TWO && rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + rb * DH + c)) : 0u;
-      qf[ks][2] = ra < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + ra * DH + c + 8)) : 0u;
-      qf[ks][3] = TWO && rb < G ? __ldcg(reinterpret_cast<const uint32_t*>(qrow + rb * DH + c + 8)) : 0u;
-    }
-    Attend<DH> at;
+    Heads<DH, TWO> at;
+    at.load_q(qrow, G, lane);
     at.clear();
-    float (&o_acc)[DH / 8][4] = at.o;
     bool ok = true;
 
     for (int pi = 0; pi < n_pages; ++pi) {
@@ -454,15 +600,15 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
       const uint32_t v_base = k_base + G_::PAGE_BYTES;
       if (++cur == DC_STAGES) { cur = 0; cur_phase ^= 1; }
       const int n_valid = k1 - (k0 + pi * 16);            // keys of this page that belong to the item
-      attend_page<DH, TWO>(at, qf, k_base, v_base, n_valid, lane, scale_log2);
+      at.page(k_base, v_base, n_valid, lane, scale_log2);
       __syncwarp();                         // every lane is done with this slot before lane 0 refills it
     }
     if (!ok && !group_mode) break;
 
-    const float m_a = at.m_a, m_b = at.m_b, l_a = quad_sum(at.l_a), l_b = quad_sum(at.l_b);
     __nv_bfloat16* orow = p.o + size_t(tok) * q_dim + size_t(hk) * G * DH;
     if (group_mode) {
-      slice_partial<DH, 16>(slots, at.o, m_a, m_b, l_a, l_b, G, lane);
+      // this slice's part into the warp's own (now idle) page ring
+      at.put(reinterpret_cast<float*>(slots), kPartPitch<DH>, reinterpret_cast<float2*>(slots + kRows * kPartPitch<DH> * 4), G, lane);
       const bool failed = __syncthreads_or(!ok) != 0;      // the same answer in every warp of the block
       if (!failed) {
         // the eight partials are merged in order by the whole block: a thread per pair of output columns
@@ -478,7 +624,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
         for (int e = threadIdx.x; e < G * (DH / 2); e += DC_THREADS) {
           const int g = e / (DH / 2), col = 2 * (e - g * (DH / 2));
           float mm, ll, o0, o1;
-          merge_eight<DH, 16, DC_STAGES * SLOT_BYTES>(smem, g, col, mm, ll, o0, o1);
+          merge_eight<DH, kRows, DC_STAGES * SLOT_BYTES>(smem, g, col, mm, ll, o0, o1);
           if (!SLICED || splits == 1) {
             store(g, col, o0, o1, ll);
           } else {
@@ -524,45 +670,11 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
     }
     if (splits == 1) {
       // the whole key range was this item: normalise and write the output rows directly
-      const float inv_a = 1.f / l_a, inv_b = 1.f / l_b;
-      if (p.o_f16) {                        // saturation report of the fp16 output (see note_f16_saturation)
-        float mx_oa = 0.f, mx_ob = 0.f;
-#pragma unroll
-        for (int j = 0; j < DH / 8; ++j) {
-          mx_oa = fmaxf(mx_oa, fmaxf(fabsf(o_acc[j][0]), fabsf(o_acc[j][1])));
-          mx_ob = fmaxf(mx_ob, fmaxf(fabsf(o_acc[j][2]), fabsf(o_acc[j][3])));
-        }
-        if ((ra < G && mx_oa * inv_a > 65504.f) || (rb < G && mx_ob * inv_b > 65504.f)) {
-          int c = 0;
-#pragma unroll
-          for (int j = 0; j < DH / 8; ++j) {
-            if (ra < G) c += (fabsf(o_acc[j][0] * inv_a) > 65504.f) + (fabsf(o_acc[j][1] * inv_a) > 65504.f);
-            if (rb < G) c += (fabsf(o_acc[j][2] * inv_b) > 65504.f) + (fabsf(o_acc[j][3] * inv_b) > 65504.f);
-          }
-          atomicAdd(p.status + 1, c);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < DH / 8; ++j) {
-        const int col = 8 * j + 2 * (lane & 3);
-        if (ra < G) *reinterpret_cast<uint32_t*>(orow + ra * DH + col) = pack_act(o_acc[j][0] * inv_a, o_acc[j][1] * inv_a, p.o_f16 != 0);
-        if (rb < G) *reinterpret_cast<uint32_t*>(orow + rb * DH + col) = pack_act(o_acc[j][2] * inv_b, o_acc[j][3] * inv_b, p.o_f16 != 0);
-      }
+      at.store(orow, p.o_f16 != 0, p.status, G, lane);
       continue;
     }
     // the item's partial: unnormalised output, running max (log2 domain) and sum, rows = query heads
-    float* po = p.part_o + size_t(part) * 16 * DH;
-    float* pml = p.part_ml + size_t(part) * 16 * 2;
-#pragma unroll
-    for (int j = 0; j < DH / 8; ++j) {
-      const int col = 8 * j + 2 * (lane & 3);
-      if (ra < G) *reinterpret_cast<float2*>(po + ra * DH + col) = make_float2(o_acc[j][0], o_acc[j][1]);
-      if (rb < G) *reinterpret_cast<float2*>(po + rb * DH + col) = make_float2(o_acc[j][2], o_acc[j][3]);
-    }
-    if ((lane & 3) == 0) {
-      if (ra < G) { pml[ra * 2] = m_a; pml[ra * 2 + 1] = l_a; }
-      if (rb < G) { pml[rb * 2] = m_b; pml[rb * 2 + 1] = l_b; }
-    }
+    at.put(p.part_o + size_t(part) * 16 * DH, DH, reinterpret_cast<float2*>(p.part_ml) + size_t(part) * 16, G, lane);
     // The warp that completes the last split of a (sequence, KV head) merges all of its splits, always in
     // split order, so the result does not depend on which warp that is.
     __threadfence();

@@ -37,7 +37,7 @@ constexpr int kTile = kChunk * SK_WARPS * 512, kSlot = 2 * kTile;    // bytes of
 static_assert(kSlot == SK_WARPS * PAGE2, "a slot holds a piece's chunk, or a page for every warp");
 constexpr int kRing = 5;                                      // slots
 constexpr int kTileRows = 64, kPartRow = 20;                  // rows of all the partial tiles reduced at a time; floats between two
-constexpr int kGroupRows = 8, kSlicePitch = kGroupRows * DH * 4 + kGroupRows * 8;     // most heads of a group; a warp's part of a slice
+constexpr int kGroupRows = 8, kSlicePitch = kGroupRows * kPartPitch<DH> * 4 + kGroupRows * 8;     // most heads of a group; a warp's part of a slice
 constexpr int kPartBytes = SK_WARPS * kTileRows * kPartRow * 4, kPartAt = kRing * kSlot, kTailAt = kPartAt + kPartBytes;
 constexpr int kBarriers = 2 * kRing + 2, kSmallSmem = 1024 + kTailAt + kBarriers * 8 + 256;
 static_assert(SK_WARPS * kSlicePitch <= kPartBytes, "the parts of a slice lie where the partial tiles do");
@@ -598,28 +598,27 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_step_kernel(const __gr
       const Slice s = i == block ? mine : slice_of(i);
       const int hk = s.it.y, k0 = s.it.z, k1 = s.it.w, tok = s.dr.y, splits = s.dr.w & 0xffff, n_pages = (k1 - k0 + 15) >> 4;
       // q of the group's heads, and for the warp with the last key the new token's key and value (16 bytes a lane)
-      uint32_t qf[DH / 16][4];
+      HeadsAsColumns<DH> at;
+      at.clear();
       uint4 kv = make_uint4(0u, 0u, 0u, 0u);
       const bool has_new = n_pages > 0 && k1 == __ldg(p.seq_ctx + s.dr.x) + 1;
       const int need_q = n_pages > 0 && g < G ? 1 : 0, need_kv = has_new ? 16 : 0;
 #pragma unroll
-      for (int ks = 0; ks < DH / 16; ++ks) qf[ks][0] = qf[ks][1] = qf[ks][2] = qf[ks][3] = 0u;
+      for (int ks = 0; ks < DH / 16; ++ks) at.qf[ks][0] = at.qf[ks][1] = 0u;
       const uint8_t* q_src = now + p.at.q + uint32_t(tok * p.q_dim + (hk * G + g) * DH + 2 * t) * 2;
       const uint8_t* kv_src = now + (lane < 8 ? p.at.k : p.at.v) + uint32_t(tok * p.kv_dim + hk * DH + (lane & 7) * 8) * 2;
       uint32_t most;
       do {
 #pragma unroll
         for (int ks = 0; ks < DH / 16; ++ks) {
-          load_below(qf[ks][0], q_src + ks * 32, 0, need_q);
-          load_below(qf[ks][2], q_src + ks * 32 + 16, 0, need_q);
+          load_below(at.qf[ks][0], q_src + ks * 32, 0, need_q);
+          load_below(at.qf[ks][1], q_src + ks * 32 + 16, 0, need_q);
         }
         load_below(kv, kv_src, lane, need_kv);
         most = largest(0u, kv);
 #pragma unroll
-        for (int ks = 0; ks < DH / 16; ++ks) most = max(most, max(qf[ks][0], qf[ks][2]));
+        for (int ks = 0; ks < DH / 16; ++ks) most = max(most, max(at.qf[ks][0], at.qf[ks][1]));
       } while (again(most == kEmpty, gave_up));
-      Attend<DH> at;
-      at.clear();
       bool ok = true;
 #pragma unroll 1
       for (int c = 0; c < s.columns; ++c) {
@@ -634,11 +633,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_step_kernel(const __gr
             __syncwarp();
           }
           const uint32_t k_base = smem_u32(page);
-          attend_page<DH, false>(at, qf, k_base, k_base + Geom<DH>::PAGE_BYTES, n_valid, lane, scale_log2);
+          at.page(k_base, k_base + Geom<DH>::PAGE_BYTES, n_valid, lane, scale_log2);
         }
         release();
       }
-      slice_partial<DH, kGroupRows>(smem + kPartAt + warp * kSlicePitch, at.o, at.m_a, 0.f, quad_sum(at.l_a), 0.f, min(G, 8), lane);
+      uint8_t* part = smem + kPartAt + warp * kSlicePitch;
+      at.put(reinterpret_cast<float*>(part), kPartPitch<DH>, reinterpret_cast<float2*>(part + kGroupRows * kPartPitch<DH> * 4), G, lane);
       if (block_any(!ok)) return;
 #pragma unroll 1
       for (int e = tid; e < G * (DH / 2); e += SK_THREADS) {
