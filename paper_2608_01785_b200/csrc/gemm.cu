@@ -600,14 +600,6 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
             const int col0 = n * p.bn + c * 32;
             const int xi = c % 3;
             uint8_t* bx = landing(xi);
-            if (lane == 0 && c > 0) {
-              bulk_wait_read<0>();                         // the stores of the previous chunk have read their blocks
-              if (c + 2 < n_chunks) {                      // ... so its landing block can take the chunk two further on
-                const int xn = (c + 2) % 3;
-                mbar_expect_tx(&xb_bar[xn], EPI_BUF_BYTES);
-                tma_load_2d(landing(xn), &p.tm_out, &xb_bar[xn], col0 + 64, row_base);
-              }
-            }
             tmem_ld32(taddr + c * 32, r0);
             uint4 gw[4];                               // 32 gains (bf16), the same for every row
             const int nv = p.N - col0 >= 32 ? 8 : (p.N - col0) >> 2;
@@ -629,6 +621,16 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
               r0[4 * u] = __float_as_uint(x0); r0[4 * u + 1] = __float_as_uint(x1);
               r0[4 * u + 2] = __float_as_uint(x2); r0[4 * u + 3] = __float_as_uint(x3);
             }
+            // (here and not at the chunk's start, where that wait was 600 cycles of every chunk's 2300)
+            if (lane == 0 && c > 0) {
+              bulk_wait_read<0>();                         // the stores of the previous chunk have read their blocks
+              if (c + 2 < n_chunks) {                      // ... so its landing block can take the chunk two further on
+                const int xn = (c + 2) % 3;
+                mbar_expect_tx(&xb_bar[xn], EPI_BUF_BYTES);
+                tma_load_2d(landing(xn), &p.tm_out, &xb_bar[xn], col0 + 64, row_base);
+              }
+            }
+            __syncwarp();
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const uint32_t pk[4] = {gw[e].x, gw[e].y, gw[e].z, gw[e].w};
