@@ -195,13 +195,17 @@ __device__ __forceinline__ void scale32(uint32_t (&r)[32], float s) {
 __device__ __forceinline__ void finish_row_norm(const GemmParams& p, int row, bool row_ok, int row_group, int n,
                                                 int n_n_tiles, float ss, int lane) {
   if (row_ok) p.row_ss[size_t(row) * p.ss_stride + n] = ss;
-  __threadfence();
   __syncwarp();
+  // (One lane's count releases the warp's partials and acquires the others'.  A fence of every lane on both sides: out and down of a
+  // small backbone, 5776 rows, 61.6 and 99.7 us instead of 60.6 and 98.7.)
   int last = 0;
-  if (lane == 0) last = atomicAdd(p.row_group_done + row_group, 1) == n_n_tiles - 1;
+  if (lane == 0) {
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(last) : "l"(p.row_group_done + row_group) : "memory");
+    last = last == n_n_tiles - 1;
+  }
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) return;
-  __threadfence();
+  __syncwarp();
   if (row_ok) {
     float sum = 0.f;
     for (int i = 0; i < n_n_tiles; ++i) sum += __ldcg(p.row_ss + size_t(row) * p.ss_stride + i);
