@@ -180,6 +180,8 @@ int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K);
  * Returns -1 for M, K or sm_budget < 1, or N < 64.
  */
 int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
+/* The same of more than 128 rows, on pairs or single blocks as a device of 148 SMs has them; -1 for M <= 128, N < 64 or sm_budget < 1. */
+int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget);
 
 /*
  * Host-only: weight rows per block of the weight-streaming kernel for a residual GEMM of M rows, width N and contraction length

@@ -557,6 +557,10 @@ int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget) 
   return M < 1 || N < 64 || K < 1 || sm_budget < 1 ? -1 : gemm_pick_gu_width(M, N, K, sm_budget);
 }
 
+int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget) {
+  return M <= 128 || N < 64 || sm_budget < 1 ? -1 : gemm_pick_tall_gu_width(M, N, sm_budget, on_pairs(M, 2 * N, 256, 148));
+}
+
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
   return sm_budget < 1 || !gemm_skinny_supports(M, K, N, kGemmResid, 0) ? -1 : gemm_skinny_rows(M, K, N, kGemmResid, 0, sm_budget);
 }
@@ -631,7 +635,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   auto pair_for = [&](int n_cols, int single_bn) { return on_pairs(T, n_cols, single_bn, s->sm_count); };
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
-  const int gu_width = gemm_pick_gu_width(T, F, d, sm_budget);      // (the results do not depend on it)
+  const int gu_width = use_pair ? gemm_pick_tall_gu_width(T, F, sm_budget, pair_gu) : gemm_pick_gu_width(T, F, d, sm_budget);   // (the results do not depend on it)
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // A operands of a small step are fetched with boxes of 64 or 32 rows instead of 128
   const int a_rows = use_pair ? 128 : (T <= 32 ? 32 : T <= 64 ? 64 : 128);
@@ -944,7 +948,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
       else k.in_row_rs = gu.in_row_rs;
       LaunchTimer t(s, 6, stream); where = "gate/up gemm"; e = launch_gemm_skinny(k, sm_budget, stream);
     } else {
-      if (!pair_gu && gu_width != 128) {
+      if (gu_width != 128) {
         gu.gu_width = gu_width;
         for (int i = 0; i < 2; ++i) gu.tm_b[i] = m.gu_narrow[(gu_width - kGuMinWidth) / 16][i];
       }

@@ -59,12 +59,11 @@ static_assert(GEMM_SMEM >= kMinSmemBytes, "one block per SM");
 // tile never straddles q | k | v (their widths are multiples of 128) and holds whole heads.
 __host__ __device__ __forceinline__ int gemm_qkv_width(const GemmParams& p) { return p.bn == 128 && !p.pair ? 128 : BN; }
 
-// GateUp mode: activation columns of a tile, 128, or on single blocks p.gu_width.
-__host__ __device__ __forceinline__ int gemm_gu_width(const GemmParams& p) { return p.gu_width > 0 && !p.pair ? p.gu_width : 128; }
+// GateUp mode: activation columns of a tile, 128 or p.gu_width.
+__host__ __device__ __forceinline__ int gemm_gu_width(const GemmParams& p) { return p.gu_width > 0 ? p.gu_width : 128; }
 
 // Output-tile width: 256 virtual columns, except in Resid mode where the launcher picks p.bn (a multiple
-// of 32 in [128, 256]) from the problem shape so that the tile count fills whole waves of SMs, and in GateUp mode on
-// single blocks.
+// of 32 in [128, 256]) from the problem shape so that the tile count fills whole waves of SMs, and in GateUp mode.
 __host__ __device__ __forceinline__ int gemm_n_tiles(const GemmParams& p) {
   if (p.mode == kGemmGateUp) return (p.N + gemm_gu_width(p) - 1) / gemm_gu_width(p);
   const int bn = p.mode == kGemmResid ? p.bn : gemm_qkv_width(p);
@@ -314,8 +313,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // small step buy depth -- 8 or 9 stages instead of 4.
   const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) > 128;
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
-  // (a narrow GateUp tile: its gate rows, and right behind them its up rows, one operand of 2 gu_w rows)
-  const int gu_w = MODE == kGemmGateUp && !PAIR ? gemm_gu_width(p) : 128, bh_bytes = gu_w * BK * 2;
+  // (a narrow GateUp tile: its gate rows, and right behind them -- in a pair, in the other block -- its up rows, one operand of
+  // 2 gu_w rows)
+  const int gu_w = MODE == kGemmGateUp ? gemm_gu_width(p) : 128, bh_bytes = gu_w * BK * 2;
   const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * bh_bytes;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
@@ -399,7 +399,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   auto load_b = [&](int s, int kb, const BSource& b0, const BSource& b1) {
     uint8_t* st = smem + s * STAGE_BYTES;
     if (PAIR) {
-      if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
+      if (rank == 0) mbar_expect_tx(&full[s], 2 * (A_BYTES + bh_bytes));
       tma_load_2d_pair(st + b_off, &p.tm_b[b0.map], mapa_u32(smem_u32(&full[s]), 0), kb * BK, b0.row);
     } else {
       mbar_expect_tx(&full[s], a_bytes + (two_halves ? 2 * bh_bytes : bh_bytes));
@@ -462,7 +462,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
-                                                 PAIR ? BN : MODE == kGemmResid ? p.bn : MODE == kGemmQkv ? gemm_qkv_width(p) : 2 * gu_w) &
+                                                 MODE == kGemmGateUp ? 2 * gu_w : PAIR ? BN : MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) &
                              (p.ab_f16 ? ~(63u << 7) : ~0u);
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
@@ -1080,7 +1080,7 @@ int gemm_pick_stream_k(int M, int N, int K, int sm_count) {
   return double(tiles) / W < 0.92 * rounds ? W : 0;
 }
 
-// Activation columns of a GateUp tile on single blocks, from the SMs the launch gets: an output element's sum is the same
+// Activation columns of a GateUp tile of at most 128 rows, from the SMs the launch gets: an output element's sum is the same
 // whatever the tile's width, so this choice may look at the budget.  Tiles of 128 columns at 7B dimensions, 148 of them, are
 // one round on the whole device but two on 96 to 147 SMs.  Time per K block: the larger of issue, shared memory, an SM's intake
 // -- 80 KB/us of the weights and 4.5 KB more, which is what narrow boxes pay -- and its share of the HBM; 1.1 us per further
@@ -1100,6 +1100,26 @@ int gemm_pick_gu_width(int M, int N, int K, int sms) {
     };
     const int rest = tiles - (rounds - 1) * sms;
     const double us = k_blocks * ((rounds - 1) * k_block_us(sms) + k_block_us(rest)) + (rounds - 1) * 1.1;
+    if (us < best_us * 0.97) { best_us = us; best = w; }
+  }
+  return best;
+}
+
+// The same for more than 128 rows: rounds, times the longer of the tensor core's time and of an SM's intake per K block (127 KB/us out of
+// the L2; a block has its rows and, of a pair, half of the weight rows).  Tiles of 128 columns left the last round of 1024 rows and d_ffn
+// 2816 nearly empty -- 88 tiles on 74 pairs.  Measured on B200, us per launch there (K = 1024), 128 / 112 / 96 / 80 / 64 / 48 columns: 17.4 /
+// 16.4 / 15.5 / 15.3 (taken) / 17.8 / 20.8.  Steps, 128 columns -> the width taken: that one 925 -> 908; 400 rows on 148 / 120 / 112 / 74 / 37
+// SMs 730 -> 708 (80), 745 -> 728 (96), 746 -> 739 (112), 942 -> 910 (80), 1189 -> 1167 (112); 504 rows of a small backbone (d_ffn 5632) on
+// 148 SMs 395 -> 378 (80).  On single blocks, 256 rows, 148 / 120 / 96 / 74 SMs: 679 -> 657 (48), 758 -> 731 (48), 759 -> 732 (64), 759 -> 738
+// (80).  5776 rows of the backbone keep 128 (16 rounds of 112 columns for 14 are 2.5 us slower).
+int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair) {
+  const int units = pair ? sms / 2 : sms, m_tiles = (M + (pair ? 2 : 1) * BM - 1) / ((pair ? 2 : 1) * BM);
+  if (units < 1) return 128;
+  int best = 128;
+  double best_us = 1e30;
+  for (int w = 128; w >= kGuMinWidth; w -= 16) {
+    const int rounds = (m_tiles * ((N + w - 1) / w) + units - 1) / units;
+    const double us = rounds * std::max(0.275 * w / 128, (A_BYTES + (pair ? 1 : 2) * w * BK * 2) / 127e3);
     if (us < best_us * 0.97) { best_us = us; best = w; }
   }
   return best;

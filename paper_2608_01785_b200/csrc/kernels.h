@@ -67,7 +67,7 @@ struct GemmParams {
   int gate_which;
   // GateUp
   CUtensorMap tm_act;        // bf16 act [M, N], box 64 x 32, 128-byte swizzle
-  int gu_width;              // single blocks: activation columns per tile when not 128 (gemm_pick_gu_width); then tm_b has
+  int gu_width;              // activation columns per tile when not 128 (gemm_pick_gu_width); then tm_b has
   __nv_bfloat16* act;        // boxes of as many rows, and act [M, N] is written with plain stores
   int* status;               // device status word; with act_f16 the word after it counts saturated act values
   int act_f16;               // GateUp: 1 = write act as fp16, 0 = bf16
@@ -97,9 +97,11 @@ cudaError_t gemm_set_attributes();
 // Tile width for a Resid-mode GEMM of this shape on a device with sm_count SMs (budget independent).
 int gemm_pick_bn(int M, int N, int sm_count);
 int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count);
-// Activation columns per tile of a GateUp GEMM on single blocks with `sms` SMs: 128, or kGuMinWidth + 16 i, i < kGuNarrow.
+// Activation columns per tile of a GateUp GEMM with `sms` SMs: 128, or kGuMinWidth + 16 i, i < kGuNarrow.  Of at most 128 rows (128 for
+// more), and of more, on pairs or on single blocks.
 constexpr int kGuMinWidth = 48, kGuNarrow = 5;
 int gemm_pick_gu_width(int M, int N, int K, int sms);
+int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair);
 // Where split i (0 .. ks) of a tile's k_blocks begins.  The splits add their sums one after the other, a link of that
 // chain costing about as long as kSplitSkew K blocks take to stream; so each split is that much longer than the one
 // before it and finishes just when its turn comes, instead of all finishing together and then queueing.  Equal
