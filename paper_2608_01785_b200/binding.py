@@ -30,7 +30,7 @@ EXPORTS = ("hs_status_str", "hs_kv_pool_bytes", "hs_workspace_bytes", "hs_stage_
            "hs_head_destroy", "hs_op_embed", "hs_temporal_create", "hs_temporal_step", "hs_temporal_destroy",
            "hs_stage_set_qkv_bias", "hs_stage_set_modulation", "hs_stage_saturation_count", "hs_op_wait_probe",
            "hs_op_decode_attention_noalloc_status", "hs_stage_plan_attention", "hs_op_gemm_split_begin",
-           "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width", "hs_op_gate_up_tile",
+           "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width", "hs_op_gate_up_tile", "hs_op_qkv_tile",
            "hs_op_weight_streaming_rows", "hs_op_one_launch_step")
 PROFILE_CLASSES = ("rmsnorm", "gemm_qkv", "attn_prefill", "attn_decode", "attn_combine", "gemm_out", "gemm_gateup",
                    "gemm_down")
@@ -122,6 +122,8 @@ def lib() -> C.CDLL:
         l.hs_op_gate_up_width.restype = C.c_int32
         l.hs_op_gate_up_tile.argtypes = [C.c_int32] * 3
         l.hs_op_gate_up_tile.restype = C.c_int32
+        l.hs_op_qkv_tile.argtypes = [C.c_int32] * 3
+        l.hs_op_qkv_tile.restype = C.c_int32
         l.hs_op_one_launch_step.argtypes = [C.c_int32] * 8
         l.hs_op_one_launch_step.restype = C.c_int32
         l.hs_op_weight_streaming_rows.argtypes = [C.c_int32] * 4
@@ -289,6 +291,10 @@ def hs_op_gate_up_width(M: int, N: int, K: int, sm_budget: int) -> int:
 
 def hs_op_gate_up_tile(M: int, N: int, sm_budget: int) -> int:
     return int(lib().hs_op_gate_up_tile(M, N, sm_budget))
+
+
+def hs_op_qkv_tile(M: int, N: int, sm_budget: int) -> int:
+    return int(lib().hs_op_qkv_tile(M, N, sm_budget))
 
 
 def hs_op_one_launch_step(rows: int, dims, sm_budget: int) -> int:

@@ -159,6 +159,7 @@ bool encode_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, u
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, wgate, wup, wdown;
   CUtensorMap gu_narrow[kGuNarrow][2];     // gate and up weights in boxes of kGuMinWidth + 16 i rows
+  CUtensorMap qkv_narrow[3];               // q, k and v weights in boxes of 32 rows
 };
 
 struct DeviceGuard {
@@ -417,7 +418,8 @@ hs_status_t hs_stage_create(const hs_stage_config_t* cfg, const hs_layer_weights
     ok = encode_2d(&m.wq, w.w_q, q_dim, d, 128) && encode_2d(&m.wk, w.w_k, kv_dim, d, 128) &&
          encode_2d(&m.wv, w.w_v, kv_dim, d, 128) && encode_2d(&m.wo, w.w_o, d, q_dim, 128) &&
          encode_2d(&m.wgate, w.w_gate, F, d, 128) && encode_2d(&m.wup, w.w_up, F, d, 128) &&
-         encode_2d(&m.wdown, w.w_down, d, F, 128);
+         encode_2d(&m.wdown, w.w_down, d, F, 128) && encode_2d(&m.qkv_narrow[0], w.w_q, q_dim, d, 32) &&
+         encode_2d(&m.qkv_narrow[1], w.w_k, kv_dim, d, 32) && encode_2d(&m.qkv_narrow[2], w.w_v, kv_dim, d, 32);
     for (int i = 0; i < kGuNarrow && ok; ++i)
       ok = encode_2d(&m.gu_narrow[i][0], w.w_gate, F, d, kGuMinWidth + 16 * i) && encode_2d(&m.gu_narrow[i][1], w.w_up, F, d, kGuMinWidth + 16 * i);
   }
@@ -561,6 +563,10 @@ int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget) {
   return M <= 128 || N < 64 || sm_budget < 1 ? -1 : gemm_pick_tall_gu_width(M, N, sm_budget, on_pairs(M, 2 * N, 256, 148));
 }
 
+int32_t hs_op_qkv_tile(int32_t M, int32_t N, int32_t sm_budget) {
+  return M <= 128 || N < 128 || sm_budget < 1 || !on_pairs(M, N, 128, 148) ? -1 : gemm_pick_pair_qkv_width(M, N, sm_budget);
+}
+
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
   return sm_budget < 1 || !gemm_skinny_supports(M, K, N, kGemmResid, 0) ? -1 : gemm_skinny_rows(M, K, N, kGemmResid, 0, sm_budget);
 }
@@ -636,6 +642,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
   const int gu_width = use_pair ? gemm_pick_tall_gu_width(T, F, sm_budget, pair_gu) : gemm_pick_gu_width(T, F, d, sm_budget);   // (the results do not depend on it)
+  const int qkv_width = gemm_pick_pair_qkv_width(T, q_dim + 2 * kv_dim, sm_budget);
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // A operands of a small step are fetched with boxes of 64 or 32 rows instead of 128
   const int a_rows = use_pair ? 128 : (T <= 32 ? 32 : T <= 64 ? 64 : 128);
@@ -830,12 +837,14 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     g.tm_a = a_rows == 128 ? s->tm_h : s->tm_h_s[a_sel];
     g.a_box_rows = a_rows;
     g.tm_b[0] = m.wq; g.tm_b[1] = m.wk; g.tm_b[2] = m.wv;
+    if (pair_qkv && qkv_width != 256)
+      for (int i = 0; i < 3; ++i) g.tm_b[i] = m.qkv_narrow[i];
     g.M = T; g.N = q_dim + 2 * kv_dim; g.K = d;
     g.mode = kGemmQkv;
     g.ab_f16 = f16;
     g.overlap = overlap;
     g.pair = pair_qkv;
-    g.bn = pair_qkv ? 256 : 128;     // small steps: 128-column tiles, twice as many SMs stream the weights
+    g.bn = pair_qkv ? qkv_width : 128;     // small steps: 128-column tiles, twice as many SMs stream the weights
     g.q_dim = q_dim; g.kv_dim = kv_dim; g.head_dim = Dh; g.n_kv_heads = c.n_kv_heads;
     g.q_out = q;
     g.k_cache = s->kv_pool + (size_t(l) * 2 + 0) * layer_kv_elems;

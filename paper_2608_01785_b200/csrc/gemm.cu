@@ -57,7 +57,17 @@ static_assert(GEMM_SMEM >= kMinSmemBytes, "one block per SM");
 // Qkv mode, single blocks: tiles of 128 virtual columns (one B box) when p.bn says so -- the launcher asks for
 // them at small M, where the tile count decides how many SMs stream weights; 256 otherwise.  A 128-column
 // tile never straddles q | k | v (their widths are multiples of 128) and holds whole heads.
-__host__ __device__ __forceinline__ int gemm_qkv_width(const GemmParams& p) { return p.bn == 128 && !p.pair ? 128 : BN; }
+// Pairs: 256, or 192 where p.bn says so (gemm_pick_pair_qkv_width).  Such a tile is three units of two 32-column pieces that rotate
+// with each other, 32 p .. of the two halves of a head; each piece is a B box of its own, so that a tile may begin and end inside a
+// head or a projection.
+constexpr int QKV_NARROW = 192;
+__host__ __device__ __forceinline__ int gemm_qkv_width(const GemmParams& p) {
+  return p.pair ? (p.bn == QKV_NARROW ? QKV_NARROW : BN) : p.bn == 128 ? 128 : BN;
+}
+// First column of unit u of [q | k | v]; its partners are half a head further.
+__device__ __forceinline__ int qkv_unit_col(const GemmParams& p, int u) {
+  return p.head_dim == 128 ? (u >> 1) * 128 + (u & 1) * 32 : u * 64;
+}
 
 // GateUp mode: activation columns of a tile, 128 or p.gu_width.
 __host__ __device__ __forceinline__ int gemm_gu_width(const GemmParams& p) { return p.gu_width > 0 ? p.gu_width : 128; }
@@ -71,14 +81,20 @@ __host__ __device__ __forceinline__ int gemm_n_tiles(const GemmParams& p) {
 }
 
 struct BSource { int map, row; };
-__device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int half) {
-  if (p.mode == kGemmResid) return {0, n_tile * p.bn + half * 128};
-  if (p.mode == kGemmGateUp) return {half, n_tile * gemm_gu_width(p)};
-  int v = n_tile * gemm_qkv_width(p) + half * 128;
+__device__ __forceinline__ BSource qkv_source(const GemmParams& p, int v) {
   if (v < p.q_dim) return {0, v};
   v -= p.q_dim;
   if (v < p.kv_dim) return {1, v};
   return {2, v - p.kv_dim};
+}
+__device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int half) {
+  if (p.mode == kGemmResid) return {0, n_tile * p.bn + half * 128};
+  if (p.mode == kGemmGateUp) return {half, n_tile * gemm_gu_width(p)};
+  return qkv_source(p, n_tile * gemm_qkv_width(p) + half * 128);
+}
+// Piece `piece` (0 .. 5) of a 192-column tile (past the end of v the boxes lie outside the matrix and read zeros)
+__device__ __forceinline__ BSource qkv_piece(const GemmParams& p, int n_tile, int piece) {
+  return qkv_source(p, qkv_unit_col(p, n_tile * 3 + (piece >> 1)) + (piece & 1) * (p.head_dim >> 1));
 }
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -315,7 +331,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
   // (a narrow GateUp tile: its gate rows, and right behind them -- in a pair, in the other block -- its up rows, one operand of
   // 2 gu_w rows)
-  const int gu_w = MODE == kGemmGateUp ? gemm_gu_width(p) : 128, bh_bytes = gu_w * BK * 2;
+  const int gu_w = MODE == kGemmGateUp ? gemm_gu_width(p) : 128;
+  const int bh_bytes = (PAIR && MODE == kGemmQkv ? gemm_qkv_width(p) / 2 : gu_w) * BK * 2;
+  const bool qkv_narrow = PAIR && MODE == kGemmQkv && gemm_qkv_width(p) == QKV_NARROW;
   const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * bh_bytes;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
@@ -396,11 +414,16 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   const bool two_halves = b_two;
   // One stage's requests of the producer thread: the weight boxes (which also arm the barrier) and the A box.  In a
   // pair both blocks' bytes are counted on the leader's barrier, which the leader arms for both.
-  auto load_b = [&](int s, int kb, const BSource& b0, const BSource& b1) {
+  auto load_b = [&](int s, int kb, const BSource& b0, const BSource& b1, const BSource& b2) {
     uint8_t* st = smem + s * STAGE_BYTES;
     if (PAIR) {
       if (rank == 0) mbar_expect_tx(&full[s], 2 * (A_BYTES + bh_bytes));
-      tma_load_2d_pair(st + b_off, &p.tm_b[b0.map], mapa_u32(smem_u32(&full[s]), 0), kb * BK, b0.row);
+      const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
+      tma_load_2d_pair(st + b_off, &p.tm_b[b0.map], bar, kb * BK, b0.row);
+      if (qkv_narrow) {
+        tma_load_2d_pair(st + b_off + 32 * BK * 2, &p.tm_b[b1.map], bar, kb * BK, b1.row);
+        tma_load_2d_pair(st + b_off + 64 * BK * 2, &p.tm_b[b2.map], bar, kb * BK, b2.row);
+      }
     } else {
       mbar_expect_tx(&full[s], a_bytes + (two_halves ? 2 * bh_bytes : bh_bytes));
       tma_load_2d(st + b_off, &p.tm_b[b0.map], &full[s], kb * BK, b0.row);
@@ -420,10 +443,12 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     have_unit = walk.next(un);
     if (have_unit) {
       const int n = un.tile / n_m_tiles;
-      const BSource b0 = b_source(p, n, PAIR ? int(rank) : 0), b1 = b_source(p, n, 1);
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b2 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 2) : b1;
       b_ahead = un.kb_end - un.kb_begin < STAGES ? un.kb_end - un.kb_begin : STAGES;
       if (elect_one())
-        for (int i = 0; i < b_ahead; ++i) load_b(i, un.kb_begin + i, b0, b1);
+        for (int i = 0; i < b_ahead; ++i) load_b(i, un.kb_begin + i, b0, b1, b2);
     }
   }
   griddep_wait();                 // everything above is set-up; the operands belong to the previous kernel until here
@@ -442,13 +467,15 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     while (ok && have_unit) {
       const int tile = un.tile;
       const int m = tile % n_m_tiles, n = tile / n_m_tiles;
-      const BSource b0 = b_source(p, n, PAIR ? int(rank) : 0), b1 = b_source(p, n, 1);
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b2 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 2) : b1;
       const int kb_end = un.kb_end;
       for (int kb = un.kb_begin; kb < kb_end; ++kb) {
         ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         if (elect_one()) {
-          if (b_ahead == 0) load_b(s, kb, b0, b1);
+          if (b_ahead == 0) load_b(s, kb, b0, b1, b2);
           load_a(s, kb, m, un.half);
         }
         if (b_ahead > 0) --b_ahead;
@@ -462,7 +489,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
-                                                 MODE == kGemmGateUp ? 2 * gu_w : PAIR ? BN : MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) &
+                                                 MODE == kGemmGateUp ? 2 * gu_w : MODE == kGemmQkv ? gemm_qkv_width(p) : PAIR ? BN : p.bn) &
                              (p.ab_f16 ? ~(63u << 7) : ~0u);
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
@@ -535,7 +562,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           pos = p.tok_pos[row];
           slot = p.tok_slot[row];
         }
-        const float2* cs = p.rope + size_t(pos) * (Dh >> 1) + (Dh == 128 ? 32 * cg : 0);
+        const float2* cs = p.rope + size_t(pos) * (Dh >> 1) + (Dh == 128 ? 32 * ((n * (gemm_qkv_width(p) / 64) + cg) & 1) : 0);
         asm volatile("prefetch.global.L1 [%0];\n\tprefetch.global.L1 [%0 + 128];" ::"l"(cs));
       }
       // folded RMSNorm, producing side: the first two blocks of this warp's rows of y are on their way before the
@@ -818,30 +845,30 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           }
         }
       } else {
-        const int half_dh = Dh >> 1;
-        const int qkv_w = gemm_qkv_width(p);
-        for (int half = 0; half < qkv_w / 128; ++half) {
-          int vcol = n * qkv_w + half * 128;      // virtual column of this half in [q | k | v]
+        // units of two 32-column pieces that rotate with each other, every other one this warp's
+        const int half_dh = Dh >> 1, n_units = gemm_qkv_width(p) / 64;
+        const bool apart = Dh == 128 && !qkv_narrow;           // (whole heads of 128: the partners are 64 columns apart)
+        for (int i = cg; i < n_units; i += 2) {
+          const int unit = n * n_units + i, vcol = qkv_unit_col(p, unit), part = Dh == 128 ? unit & 1 : 0;   // column of [q | k | v]
           if (vcol >= p.N) break;
-          int region = 0;
-          if (vcol >= p.q_dim) { region = 1; vcol -= p.q_dim; }
-          if (region == 1 && vcol >= p.kv_dim) { region = 2; vcol -= p.kv_dim; }
+          int region = 0, col = vcol;
+          if (col >= p.q_dim) { region = 1; col -= p.q_dim; }
+          if (region == 1 && col >= p.kv_dim) { region = 2; col -= p.kv_dim; }
           const __nv_bfloat16* bias = p.qkv_bias[region];      // of this region's projection, or null
-          // this warp's two 32-column chunks of the half: rotation partners (q and k heads; the same pairs in both halves)
-          const int lo = Dh == 128 ? cg : 2 * cg, hi = lo + (Dh == 128 ? 2 : 1);
-          tmem_ld32(taddr + half * 128 + lo * 32, r0);
-          tmem_ld32(taddr + half * 128 + hi * 32, r1);
+          const int at = apart ? (i >> 1) * 128 + (i & 1) * 32 : i * 64;
+          tmem_ld32(taddr + at, r0);
+          tmem_ld32(taddr + at + (apart ? 64 : 32), r1);
           tmem_ld_wait();
           if (p.in_row_rs) {
             scale32(r0, rs);
             scale32(r1, rs);
           }
           if (bias) {                                          // the bias comes before the rotation
-            add_bias32(r0, bias + vcol + lo * 32);
-            add_bias32(r1, bias + vcol + hi * 32);
+            add_bias32(r0, bias + col);
+            add_bias32(r1, bias + col + half_dh);
           }
           if (region != 2) {
-            const float2* cs = p.rope + size_t(pos) * half_dh + (Dh == 128 ? 32 * cg : 0);
+            const float2* cs = p.rope + size_t(pos) * half_dh + 32 * part;
 #pragma unroll
             for (int e = 0; e < 32; e += 4) {
               float t[8];                                      // cos, sin of pairs e .. e + 3
@@ -856,16 +883,10 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
             }
           }
           if (row_ok) {
-            const int col_lo = vcol + lo * 32, col_hi = vcol + hi * 32;
-            if (region == 0) {
-              __nv_bfloat16* qrow = p.q_out + size_t(row) * p.q_dim;
-              store_bf16x32(qrow + col_lo, r0);
-              store_bf16x32(qrow + col_hi, r1);
-            } else {
-              __nv_bfloat16* cache = region == 1 ? p.k_cache : p.v_cache;
-              store_bf16x32(cache_ptr(cache, slot, col_lo / Dh, p.n_kv_heads, Dh, col_lo % Dh), r0);
-              store_bf16x32(cache_ptr(cache, slot, col_hi / Dh, p.n_kv_heads, Dh, col_hi % Dh), r1);
-            }
+            __nv_bfloat16* to = region == 0 ? p.q_out + size_t(row) * p.q_dim + col
+                                            : cache_ptr(region == 1 ? p.k_cache : p.v_cache, slot, col / Dh, p.n_kv_heads, Dh, col % Dh);
+            store_bf16x32(to, r0);
+            store_bf16x32(to + half_dh, r1);
           }
         }
       }
@@ -1123,6 +1144,23 @@ int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair) {
     if (us < best_us * 0.97) { best_us = us; best = w; }
   }
   return best;
+}
+
+// Columns of a pair's Qkv tile, 256 or 192, by the same rounds and times: 48 tiles of 256 columns (1024 rows, 3072 columns) leave a third of
+// the 74 pairs idle, 64 of 192 do not and are shorter (15.6 -> 13.8 us a launch); 162 tiles (2112 rows, 4608 columns) are 2.19 rounds run
+// as three, 216 are 2.92 (75 -> 68 us).  Steps on B200, 256 -> 192 columns: denoising, 1024 rows, 909 -> 887 us; a small backbone (K = 2048,
+// 3072 columns), 1004 and 2104 rows 537 -> 526, 834 -> 816; 7B dimensions, 4 layers, 604, 1104, 1504, 2052 rows 1353 -> 1337, 2053 ->
+// 2035, 2519 -> 2463, 3657 -> 3617; 2 layers on 96 SMs, 904 and 1504 rows 1112 -> 1086, 1601 -> 1583.  Not where the last round of 256
+// columns is nearly empty, which is then a fast one: 1254 rows of the small backbone on 112 SMs (60 tiles on 56 pairs) 779 -> 797, 3204 rows
+// on 148 (156 on 74) 1198 -> 1207; nor for more rounds (5404 rows, five for four, 1892 -> 1935).
+int gemm_pick_pair_qkv_width(int M, int N, int sms) {
+  const int pairs = sms / 2, m_tiles = (M + 2 * BM - 1) / (2 * BM);
+  if (pairs < 1) return BN;
+  auto tiles = [&](int w) { return m_tiles * ((N + w - 1) / w); };
+  auto cost = [&](int w) { return (tiles(w) + pairs - 1) / pairs * std::max(0.275 * w / BN, (A_BYTES + w * BK) / 127e3); };
+  const int rest = tiles(BN) % pairs;
+  if (tiles(BN) > pairs && rest > 0 && rest * 8 < pairs) return BN;
+  return cost(QKV_NARROW) < 0.97 * cost(BN) ? QKV_NARROW : BN;
 }
 
 cudaError_t launch_gemm(const GemmParams& p, int sm_budget, cudaStream_t stream) {

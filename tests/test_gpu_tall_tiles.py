@@ -1,6 +1,8 @@
-"""Gate/up GEMM of more than 128 rows: the width of its tiles follows the budget, on pairs of SMs and on single blocks; the results do not."""
+"""GEMMs of more than 128 rows whose tiles' width follows the budget -- gate/up on pairs of SMs and on single blocks, QKV on pairs --
+while the results do not."""
 import numpy as np
 import pytest
+import torch
 
 from oracle.oracle import Oracle
 from paper_2608_01785_b200 import binding as B
@@ -32,6 +34,45 @@ def test_tile_width_does_not_reach_the_output(name, flags):
     y_ref = Oracle("f32").step(case.cfg, case.weights, case.kv_pool.copy(), q_len, ctx_len, case.block_tables, case.x)
     st = make_stage(case, flags=flags)
     try:
+        first = None
+        for budget in BUDGETS:
+            st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
+            out = run_step(st, case, budget)
+            first = out if first is None else first
+            assert np.array_equal(out[0], first[0]) and np.array_equal(out[1], first[1]), budget
+        assert rel_err(first[0], y_ref) <= 2e-2        # the rule of every parity test (16-bit operands)
+    finally:
+        st.close()
+
+
+# QKV on pairs: heads of 64 and of 128, tiles that end inside a head and a projection, a last tile of one or two units of three, a ragged
+# row tile; with biases and behind a folded norm.
+QKV_CASES = {
+    "dh128_split_heads": (wl.StageDims(1, 256, 28, 4, 128, 256), [600], [0], False),
+    "dh128_bias_ragged": (wl.StageDims(1, 264, 22, 2, 128, 264), [500, 77, 1], [0, 30, 5], True),
+    "dh64_projections_inside_a_tile": (wl.StageDims(1, 256, 40, 4, 64, 256), [1000, 1], [0, 9], True),
+    "dh128_folded": (wl.StageDims(2, 2048, 16, 4, 128, 2816), [1025], [3], False),
+}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, B.HS_FLAG_BF16_ACTIVATIONS])
+@pytest.mark.parametrize("name", sorted(QKV_CASES))
+def test_qkv_tile_width_does_not_reach_the_output(name, flags):
+    dims, q_len, ctx_len, bias = QKV_CASES[name]
+    n = (dims.n_q_heads + 2 * dims.n_kv_heads) * dims.head_dim
+    assert {B.hs_op_qkv_tile(sum(q_len), n, k) for k in BUDGETS} == {192, 256}
+    case = make_case(dims, wl.BatchSpec(q_len, ctx_len), seed=83, kv_fill=True)
+    st = make_stage(case, flags=flags)
+    try:
+        weights = case.weights
+        if bias:
+            g = torch.Generator().manual_seed(7)
+            for l in range(dims.n_layers):
+                b = [(torch.randn(k * dims.head_dim, generator=g) * 0.5).to(torch.bfloat16) for k in (dims.n_q_heads, dims.n_kv_heads, dims.n_kv_heads)]
+                st.set_qkv_bias(l, *[t.to(st.device) for t in b])
+                weights = weights[:l] + [dict(weights[l], **{k: t.float().numpy() for k, t in zip(("b_q", "b_k", "b_v"), b)})] + weights[l + 1:]
+        y_ref = Oracle("f32").step(case.cfg, weights, case.kv_pool.copy(), q_len, ctx_len, case.block_tables, case.x)
         first = None
         for budget in BUDGETS:
             st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
