@@ -22,7 +22,8 @@
 // stands and the row put in place in shared memory.
 // Measured on B200, talker step, separate launches -> this, on 148 / 96 / 52 / 28 SMs: one row 245 -> 207, 295 -> 207, 339 -> 240,
 // 484 -> 317 us; eight 262 -> 222, 313 -> 222, 354 -> 273, 529 -> 369; eleven 297 -> 278, 342 -> 288, 384 -> 371, 594 -> 556; sixteen
-// 277 -> 267, 326 -> 285, 411 -> 406, 602 -> 572.
+// 277 -> 267, 326 -> 285, 411 -> 406, 602 -> 572.  With a kernel that fetches the metadata and the heads as columns: one row 183, sixteen
+// 263, eleven on 52 SMs 363.
 #include "attention_decode.cuh"
 #include "hs_internal.h"
 #include "weight_stream.cuh"
