@@ -182,8 +182,8 @@ int32_t hs_op_gemm_part_splits(int32_t M, int32_t N, int32_t K);
 int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
 /* The same of more than 128 rows, on pairs or single blocks as a device of 148 SMs has them; -1 for M <= 128, N < 64 or sm_budget < 1. */
 int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget);
-/* Host-only: columns (256 or 192) per tile of the QKV GEMM of M rows and N = q + k + v columns where a device of 148 SMs has it on pairs
- * of SMs, on sm_budget of them; -1 where it has not, or for M <= 128, N < 128 or sm_budget < 1.  The results do not depend on it. */
+/* Host-only: columns per tile of the QKV GEMM of M rows and N = q + k + v columns on sm_budget SMs: 256 or 192 where a device of 148 SMs
+ * has it on pairs, else 128 or 64; -1 for M <= 64, N < 128 or sm_budget < 1.  The results do not depend on it. */
 int32_t hs_op_qkv_tile(int32_t M, int32_t N, int32_t sm_budget);
 
 /*

@@ -564,7 +564,7 @@ int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget) {
 }
 
 int32_t hs_op_qkv_tile(int32_t M, int32_t N, int32_t sm_budget) {
-  return M <= 128 || N < 128 || sm_budget < 1 || !on_pairs(M, N, 128, 148) ? -1 : gemm_pick_pair_qkv_width(M, N, sm_budget);
+  return M <= 64 || N < 128 || sm_budget < 1 ? -1 : (on_pairs(M, N, 128, 148) ? gemm_pick_pair_qkv_width : gemm_pick_qkv_width)(M, N, sm_budget);
 }
 
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {
@@ -642,7 +642,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   const bool pair_qkv = pair_for(q_dim + 2 * kv_dim, 128), pair_gu = pair_for(2 * F, 256);
   const bool pair_d = pair_for(d, gemm_pick_bn(T, d, s->sm_count));
   const int gu_width = use_pair ? gemm_pick_tall_gu_width(T, F, sm_budget, pair_gu) : gemm_pick_gu_width(T, F, d, sm_budget);   // (the results do not depend on it)
-  const int qkv_width = gemm_pick_pair_qkv_width(T, q_dim + 2 * kv_dim, sm_budget);
+  const int qkv_width = (pair_qkv ? gemm_pick_pair_qkv_width : gemm_pick_qkv_width)(T, q_dim + 2 * kv_dim, sm_budget);
   const int f16 = (c.flags & HS_FLAG_BF16_ACTIVATIONS) ? 0 : 1;   // format of h, o, act
   // A operands of a small step are fetched with boxes of 64 or 32 rows instead of 128
   const int a_rows = use_pair ? 128 : (T <= 32 ? 32 : T <= 64 ? 64 : 128);
@@ -837,14 +837,14 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     g.tm_a = a_rows == 128 ? s->tm_h : s->tm_h_s[a_sel];
     g.a_box_rows = a_rows;
     g.tm_b[0] = m.wq; g.tm_b[1] = m.wk; g.tm_b[2] = m.wv;
-    if (pair_qkv && qkv_width != 256)
+    if (qkv_width != (pair_qkv ? 256 : 128))
       for (int i = 0; i < 3; ++i) g.tm_b[i] = m.qkv_narrow[i];
     g.M = T; g.N = q_dim + 2 * kv_dim; g.K = d;
     g.mode = kGemmQkv;
     g.ab_f16 = f16;
     g.overlap = overlap;
     g.pair = pair_qkv;
-    g.bn = pair_qkv ? qkv_width : 128;     // small steps: 128-column tiles, twice as many SMs stream the weights
+    g.bn = qkv_width;
     g.q_dim = q_dim; g.kv_dim = kv_dim; g.head_dim = Dh; g.n_kv_heads = c.n_kv_heads;
     g.q_out = q;
     g.k_cache = s->kv_pool + (size_t(l) * 2 + 0) * layer_kv_elems;

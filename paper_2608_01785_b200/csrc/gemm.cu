@@ -54,15 +54,15 @@ constexpr int GEMM_SMEM = 1024 + RING_BYTES + EPI_BYTES + 384;
 static_assert(GEMM_SMEM <= 227 * 1024, "fits one SM");
 static_assert(GEMM_SMEM >= kMinSmemBytes, "one block per SM");
 
-// Qkv mode, single blocks: tiles of 128 virtual columns (one B box) when p.bn says so -- the launcher asks for
-// them at small M, where the tile count decides how many SMs stream weights; 256 otherwise.  A 128-column
+// Qkv mode, single blocks: tiles of 128 virtual columns (one B box) when p.bn says so -- a step asks for
+// them, since the tile count decides how many SMs stream weights; 256 otherwise.  A 128-column
 // tile never straddles q | k | v (their widths are multiples of 128) and holds whole heads.
 // Pairs: 256, or 192 where p.bn says so (gemm_pick_pair_qkv_width).  Such a tile is three units of two 32-column pieces that rotate
 // with each other, 32 p .. of the two halves of a head; each piece is a B box of its own, so that a tile may begin and end inside a
-// head or a projection.
-constexpr int QKV_NARROW = 192;
+// head or a projection.  Single blocks also have tiles of one such unit (gemm_pick_qkv_width).
+constexpr int QKV_NARROW = 192, QKV_UNIT = 64;
 __host__ __device__ __forceinline__ int gemm_qkv_width(const GemmParams& p) {
-  return p.pair ? (p.bn == QKV_NARROW ? QKV_NARROW : BN) : p.bn == 128 ? 128 : BN;
+  return p.pair ? (p.bn == QKV_NARROW ? QKV_NARROW : BN) : p.bn == 128 || p.bn == QKV_UNIT ? p.bn : BN;
 }
 // First column of unit u of [q | k | v]; its partners are half a head further.
 __device__ __forceinline__ int qkv_unit_col(const GemmParams& p, int u) {
@@ -92,9 +92,9 @@ __device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int
   if (p.mode == kGemmGateUp) return {half, n_tile * gemm_gu_width(p)};
   return qkv_source(p, n_tile * gemm_qkv_width(p) + half * 128);
 }
-// Piece `piece` (0 .. 5) of a 192-column tile (past the end of v the boxes lie outside the matrix and read zeros)
-__device__ __forceinline__ BSource qkv_piece(const GemmParams& p, int n_tile, int piece) {
-  return qkv_source(p, qkv_unit_col(p, n_tile * 3 + (piece >> 1)) + (piece & 1) * (p.head_dim >> 1));
+// Piece `piece` of a tile of `units` units (past the end of v the boxes lie outside the matrix and read zeros)
+__device__ __forceinline__ BSource qkv_piece(const GemmParams& p, int n_tile, int units, int piece) {
+  return qkv_source(p, qkv_unit_col(p, n_tile * units + (piece >> 1)) + (piece & 1) * (p.head_dim >> 1));
 }
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -327,13 +327,14 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // when the step is that small) and one or two 128-row B boxes, and the ring holds as many stages as fit (at
   // most kMaxStages): a block's streaming rate is stages in flight / memory latency, so the small stages of a
   // small step buy depth -- 8 or 9 stages instead of 4.
-  const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn : gemm_qkv_width(p)) > 128;
+  const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn > 128 : gemm_qkv_width(p) != 128);   // (64 columns: two pieces of 32)
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
   // (a narrow GateUp tile: its gate rows, and right behind them -- in a pair, in the other block -- its up rows, one operand of
   // 2 gu_w rows)
   const int gu_w = MODE == kGemmGateUp ? gemm_gu_width(p) : 128;
-  const int bh_bytes = (PAIR && MODE == kGemmQkv ? gemm_qkv_width(p) / 2 : gu_w) * BK * 2;
-  const bool qkv_narrow = PAIR && MODE == kGemmQkv && gemm_qkv_width(p) == QKV_NARROW;
+  const int bh_bytes = (MODE != kGemmQkv ? gu_w : PAIR ? gemm_qkv_width(p) / 2 : gemm_qkv_width(p) < 128 ? 32 : 128) * BK * 2;
+  constexpr int narrow_units = PAIR ? 3 : 1, pieces = PAIR ? 3 : 2;      // of a narrow tile, and of those a block's
+  const bool qkv_narrow = MODE == kGemmQkv && gemm_qkv_width(p) == narrow_units * QKV_UNIT;
   const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * bh_bytes;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
@@ -443,9 +444,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     have_unit = walk.next(un);
     if (have_unit) {
       const int n = un.tile / n_m_tiles;
-      const BSource b0 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
-      const BSource b1 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 1) : b_source(p, n, 1);
-      const BSource b2 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 2) : b1;
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b2 = PAIR && qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 2) : b1;
       b_ahead = un.kb_end - un.kb_begin < STAGES ? un.kb_end - un.kb_begin : STAGES;
       if (elect_one())
         for (int i = 0; i < b_ahead; ++i) load_b(i, un.kb_begin + i, b0, b1, b2);
@@ -467,9 +468,9 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     while (ok && have_unit) {
       const int tile = un.tile;
       const int m = tile % n_m_tiles, n = tile / n_m_tiles;
-      const BSource b0 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
-      const BSource b1 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 1) : b_source(p, n, 1);
-      const BSource b2 = qkv_narrow ? qkv_piece(p, n, 3 * int(rank) + 2) : b1;
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b2 = PAIR && qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 2) : b1;
       const int kb_end = un.kb_end;
       for (int kb = un.kb_begin; kb < kb_end; ++kb) {
         ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status);
@@ -1144,6 +1145,16 @@ int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair) {
     if (us < best_us * 0.97) { best_us = us; best = w; }
   }
   return best;
+}
+
+// Columns of a single block's Qkv tile, 128 or 64, by rounds and an SM's intake per K block -- 64 where that is one round still.  Steps on
+// B200, 128 -> 64 columns: denoising, one image, 70 rows 538 -> 524 us, 256 on 148 / 120 / 96 SMs 670 -> 655, 743 -> 728, 745 -> 730; 128 decode
+// rows of the talker 709 -> 689, at 7B dimensions (2 layers) 320 -> 315; a small backbone, 84 rows 266 -> 260.  In two rounds 64 columns
+// lose: 256 rows of the denoising stage on 74 SMs 751 -> 778, 400 on 148 740 -> 759.
+int gemm_pick_qkv_width(int M, int N, int sms) {
+  const int a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2, m_tiles = (M + BM - 1) / BM;
+  auto cost = [&](int w) { return (m_tiles * ((N + w - 1) / w) + sms - 1) / sms * double(a_bytes + w * BK * 2); };
+  return cost(QKV_UNIT) < 0.97 * cost(128) ? QKV_UNIT : 128;
 }
 
 // Columns of a pair's Qkv tile, 256 or 192, by the same rounds and times: 48 tiles of 256 columns (1024 rows, 3072 columns) leave a third of

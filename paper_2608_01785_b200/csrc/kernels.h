@@ -102,8 +102,9 @@ int gemm_pick_ksplit(int M, int N, int K, int bn, int sm_count);
 constexpr int kGuMinWidth = 48, kGuNarrow = 5;
 int gemm_pick_gu_width(int M, int N, int K, int sms);
 int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair);
-// Columns per tile of a Qkv GEMM on pairs with `sms` SMs: 256, or 192 (then tm_b has boxes of 32 rows).
+// Columns per tile of a Qkv GEMM with `sms` SMs, on pairs 256 or 192, on single blocks 128 or 64 (192 and 64: tm_b has boxes of 32 rows).
 int gemm_pick_pair_qkv_width(int M, int N, int sms);
+int gemm_pick_qkv_width(int M, int N, int sms);
 // Where split i (0 .. ks) of a tile's k_blocks begins.  The splits add their sums one after the other, a link of that
 // chain costing about as long as kSplitSkew K blocks take to stream; so each split is that much longer than the one
 // before it and finishes just when its turn comes, instead of all finishing together and then queueing.  Equal

@@ -1,5 +1,5 @@
-"""GEMMs of more than 128 rows whose tiles' width follows the budget -- gate/up on pairs of SMs and on single blocks, QKV on pairs --
-while the results do not."""
+"""GEMMs of more than 64 rows whose tiles' width follows the budget -- gate/up and QKV, on pairs of SMs and on single blocks -- while the
+results do not."""
 import numpy as np
 import pytest
 import torch
@@ -45,13 +45,16 @@ def test_tile_width_does_not_reach_the_output(name, flags):
         st.close()
 
 
-# QKV on pairs: heads of 64 and of 128, tiles that end inside a head and a projection, a last tile of one or two units of three, a ragged
+# QKV on pairs and (the last three) on single blocks: heads of 64 and of 128, tiles that end inside a head and a projection, a last tile of one or two units of three, a ragged
 # row tile; with biases and behind a folded norm.
 QKV_CASES = {
     "dh128_split_heads": (wl.StageDims(1, 256, 28, 4, 128, 256), [600], [0], False),
     "dh128_bias_ragged": (wl.StageDims(1, 264, 22, 2, 128, 264), [500, 77, 1], [0, 30, 5], True),
     "dh64_projections_inside_a_tile": (wl.StageDims(1, 256, 40, 4, 64, 256), [1000, 1], [0, 9], True),
     "dh128_folded": (wl.StageDims(2, 2048, 16, 4, 128, 2816), [1025], [3], False),
+    "singles_dh64_200_rows": (wl.StageDims(1, 256, 24, 4, 64, 256), [199, 1], [0, 20], True),
+    "singles_dh128_70_rows": (wl.StageDims(1, 264, 7, 1, 128, 264), [70], [5], True),
+    "singles_decode_65_rows": (wl.StageDims(1, 512, 8, 2, 64, 512), [1] * 65, [i % 19 for i in range(65)], False),
 }
 
 
@@ -61,7 +64,7 @@ QKV_CASES = {
 def test_qkv_tile_width_does_not_reach_the_output(name, flags):
     dims, q_len, ctx_len, bias = QKV_CASES[name]
     n = (dims.n_q_heads + 2 * dims.n_kv_heads) * dims.head_dim
-    assert {B.hs_op_qkv_tile(sum(q_len), n, k) for k in BUDGETS} == {192, 256}
+    assert {B.hs_op_qkv_tile(sum(q_len), n, k) for k in BUDGETS} == ({64, 128} if name.startswith("singles") else {192, 256})
     case = make_case(dims, wl.BatchSpec(q_len, ctx_len), seed=83, kv_fill=True)
     st = make_stage(case, flags=flags)
     try:
