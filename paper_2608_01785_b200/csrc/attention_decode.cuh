@@ -53,14 +53,13 @@ __device__ __forceinline__ float quad_sum(float v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
-// The same over the eight lanes that share lane % 4.
+// The same over the eight lanes that share lane % 4, and over the four of those that share lane % 8.
 __device__ __forceinline__ float column_max(float v) {
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
   return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
 }
-__device__ __forceinline__ float column_sum(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
+__device__ __forceinline__ float half_column_sum(float v) {
   v += __shfl_xor_sync(0xffffffffu, v, 8);
   return v + __shfl_xor_sync(0xffffffffu, v, 16);
 }
@@ -221,17 +220,20 @@ struct HeadsAsRows {
 // columns, so that no half of a tile is padding: half the MMAs, and as an MMA takes its scheduler ten cycles, they were most of a
 // page (in shared memory, cycles at head_dim 128 / 64: 784 -> 597, 473 -> 392).  This lane has heads 2 (lane % 4) and the next one; keys, and
 // dimensions, lane / 4 and lane / 4 + 8.  The scores become the second product's operand by two 8 x 8 transpositions.
+// The weights of a head are added in the order of HeadsAsRows, so that a group's bits do not depend on the form: keys 2 i, 2 i + 1,
+// 2 i + 8 and 2 i + 9 of a page in one lane, page after page, then the four lanes.  Lanes 8 i .. 8 i + 3 do that for their even head,
+// lanes 8 i + 4 .. 8 i + 7 for the odd one; they give each other what they lack.
 // Steps, us: eleven rows of the talker on 52 SMs 368 -> 364, 16 on 148 260.2 -> 259.6; at 7B dimensions 29 rows on 96 SMs 642 -> 639, 64
 // rows 4801 -> 4787.
 template <int DH>
 struct HeadsAsColumns {
   uint32_t qf[DH / 16][2];
-  float o[DH / 16][4], m[2], l[2];
+  float o[DH / 16][4], m[2], l;               // (l: of the even head in lanes with an even key, of the odd one in the others)
   __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int j = 0; j < DH / 16; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
     m[0] = m[1] = -INFINITY;
-    l[0] = l[1] = 0.f;
+    l = 0.f;
   }
   __device__ __forceinline__ void load_q(const __nv_bfloat16* q, int G, int lane) {
     const int h = lane >> 2;
@@ -242,6 +244,7 @@ struct HeadsAsColumns {
   }
   __device__ __forceinline__ void page(uint32_t k_base, uint32_t v_base, int n_valid, int lane, float scale_log2) {
     const int key = lane >> 2;
+    const bool odd = (lane & 4) != 0;
     float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
     {
       const int kk = (lane & 7) + ((lane >> 3) & 1) * 8, cc = lane >> 4;
@@ -276,8 +279,7 @@ struct HeadsAsColumns {
       const float al0 = fast_exp2(m[0] - mn0), al1 = fast_exp2(m[1] - mn1);
       m[0] = mn0;
       m[1] = mn1;
-      l[0] *= al0;
-      l[1] *= al1;
+      l *= odd ? al1 : al0;
 #pragma unroll
       for (int j = 0; j < DH / 16; ++j) {
         o[j][0] *= al0; o[j][1] *= al1;
@@ -286,32 +288,35 @@ struct HeadsAsColumns {
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) s[e] = fast_exp2(fmaf(s[e], scale_log2, -m[e & 1]));
-    l[0] += s[0] + s[2];
-    l[1] += s[1] + s[3];
+    const float near_ = (odd ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 4);
+    const float far_ = (odd ? s[3] : s[2]) + __shfl_xor_sync(0xffffffffu, odd ? s[2] : s[3], 4);
+    l += near_ + far_;
     const uint32_t p0 = transpose_8x8(pack_bf16(s[0], s[1])), p1 = transpose_8x8(pack_bf16(s[2], s[3]));
 #pragma unroll
     for (int dp = 0; dp < DH / 16; ++dp) mma_bf16_16816(o[dp], vf[dp], p0, p1);
   }
   __device__ __forceinline__ void put(float* po, int pitch, float2* pml, int G, int lane) {
     const int d = lane >> 2, h = 2 * (lane & 3);
+    l = half_column_sum(l);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      l[e] = column_sum(l[e]);
       if (h + e < G) {
 #pragma unroll
         for (int j = 0; j < DH / 16; ++j) {
           po[(h + e) * pitch + 16 * j + d] = o[j][e];
           po[(h + e) * pitch + 16 * j + d + 8] = o[j][e + 2];
         }
-        if (d == 0) pml[h + e] = make_float2(m[e], l[e]);
+        if (d == e) pml[h + e] = make_float2(m[e], l);
       }
     }
   }
   __device__ __forceinline__ void store(__nv_bfloat16* out, bool f16, int* status, int G, int lane) {
     const int d = lane >> 2, h = 2 * (lane & 3);
+    l = half_column_sum(l);
+    const float other = __shfl_xor_sync(0xffffffffu, l, 4);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const float inv = 1.f / column_sum(l[e]);
+      const float inv = 1.f / ((d & 1) == e ? l : other);
       if (h + e < G) {
 #pragma unroll
         for (int j = 0; j < DH / 16; ++j) {
