@@ -97,6 +97,11 @@ __device__ __forceinline__ void drain_after_abort() {
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
+// Before the first use of a tensor map that lies in global memory, where the host has written it: the unit that reads maps has a
+// cache of its own, which may still hold what stood there before.  (Maps among a kernel's parameters need none.)
+__device__ __forceinline__ void tma_acquire_desc(const CUtensorMap* m) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+}
 // 2-D tiled load global -> this block's shared memory; completion is signalled on `bar` in bytes.
 // c0 is the innermost coordinate (elements); c0 * element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1) {

@@ -173,6 +173,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_step_kernel(const __gr
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kServiceRegs));
     if (tid == SK_THREADS + 32) watch(all_done, progress, gave_up, p.sync + 1, p.status);
     if (warp != SK_WARPS) return;
+    // (the maps lie in the stage's workspace, where another stage's may have been before)
+    for (int i = lane; i < L * 7; i += 32) tma_acquire_desc(p.maps + i);
+    __syncwarp();
     int slot = 0;
     uint32_t parity = 1;                                        // (a fresh barrier's phase before the first counts as done)
     bool ok = true;

@@ -89,6 +89,30 @@ def test_steps_of_other_sizes_leave_nothing_behind_for_the_next():
         st.close()
 
 
+@pytest.mark.gpu
+def test_a_second_stage_in_the_same_workspace_streams_its_own_weights():
+    """The weights' tensor maps lie in the workspace.  (With bf16 activations the stages read the caller's tensors, so the two sets of
+    maps differ; both sets of weights stay allocated.)"""
+    dims = D(3, 1024, 16, 4, 64, 2816)
+    ctx = [100, 37, 260]
+    cases = [make_case(dims, wl.BatchSpec([1] * 3, ctx), seed=k, kv_fill=True) for k in (64, 65)]
+    stages = [make_stage(c, flags=B.HS_FLAG_BF16_ACTIVATIONS) for c in cases]
+    try:
+        shared = stages[0]
+        want = [_step(st, cases[0], shared.sm_count) for st in stages]
+        assert not np.array_equal(want[0][0], want[1][0])
+        for i in (1, 0, 1):
+            B.hs_stage_destroy(shared.handle)
+            shared.handle = 0
+            ptrs = [{k: v.data_ptr() for k, v in lw.items()} for lw in stages[i].weights]
+            shared.handle = B.hs_stage_create(shared.cfg, ptrs, shared.kv_pool.data_ptr(), shared.workspace.data_ptr())
+            for a, b in zip(_step(shared, cases[0], shared.sm_count), want[i]):
+                assert np.array_equal(a, b), i
+    finally:
+        for st in stages:
+            st.close()
+
+
 def test_the_rule_that_takes_the_one_launch():
     t = wl.DIMS["c4_talker"]
     assert [B.hs_op_one_launch_step(n, t, 148) for n in (1, 8, 9, 16, 17)] == [1, 1, 1, 1, 0]
