@@ -202,6 +202,25 @@ int32_t hs_op_one_launch_step(int32_t rows, int32_t d_model, int32_t n_q_heads, 
                               int32_t n_layers, int32_t sm_budget);
 
 /*
+ * Diagnosis of the one-launch step's ways out, as hs_op_wait_probe is of the other kernels' waits.  Until the next call the
+ * one-launch steps of the stage
+ *   HS_FAULT_NONE      run as they should;
+ *   HS_FAULT_REFUSED   find that the context does not hold their blocks at once, and take the separate launches;
+ *   HS_FAULT_MISSING   wait for one block more than there is: after limit_ns nanoseconds (1 us .. 100 ms) without progress, in place
+ *                      of the kernels' 2 s, the step gives up, stores nothing of what it has not got, and leaves HS_ERR_TIMEOUT in
+ *                      the stage's status (hs_stage_status);
+ *   HS_FAULT_GAVE_UP   find that another block has given up, and leave wherever they are; y_out and the new tokens' cache rows then hold
+ *                      what the step had come to (its status is the other block's to set: here nothing does).
+ * The next step of the stage starts from nothing that such a step leaves.
+ * Errors: INVALID_ARG (NULL stage, unknown fault, limit out of range), NO_DEVICE.
+ */
+#define HS_FAULT_NONE 0
+#define HS_FAULT_REFUSED 1
+#define HS_FAULT_MISSING 2
+#define HS_FAULT_GAVE_UP 3
+hs_status_t hs_stage_one_launch_fault(hs_stage_t *stage, int32_t fault, uint64_t limit_ns);
+
+/*
  * Host-only: the K block (of 64) at which split i (0 .. ks; i = ks gives k_blocks) of a small step's residual GEMM
  * begins when its k_blocks are cut into ks splits.  Each split is ten K blocks longer than the one before it (the
  * splits add their sums one after the other, and a link of that chain takes about as long as ten K blocks take to

@@ -256,6 +256,8 @@ struct hs_stage {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool ev_pending[kRing] = {};
   int ring_pos = 0;
+  int one_launch_fault = HS_FAULT_NONE;       // hs_stage_one_launch_fault
+  uint64_t one_launch_limit_ns = 0;
   // optional per-kernel timing
   bool census = false;      // record SM placement of the last step's launches
   bool profile = false;
@@ -612,6 +614,13 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   // OverlapMode).  (Not while the per-kernel timers run: an event between two kernels serialises them anyway.)
   const int overlap = s->profile ? kOverlapNone : sm_budget == s->sm_count ? kOverlapEarly : kOverlapLate;
   int32_t* meta = reinterpret_cast<int32_t*>(s->ws_dev + s->ws.meta);
+  // The whole step in one launch, with the bits of the launches below.  Not while those are timed or counted one by one, nor for a
+  // conditioned stage.
+  const bool whole = plan.n_prefill_items == 0 && plan.decode_group && !s->modulation && !s->profile && !s->census && one_launch(c, plan.n_tokens, s->sm_count, sm_budget);
+  if (whole) {                 // (its two words, see SmallStepParams: blocks that have arrived, a flag of blocks that gave up)
+    s->pinned[slot][s->ml.counters] = s->one_launch_fault == HS_FAULT_MISSING ? -1 : 0;
+    s->pinned[slot][s->ml.counters + 1] = s->one_launch_fault == HS_FAULT_GAVE_UP ? 1 : 0;
+  }
   // the slot may be planned into again when the step is through (an event behind the first kernel would keep the second one's
   // set-up from overlapping it)
   struct SlotInUse {
@@ -774,9 +783,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     a.smid_log = slots(2);       // prefill in class 2, decode in class 3 (the next slots)
     return a;
   };
-  // The whole step in one launch, with the bits of the launches below.  Not while those are timed or counted one by one, nor for a
-  // conditioned stage.
-  if (plan.n_prefill_items == 0 && plan.decode_group && !s->modulation && !s->profile && !s->census && one_launch(c, T, s->sm_count, sm_budget)) {
+  if (whole) {
     SmallStepParams k{};
     k.tm_kv_page = s->tm_kv_page;
     for (int l = 0; l < c.n_layers; ++l) {
@@ -799,10 +806,11 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     k.rope = reinterpret_cast<const float2*>(s->ws_dev + s->ws.rope);
     k.sync = meta + s->ml.counters;
     k.status = status;
-    e = launch_small_step(k, sm_budget, stream);
+    k.wait_limit_ns = s->one_launch_fault == HS_FAULT_NONE ? 0 : s->one_launch_limit_ns;
+    e = s->one_launch_fault == HS_FAULT_REFUSED ? cudaErrorCooperativeLaunchTooLarge : launch_small_step(k, sm_budget, stream);
     if (e == cudaSuccess) return HS_OK;
     // a context that does not hold so many blocks at once takes the separate launches
-    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return cuda_fail("small step", e);
+    if ((e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) || s->one_launch_fault > HS_FAULT_REFUSED) return cuda_fail("small step", e);
     cudaGetLastError();
     e = cudaSuccess;
   }
@@ -1067,6 +1075,15 @@ hs_status_t hs_stage_profile_read(hs_stage_t* s, float* ms, int32_t* launches) {
   }
   s->timed.clear();
   return st;
+}
+
+hs_status_t hs_stage_one_launch_fault(hs_stage_t* s, int32_t fault, uint64_t limit_ns) {
+  if (!s || fault < HS_FAULT_NONE || fault > HS_FAULT_GAVE_UP) return HS_ERR_INVALID_ARG;
+  if (s->cfg.device < 0) return HS_ERR_NO_DEVICE;
+  if (fault != HS_FAULT_NONE && (limit_ns < 1000 || limit_ns > 100000000ull)) return HS_ERR_INVALID_ARG;
+  s->one_launch_fault = fault;
+  s->one_launch_limit_ns = limit_ns;
+  return HS_OK;
 }
 
 hs_status_t hs_stage_debug_buffer(hs_stage_t* s, const char* name, void** dev_ptr, size_t* bytes) {

@@ -233,6 +233,7 @@ struct SmallStepParams {
   const float2* rope;
   int* sync;                       // two words, zero at entry: blocks that have arrived, and a flag of blocks that gave up
   int* status;
+  unsigned long long wait_limit_ns;    // without progress, before a block gives up; 0: kWaitLimitNs
 };
 // Tensor map of a 16-bit weight matrix [rows, K], K a multiple of 256, from which one copy brings eight rows of four consecutive
 // 256-column blocks as [block][eighth of it: one warp's 32 columns][row][64 bytes].

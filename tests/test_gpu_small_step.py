@@ -113,6 +113,52 @@ def test_a_second_stage_in_the_same_workspace_streams_its_own_weights():
             st.close()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["one_row_sliced", "first_token", "eight_heads_a_group", "sixteen_rows"])
+def test_every_way_out_of_the_one_launch(name):
+    """A launch that the context refuses becomes the chain.  A step whose wait runs out ends by itself and stores nothing that it has not got:
+    no block leaves the first barrier, so neither the output nor the cache is touched.  What such a step leaves does not reach the
+    next one."""
+    dims, ctx = CASES[name]
+    case = make_case(dims, wl.BatchSpec([1] * len(ctx), ctx), seed=66, kv_fill=True)
+    st = make_stage(case)
+    try:
+        for budget in _budgets(len(ctx), dims, st.sm_count)[:3]:
+            want = _step(st, case, budget)
+            B.hs_stage_one_launch_fault(st.handle, B.HS_FAULT_REFUSED)
+            for a, b in zip(_step(st, case, budget), want):
+                assert np.array_equal(a, b), budget
+            B.hs_stage_one_launch_fault(st.handle, B.HS_FAULT_GAVE_UP)
+            for _ in range(3):
+                _step(st, case, budget)
+            B.hs_stage_one_launch_fault(st.handle, B.HS_FAULT_NONE)
+            for a, b in zip(_step(st, case, budget), want):
+                assert np.array_equal(a, b), budget
+        x = case.x_t.to(st.device)
+        for budget in _budgets(len(ctx), dims, st.sm_count)[:3]:      # (from here on the stage's status says what happened)
+            st.kv_pool.copy_(wl.bits_to_bf16_tensor(case.kv_pool, st.device))
+            y = torch.full((len(ctx), dims.d_model), -7.0, device=st.device)
+            b = st.make_batch([1] * len(ctx), ctx, case.block_tables, x, y)
+            B.hs_stage_one_launch_fault(st.handle, B.HS_FAULT_MISSING, 2_000_000)
+            t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda.synchronize()
+            t[0].record()
+            st.step(b, budget)
+            t[1].record()
+            torch.cuda.synchronize()
+            assert st.status() == B.HS_ERR_TIMEOUT and 2.0 <= t[0].elapsed_time(t[1]) < 50.0
+            assert (y == -7.0).all() and np.array_equal(wl.bf16_bits_numpy(st.kv_pool).reshape(-1), case.kv_pool)
+            B.hs_stage_one_launch_fault(st.handle, B.HS_FAULT_NONE)
+            st.step(b, budget)
+            torch.cuda.synchronize()
+            assert np.array_equal(y.cpu().numpy(), want[0]) and np.array_equal(wl.bf16_bits_numpy(st.kv_pool).reshape(-1), want[1])
+        for bad in ((-1, 1000), (4, 1000), (B.HS_FAULT_MISSING, 10), (B.HS_FAULT_MISSING, 10**9)):
+            with pytest.raises(B.HsError):
+                B.hs_stage_one_launch_fault(st.handle, *bad)
+    finally:
+        st.close()
+
+
 def test_the_rule_that_takes_the_one_launch():
     t = wl.DIMS["c4_talker"]
     assert [B.hs_op_one_launch_step(n, t, 148) for n in (1, 8, 9, 16, 17)] == [1, 1, 1, 1, 0]
