@@ -196,6 +196,8 @@ hs_status_t hs_stage_plan(hs_stage_t *stage, const hs_batch_t *batch, int32_t *t
  * blocks (at most 120) are free together; a context that cannot hold them gets the separate launches.  With both prefill and
  * decode work in a step the two attention kernels of a layer run side by side on two shares of the budget, the decode kernel on
  * a stream of the stage's own that is forked from and joined to cuda_stream by events.
+ * The call returns when the step is enqueued.  Five steps of a stage may be on their way at a time: the sixth call waits on the host
+ * until the first one's step has ended.
  * Errors (nothing launched): INVALID_ARG, INVALID_BUDGET, BAD_BLOCK_TABLE, NO_DEVICE, CUDA.
  */
 hs_status_t hs_stage_step(hs_stage_t *stage, const hs_batch_t *batch, int32_t sm_budget, void *cuda_stream);

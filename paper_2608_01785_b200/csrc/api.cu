@@ -18,7 +18,9 @@
 namespace hs {
 namespace {
 
-constexpr int kRing = 4;   // pinned staging slots for step metadata
+// Pinned staging slots for step metadata.  A slot is a step's until the step has ended, so a call waits on the host only where the
+// stage's fifth step before it has not.
+constexpr int kRing = 5;
 constexpr int kRowSsStride = 64;   // partial sums of x^2 kept per token: one per 128-column tile of d_model at most
 
 struct WsLayout {
@@ -586,6 +588,8 @@ int32_t hs_op_gemm_split_begin(int32_t k_blocks, int32_t ks, int32_t i) {
   return gemm_split_begin(k_blocks, ks, i);
 }
 
+static hs_status_t enqueue_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget, cudaStream_t stream, const StepPlan& plan, int slot);
+
 hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget, void* cuda_stream) {
   if (!s || !b) return HS_ERR_INVALID_ARG;
   if (s->cfg.device < 0) return HS_ERR_NO_DEVICE;
@@ -597,7 +601,7 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   DeviceGuard guard(c.device);
   if (!guard.ok) return HS_ERR_CUDA;
 
-  // plan into the next pinned slot (waiting for the copy that last used it)
+  // plan into the next pinned slot (waiting for the step that last used it)
   const int slot = s->ring_pos;
   if (s->ev_pending[slot]) {
     if (cudaEventSynchronize(s->ev[slot]) != cudaSuccess) return HS_ERR_CUDA;
@@ -607,7 +611,18 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
   hs_status_t st = plan_step(c, s->ml, *b, s->sm_count, sm_budget, !s->profile, s->page_stamp, ++s->stamp, s->pinned[slot], nullptr, &plan);
   if (st != HS_OK) return st;
   s->ring_pos = (slot + 1) % kRing;
+  st = enqueue_step(s, b, sm_budget, stream, plan, slot);
+  // The slot may be planned into again when the step is through, whatever became of it.  (An event behind the kernel that fetches it
+  // would keep the next one's set-up from overlapping that.)
+  const cudaError_t marked = cudaEventRecord(s->ev[slot], stream);
+  if (marked != cudaSuccess) return st != HS_OK ? st : cuda_fail("hs_stage_step: the metadata slot's event", marked);
+  s->ev_pending[slot] = true;
+  return st;
+}
 
+// Everything of a planned step that goes to the device.
+static hs_status_t enqueue_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget, cudaStream_t stream, const StepPlan& plan, int slot) {
+  const hs_stage_config_t& c = s->cfg;
   // With the whole device as its budget a step has no neighbour to take SMs from, so each kernel is launched
   // such that its set-up overlaps the previous kernel's drain.  With a smaller budget the blocks of the next
   // kernel would wait on SMs outside the budget, so they are placed only when the last block in front has left (see
@@ -621,14 +636,6 @@ hs_status_t hs_stage_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_budget,
     s->pinned[slot][s->ml.counters] = s->one_launch_fault == HS_FAULT_MISSING ? -1 : 0;
     s->pinned[slot][s->ml.counters + 1] = s->one_launch_fault == HS_FAULT_GAVE_UP ? 1 : 0;
   }
-  // the slot may be planned into again when the step is through (an event behind the first kernel would keep the second one's
-  // set-up from overlapping it)
-  struct SlotInUse {
-    hs_stage* s;
-    int slot;
-    cudaStream_t stream;
-    ~SlotInUse() { s->ev_pending[slot] = cudaEventRecord(s->ev[slot], stream) == cudaSuccess; }
-  } slot_in_use{s, slot, stream};
   if (const cudaError_t fetched = launch_fetch_metadata(s->pinned[slot], meta, plan.meta_words, overlap, sm_budget, stream); fetched != cudaSuccess)
     return cuda_fail("metadata", fetched);
 

@@ -46,5 +46,15 @@ def test_back_to_back_steps_find_their_own_metadata(budget):
         assert st.status() == 0
         for i, y in got:
             assert torch.isfinite(y).all() and torch.equal(y, want[i]), i
+        # five steps are enqueued without a wait on the host, behind whatever the stream is doing
+        ys, busy = [torch.empty_like(want[i]) for i in range(5)], torch.cuda.Event()
+        args = [st.make_batch(batches[i].q_len, batches[i].ctx_len, tables[i], xs[i], ys[i]) for i in range(5)]
+        torch.cuda._sleep(1_000_000_000)
+        busy.record()
+        for a in args:
+            st.step(a, budget)
+        assert not busy.query()
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, want[i]) for i, y in enumerate(ys))
     finally:
         st.close()
