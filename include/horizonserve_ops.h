@@ -183,7 +183,8 @@ int32_t hs_op_gate_up_width(int32_t M, int32_t N, int32_t K, int32_t sm_budget);
 /* The same of more than 128 rows, on pairs or single blocks as a device of 148 SMs has them; -1 for M <= 128, N < 64 or sm_budget < 1. */
 int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget);
 /* Host-only: columns per tile of the QKV GEMM of M rows and N = q + k + v columns on sm_budget SMs: 256 or 192 where a device of 148 SMs
- * has it on pairs, else 128 or 64; -1 for M <= 64, N < 128 or sm_budget < 1.  The results do not depend on it. */
+ * has it on pairs, else 128 or, of more than 64 rows, 64; -1 for M < 1, N < 128 or sm_budget < 1.  (Up to 64 rows the weight-streaming
+ * kernel takes it in most shapes instead.)  The results do not depend on it. */
 int32_t hs_op_qkv_tile(int32_t M, int32_t N, int32_t sm_budget);
 
 /*

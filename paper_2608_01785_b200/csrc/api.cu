@@ -568,7 +568,7 @@ int32_t hs_op_gate_up_tile(int32_t M, int32_t N, int32_t sm_budget) {
 }
 
 int32_t hs_op_qkv_tile(int32_t M, int32_t N, int32_t sm_budget) {
-  return M <= 64 || N < 128 || sm_budget < 1 ? -1 : (on_pairs(M, N, 128, 148) ? gemm_pick_pair_qkv_width : gemm_pick_qkv_width)(M, N, sm_budget);
+  return M < 1 || N < 128 || sm_budget < 1 ? -1 : (on_pairs(M, N, 128, 148) ? gemm_pick_pair_qkv_width : gemm_pick_qkv_width)(M, N, sm_budget);
 }
 
 int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_budget) {

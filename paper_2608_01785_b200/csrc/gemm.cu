@@ -1150,10 +1150,12 @@ int gemm_pick_tall_gu_width(int M, int N, int sms, bool pair) {
 // Columns of a single block's Qkv tile, 128 or 64, by rounds and an SM's intake per K block -- 64 where that is one round still.  Steps on
 // B200, 128 -> 64 columns: denoising, one image, 70 rows 538 -> 524 us, 256 on 148 / 120 / 96 SMs 670 -> 655, 743 -> 728, 745 -> 730; 128 decode
 // rows of the talker 709 -> 689, at 7B dimensions (2 layers) 320 -> 315; a small backbone, 84 rows 266 -> 260.  In two rounds 64 columns
-// lose: 256 rows of the denoising stage on 74 SMs 751 -> 778, 400 on 148 740 -> 759.
+// lose: 256 rows of the denoising stage on 74 SMs 751 -> 778, 400 on 148 740 -> 759.  Not for at most 64 rows, whose A boxes of 64 or
+// 32 rows would leave a stage (12 KB) shorter than the 128 rows that an MMA reads.
 int gemm_pick_qkv_width(int M, int N, int sms) {
-  const int a_bytes = (M <= 32 ? 32 : M <= 64 ? 64 : 128) * BK * 2, m_tiles = (M + BM - 1) / BM;
-  auto cost = [&](int w) { return (m_tiles * ((N + w - 1) / w) + sms - 1) / sms * double(a_bytes + w * BK * 2); };
+  if (M <= 64) return 128;
+  const int m_tiles = (M + BM - 1) / BM;
+  auto cost = [&](int w) { return (m_tiles * ((N + w - 1) / w) + sms - 1) / sms * double(A_BYTES + w * BK * 2); };
   return cost(QKV_UNIT) < 0.97 * cost(128) ? QKV_UNIT : 128;
 }
 

@@ -85,3 +85,12 @@ def test_qkv_tile_width_does_not_reach_the_output(name, flags):
         assert rel_err(first[0], y_ref) <= 2e-2        # the rule of every parity test (16-bit operands)
     finally:
         st.close()
+
+
+def test_few_rows_keep_whole_qkv_tiles():
+    """A tile of 64 columns behind an A box of fewer than 128 rows would be a stage shorter than what an MMA reads of it."""
+    for n in (1536, 4608, 6144):
+        for rows in (1, 20, 32, 33, 50, 64):
+            assert {B.hs_op_qkv_tile(rows, n, k) for k in BUDGETS} == {128}, (rows, n)
+        assert B.hs_op_qkv_tile(65, n, 148) == 64
+    assert B.hs_op_qkv_tile(0, 1536, 148) == B.hs_op_qkv_tile(65, 64, 148) == B.hs_op_qkv_tile(65, 1536, 0) == -1
