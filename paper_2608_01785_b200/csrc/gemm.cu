@@ -87,10 +87,10 @@ __device__ __forceinline__ BSource qkv_source(const GemmParams& p, int v) {
   if (v < p.kv_dim) return {1, v};
   return {2, v - p.kv_dim};
 }
-__device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int half) {
+__device__ __forceinline__ BSource b_source(const GemmParams& p, int n_tile, int half, int qkv_width) {
   if (p.mode == kGemmResid) return {0, n_tile * p.bn + half * 128};
   if (p.mode == kGemmGateUp) return {half, n_tile * gemm_gu_width(p)};
-  return qkv_source(p, n_tile * gemm_qkv_width(p) + half * 128);
+  return qkv_source(p, n_tile * qkv_width + half * 128);
 }
 // Piece `piece` of a tile of `units` units (past the end of v the boxes lie outside the matrix and read zeros)
 __device__ __forceinline__ BSource qkv_piece(const GemmParams& p, int n_tile, int units, int piece) {
@@ -320,21 +320,24 @@ struct UnitWalk {
   }
 };
 
-// (one instantiation per mode: an epilogue does not pay with registers for the others)
-template <bool PAIR, int MODE>
+// (One instantiation per mode: an epilogue does not pay with registers for the others.  UNIT: Qkv tiles of 64 columns on single blocks.  In
+// one instantiation with the others, and with a tile width that the pairs' read from the parameters alike, those cost every launch:
+// denoising step, 1024 rows on pairs 892.2 -> 884.5 us.)
+template <bool PAIR, int MODE, bool UNIT = false>
 __device__ __forceinline__ void gemm_body(const GemmParams& p) {
+  const int qkv_width = PAIR ? (p.bn == QKV_NARROW ? QKV_NARROW : BN) : UNIT ? QKV_UNIT : p.bn == 128 ? 128 : BN;      // (Qkv mode)
   // Ring geometry.  Pairs: 6 stages of 32 KB.  Single blocks: a stage holds the A box (128 rows, or only 64 / 32
   // when the step is that small) and one or two 128-row B boxes, and the ring holds as many stages as fit (at
   // most kMaxStages): a block's streaming rate is stages in flight / memory latency, so the small stages of a
   // small step buy depth -- 8 or 9 stages instead of 4.
-  const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn > 128 : gemm_qkv_width(p) != 128);   // (64 columns: two pieces of 32)
+  const bool b_two = MODE == kGemmGateUp || (MODE == kGemmResid ? p.bn > 128 : UNIT || qkv_width > 128);   // (64 columns: two pieces of 32)
   const int a_bytes = (p.a_box_rows > 0 && !PAIR ? p.a_box_rows : BM) * BK * 2;
   // (a narrow GateUp tile: its gate rows, and right behind them -- in a pair, in the other block -- its up rows, one operand of
   // 2 gu_w rows)
   const int gu_w = MODE == kGemmGateUp ? gemm_gu_width(p) : 128;
-  const int bh_bytes = (MODE != kGemmQkv ? gu_w : PAIR ? gemm_qkv_width(p) / 2 : gemm_qkv_width(p) < 128 ? 32 : 128) * BK * 2;
+  const int bh_bytes = (MODE != kGemmQkv ? gu_w : PAIR ? qkv_width / 2 : UNIT ? 32 : 128) * BK * 2;
   constexpr int narrow_units = PAIR ? 3 : 1, pieces = PAIR ? 3 : 2;      // of a narrow tile, and of those a block's
-  const bool qkv_narrow = MODE == kGemmQkv && gemm_qkv_width(p) == narrow_units * QKV_UNIT;
+  const bool qkv_narrow = UNIT || (PAIR && MODE == kGemmQkv && qkv_width == narrow_units * QKV_UNIT);
   const int STAGE_BYTES = PAIR ? Ring<true>::STAGE_BYTES : a_bytes + (b_two ? 2 : 1) * bh_bytes;
   // (a pair kernel that folds the following RMSNorm into its epilogue runs its ring one stage short and uses the last
   // stage's 32 KB as landing blocks for the residual stream: see the epilogue)
@@ -367,7 +370,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
   // a single block that stands in for a pair (stream-K form at sm_budget 1) walks the pair's 256-row tiles
   const bool emulate_pair = !PAIR && p.pair && MODE == kGemmResid && p.stream_k_slots > 0;
   const int n_m_tiles = PAIR || emulate_pair ? (p.M + 2 * BM - 1) / (2 * BM) : (p.M + BM - 1) / BM;
-  const int n_n_tiles = gemm_n_tiles(p);
+  const int n_n_tiles = MODE == kGemmQkv ? (p.N + qkv_width - 1) / qkv_width : gemm_n_tiles(p);
   const int n_tiles = n_m_tiles * n_n_tiles;
   const int k_blocks = (p.K + BK - 1) / BK;
   // Work unit = (output tile, run of K blocks): see UnitWalk.  Runs shorter than the whole K range exist only in
@@ -444,8 +447,8 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     have_unit = walk.next(un);
     if (have_unit) {
       const int n = un.tile / n_m_tiles;
-      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
-      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0, qkv_width);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1, qkv_width);
       const BSource b2 = PAIR && qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 2) : b1;
       b_ahead = un.kb_end - un.kb_begin < STAGES ? un.kb_end - un.kb_begin : STAGES;
       if (elect_one())
@@ -468,8 +471,8 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
     while (ok && have_unit) {
       const int tile = un.tile;
       const int m = tile % n_m_tiles, n = tile / n_m_tiles;
-      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0);
-      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1);
+      const BSource b0 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank)) : b_source(p, n, PAIR ? int(rank) : 0, qkv_width);
+      const BSource b1 = qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 1) : b_source(p, n, 1, qkv_width);
       const BSource b2 = PAIR && qkv_narrow ? qkv_piece(p, n, narrow_units, pieces * int(rank) + 2) : b1;
       const int kb_end = un.kb_end;
       for (int kb = un.kb_begin; kb < kb_end; ++kb) {
@@ -490,7 +493,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
       // both operands are fp16 or both bf16 (one MMA cannot mix the two): the format fields of A (bits 7..9)
       // and B (bits 10..12) are 0 for fp16 and 1 for bf16
       const uint32_t idesc = umma_idesc_bf16_f32(PAIR ? 2 * BM : BM,
-                                                 MODE == kGemmGateUp ? 2 * gu_w : MODE == kGemmQkv ? gemm_qkv_width(p) : PAIR ? BN : p.bn) &
+                                                 MODE == kGemmGateUp ? 2 * gu_w : MODE == kGemmQkv ? qkv_width : PAIR ? BN : p.bn) &
                              (p.ab_f16 ? ~(63u << 7) : ~0u);
       int s = 0, acc = 0;
       uint32_t ph = 0, acc_ph = 0;
@@ -563,7 +566,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
           pos = p.tok_pos[row];
           slot = p.tok_slot[row];
         }
-        const float2* cs = p.rope + size_t(pos) * (Dh >> 1) + (Dh == 128 ? 32 * ((n * (gemm_qkv_width(p) / 64) + cg) & 1) : 0);
+        const float2* cs = p.rope + size_t(pos) * (Dh >> 1) + (Dh == 128 ? 32 * ((n * (qkv_width / 64) + cg) & 1) : 0);
         asm volatile("prefetch.global.L1 [%0];\n\tprefetch.global.L1 [%0 + 128];" ::"l"(cs));
       }
       // folded RMSNorm, producing side: the first two blocks of this warp's rows of y are on their way before the
@@ -847,7 +850,7 @@ __device__ __forceinline__ void gemm_body(const GemmParams& p) {
         }
       } else {
         // units of two 32-column pieces that rotate with each other, every other one this warp's
-        const int half_dh = Dh >> 1, n_units = gemm_qkv_width(p) / 64;
+        const int half_dh = Dh >> 1, n_units = qkv_width / 64;
         const bool apart = Dh == 128 && !qkv_narrow;           // (whole heads of 128: the partners are 64 columns apart)
         for (int i = cg; i < n_units; i += 2) {
           const int unit = n * n_units + i, vcol = qkv_unit_col(p, unit), part = Dh == 128 ? unit & 1 : 0;   // column of [q | k | v]
@@ -935,6 +938,9 @@ template <int MODE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
   gemm_body<false, MODE>(p);
 }
+__global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_qkv_unit_kernel(const __grid_constant__ GemmParams p) {
+  gemm_body<false, kGemmQkv, true>(p);
+}
 // Two blocks per cluster, one 256 x 256 tile per pair.
 template <int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
@@ -958,7 +964,7 @@ cudaError_t gemm_set_attributes() {
     });
     if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  return set_kernel_smem(gemm_qkv_unit_kernel, GEMM_SMEM);
 }
 
 int gemm_pick_bn(int M, int N, int sm_count) {
@@ -1192,6 +1198,8 @@ cudaError_t launch_gemm(const GemmParams& p, int sm_budget, cudaStream_t stream)
     });
   }
   const int grid = n_tiles < sm_budget ? n_tiles : sm_budget;
+  if (p.mode == kGemmQkv && gemm_qkv_width(p) == QKV_UNIT)
+    return launch_step_kernel(gemm_qkv_unit_kernel, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
   return by_mode(p.mode, [&](auto m) {
     return launch_step_kernel(gemm_kernel<decltype(m)::value>, grid, GEMM_THREADS, GEMM_SMEM, stream, p.overlap != 0, p);
   });
