@@ -13,10 +13,12 @@ BATCHES = [([1], [7]), ([1, 1, 1], [300, 17, 33]), ([40], [0]), ([130, 1, 1], [5
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("budget", [148, 40, 1])
-def test_back_to_back_steps_find_their_own_metadata(budget):
+@pytest.mark.parametrize("budget,pages", [(148, 0), (40, 0), (1, 0), (148, 4096), (16, 4096), (3, 4096), (1, 4096)])
+def test_back_to_back_steps_find_their_own_metadata(budget, pages):
+    """`pages`: width of the block tables, if more than the longest sequence takes: 320 KB of them are one or several rounds of the
+    kernel that fetches them, or a copy."""
     batches = [wl.BatchSpec(list(q), list(c)) for q, c in BATCHES]
-    mpps = max(-(-t // 16) for b in batches for t in b.total_len())
+    mpps = max(pages, max(-(-t // 16) for b in batches for t in b.total_len()))
     tables, n_pages = [], 0                       # every batch has pages of its own: its step gives the same whenever it runs
     for b in batches:
         t = np.full((b.n_seqs, mpps), -1, dtype=np.int32)
