@@ -202,6 +202,9 @@ int32_t hs_op_weight_streaming_rows(int32_t M, int32_t N, int32_t K, int32_t sm_
 int32_t hs_op_one_launch_step(int32_t rows, int32_t d_model, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int32_t d_ffn,
                               int32_t n_layers, int32_t sm_budget);
 
+/* Host-only: 1 if the stage's last step was the one cooperative launch, 0 if it was a chain of launches, -1 before the first step. */
+int32_t hs_stage_last_step_one_launch(const hs_stage_t *stage);
+
 /*
  * Diagnosis of the one-launch step's ways out, as hs_op_wait_probe is of the other kernels' waits.  Until the next call the
  * one-launch steps of the stage

@@ -31,7 +31,8 @@ EXPORTS = ("hs_status_str", "hs_kv_pool_bytes", "hs_workspace_bytes", "hs_stage_
            "hs_stage_set_qkv_bias", "hs_stage_set_modulation", "hs_stage_saturation_count", "hs_op_wait_probe",
            "hs_op_decode_attention_noalloc_status", "hs_stage_plan_attention", "hs_op_gemm_split_begin",
            "hs_op_gemm_part_splits", "hs_stage_plan_shares", "hs_op_gate_up_width", "hs_op_gate_up_tile", "hs_op_qkv_tile",
-           "hs_op_weight_streaming_rows", "hs_op_one_launch_step", "hs_stage_one_launch_fault")
+           "hs_op_weight_streaming_rows", "hs_op_one_launch_step", "hs_stage_one_launch_fault",
+           "hs_stage_last_step_one_launch")
 PROFILE_CLASSES = ("rmsnorm", "gemm_qkv", "attn_prefill", "attn_decode", "attn_combine", "gemm_out", "gemm_gateup",
                    "gemm_down")
 
@@ -126,6 +127,8 @@ def lib() -> C.CDLL:
         l.hs_op_qkv_tile.restype = C.c_int32
         l.hs_op_one_launch_step.argtypes = [C.c_int32] * 8
         l.hs_op_one_launch_step.restype = C.c_int32
+        l.hs_stage_last_step_one_launch.argtypes = [C.c_void_p]
+        l.hs_stage_last_step_one_launch.restype = C.c_int32
         l.hs_stage_one_launch_fault.argtypes = [C.c_void_p, C.c_int32, C.c_uint64]
         l.hs_op_weight_streaming_rows.argtypes = [C.c_int32] * 4
         l.hs_op_weight_streaming_rows.restype = C.c_int32
@@ -301,6 +304,11 @@ def hs_op_qkv_tile(M: int, N: int, sm_budget: int) -> int:
 def hs_op_one_launch_step(rows: int, dims, sm_budget: int) -> int:
     return int(lib().hs_op_one_launch_step(rows, dims.d_model, dims.n_q_heads, dims.n_kv_heads, dims.head_dim, dims.d_ffn, dims.n_layers,
                                            sm_budget))
+
+
+def hs_stage_last_step_one_launch(stage: int) -> int:
+    """1: the last step was the one cooperative launch; 0: a chain of launches; -1: there was none."""
+    return int(lib().hs_stage_last_step_one_launch(C.c_void_p(stage)))
 
 
 HS_FAULT_NONE, HS_FAULT_REFUSED, HS_FAULT_MISSING, HS_FAULT_GAVE_UP = range(4)

@@ -258,6 +258,7 @@ struct hs_stage {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool ev_pending[kRing] = {};
   int ring_pos = 0;
+  int last_one_launch = -1;                   // hs_stage_last_step_one_launch
   int one_launch_fault = HS_FAULT_NONE;       // hs_stage_one_launch_fault
   uint64_t one_launch_limit_ns = 0;
   // optional per-kernel timing
@@ -790,6 +791,7 @@ static hs_status_t enqueue_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_b
     a.smid_log = slots(2);       // prefill in class 2, decode in class 3 (the next slots)
     return a;
   };
+  s->last_one_launch = 0;
   if (whole) {
     SmallStepParams k{};
     k.tm_kv_page = s->tm_kv_page;
@@ -815,6 +817,7 @@ static hs_status_t enqueue_step(hs_stage_t* s, const hs_batch_t* b, int32_t sm_b
     k.status = status;
     k.wait_limit_ns = s->one_launch_fault == HS_FAULT_NONE ? 0 : s->one_launch_limit_ns;
     e = s->one_launch_fault == HS_FAULT_REFUSED ? cudaErrorCooperativeLaunchTooLarge : launch_small_step(k, sm_budget, stream);
+    s->last_one_launch = e == cudaSuccess ? 1 : 0;
     if (e == cudaSuccess) return HS_OK;
     // a context that does not hold so many blocks at once takes the separate launches
     if ((e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) || s->one_launch_fault > HS_FAULT_REFUSED) return cuda_fail("small step", e);
@@ -1083,6 +1086,8 @@ hs_status_t hs_stage_profile_read(hs_stage_t* s, float* ms, int32_t* launches) {
   s->timed.clear();
   return st;
 }
+
+int32_t hs_stage_last_step_one_launch(const hs_stage_t* s) { return s ? s->last_one_launch : -1; }
 
 hs_status_t hs_stage_one_launch_fault(hs_stage_t* s, int32_t fault, uint64_t limit_ns) {
   if (!s || fault < HS_FAULT_NONE || fault > HS_FAULT_GAVE_UP) return HS_ERR_INVALID_ARG;
