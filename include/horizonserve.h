@@ -193,7 +193,10 @@ hs_status_t hs_stage_plan(hs_stage_t *stage, const hs_batch_t *batch, int32_t *t
  * previous one has left, so that no block of the step ever sits on an SM outside the budget; with sm_budget == SM
  * count (no co-running neighbour) each kernel's set-up overlaps the previous kernel's drain.  A decode-only step of at most
  * 16 rows of a narrow stage (hs_op_one_launch_step) is one cooperative launch instead, which starts when as many SMs as it has
- * blocks (at most 120) are free together; a context that cannot hold them gets the separate launches.  With both prefill and
+ * blocks (at most 120) are free together; a context that cannot hold them gets the separate launches.  So beside a stage whose budget
+ * overlaps its own it finds its place between two of that stage's kernels, once for the whole step; but one-launch steps of two
+ * stages whose blocks the device does not hold together run one after the other: give stages that run beside each other
+ * budgets that add up to the device.  With both prefill and
  * decode work in a step the two attention kernels of a layer run side by side on two shares of the budget, the decode kernel on
  * a stream of the stage's own that is forked from and joined to cuda_stream by events.
  * The call returns when the step is enqueued.  Five steps of a stage may be on their way at a time: the sixth call waits on the host

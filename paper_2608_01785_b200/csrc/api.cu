@@ -1276,7 +1276,7 @@ hs_status_t hs_head_step(hs_head_t* h, const float* y, const int32_t* rows, int3
   np.sm_count = h->sm_count;
   np.status = status;
   // The norm reads the gains in front of its wait, and what is in front of it is the caller's: an update of the gains in
-  // place has to be behind it.  (In a stage step the copy of the metadata stands between; the vocabulary GEMM is behind a
+  // place has to be behind it.  (In a stage step the kernel that fetches the metadata stands between; the vocabulary GEMM is behind a
   // norm all of whose blocks have waited.)
   const int overlap = sm_budget == h->sm_count ? kOverlapEarly : kOverlapLate;
   np.overlap = overlap == kOverlapEarly ? kOverlapFirst : kOverlapNone;

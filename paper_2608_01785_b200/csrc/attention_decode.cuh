@@ -224,7 +224,8 @@ struct HeadsAsRows {
 // 2 i + 8 and 2 i + 9 of a page in one lane, page after page, then the four lanes.  Lanes 8 i .. 8 i + 3 do that for their even head,
 // lanes 8 i + 4 .. 8 i + 7 for the odd one; they give each other what they lack.
 // Steps, us: eleven rows of the talker on 52 SMs 368 -> 364, 16 on 148 260.2 -> 259.6; at 7B dimensions 29 rows on 96 SMs 642 -> 639, 64
-// rows 4801 -> 4787.
+// rows 4801 -> 4787.  (Of that the order of the weights takes back 0 to 0.2 %: against eight lanes that add two keys each, 64 rows
+// 4622.8 -> 4628.3, 29 rows on 96 SMs 633.3 -> 634.1, sixteen of the talker 260.2 -> 260.2.)
 template <int DH>
 struct HeadsAsColumns {
   uint32_t qf[DH / 16][2];
@@ -524,7 +525,7 @@ __device__ __forceinline__ void attn_decode_body(const AttnParams& p, uint8_t* s
   // A warp's first item is its own index in the grid (no round trip to the queue head before the first page request);
   // the queue hands out the items after those.  The first item's record, its page ids and those of its first pages
   // that lie wholly inside the cached context are fetched before the wait for the previous kernel: the step's
-  // metadata was copied before any kernel of the step started, and this step writes K / V at positions >= ctx only.
+  // metadata is there since two launches at least (see launch_fetch_metadata), and this step writes K / V at positions >= ctx only.
   int item = block * DC_WARPS + warp;
   int4 it = make_int4(0, 0, 0, 0), dr = it;
   int my_page = 0, ahead = 0;             // ahead: pages of the current item already requested

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_skinny_kernel(const Skinny
     first_b();
   }
   // This thread's part of the epilogue -- its row, and in Resid mode 2 Q consecutive columns, else Q columns of the first
-  // half and their partners -- and what it needs from the step's metadata (written before the step's first kernel).
+  // half and their partners -- and what it needs from the step's metadata (there since two launches at least, see launch_fetch_metadata).
   constexpr int Q = MT == 1 && P <= 4 ? 2 : 4, TPR = 16 * P / (2 * Q);  // threads of a row
   static_assert(MT * 16 * TPR <= SK_THREADS, "one epilogue task per thread");
   const int e_row = threadIdx.x / TPR, e_q = threadIdx.x - e_row * TPR;

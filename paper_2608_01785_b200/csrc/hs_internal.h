@@ -46,8 +46,8 @@ class PageAllocator {
 };
 
 // --------------------------------------------------------- step metadata --
-// Offsets (in int32 units) of the arrays inside the per-step metadata block that is copied to the
-// device once per step.  Fixed at stage creation from the configuration's maxima.
+// Offsets (in int32 units) of the arrays inside the per-step metadata block that the device
+// fetches once per step.  Fixed at stage creation from the configuration's maxima.
 struct MetaLayout {
   int tok_pos, tok_slot, tok_seq;    // [max_tokens]      absolute position / cache slot / sequence index of each new token
   int seq_tok0, seq_ctx, seq_qlen;   // [max_seqs]        first token row, cached tokens, new tokens

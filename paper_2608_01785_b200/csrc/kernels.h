@@ -193,7 +193,11 @@ cudaError_t launch_gemm_skinny(const SkinnyParams& p, int sm_budget, cudaStream_
 cudaError_t gemm_skinny_set_attributes();
 constexpr int kGemmTurnWords = 8192;   // capacity of the whose-turn array: splits are used only when tiles * 8 fits
 
-// The step's metadata from pinned host memory (a multiple of four words, 16-byte aligned).
+// The step's metadata from pinned host memory (a multiple of four words, 16-byte aligned), as the step's first launch.
+// The kernels of a step may read work lists, positions and slots in front of their own wait for the kernel before them, which this
+// launch allows to all but the kernel directly behind it: that one may be running while the block is written.  So (1) the kernel
+// behind it, the first RMSNorm or the one-launch step, touches no metadata before it has waited, and (2) like every kernel of a step it
+// lets its successor go behind that wait only, when the block is complete.
 cudaError_t launch_fetch_metadata(const void* host, void* dev, int words, int overlap, int sm_budget, cudaStream_t stream);
 cudaError_t metadata_set_attributes();
 
@@ -251,6 +255,8 @@ bool small_step_supports(int T, int d, int q_dim, int kv_dim, int F, int head_di
 // Where it is the faster form.  Up to eight rows at every budget tried (2 .. 148 SMs).  With more, a block's load of the rows is
 // what a phase waits for, which wide rows and few blocks lengthen: 13 rows, d_model 2048, on 148 SMs 229 -> 255 us; the talker's 13 on
 // 28 / 8 / 2 540 -> 507, 1325 -> 1379, 4524 -> 5031; d_model 768 on 148 / 52 / 28 162 -> 161, 204 -> 187, 297 -> 273; 512 on 28 201 -> 209.
+// 75 steps drawn over the sizes that it takes (d_model 256 .. 2048, q_dim 256 .. 2048, d_ffn 256 .. 3072, 4 .. 12 layers, 1 .. 16 rows of up to 4000
+// keys, 2 .. 148 SMs; the chain where this says so): 1.00 to 1.7 times as fast as the chain with a copied block of metadata, 1.29 on average.
 // The results are the same bits, so the choice may look at the budget.
 bool small_step_wins(int T, int d, int q_dim, int sm_budget);
 cudaError_t launch_small_step(const SmallStepParams& p, int sm_budget, cudaStream_t stream);

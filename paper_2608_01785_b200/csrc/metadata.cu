@@ -13,7 +13,7 @@ constexpr int META_THREADS = 256, META_AHEAD = 8;      // 16-byte groups that a 
 // thread 31.8 / 36.9 / 57.6 / 152.3, with eight 31.9 / 37.0 / 48.3 / 110.7; 1 MB 54.3 / 60.2 / 72.4 / 126.6, 50.8 / 61.5 / 145.8 / 498.9, 47.7 /
 // 54.3 / 68.4 / 172.7.
 // (The kernel behind is let go after the wait too: it reads weights ahead of its own, and what is in front of a step may be
-// writing them.)  A copy by the copy engine costs two changes between engine and SMs: from the end of one step to the end of the
+// writing them.  It is let go before the block is written: see launch_fetch_metadata for what that asks of it.)  A copy by the copy engine costs two changes between engine and SMs: from the end of one step to the end of the
 // next one's first RMSNorm 21 us (denoising) and 19 (nine decode rows at 7B dimensions), with this kernel behind the step in front
 // 13.5 and 11.3, ahead of its end 7.9 and 5.7.
 __global__ void __launch_bounds__(META_THREADS, 1) fetch_metadata_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n, int overlap) {

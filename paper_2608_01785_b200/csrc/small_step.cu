@@ -20,10 +20,10 @@
 // same order; the attention is the group mode of attention_decode.cuh, slice by slice.  So the bits are those of the separate
 // launches, whatever the grid.  The new token's key and value come from the exchange buffer too: its page is fetched as it
 // stands and the row put in place in shared memory.
-// Measured on B200, talker step, separate launches -> this, on 148 / 96 / 52 / 28 SMs: one row 245 -> 207, 295 -> 207, 339 -> 240,
-// 484 -> 317 us; eight 262 -> 222, 313 -> 222, 354 -> 273, 529 -> 369; eleven 297 -> 278, 342 -> 288, 384 -> 371, 594 -> 556; sixteen
-// 277 -> 267, 326 -> 285, 411 -> 406, 602 -> 572.  With a kernel that fetches the metadata and the heads as columns: one row 183, sixteen
-// 263, eleven on 52 SMs 363.
+// Measured on B200, talker step, rows of 128 .. 1024 cached tokens (eleven: .. 1500), separate launches behind a copy of the metadata -> this
+// behind the kernel that fetches it, on 148 / 96 / 52 / 28 SMs: one row 223 -> 174, 270 -> 174, 316 -> 210, 461 -> 288 us; eight 258 -> 206,
+// 309 -> 208, 350 -> 260, 536 -> 374; eleven 297 -> 280, 344 -> 281, 384 -> 371, 595 -> 575; sixteen 281 -> 260, 326 -> 266, 411 -> 399,
+// 609 -> 590.
 #include "attention_decode.cuh"
 #include "hs_internal.h"
 #include "weight_stream.cuh"
@@ -62,7 +62,7 @@ __device__ __forceinline__ void load_below(uint32_t& v, const void* at, int i, i
   asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %2, %3;\n\t@p ld.relaxed.gpu.global.u32 %0, [%1];\n\t}\n"
                : "+r"(v) : "l"(at), "r"(i), "r"(n) : "memory");
 }
-__device__ __forceinline__ uint32_t load_words(const void* at, uint32_t) {
+__device__ __forceinline__ uint32_t load_word(const void* at) {
   uint32_t v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(at) : "memory");
   return v;
@@ -105,7 +105,7 @@ __device__ __forceinline__ void watch(uint64_t* done, volatile int* progress, vo
     const unsigned long long now = globaltimer_ns();
     if (at != seen) { seen = at; t0 = now; }
     const bool late = now - t0 > limit_ns;
-    if (late || load_words(all_gave_up, 0u) != 0) {
+    if (late || load_word(all_gave_up) != 0) {
       if (late) {
         atomicExch(status, kErrTimeout);
         put1(all_gave_up, 1u);
